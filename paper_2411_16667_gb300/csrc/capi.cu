@@ -759,7 +759,8 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
     if (e2 != cudaSuccess) return cuda_fail(e2, "batch status copy");
     if (e3 != cudaSuccess) return cuda_fail(e3, "multi-query kernel");
   }
-  if (hM2.error) return fail((int)hM2.error, "multi-query kernel stopped with error %u", hM2.error);
+  if (hM2.bar.error)
+    return fail((int)hM2.bar.error, "multi-query kernel stopped with error %u", hM2.bar.error);
   const bool paths = !(o.flags & OPMOS_FLAG_NO_PATHS);
   const uint64_t total_ns = (uint64_t)std::chrono::duration_cast<std::chrono::nanoseconds>(
                                 std::chrono::steady_clock::now() - t0).count();

@@ -27,7 +27,8 @@ struct MQuery {    // a queued query
 };
 
 struct MCtl {      // grid-wide control of the multi-query kernel
-  unsigned bar_count, bar_gen, error, done;
+  BarWord bar;  // the grid barrier
+  unsigned done, pad;
   unsigned q_next, iter, qcap, hold;  // hold: keep slots until the host releases them
 };
 

@@ -2262,33 +2262,12 @@ struct SubTeam {
   __device__ __forceinline__ bool leader() const { return j == 0 && threadIdx.x == 0; }
 };
 
-__device__ inline bool mq_barrier(MCtl* M) {
+__device__ inline bool mq_barrier(MCtl* M, unsigned& target) {
   __shared__ unsigned s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned gen = ld_volatile(&M->bar_gen);
-    __threadfence();
-    const unsigned arrived = atomicAdd(&M->bar_count, 1u);
-    if (arrived == gridDim.x - 1) {
-      atomicExch(&M->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&M->bar_gen, 1u);
-    } else {
-      const unsigned long long t0 = globaltimer();
-      unsigned spins = 0;
-      while (ld_volatile(&M->bar_gen) == gen) {
-        if (++spins > 64) __nanosleep(64);
-        if ((spins & 255u) == 0) {
-          if (ld_volatile(&M->error) != 0) break;
-          if (globaltimer() - t0 > kBarrierTimeoutNs) {
-            atomicCAS(&M->error, 0u, (unsigned)OPMOS_ERR_TIMEOUT);
-            break;
-          }
-        }
-      }
-    }
-    __threadfence();
-    s_ok = ld_volatile(&M->error) == 0;
+    target += gridDim.x;
+    s_ok = grid_barrier(&M->bar, target) == 0u;
   }
   __syncthreads();
   return s_ok != 0;
@@ -2524,12 +2503,13 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
                  const GraphDev* graphs, QResult* results, unsigned* done_flags, MCtl* M) {
   __shared__ Shared S;
   __shared__ unsigned s_pref[kMaxSlots + 1];
+  unsigned target = 0;
   for (;;) {
     if (blockIdx.x == 0) mq_schedule<D>(slots, ctls, nslots, queue, hctl, graphs, M, results, done_flags);
-    if (!mq_barrier(M)) return;
+    if (!mq_barrier(M, target)) return;
     if (ld_volatile(&M->done)) return;
     mq_phase<D>(slots, ctls, nslots, S, s_pref);
-    if (!mq_barrier(M)) return;
+    if (!mq_barrier(M, target)) return;
   }
 }
 
