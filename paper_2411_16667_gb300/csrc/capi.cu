@@ -223,7 +223,7 @@ int plan_arena(const opmos_graph* g, uint32_t D, uint32_t window, size_t budget,
   pl->plog_cap = batch ? (1u << 16) : (1u << 20);
   const size_t ptiles = pl->plog_cap / 32 + 1;
   // per node: fbase, fcount, fcap, then per candidate set ncand, list heads, heavy flag,
-  // part count, slots; per candidate (two sets): node, parent, arc, list link, two touched
+  // part count, slots; per candidate (two sets): parent, arc, list link, two touched
   // entries, part count, flag, cost vector; the parts of split merges (two sets)
   pl->lsub = batch ? kLSubBatch : kLSubGrid;
   pl->nslots = kNodeSlots;
@@ -235,7 +235,7 @@ int plan_arena(const opmos_graph* g, uint32_t D, uint32_t window, size_t budget,
     pl->xcap = kPartsMax * (uint32_t)std::min<size_t>(n + 1, pl->cand_cap);
   }
   size_t fixed = (n + 1) * (8 + 4 + 4 + 2 * (4 + (4u << pl->lsub) + 4 + 4 + 4 * (size_t)pl->nslots)) + 3 * kNB * 4 +
-                 2 * (size_t)pl->cand_cap * (32 + 4 * D) + 2 * (size_t)pl->xcap * 4 + (size_t)pl->plog_cap * 4 * D +
+                 2 * (size_t)pl->cand_cap * (28 + 4 * D) + 2 * (size_t)pl->xcap * 4 + (size_t)pl->plog_cap * 4 * D +
                  2 * ((size_t)pl->plog_cap + ptiles) * 4 * D + kPSMax * 4 + 96 * 256;
   pl->fixed = fixed;
   if (budget < fixed + (8u << 20))
@@ -268,7 +268,6 @@ void layout_arena(const opmos_graph* g, uint32_t D, const ArenaPlan& pl, char* b
     cs.xpart = carve<uint32_t>(p, std::max<uint32_t>(pl.xcap, 1));
     cs.cflag = carve<uint32_t>(p, pl.cand_cap);
     cs.cslot = carve<int32_t>(p, n * pl.nslots);
-    cs.cnode = carve<uint32_t>(p, pl.cand_cap);
     cs.cparent = carve<uint32_t>(p, pl.cand_cap);
     cs.cedge = carve<uint32_t>(p, pl.cand_cap);
     cs.cnext = carve<int32_t>(p, pl.cand_cap);

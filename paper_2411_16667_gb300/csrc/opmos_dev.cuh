@@ -34,7 +34,7 @@ constexpr uint32_t kAlive = 0xFFFFFFFFu;  // ldead of a label that has not been 
 constexpr int32_t kNil = -1;
 constexpr int kNB = 4096;    // histogram bins of one OPEN array (the last one collects the rest)
 constexpr int kSub = 256;    // F[1] cells per F[0] bucket; a bin is 2^s2 consecutive cells
-constexpr unsigned kChunk = 32;       // OPEN entries per extraction work item
+constexpr unsigned kChunk = 32;       // most OPEN entries per extraction work item
 constexpr unsigned kRankQ = 1024;     // P entries per rank work item of an index rebuild
 constexpr unsigned kPSMax = 32768;    // largest P indexed by the sorted snapshot
 // candidates x frontier entries from which a node's merge takes a whole block:
@@ -210,7 +210,6 @@ struct CandSet {
   uint32_t* hsplit;    // cand_cap: parts the h-th heavy node's merge is split into (1: not split)
   uint32_t* xpart;     // parts of split merges, h << 4 | part (kPartsMax per heavy node at most)
   uint32_t* cflag;     // cand_cap: candidate dropped by a part of a split merge
-  uint32_t* cnode;
   uint32_t* cparent;
   uint32_t* cedge;
   int32_t* cnext;
@@ -389,6 +388,8 @@ struct GridTeam {
   __device__ __forceinline__ unsigned nthreads() const { return gridDim.x * blockDim.x; }
   __device__ __forceinline__ unsigned wid() const { return tid() >> 5; }
   __device__ __forceinline__ unsigned nwarps() const { return nthreads() >> 5; }
+  __device__ __forceinline__ unsigned block() const { return blockIdx.x; }
+  __device__ __forceinline__ unsigned nblocks() const { return gridDim.x; }
   __device__ __forceinline__ bool leader_block() const { return blockIdx.x == 0; }
   __device__ __forceinline__ bool leader() const { return blockIdx.x == 0 && threadIdx.x == 0; }
   // Returns false when the query has an error set; the decision is read once

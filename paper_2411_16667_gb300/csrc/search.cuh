@@ -30,6 +30,7 @@ struct MCtl {      // grid-wide control of the multi-query kernel
   BarWord bar;  // the grid barrier
   unsigned done, pad;
   unsigned q_next, iter, qcap, hold;  // hold: keep slots until the host releases them
+  unsigned pref[kMaxSlots + 1];       // virtual blocks of the iteration: prefix sums over the slots
 };
 
 // Host control words (host-mapped memory when serving): [0] queries queued

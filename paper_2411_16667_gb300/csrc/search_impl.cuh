@@ -68,22 +68,14 @@
 namespace opmos {
 namespace detail {
 
-__device__ __forceinline__ unsigned warp_min(unsigned x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = min(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
+__device__ __forceinline__ unsigned warp_min(unsigned x) { return __reduce_min_sync(0xffffffffu, x); }
 
-__device__ __forceinline__ unsigned warp_max(unsigned x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
+__device__ __forceinline__ unsigned warp_max(unsigned x) { return __reduce_max_sync(0xffffffffu, x); }
 
 __device__ __forceinline__ unsigned long long warp_min64(unsigned long long x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = min(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
+  const unsigned hi = warp_min((unsigned)(x >> 32));
+  const unsigned lo = warp_min((unsigned)(x >> 32) == hi ? (unsigned)x : 0xffffffffu);
+  return (unsigned long long)hi << 32 | lo;
 }
 
 __device__ __forceinline__ void flush_stats(QCtl* C, unsigned long long (&st)[kNStat]) {
@@ -133,7 +125,11 @@ struct Shared {
   unsigned warp[33];
   unsigned f_min, b1_max, bstar;
   unsigned pmax[3];
-  unsigned claim;
+  unsigned claim[2];
+  // what this block's extraction items found (next bins), added to the global
+  // record once a step
+  unsigned long long min_key;
+  unsigned win_min, win_max, f1lo, f1hi;
   PIdx pd;             // the P index as this step sees it
   // the candidates of a block-merged node (up to kHC at a time)
   uint32_t hc[OPMOS_MAX_D][kHC];
@@ -158,7 +154,8 @@ struct BinParams {
 };
 __device__ __forceinline__ unsigned bin_of(uint64_t key, const BinParams& bp) {
   const uint32_t F0 = (uint32_t)(key >> 32), F1 = (uint32_t)key;
-  const uint64_t q = F0 > bp.b0 ? (F0 - bp.b0) / bp.delta : 0u;
+  const uint32_t f = F0 > bp.b0 ? F0 - bp.b0 : 0u;
+  const uint64_t q = bp.delta == 1u ? f : f / bp.delta;
   const uint32_t x = F1 > bp.b1 ? min((F1 - bp.b1) >> bp.s1, (unsigned)kSub - 1) : 0u;
   return (unsigned)min((q * kSub + x) >> bp.s2, (uint64_t)(kNB - 1));
 }
@@ -390,21 +387,33 @@ struct Search {
   // range of the entries carried into OPEN_i in 256 cells. Cells per bin: the
   // bins cover the F[0] buckets from the origin to window i's largest F[0]
   // and three times window i's F[0] extent beyond.
-  __device__ BinParams next_bins(const CycleCtl& K) const {
-    const unsigned long long mk = ld_volatile64(&K.min_key.v);
-    const unsigned lo = ld_volatile(&K.f1lo.v), hi = ld_volatile(&K.f1hi.v);
+  struct Measured {
+    unsigned long long min_key;
+    unsigned f1lo, f1hi, wmin, wprev, wmax;
+  };
+  __device__ __forceinline__ Measured measured(const CycleCtl& K) const {
+    return Measured{ld_volatile64(&K.min_key.v), ld_volatile(&K.f1lo.v),      ld_volatile(&K.f1hi.v),
+                    ld_volatile(&K.win_min.v),   ld_volatile(&K.win_min_prev), ld_volatile(&K.win_max.v)};
+  }
+  __device__ BinParams next_bins(const Measured& m) const {
     BinParams b;
-    b.b0 = min(min((uint32_t)(mk >> 32), ld_volatile(&K.win_min.v)), ld_volatile(&K.win_min_prev));
+    b.b0 = min(min((uint32_t)(m.min_key >> 32), m.wmin), m.wprev);
     if (b.b0 == kInf) b.b0 = 0;
-    b.b1 = lo <= hi ? lo : (mk != ~0ull ? (uint32_t)mk : 0u);
-    const unsigned span = lo <= hi ? hi - lo : 0u;
-    b.s1 = 0;
-    while ((span >> b.s1) >= (unsigned)kSub) ++b.s1;
+    b.b1 = m.f1lo <= m.f1hi ? m.f1lo : (m.min_key != ~0ull ? (uint32_t)m.min_key : 0u);
+    const unsigned span = m.f1lo <= m.f1hi ? m.f1hi - m.f1lo : 0u;
+    constexpr int kSubBits = 8;
+    static_assert(kSub == 1 << kSubBits, "cells per bucket");
+    b.s1 = (unsigned)max(0, 32 - kSubBits - __clz((int)span));  // the smallest with span >> s1 < kSub
     b.delta = P.delta;
-    const uint32_t wmax = ld_volatile(&K.win_max.v), wmin = min(ld_volatile(&K.win_min.v), wmax);
-    const uint64_t rows = (wmax > b.b0 ? (wmax - b.b0) / b.delta : 0u) + 1 + 3ull * ((wmax - wmin) / b.delta + 1);
+    const uint32_t wmin = min(m.wmin, m.wmax);
+    uint32_t q0 = m.wmax > b.b0 ? m.wmax - b.b0 : 0u, q1 = m.wmax - wmin;
+    if (b.delta != 1u) {
+      q0 /= b.delta;
+      q1 /= b.delta;
+    }
+    const uint64_t rows = (uint64_t)q0 + 1 + 3ull * ((uint64_t)q1 + 1);
     b.s2 = 0;
-    while (b.s2 < 30 && ((uint64_t)(kNB - 1) << b.s2) / kSub < rows) ++b.s2;
+    while (b.s2 < 30 && ((uint64_t)(kNB - 1) << b.s2) >> kSubBits < rows) ++b.s2;
     return b;
   }
 
@@ -415,22 +424,32 @@ struct Search {
   }
 
   // ---------------- expansion (Algorithm 1) ----------------
-  __device__ __forceinline__ void add_candidate(const CandSet& cs, CycleCtl& K1, uint32_t v2, uint32_t parent,
-                                                uint32_t e, const uint32_t (&g2)[D]) {
-    const unsigned c = agg_inc(&K1.cand_count.v);
-    cs.cnode[c] = v2;
-    cs.cparent[c] = parent;
-    cs.cedge[c] = e;
-    cs.cflag[c] = 0u;
+  // The candidates of one round of the whole warp (lane's candidate when
+  // alive: target v2, parent, arc e, costs g2; fc = fcount[v2]). The two
+  // returning atomics a candidate needs -- its record and its rank at the
+  // node -- are in flight together.
+  __device__ __forceinline__ void add_candidates(const CandSet& cs, CycleCtl& K1, bool alive, uint32_t v2,
+                                                 uint32_t parent, uint32_t e, const uint32_t (&g2)[D], unsigned fc) {
+    const unsigned am = __ballot_sync(0xffffffffu, alive);
+    if (!am) return;
+    const unsigned lead = __ffs(am) - 1;
+    unsigned c = 0, pos = 0;
+    if (lane_id() == lead) c = atomicAdd(&K1.cand_count.v, __popc(am));
+    if (alive) pos = atomicAdd(&cs.ncand[v2], 1u);
+    c = __shfl_sync(0xffffffffu, c, lead) + __popc(am & lanemask_lt());
+    if (alive) {
+      cs.cparent[c] = parent;
+      cs.cedge[c] = e;
+      cs.cflag[c] = 0u;
 #pragma unroll
-    for (int k = 0; k < D; ++k) cs.cg[(size_t)k * A.cand_cap + c] = g2[k];
-    const unsigned pos = atomicAdd(&cs.ncand[v2], 1u);
-    if (pos < A.nslots) {
-      cs.cslot[(size_t)v2 * A.nslots + pos] = (int)c;
-    } else {  // list (pos - nslots) mod 2^lsub of the node, so all its lists grow evenly
-      const unsigned j = (pos - A.nslots) & ((1u << A.lsub) - 1u);
-      cs.cnext[c] = atomicExch(&cs.node_head[((size_t)v2 << A.lsub) + j], (int)c);
-      st[S_OVF]++;
+      for (int k = 0; k < D; ++k) cs.cg[(size_t)k * A.cand_cap + c] = g2[k];
+      if (pos < A.nslots) {
+        cs.cslot[(size_t)v2 * A.nslots + pos] = (int)c;
+      } else {  // list (pos - nslots) mod 2^lsub of the node, so all its lists grow evenly
+        const unsigned j = (pos - A.nslots) & ((1u << A.lsub) - 1u);
+        cs.cnext[c] = atomicExch(&cs.node_head[((size_t)v2 << A.lsub) + j], (int)c);
+        st[S_OVF]++;
+      }
     }
     // Every node is listed among the light ones (one warp each) on its
     // first candidate. A node with a large frontier, or reached by many
@@ -438,20 +457,28 @@ struct Search {
     // (hflag decides; the array holds 2 * cand_cap entries) and merged by
     // whole blocks; its light item then only clears hflag. Only light items
     // touch hflag during the merge, so a block merge never races a warp.
-    if (pos == 0) cs.touched[agg_inc(&K1.touched_count.v)] = v2;
+    const unsigned fm = __ballot_sync(0xffffffffu, alive && pos == 0);
+    if (fm) {
+      const unsigned l0 = __ffs(fm) - 1;
+      unsigned t = 0;
+      if (lane_id() == l0) t = atomicAdd(&K1.touched_count.v, __popc(fm));
+      t = __shfl_sync(0xffffffffu, t, l0) + __popc(fm & lanemask_lt());
+      if (alive && pos == 0) cs.touched[t] = v2;
+    }
     // A node is merged by a whole block once its candidates x frontier
     // entries reach P.heavy_work (checked at 1, 4, 8 and 16 candidates: the
     // work of a one-warp merge grows with that product; at the goal node n,
     // with candidates x P), and always past kHeavyCands candidates (a warp
     // would take them in two batches).
-    const unsigned nc = pos + 1u;
-    const bool list = pos == kHeavyCands ||
-                      ((nc == 1u || nc == 4u || nc == 8u || nc == 16u) &&
-                       (unsigned long long)nc * A.fcount[v2] >= P.heavy_work);
-    // at 64, 128, 256, ... candidates the merge may be split further
-    const bool grow = A.kparts > 1u && pos > kHeavyCands && ((pos + 1u) & pos) == 0u;
-    // (the P test of a goal candidate skips most of P through the index tiles)
-    if (list || grow) heavy_list(cs, K1, v2, parts_for(pos + 1u, A.fcount[v2] >> (v2 == G.n ? 3 : 0)), list);
+    if (alive) {
+      const unsigned nc = pos + 1u;
+      const bool list = pos == kHeavyCands || ((nc == 1u || nc == 4u || nc == 8u || nc == 16u) &&
+                                               (unsigned long long)nc * fc >= P.heavy_work);
+      // at 64, 128, 256, ... candidates the merge may be split further
+      const bool grow = A.kparts > 1u && pos > kHeavyCands && ((pos + 1u) & pos) == 0u;
+      // (the P test of a goal candidate skips most of P through the index tiles)
+      if (list || grow) heavy_list(cs, K1, v2, parts_for(pos + 1u, fc >> (v2 == G.n ? 3 : 0)), list);
+    }
   }
 
   // Parts a block merge of nc candidates against F frontier entries is split
@@ -503,48 +530,113 @@ struct Search {
     }
   }
 
-  // Expansion of up to 32 / L window labels, one per lane group of L lanes
-  // (has: the lane's group holds label lid), one round of out-arcs at a time
-  // with every lane of the warp taking part: g' = g + c(e), dropped when h(v')
-  // is infinite (Algorithm 1). A goal label is not expanded (Algorithm 1); it
-  // becomes a candidate at the virtual node n.
-  __device__ void expand_labels(uint32_t lid, bool has, unsigned gl, unsigned L, const CandSet& cs, CycleCtl& K1,
-                                unsigned long long& pcmp) {
-    uint32_t v = 0, e0 = 0, e1 = 0;
+  // A window label as its lane holds it.
+  struct Label {
+    uint32_t id, v;
+    uint32_t e0, e1;  // its out-arcs
     uint32_t g[D];
+    unsigned since;   // P-log length at its last F-against-P test
+  };
+  // Everything extraction needs of label id, in two rounds of loads.
+  __device__ __forceinline__ Label load_label(bool want, uint32_t id) const {
+    Label l;
+    l.id = id;
+    l.v = l.e0 = l.e1 = 0;
+    l.since = kInf;
 #pragma unroll
-    for (int k = 0; k < D; ++k) g[k] = 0;
-    if (has) {
-      v = A.lnode[lid];
+    for (int k = 0; k < D; ++k) l.g[k] = 0;
+    if (want) {
+      l.v = A.lnode[id];
 #pragma unroll
-      for (int k = 0; k < D; ++k) g[k] = A.lg[(size_t)k * A.label_cap + lid];
+      for (int k = 0; k < D; ++k) l.g[k] = A.lg[(size_t)k * A.label_cap + id];
+      l.since = A.lpver[id];
+      l.e0 = __ldg(G.rowptr + l.v);
+      l.e1 = __ldg(G.rowptr + l.v + 1);
     }
-    const bool goal = has && v == P.goal;
-    if (goal && gl == 0) add_candidate(cs, K1, G.n, A.lparent[lid], A.ledge[lid], g);
-    if (has && !goal) {
-      e0 = __ldg(G.rowptr + v);
-      e1 = __ldg(G.rowptr + v + 1);
+    return l;
+  }
+  // Lazy PruneOPEN: F against the goal costs logged since the label's last
+  // check (through the P index when that check predates it).
+  __device__ __forceinline__ bool still_open(bool want, const Label& l, unsigned long long& pcmp) {
+    const unsigned since = warp_min(want ? l.since : kInf);
+    bool alive = want;
+    if (since < psnap) {
+      const PIdx& pd = S.pd;
+      uint32_t F[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) F[k] = want ? l.g[k] + hk(k, l.v) : 0u;
+      if (pd.count && since < pd.mark)
+        p_filter(alive, F, pd.mark, psnap, pd.count, pd.ntiles, pd.cur, pcmp);
+      else
+        p_filter(alive, F, since, psnap, 0, 0, 0, pcmp);
     }
-    const PIdx& pd = S.pd;
-    for (uint32_t r = 0;; r += L) {
-      const uint32_t e = e0 + gl + r;
-      const bool valid = has && !goal && e < e1;
-      if (!__any_sync(0xffffffffu, valid)) break;
-      uint32_t v2 = 0, g2[D];
-      bool alive = false;
-      if (valid) {
-        v2 = __ldg(G.col + e);
-        st[S_CAND]++;
-        alive = hk(0, v2) != kInf;  // else the goal is unreachable from v2
+    return alive;
+  }
+
+  // Expansion of the window labels the warp's lanes hold (take): 32 / L of
+  // them side by side, one per group of L lanes, one round of out-arcs at a
+  // time with every lane taking part: g' = g + c(e), dropped when h(v') is
+  // infinite (Algorithm 1). A goal label is not expanded (Algorithm 1); it
+  // becomes a candidate at the virtual node n. L is P.lanes, or more when the
+  // labels leave lane groups idle (one label on a node of degree 24: one round
+  // of 32 lanes instead of three of 8).
+  __device__ void expand_labels(bool take, const Label& own, const CandSet& cs, CycleCtl& K1) {
+    unsigned hits = __ballot_sync(0xffffffffu, take);
+    unsigned L = P.lanes;
+    while (L < 32u && __popc(hits) * L <= 16u) L <<= 1;
+    const unsigned lane = lane_id(), groups = 32u / L, grp = lane / L, gl = lane % L;
+    while (hits) {
+      const unsigned src = nth_bit(hits, grp);
+      const bool has = src < 32u;
+      const unsigned from = has ? src : 0u;
+      const uint32_t lid = __shfl_sync(0xffffffffu, own.id, from), v = __shfl_sync(0xffffffffu, own.v, from);
+      const uint32_t e0 = __shfl_sync(0xffffffffu, own.e0, from), e1 = __shfl_sync(0xffffffffu, own.e1, from);
+      uint32_t g[D];
+#pragma unroll
+      for (int k = 0; k < D; ++k) g[k] = __shfl_sync(0xffffffffu, own.g[k], from);
+      const bool goal = has && v == P.goal;
+      const unsigned deg = has ? (goal ? 1u : e1 - e0) : 0u;
+      const unsigned rounds = warp_max(deg);
+      for (unsigned r = 0; r < rounds; r += L) {
+        bool alive = gl + r < deg;
+        uint32_t v2 = G.n, par = lid, e = e0 + gl + r, g2[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) g2[k] = g[k];
+        unsigned fc = 0;
+        if (alive) {
+          if (goal) {
+            par = A.lparent[lid];
+            e = A.ledge[lid];
+          } else {
+            v2 = __ldg(G.col + e);
+#pragma unroll
+            for (int k = 0; k < D; ++k) g2[k] += ck(k, e);
+            st[S_CAND]++;
+          }
+          fc = A.fcount[v2];
+          if (!goal) alive = hk(0, v2) != kInf;  // else the goal is unreachable from v2
+        }
+        add_candidates(cs, K1, alive, v2, par, e, g2, fc);
       }
-#pragma unroll
-      for (int k = 0; k < D; ++k) g2[k] = alive ? g[k] + ck(k, e) : 0u;
-      if (alive) add_candidate(cs, K1, v2, lid, e, g2);
+      for (unsigned r = 0; r < groups && hits; ++r) hits &= hits - 1;
     }
   }
 
   // ---------------- extraction of window i+1 from OPEN_i ----------------
-  // One warp, the kChunk entries chunk, chunk + nchunks, chunk + 2 nchunks,
+  // Entries one work item (one warp) takes: as many labels as one round of
+  // the warp's lanes expands (an item of 32 labels is eight rounds of
+  // dependent loads and atomics one after the other: 10 us at 8 lanes a label
+  // and degree 8, 45 us at degree 24, while most of the warps had no item),
+  // more only when there are more entries than warps hold then.
+  // Measured: longest extraction item of a step 10 -> 3 us and step 22 -> 13 us
+  // (97x89 ship grid, d = 3), 17 -> 2.4 us and 34 -> 17 us (241-node route, d = 8).
+  __device__ __forceinline__ unsigned item_entries(unsigned n, unsigned nwarps) const {
+    unsigned per = 32u;
+    while (per > 1u && (32u / per) < G.maxdeg) per >>= 1;
+    return min(kChunk, max(per, (n + nwarps - 1) / nwarps));
+  }
+
+  // One warp, the `per` entries chunk, chunk + nchunks, chunk + 2 nchunks,
   // ... (a merge appends a node's new labels side by side and they tend to
   // fall in the same window, so strided chunks spread the window's labels
   // over the work items): dead entries are dropped (lazy OPEN delete), window
@@ -552,169 +644,110 @@ struct Search {
   // PruneOPEN), the other window entries are taken and expanded at once by
   // lane groups; every other entry is carried to OPEN_{i+1} and counted in
   // its histogram.
-  __device__ void extract_chunk(unsigned chunk, unsigned n_in, const BinParams& bp, CycleCtl& K1) {
+  __device__ void extract_chunk(unsigned chunk, unsigned n_in, unsigned per, const BinParams& bp, CycleCtl& K1) {
     const unsigned cur = cyc & 1u, nxt = cur ^ 1u;
-    const uint64_t* in = A.okey[cur];
-    const uint32_t* in_id = A.oid[cur];
-    uint64_t* out = A.okey[nxt];
-    uint32_t* out_id = A.oid[nxt];
     const CandSet& cs = A.cs[nxt];
-    const PIdx& pd = S.pd;
-    const unsigned bstar = S.bstar;
     const unsigned lane = lane_id();
-    const unsigned L = P.lanes, G_per = 32 / L, grp = lane / L, gl = lane % L;
-    unsigned long long kmin = ~0ull, pcmp = 0;
-    unsigned wmin = kInf, wmax = 0, f1lo = kInf, f1hi = 0;
-    const unsigned nchunks = (n_in + kChunk - 1) / kChunk;
-    for (unsigned r = 0; r < kChunk; r += 32) {
-      const unsigned i = chunk + (r + lane) * nchunks;
-      const bool valid = i < n_in;
-      uint64_t key = 0;
-      uint32_t id = 0;
-      bool keep = false, want = false;
-      if (valid) {
-        key = in[i];
-        id = in_id[i];
-        st[S_OSCAN]++;
-        if (dead_now(id))
-          st[S_DEAD]++;
-        else if (bin_of(key, bp) <= bstar)
-          want = true;
-        else
-          keep = true;
-      }
-      // lazy PruneOPEN: F against the goal costs logged since the label's
-      // last check (through the P index when that check predates it)
-      uint32_t F[D];
-      unsigned since = kInf;
-      if (want) {
-        const uint32_t v = A.lnode[id];
-#pragma unroll
-        for (int k = 0; k < D; ++k) F[k] = A.lg[(size_t)k * A.label_cap + id] + hk(k, v);
-        since = A.lpver[id];
+    const unsigned nchunks = (n_in + per - 1) / per;
+    const unsigned i = chunk + lane * nchunks;
+    const bool valid = lane < per && i < n_in;
+    uint64_t key = 0;
+    uint32_t id = 0;
+    unsigned dead = 0;
+    bool want = false, keep = false;
+    if (valid) {
+      key = A.okey[cur][i];
+      id = A.oid[cur][i];
+      dead = A.ldead[id];
+      want = bin_of(key, bp) <= S.bstar;
+      st[S_OSCAN]++;
+    }
+    const Label own = load_label(want, id);
+    if (valid) {
+      if (dead < cyc) {
+        st[S_DEAD]++;
+        want = false;
       } else {
-#pragma unroll
-        for (int k = 0; k < D; ++k) F[k] = 0;
+        keep = !want;
       }
-      since = warp_min(since);
-      bool alive = want;
-      if (since < psnap) {
-        if (pd.count && since < pd.mark)
-          p_filter(alive, F, pd.mark, psnap, pd.count, pd.ntiles, pd.cur, pcmp);
-        else
-          p_filter(alive, F, since, psnap, 0, 0, 0, pcmp);
+    }
+    unsigned long long pcmp = 0;
+    bool take = still_open(want, own, pcmp);
+    st[S_PCMP] += pcmp;
+    if (want && !take) st[S_GOALPRUNED]++;
+    if (n_in > A.win_cap && take) {  // else the window cannot be full
+      if (agg_inc(&K1.win_count.v) >= A.win_cap) {
+        take = false;
+        keep = true;  // window full: stays in OPEN for the next step
       }
-      bool take = false;
-      if (want && !alive) {
-        st[S_GOALPRUNED]++;
-      } else if (want) {
-        if (agg_inc(&K1.win_count.v) < A.win_cap) {
-          st[S_EXTRACTED]++;
-          take = true;
-          wmin = min(wmin, (uint32_t)(key >> 32));
-          wmax = max(wmax, (uint32_t)(key >> 32));
-        } else {
-          keep = true;  // window full: stays in OPEN for the next step
-        }
+    }
+    // places in the next OPEN are claimed before the expansion and used
+    // after it
+    const unsigned km = __ballot_sync(0xffffffffu, keep);
+    unsigned ob = 0;
+    if (km && lane == 0) ob = atomicAdd(&K1.open_count.v, __popc(km));
+    const unsigned tm = __ballot_sync(0xffffffffu, take);
+    if (tm) {
+      if (take) st[S_EXTRACTED]++;
+      const unsigned wmin = warp_min(take ? (unsigned)(key >> 32) : kInf);
+      const unsigned wmax = warp_max(take ? (unsigned)(key >> 32) : 0u);
+      if (lane == 0) {
+        atomicMin(&S.win_min, wmin);
+        atomicMax(&S.win_max, wmax);
       }
+      expand_labels(take, own, cs, K1);
+    }
+    if (km) {
+      const unsigned o = __shfl_sync(0xffffffffu, ob, 0) + __popc(km & lanemask_lt());
+      bool inbins = false;
       if (keep) {
-        const unsigned o = agg_inc(&K1.open_count.v);
         if (o < A.open_cap) {
-          out[o] = key;
-          out_id[o] = id;
+          A.okey[nxt][o] = key;
+          A.oid[nxt][o] = id;
           st[S_OKEEP]++;
-          kmin = min(kmin, (unsigned long long)key);
           const unsigned b = bin_of(key, bpn);
           atomicAdd(&S.hist[b], 1u);
-          if (b < (unsigned)kNB - 1) {
-            f1lo = min(f1lo, (uint32_t)key);
-            f1hi = max(f1hi, (uint32_t)key);
-          }
+          inbins = b < (unsigned)kNB - 1;
         } else {
           set_error(C, OPMOS_ERR_CAPACITY);
         }
       }
-      unsigned hits = __ballot_sync(0xffffffffu, take);
-      while (hits) {
-        const unsigned src = nth_bit(hits, grp);
-        const uint32_t lid = __shfl_sync(0xffffffffu, id, src < 32 ? src : 0);
-        expand_labels(lid, src < 32, gl, L, cs, K1, pcmp);
-        for (unsigned r = 0; r < G_per && hits; ++r) hits &= hits - 1;
-      }
-    }
-    st[S_PCMP] += pcmp;
-    kmin = warp_min64(kmin);
-    wmin = warp_min(wmin);
-    wmax = warp_max(wmax);
-    f1lo = warp_min(f1lo);
-    f1hi = warp_max(f1hi);
-    if (lane == 0) {
-      if (kmin != ~0ull) atomicMin(&K1.min_key.v, kmin);
-      if (wmin != kInf) {
-        atomicMin(&K1.win_min.v, wmin);
-        atomicMax(&K1.win_max.v, wmax);
-      }
-      if (f1lo != kInf) {
-        atomicMin(&K1.f1lo.v, f1lo);
-        atomicMax(&K1.f1hi.v, f1hi);
+      const unsigned long long kmin = warp_min64(keep ? key : ~0ull);
+      const unsigned f1lo = warp_min(inbins ? (uint32_t)key : kInf), f1hi = warp_max(inbins ? (uint32_t)key : 0u);
+      if (lane == 0) {
+        atomicMin(&S.min_key, kmin);
+        if (f1lo != kInf) {
+          atomicMin(&S.f1lo, f1lo);
+          atomicMax(&S.f1hi, f1hi);
+        }
       }
     }
   }
 
   // FIFO order (OPMOS_FLAG_FIFO): one warp takes the ring positions
-  // [p0, p1) of window i+1 -- the oldest entries -- and expands every one
-  // that is alive and not dominated by a logged solution on F. Nothing is
-  // carried: the rest of the ring stays where it is.
+  // [p0, p1) of window i+1 (at most 32) -- the oldest entries -- and expands
+  // every one that is alive and not dominated by a logged solution on F.
+  // Nothing is carried: the rest of the ring stays where it is.
   __device__ void extract_fifo(unsigned p0, unsigned p1, CycleCtl& K1) {
     const CandSet& cs = A.cs[(cyc & 1u) ^ 1u];
-    const PIdx& pd = S.pd;
-    const unsigned lane = lane_id();
-    const unsigned L = P.lanes, G_per = 32 / L, grp = lane / L, gl = lane % L;
-    unsigned long long pcmp = 0;
-    const unsigned pos = p0 + lane;
-    const bool valid = pos < p1;
+    const unsigned pos = p0 + lane_id();
     uint32_t id = 0;
-    bool want = false;
+    unsigned dead = 0;
+    const bool valid = pos < p1;
     if (valid) {
       id = A.oid[0][pos % A.open_cap];
+      dead = A.ldead[id];
       st[S_OSCAN]++;
-      if (dead_now(id))
-        st[S_DEAD]++;
-      else
-        want = true;
     }
-    uint32_t F[D];
-    unsigned since = kInf;
-    if (want) {
-      const uint32_t v = A.lnode[id];
-#pragma unroll
-      for (int k = 0; k < D; ++k) F[k] = A.lg[(size_t)k * A.label_cap + id] + hk(k, v);
-      since = A.lpver[id];
-    } else {
-#pragma unroll
-      for (int k = 0; k < D; ++k) F[k] = 0;
-    }
-    since = warp_min(since);
-    bool alive = want;
-    if (since < psnap) {
-      if (pd.count && since < pd.mark)
-        p_filter(alive, F, pd.mark, psnap, pd.count, pd.ntiles, pd.cur, pcmp);
-      else
-        p_filter(alive, F, since, psnap, 0, 0, 0, pcmp);
-    }
-    if (want && !alive) st[S_GOALPRUNED]++;
-    if (alive) {
-      st[S_EXTRACTED]++;
-      agg_inc(&K1.win_count.v);
-    }
-    unsigned hits = __ballot_sync(0xffffffffu, alive);
-    while (hits) {
-      const unsigned src = nth_bit(hits, grp);
-      const uint32_t lid = __shfl_sync(0xffffffffu, id, src < 32 ? src : 0);
-      expand_labels(lid, src < 32, gl, L, cs, K1, pcmp);
-      for (unsigned r = 0; r < G_per && hits; ++r) hits &= hits - 1;
-    }
+    const Label own = load_label(valid, id);
+    const bool want = valid && dead >= cyc;
+    if (valid && !want) st[S_DEAD]++;
+    unsigned long long pcmp = 0;
+    const bool take = still_open(want, own, pcmp);
     st[S_PCMP] += pcmp;
+    if (want && !take) st[S_GOALPRUNED]++;
+    if (take) st[S_EXTRACTED]++;
+    expand_labels(take, own, cs, K1);
   }
 
   // F against the P index + the logged goal costs log[t0, t1): clears alive
@@ -1013,7 +1046,7 @@ struct Search {
         }
         unsigned plen = 0;
         if (is_goal) {
-          plen = ld_volatile(&C->plog_len.v);
+          plen = __shfl_sync(0xffffffffu, ld_volatile(&C->plog_len.v), 0);  // read before lane 0 raises it
           if (plen + ns > A.plog_cap) {
             if (lane == 0) set_error(C, OPMOS_ERR_CAPACITY);
             return;
@@ -1365,7 +1398,8 @@ struct Search {
 #pragma unroll
             for (unsigned q = 0; q < NW; ++q) {
               if (q >= nwords) break;
-              unsigned am = S.halive[q] & ~S.hkill[q] & ~kill[q];
+              // one lane's view of the kills other warps add meanwhile
+              unsigned am = __shfl_sync(0xffffffffu, S.halive[q] & ~S.hkill[q] & ~kill[q], 0);
               fcmp += (unsigned long long)__popc(am) * min(32u, fc - i0);
               while (am) {
                 const unsigned j = __ffs(am) - 1;
@@ -1676,7 +1710,7 @@ struct Search {
         bool any = false;
 #pragma unroll
         for (unsigned q = 0; q < NW; ++q) any |= q < nwords && (S.halive[q] & ~S.hkill[q]) != 0u;
-        if (!any) break;
+        if (!__any_sync(0xffffffffu, any)) break;
         uint32_t m[U][D];
         uint32_t mid[U];
 #pragma unroll
@@ -1699,7 +1733,8 @@ struct Search {
 #pragma unroll
             for (unsigned q = 0; q < NW; ++q) {
               if (q >= nwords) break;
-              unsigned am = S.halive[q] & ~S.hkill[q] & ~kill[q];
+              // one lane's view of the kills other warps add meanwhile
+              unsigned am = __shfl_sync(0xffffffffu, S.halive[q] & ~S.hkill[q] & ~kill[q], 0);
               fcmp += (unsigned long long)__popc(am) * min(32u, hi - i0);
               while (am) {
                 const unsigned j = __ffs(am) - 1;
@@ -1874,6 +1909,31 @@ struct Search {
     if (threadIdx.x == 0) C->pidx[(i + 1) & 1u] = nd;
   }
 
+  // Block-merge item t of a step: a part of a split merge (t < np), or a
+  // heavy node's whole merge, skipped when it is split.
+  __device__ void heavy_item(unsigned t, unsigned np, unsigned cur, CycleCtl& K1, bool split) {
+    const unsigned x = t < np ? A.cs[cur].xpart[t] : (t - np) << 4;
+    const unsigned h = x >> 4, r = x & 15u;
+    const unsigned k = A.cs[cur].hsplit[h];
+    if (t >= np && k > 1u) return;
+    const uint32_t v = A.cs[cur].touched[2u * A.cand_cap - 1u - h];
+    if (threadIdx.x == 0 && r == 0) {  // read before the merge clears them
+      S.tmax[3] = max(S.tmax[3], A.cs[cur].ncand[v]);
+      S.tmax[4] = max(S.tmax[4], A.fcount[v]);
+    }
+    const unsigned long long t0 = globaltimer();
+    if (split && k > 1u)
+      merge_part(v, r, k, K1);
+    else
+      merge_heavy(v, K1);
+    if (threadIdx.x == 0) {
+      const unsigned long long dt = globaltimer() - t0;
+      S.tmax[0] = max(S.tmax[0], (unsigned)min(dt, 0xFFFFFFFFull));
+      st[S_NHEAVY] += r == 0;
+      st[S_SUMH] += dt;
+    }
+  }
+
   // ---------------- one step ----------------
   // Returns false (on every block alike) when the search is over: OPEN_i
   // holds no entry and window i produced no candidate.
@@ -1885,32 +1945,35 @@ struct Search {
     CycleCtl& K1 = C->cyc[r1];
     CycleCtl& K2 = C->cyc[r2];
     const bool fifo = (P.flags & OPMOS_FLAG_FIFO) != 0;
+    // everything the step reads of its record, in one round of loads
     const unsigned head = ld_volatile(&K0.head);
-    const unsigned n_in = min(ld_volatile(&K0.open_count.v) - head, A.open_cap);  // FIFO: ring tail - head
+    const unsigned tail = ld_volatile(&K0.open_count.v);
     const unsigned nt = ld_volatile(&K0.touched_count.v);
     const unsigned nh = ld_volatile(&K0.heavy_count.v);
+    const unsigned np = ld_volatile(&K0.part_count.v);
+    const unsigned plen = ld_volatile(&K0.plen.v);
+    const unsigned nlab = ld_volatile(&K0.lbase.v);
+    const Measured ms = measured(K0);
+    const BinLimits bl = C->bins[r0];
+    if (threadIdx.x < sizeof(PIdx) / 4)  // visible after select_window's block barriers
+      reinterpret_cast<unsigned*>(&S.pd)[threadIdx.x] =
+          ld_volatile(reinterpret_cast<const unsigned*>(&C->pidx[cur]) + threadIdx.x);
+    const unsigned n_in = min(tail - head, A.open_cap);  // FIFO: ring tail - head
     if (n_in == 0 && nt == 0 && nh == 0) return false;
     cyc = i;
     fifo_head = head;
     const unsigned fwin = min(n_in, P.window);  // FIFO: ring positions window i+1 takes
-    psnap = ld_volatile(&K0.plen.v);
-    lbase = ld_volatile(&K0.lbase.v);
-    const BinLimits bl = C->bins[r0];
+    psnap = plen;
+    lbase = nlab;
     const BinParams bp{bl.b0, bl.b1, bl.s1, bl.delta, bl.s2};  // bins OPEN_i's histogram was built on
-    bpn = next_bins(K0);
+    bpn = next_bins(ms);
     if (threadIdx.x == 0) {
       for (int j = 0; j < 5; ++j) S.tmax[j] = 0;
-      const volatile PIdx* src = &C->pidx[cur];
-      S.pd.cur = src->cur;
-      S.pd.count = src->count;
-      S.pd.mark = src->mark;
-      S.pd.ntiles = src->ntiles;
-      S.pd.state = src->state;
-      S.pd.nb = src->nb;
-      S.pd.k = src->k;
-      for (int j = 0; j < 3; ++j) S.pd.shift[j] = src->shift[j];
+      S.min_key = ~0ull;
+      S.win_min = S.f1lo = kInf;
+      S.win_max = S.f1hi = 0;
     }
-    select_window(A.hist + r0 * kNB, n_in <= P.window);  // has block barriers: S.pd is visible after it
+    select_window(A.hist + r0 * kNB, n_in <= P.window);
     for (unsigned x = T.tid(); x < kNB; x += T.nthreads()) A.hist[r2 * kNB + x] = 0;
     if (T.leader_block()) {
       if (threadIdx.x == 0) {
@@ -1924,7 +1987,7 @@ struct Search {
         // values step i+1 starts from; the writers of this step raise them
         atomicMax(&K1.plen.v, psnap);
         atomicMax(&K1.lbase.v, lbase);
-        K1.win_min_prev = ld_volatile(&K0.win_min.v);
+        K1.win_min_prev = ms.wmin;
         C->bins[r1] = BinLimits{bpn.b0, bpn.b1, bpn.s1, bpn.delta, bpn.s2};
         if (fifo) {
           K1.head = head + fwin;
@@ -1942,48 +2005,37 @@ struct Search {
     // block merges first (the longest single tasks): the parts of split
     // merges (recorded in xpart while the candidates arrived), then one item
     // per heavy node, skipped when the node's merge is split
-    const unsigned np = ld_volatile(&K0.part_count.v);
-    for (const unsigned nhi = np + nh; nhi;) {
-      if (threadIdx.x == 0) S.claim = atomicAdd(&K0.heavy_next.v, 1u);
+    // The first one of each block is its own number, later ones are claimed.
+    const unsigned nhi = np + nh, nblk = T.nblocks();
+    for (unsigned t = T.block(), turn = 0; t < nhi; turn ^= 1u) {
+      const unsigned mine = t;
+      heavy_item(mine, np, cur, K1, Team::kSplitMerges);
+      if (nhi <= nblk) break;
+      if (threadIdx.x == 0) S.claim[turn] = nblk + atomicAdd(&K0.heavy_next.v, 1u);
       __syncthreads();
-      const unsigned t = S.claim;
-      __syncthreads();
-      if (t >= nhi) break;
-      const unsigned x = t < np ? A.cs[cur].xpart[t] : (t - np) << 4;
-      const unsigned h = x >> 4, r = x & 15u;
-      const unsigned k = A.cs[cur].hsplit[h];
-      if (t >= np && k > 1u) continue;
-      const uint32_t v = A.cs[cur].touched[2u * A.cand_cap - 1u - h];
-      if (threadIdx.x == 0 && r == 0) {  // read before the merge clears them
-        S.tmax[3] = max(S.tmax[3], A.cs[cur].ncand[v]);
-        S.tmax[4] = max(S.tmax[4], A.fcount[v]);
-      }
-      const unsigned long long t0 = globaltimer();
-      if constexpr (Team::kSplitMerges) {
-        if (k > 1u)
-          merge_part(v, r, k, K1);
-        else
-          merge_heavy(v, K1);
-      } else {
-        merge_heavy(v, K1);
-      }
-      if (threadIdx.x == 0) {
-        const unsigned long long dt = globaltimer() - t0;
-        S.tmax[0] = max(S.tmax[0], (unsigned)min(dt, 0xFFFFFFFFull));
-        st[S_NHEAVY] += r == 0;
-        st[S_SUMH] += dt;
-      }
+      t = S.claim[turn];
     }
     // warp items: index-rank items, light merges, extraction chunks
     const PIdx& pd = S.pd;
     const unsigned nrank = (D >= 2 && pd.state == 1) ? ((pd.k + 31) / 32) * ((pd.k + kRankQ - 1) / kRankQ) : 0u;
-    const unsigned nchunks = ((fifo ? fwin : n_in) + kChunk - 1) / kChunk;
+    const unsigned nopen = fifo ? fwin : n_in, nwarps = T.nwarps();
+    const unsigned per = item_entries(nopen, nwarps);
+    const unsigned nchunks = (nopen + per - 1) / per;
     const unsigned nitems = nrank + nt + nchunks;
     const unsigned lane = lane_id();
+    // The warps of the blocks without block merges take their first items by
+    // number (a claim by every warp at once queues on one counter for 2 us);
+    // the rest is claimed.
+    const unsigned wpb = blockDim.x >> 5, own = nhi < nblk ? (nblk - nhi) * wpb : 0u;
+    bool first = T.block() >= nhi;
     for (;;) {
-      unsigned t = 0;
-      if (lane == 0) t = atomicAdd(&K0.work_next.v, 1u);
-      t = __shfl_sync(0xffffffffu, t, 0);
+      unsigned t = T.wid() - nhi * wpb;
+      if (!first) {
+        if (nitems <= own) break;
+        if (lane == 0) t = own + atomicAdd(&K0.work_next.v, 1u);
+        t = __shfl_sync(0xffffffffu, t, 0);
+      }
+      first = false;
       if (t >= nitems) break;
       const unsigned long long t0 = globaltimer();
       if (t < nrank) {
@@ -1991,7 +2043,9 @@ struct Search {
       } else if (t < nrank + nt) {
         const uint32_t v = A.cs[cur].touched[t - nrank];
         uint32_t* hf = A.cs[cur].hflag + v;
-        if (*hf) {
+        const uint32_t listed = *hf;
+        __syncwarp();  // every lane has read it before lane 0 clears it
+        if (listed) {
           if (lane == 0) *hf = 0;  // merged by a block this step
         } else {
           merge_node(v, K1);
@@ -2004,9 +2058,9 @@ struct Search {
       } else {
         const unsigned c = t - nrank - nt;
         if (fifo)
-          extract_fifo(head + c * kChunk, head + min(fwin, (c + 1) * kChunk), K1);
+          extract_fifo(head + c * per, head + min(fwin, (c + 1) * per), K1);
         else
-          extract_chunk(c, n_in, bp, K1);
+          extract_chunk(c, n_in, per, bp, K1);
         if (lane == 0) {
           const unsigned long long dt = globaltimer() - t0;
           atomicMax(&S.tmax[2], (unsigned)min(dt, 0xFFFFFFFFull));
@@ -2016,7 +2070,18 @@ struct Search {
     }
     index_strided_work(T);
     __syncthreads();
-    if (threadIdx.x < 5) atomicMax(&K0.tmax[threadIdx.x], S.tmax[threadIdx.x]);
+    if (threadIdx.x < 5 && S.tmax[threadIdx.x]) atomicMax(&K0.tmax[threadIdx.x], S.tmax[threadIdx.x]);
+    if (threadIdx.x == 32) {
+      if (S.min_key != ~0ull) atomicMin(&K1.min_key.v, S.min_key);
+      if (S.win_min != kInf) {
+        atomicMin(&K1.win_min.v, S.win_min);
+        atomicMax(&K1.win_max.v, S.win_max);
+      }
+      if (S.f1lo != kInf) {
+        atomicMin(&K1.f1lo.v, S.f1lo);
+        atomicMax(&K1.f1hi.v, S.f1hi);
+      }
+    }
     for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x)
       if (S.hist[x]) atomicAdd(&A.hist[r1 * kNB + x], S.hist[x]);
     if (T.leader() && tlap) {
@@ -2247,9 +2312,9 @@ __global__ void __launch_bounds__(NT, NB) search_grid_kernel(GraphDev G, QArena 
 //   P1  INIT slots are initialised, OUT slots write one part of their
 //       result, RUN slots run one search step (merge of window i beside the
 //       extraction of window i+1).
-// In P1 each block derives the same assignment of "virtual blocks" to slots
-// (a running slot gets a share of the grid in proportion to its work, at
-// least one block), so large and small queries advance side by side.
+// In P1 every block reads the same assignment of "virtual blocks" to slots,
+// made in P0 (a running slot gets a share of the grid in proportion to its
+// work, at least one block), so large and small queries advance side by side.
 // ---------------------------------------------------------------------------
 struct SubTeam {
   static constexpr bool kSplitMerges = false;  // a query's arena has kparts = 1
@@ -2258,6 +2323,8 @@ struct SubTeam {
   __device__ __forceinline__ unsigned nthreads() const { return nb * blockDim.x; }
   __device__ __forceinline__ unsigned wid() const { return tid() >> 5; }
   __device__ __forceinline__ unsigned nwarps() const { return nthreads() >> 5; }
+  __device__ __forceinline__ unsigned block() const { return j; }
+  __device__ __forceinline__ unsigned nblocks() const { return nb; }
   __device__ __forceinline__ bool leader_block() const { return j == 0; }
   __device__ __forceinline__ bool leader() const { return j == 0 && threadIdx.x == 0; }
 };
@@ -2309,6 +2376,62 @@ __device__ __forceinline__ bool step_empty(const QCtl* C, unsigned i) {
   const CycleCtl& K = C->cyc[i % 3];
   return ld_volatile(&K.open_count.v) == ld_volatile(&K.head) && ld_volatile(&K.touched_count.v) == 0 &&
          ld_volatile(&K.heavy_count.v) == 0;
+}
+
+// Work units of a slot that enters the iteration in state st (0: none). INIT
+// and the scan part of the output get one block; the other output parts a
+// share like search steps.
+__device__ __forceinline__ unsigned mq_weight(const MSlot& sl, const QCtl* C, unsigned st, bool& single) {
+  single = false;
+  if (st == SL_FREE || st == SL_HELD) return 0;
+  if (st == SL_INIT || st == SL_OUT3) {
+    single = true;
+    return 1u;
+  }
+  if (st >= SL_OUT1) return max(1u, ld_volatile(&C->res_count) + ld_volatile(sl.A.fcount + sl.G.n));
+  const CycleCtl& K = C->cyc[C->step % 3];
+  const unsigned w = (ld_volatile(&K.open_count.v) - ld_volatile(&K.head)) + ld_volatile(&K.touched_count.v) +
+                     8u * ld_volatile(&K.heavy_count.v);
+  return w ? w : 1u;  // a running slot always gets a block
+}
+
+// Virtual blocks of the iteration (block 0, once every slot's state is set):
+// a slot gets a share of the grid in proportion to its work, at least one
+// block; M->pref holds the prefix sums. One block computes them for all: a
+// block that read the weights for itself could see counters the iteration's
+// work already moves, and take another slot's work.
+__device__ inline void mq_assign(const MSlot* slots, const QCtl* ctls, unsigned nslots, MCtl* M) {
+  __shared__ unsigned long long s_wtot;
+  __shared__ unsigned s_scan[33];
+  if (threadIdx.x == 0) s_wtot = 0;
+  __syncthreads();
+  unsigned long long wloc = 0;
+  for (unsigned q = threadIdx.x; q < nslots; q += blockDim.x) {
+    bool single;
+    const unsigned w = mq_weight(slots[q], &ctls[q], slots[q].state, single);
+    if (!single) wloc += w;
+  }
+  if (wloc) atomicAdd(&s_wtot, wloc);
+  __syncthreads();
+  const unsigned long long wtot = s_wtot > 0 ? s_wtot : 1, B = gridDim.x;
+  unsigned carry = 0;
+  for (unsigned c0 = 0; c0 < nslots; c0 += blockDim.x) {
+    const unsigned q = c0 + threadIdx.x;
+    unsigned nbq = 0;
+    if (q < nslots) {
+      bool single;
+      const unsigned w = mq_weight(slots[q], &ctls[q], slots[q].state, single);
+      if (single)
+        nbq = 1;
+      else if (w)
+        nbq = (unsigned)min(B, max(1ull, (w * B + wtot - 1) / wtot));
+    }
+    unsigned total;
+    const unsigned ex = block_exclusive_scan(nbq, s_scan, total);
+    if (q < nslots) M->pref[q] = carry + ex;
+    carry += total;
+  }
+  if (threadIdx.x == 0) M->pref[nslots] = carry;
 }
 
 // P0: slot transitions and admission (block 0).
@@ -2390,6 +2513,7 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
     if (st != SL_FREE) atomicAdd(&s_busy, 1u);
   }
   __syncthreads();
+  mq_assign(slots, ctls, nslots, M);
   if (threadIdx.x == 0) {
     M->iter++;
     const unsigned closing = ld_volatile(&hctl[HC_CLOSING]);
@@ -2428,61 +2552,11 @@ __device__ void mq_work(MSlot* slots, QCtl* ctls, unsigned q, unsigned j, unsign
   flush_stats(C, X.st);
 }
 
-__device__ __forceinline__ unsigned A_fcount_goal(const MSlot& sl) { return sl.A.fcount[sl.G.n]; }
-
-// Work units of a slot (0: none). INIT and the scan part of the output get
-// one block; the other output parts a share like search steps.
-__device__ __forceinline__ unsigned mq_weight(const MSlot& sl, QCtl* C, bool& single) {
-  single = false;
-  const unsigned st = sl.state;
-  if (st == SL_FREE || st == SL_HELD) return 0;
-  if (st == SL_INIT || st == SL_OUT3) {
-    single = true;
-    return 1u;
-  }
-  if (st >= SL_OUT1) return max(1u, ld_volatile(&C->res_count) + A_fcount_goal(sl));
-  const CycleCtl& K = C->cyc[C->step % 3];
-  const unsigned w = (ld_volatile(&K.open_count.v) - ld_volatile(&K.head)) + ld_volatile(&K.touched_count.v) +
-                     8u * ld_volatile(&K.heavy_count.v);
-  return w ? w : 1u;  // a running slot always gets a block
-}
-
 template <int D>
-__device__ void mq_phase(MSlot* slots, QCtl* ctls, unsigned nslots, Shared& S, unsigned* s_pref) {
-  // total weight of the multi-block slots
-  __shared__ unsigned long long s_wtot;
-  if (threadIdx.x == 0) s_wtot = 0;
+__device__ void mq_phase(MSlot* slots, QCtl* ctls, unsigned nslots, MCtl* M, Shared& S, unsigned* s_pref) {
+  for (unsigned q = threadIdx.x; q <= nslots; q += blockDim.x) s_pref[q] = ld_volatile(&M->pref[q]);
   __syncthreads();
-  unsigned long long wloc = 0;
-  for (unsigned q = threadIdx.x; q < nslots; q += blockDim.x) {
-    bool single;
-    const unsigned w = mq_weight(slots[q], &ctls[q], single);
-    if (!single) wloc += w;
-  }
-  atomicAdd(&s_wtot, wloc);
-  __syncthreads();
-  const unsigned long long wtot = s_wtot > 0 ? s_wtot : 1;
   const unsigned B = gridDim.x;
-  // virtual blocks per slot, then their prefix sums (chunked block scan)
-  unsigned carry = 0;
-  for (unsigned c0 = 0; c0 < nslots; c0 += blockDim.x) {
-    const unsigned q = c0 + threadIdx.x;
-    unsigned nbq = 0;
-    if (q < nslots) {
-      bool single;
-      const unsigned w = mq_weight(slots[q], &ctls[q], single);
-      if (single)
-        nbq = 1;
-      else if (w)
-        nbq = (unsigned)min((unsigned long long)B, max(1ull, (w * (unsigned long long)B + wtot - 1) / wtot));
-    }
-    unsigned total;
-    const unsigned ex = block_exclusive_scan(nbq, S.warp, total);
-    if (q < nslots) s_pref[q] = carry + ex;
-    carry += total;
-  }
-  if (threadIdx.x == 0) s_pref[nslots] = carry;
-  __syncthreads();
   const unsigned VB = s_pref[nslots];
   for (unsigned v = blockIdx.x; v < VB; v += B) {
     unsigned lo = 0, hi = nslots;  // last q with s_pref[q] <= v
@@ -2508,7 +2582,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
     if (blockIdx.x == 0) mq_schedule<D>(slots, ctls, nslots, queue, hctl, graphs, M, results, done_flags);
     if (!mq_barrier(M, target)) return;
     if (ld_volatile(&M->done)) return;
-    mq_phase<D>(slots, ctls, nslots, S, s_pref);
+    mq_phase<D>(slots, ctls, nslots, M, S, s_pref);
     if (!mq_barrier(M, target)) return;
   }
 }

@@ -98,7 +98,6 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
     cs.hsplit = take<uint32_t>(p, cand_cap);
     cs.cflag = take<uint32_t>(p, cand_cap);
     cs.cslot = take<int32_t>(p, (size_t)(n + 1) * slots);
-    cs.cnode = take<uint32_t>(p, cand_cap);
     cs.cparent = take<uint32_t>(p, cand_cap);
     cs.cedge = take<uint32_t>(p, cand_cap);
     cs.cnext = take<int32_t>(p, cand_cap);
@@ -142,7 +141,7 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
     }
     fimg[(size_t)D * fcap0 + i] = i;
   }
-  std::vector<uint32_t> cnode(cand_cap, 0), cpar(cand_cap, 0), cedge(cand_cap, 0), cg((size_t)cand_cap * D, 0);
+  std::vector<uint32_t> cpar(cand_cap, 0), cedge(cand_cap, 0), cg((size_t)cand_cap * D, 0);
   std::vector<int32_t> cnext(cand_cap, kNil), cslot((size_t)(n + 1) * slots, kNil),
       head((size_t)(n + 1) << lsub, kNil);
   for (uint32_t j = 0; j < ncand; ++j) {
@@ -186,7 +185,6 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   up(cs.ncand, ncand_v, 8);
   up(cs.node_head, head.data(), head.size() * 4);
   up(cs.cslot, cslot.data(), cslot.size() * 4);
-  up(cs.cnode, cnode.data(), cnode.size() * 4);
   up(cs.cparent, cpar.data(), cpar.size() * 4);
   up(cs.cedge, cedge.data(), cedge.size() * 4);
   up(cs.cnext, cnext.data(), cnext.size() * 4);
@@ -258,7 +256,7 @@ __global__ void __launch_bounds__(kGridThreads, 1) window_hook_kernel(GraphDev G
   X.select_window(A.hist + 1 * kNB);  // leaves S.hist empty for the extraction
   if (threadIdx.x == 0) *bstar = S.bstar;
   const unsigned nchunks = (n + kChunk - 1) / kChunk;
-  for (unsigned c = threadIdx.x >> 5; c < nchunks; c += blockDim.x >> 5) X.extract_chunk(c, n, bp, C->cyc[2]);
+  for (unsigned c = threadIdx.x >> 5; c < nchunks; c += blockDim.x >> 5) X.extract_chunk(c, n, kChunk, bp, C->cyc[2]);
 }
 
 }  // namespace
@@ -335,7 +333,6 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
       cs.hsplit = take<uint32_t>(p, cap);
       cs.cflag = take<uint32_t>(p, cap);
       cs.cslot = take<int32_t>(p, 3 * 32);
-      cs.cnode = take<uint32_t>(p, cap);
       cs.cparent = take<uint32_t>(p, cap);
       cs.cedge = take<uint32_t>(p, cap);
       cs.cnext = take<int32_t>(p, cap);
