@@ -1308,7 +1308,7 @@ int opmos_server_submit(opmos_server* sv, uint32_t graph, uint32_t d, uint32_t s
     CK(cudaMemsetAsync(sv->hkctr, 0, 2 * sizeof(unsigned), s));
     CK(cudaMemcpyAsync(sv->djobs, jobs, D * sizeof(HJob), cudaMemcpyHostToDevice, s));
     CK(launch_heuristic(g->dev, sv->djobs, D, sv->hscratch, 5 * (size_t)sv->shape.n + 64,
-                        std::min<unsigned>(D, kServeHeurBlocks), g->delta, sv->hkctr, sv->hkctr + 1, s));
+                        std::min<unsigned>(D, kServeHeurBlocks), g->delta, sv->hkctr, sv->hkctr + 1, s, kHeurSmemServed));
     unsigned herr = 0;
     CK(cudaMemcpyAsync(&herr, sv->hkctr + 1, 4, cudaMemcpyDeviceToHost, s));
     // bounded wait: the heuristic runs on SMs the resident kernel leaves free

@@ -88,8 +88,13 @@ struct HJob {
 // Sets the calling thread's opmos_last_error() message; returns code.
 int record_error(int code, const char* msg);
 
+// smem: shared memory a block may take. kHeurSmem by default; kHeurSmemServed
+// beside a resident multi-query kernel, which leaves a block's place (its
+// shared memory, registers and threads) free on the SMs it does not fill.
+constexpr size_t kHeurSmem = 200u << 10;
+constexpr size_t kHeurSmemServed = 38u << 10;
 cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                              size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta,
-                             unsigned* next_job, unsigned* err, cudaStream_t s);
+                             unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem = kHeurSmem);
 
 }  // namespace opmos
