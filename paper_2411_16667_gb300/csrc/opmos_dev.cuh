@@ -126,26 +126,36 @@ struct alignas(128) Hot {
 // step i works on are produced then) and read during step i; step i clears
 // the slot of step i+2.
 struct CycleCtl {
+  // What step i reads, one counter to a 128-byte line in this order: lane l of
+  // a block's first warp reads counter l (kRecWords; see Search::step).
   Hot<unsigned> open_count;         // entries of step i's OPEN array (FIFO: the ring's tail)
-  Hot<unsigned long long> min_key;  // smallest key among the entries carried over by extraction
-  Hot<unsigned> win_count;          // labels of window i
-  Hot<unsigned> win_min;            // smallest F[0] among them
-  Hot<unsigned> win_max;            // largest F[0] among them
-  Hot<unsigned> cand_count;         // candidates of window i (merged in step i)
-  Hot<unsigned> touched_count;      // nodes they reach with a small frontier (one warp each)
+  Hot<unsigned> head;               // FIFO: the ring position window i+1 starts at (0 otherwise)
+  Hot<unsigned> touched_count;      // nodes window i's candidates reach with a small frontier (one warp each)
   Hot<unsigned> heavy_count;        // ... with a large frontier (one block each)
-  Hot<unsigned> work_next;          // dynamic claims: index-rank items, light merges, extraction chunks
-  Hot<unsigned> heavy_next;         // dynamic claims of heavy merges (parts first)
   Hot<unsigned> part_count;         // parts of split heavy merges listed in xpart
-  Hot<unsigned> f1lo;               // F[1] range of the carried entries the histogram's bins cover
-  Hot<unsigned> f1hi;
   Hot<unsigned> plen;               // P-log length every reader uses in step i
   Hot<unsigned> lbase;              // labels that existed when step i began
-  unsigned win_min_prev;            // win_min of window i-1
-  unsigned head;                    // FIFO: the ring position window i+1 starts at (0 otherwise)
+  Hot<unsigned> win_min;            // smallest F[0] among the labels of window i
+  Hot<unsigned> win_prev;           // win_min of window i-1
+  Hot<unsigned> win_max;            // largest F[0] among the labels of window i
+  Hot<unsigned> f1lo;               // F[1] range of the carried entries the histogram's bins cover
+  Hot<unsigned> f1hi;
+  Hot<unsigned long long> min_key;  // smallest key among the entries carried over by extraction
+  // counters claimed from
+  Hot<unsigned> win_count;          // labels of window i
+  Hot<unsigned> cand_count;         // candidates of window i (merged in step i)
+  Hot<unsigned> work_next;          // dynamic claims: index-rank items, light merges, extraction chunks
+  Hot<unsigned> heavy_next;         // dynamic claims of heavy merges (parts first)
   unsigned tmax[5];                 // longest heavy merge, light merge, extraction item of step i (ns);
                                     // most candidates and largest frontier of a heavy merge
 };
+// The record's words a step reads: the counters above (the last one in two
+// words), the bins of its histogram and the P index.
+enum RecWord {
+  RW_OPEN, RW_HEAD, RW_TOUCHED, RW_HEAVY, RW_PARTS, RW_PLEN, RW_LBASE, RW_WMIN, RW_WPREV, RW_WMAX, RW_F1LO, RW_F1HI,
+  RW_KEYLO, RW_KEYHI, RW_BINS, RW_PIDX = RW_BINS + 5, kRecWords = RW_PIDX + 10
+};
+static_assert(kRecWords <= 32, "one lane a word");
 
 // Bins of one OPEN array's histogram: F[0] origin, F[1] origin and shift,
 // F[0] bucket width, cells per bin (2^s2).

@@ -130,6 +130,7 @@ struct Shared {
   // record once a step
   unsigned long long min_key;
   unsigned win_min, win_max, f1lo, f1hi;
+  unsigned rec[32];    // the step's record (RecWord)
   PIdx pd;             // the P index as this step sees it
   // the candidates of a block-merged node (up to kHC at a time)
   uint32_t hc[OPMOS_MAX_D][kHC];
@@ -257,7 +258,7 @@ struct Search {
     K.plen.v = 0;
     K.lbase.v = 0;
     for (int j = 0; j < 5; ++j) K.tmax[j] = 0;
-    K.head = 0;
+    K.head.v = 0;
   }
 
   // l_s = (v_s, 0) into OPEN_0 and G_OP(v_s) (Algorithm 1), control reset.
@@ -292,7 +293,7 @@ struct Search {
     C->n_labels.v = 1;
     for (int r = 0; r < 3; ++r) {
       clear_cycle(C->cyc[r]);
-      C->cyc[r].win_min_prev = kInf;
+      C->cyc[r].win_prev.v = kInf;
     }
     for (int b = 0; b < 2; ++b) C->pidx[b] = PIdx{};
     const uint32_t h0 = hk(0, s);
@@ -391,10 +392,6 @@ struct Search {
     unsigned long long min_key;
     unsigned f1lo, f1hi, wmin, wprev, wmax;
   };
-  __device__ __forceinline__ Measured measured(const CycleCtl& K) const {
-    return Measured{ld_volatile64(&K.min_key.v), ld_volatile(&K.f1lo.v),      ld_volatile(&K.f1hi.v),
-                    ld_volatile(&K.win_min.v),   ld_volatile(&K.win_min_prev), ld_volatile(&K.win_max.v)};
-  }
   __device__ BinParams next_bins(const Measured& m) const {
     BinParams b;
     b.b0 = min(min((uint32_t)(m.min_key >> 32), m.wmin), m.wprev);
@@ -1915,8 +1912,8 @@ struct Search {
     const unsigned x = t < np ? A.cs[cur].xpart[t] : (t - np) << 4;
     const unsigned h = x >> 4, r = x & 15u;
     const unsigned k = A.cs[cur].hsplit[h];
-    if (t >= np && k > 1u) return;
     const uint32_t v = A.cs[cur].touched[2u * A.cand_cap - 1u - h];
+    if (t >= np && k > 1u) return;
     if (threadIdx.x == 0 && r == 0) {  // read before the merge clears them
       S.tmax[3] = max(S.tmax[3], A.cs[cur].ncand[v]);
       S.tmax[4] = max(S.tmax[4], A.fcount[v]);
@@ -1945,38 +1942,47 @@ struct Search {
     CycleCtl& K1 = C->cyc[r1];
     CycleCtl& K2 = C->cyc[r2];
     const bool fifo = (P.flags & OPMOS_FLAG_FIFO) != 0;
-    // everything the step reads of its record, in one round of loads
-    const unsigned head = ld_volatile(&K0.head);
-    const unsigned tail = ld_volatile(&K0.open_count.v);
-    const unsigned nt = ld_volatile(&K0.touched_count.v);
-    const unsigned nh = ld_volatile(&K0.heavy_count.v);
-    const unsigned np = ld_volatile(&K0.part_count.v);
-    const unsigned plen = ld_volatile(&K0.plen.v);
-    const unsigned nlab = ld_volatile(&K0.lbase.v);
-    const Measured ms = measured(K0);
-    const BinLimits bl = C->bins[r0];
-    if (threadIdx.x < sizeof(PIdx) / 4)  // visible after select_window's block barriers
-      reinterpret_cast<unsigned*>(&S.pd)[threadIdx.x] =
-          ld_volatile(reinterpret_cast<const unsigned*>(&C->pidx[cur]) + threadIdx.x);
+    // Everything the step reads of its record, by one warp a block in one round
+    // of loads, a lane a word (every warp reading every word was 36,000 loads
+    // of 15 lines a step: 2.7 us).
+    if (threadIdx.x < kRecWords) {
+      static_assert(sizeof(BinLimits) == 5 * 4 && sizeof(PIdx) == 10 * 4, "RecWord");
+      static_assert(offsetof(CycleCtl, min_key) == RW_KEYLO * 128, "RecWord");
+      const unsigned l = threadIdx.x;
+      const unsigned* src = reinterpret_cast<const unsigned*>(&K0) + l * 32u;
+      if (l == RW_KEYHI) src -= 31;
+      if (l >= RW_BINS) src = reinterpret_cast<const unsigned*>(&C->bins[r0]) + (l - RW_BINS);
+      if (l >= RW_PIDX) src = reinterpret_cast<const unsigned*>(&C->pidx[cur]) + (l - RW_PIDX);
+      const unsigned x = __ldcg(src);
+      S.rec[l] = x;
+      if (l >= RW_PIDX) reinterpret_cast<unsigned*>(&S.pd)[l - RW_PIDX] = x;
+      if (l < 5) S.tmax[l] = 0;
+      if (l == 0) {
+        S.min_key = ~0ull;
+        S.win_min = S.f1lo = kInf;
+        S.win_max = S.f1hi = 0;
+      }
+    }
+    __syncthreads();
+    const unsigned* rec = S.rec;
+    const unsigned head = rec[RW_HEAD], tail = rec[RW_OPEN];
+    const unsigned nt = rec[RW_TOUCHED], nh = rec[RW_HEAVY], np = rec[RW_PARTS];
+    const Measured ms{(unsigned long long)rec[RW_KEYHI] << 32 | rec[RW_KEYLO], rec[RW_F1LO], rec[RW_F1HI],
+                      rec[RW_WMIN], rec[RW_WPREV], rec[RW_WMAX]};
     const unsigned n_in = min(tail - head, A.open_cap);  // FIFO: ring tail - head
     if (n_in == 0 && nt == 0 && nh == 0) return false;
     cyc = i;
     fifo_head = head;
     const unsigned fwin = min(n_in, P.window);  // FIFO: ring positions window i+1 takes
-    psnap = plen;
-    lbase = nlab;
-    const BinParams bp{bl.b0, bl.b1, bl.s1, bl.delta, bl.s2};  // bins OPEN_i's histogram was built on
+    psnap = rec[RW_PLEN];
+    lbase = rec[RW_LBASE];
+    // bins OPEN_i's histogram was built on
+    const BinParams bp{rec[RW_BINS], rec[RW_BINS + 1], rec[RW_BINS + 2], rec[RW_BINS + 3], rec[RW_BINS + 4]};
     bpn = next_bins(ms);
-    if (threadIdx.x == 0) {
-      for (int j = 0; j < 5; ++j) S.tmax[j] = 0;
-      S.min_key = ~0ull;
-      S.win_min = S.f1lo = kInf;
-      S.win_max = S.f1hi = 0;
-    }
     select_window(A.hist + r0 * kNB, n_in <= P.window);
     for (unsigned x = T.tid(); x < kNB; x += T.nthreads()) A.hist[r2 * kNB + x] = 0;
     if (T.leader_block()) {
-      if (threadIdx.x == 0) {
+      if (threadIdx.x == 64) {
         // the longest tasks of step i-1 (its slot is K2)
         st[S_MAXH] += K2.tmax[0];
         st[S_MAXL] += K2.tmax[1];
@@ -1987,10 +1993,10 @@ struct Search {
         // values step i+1 starts from; the writers of this step raise them
         atomicMax(&K1.plen.v, psnap);
         atomicMax(&K1.lbase.v, lbase);
-        K1.win_min_prev = ms.wmin;
+        K1.win_prev.v = ms.wmin;
         C->bins[r1] = BinLimits{bpn.b0, bpn.b1, bpn.s1, bpn.delta, bpn.s2};
         if (fifo) {
-          K1.head = head + fwin;
+          K1.head.v = head + fwin;
           atomicMax(&K1.open_count.v, head + n_in);
         }
       }
@@ -2018,24 +2024,24 @@ struct Search {
     // warp items: index-rank items, light merges, extraction chunks
     const PIdx& pd = S.pd;
     const unsigned nrank = (D >= 2 && pd.state == 1) ? ((pd.k + 31) / 32) * ((pd.k + kRankQ - 1) / kRankQ) : 0u;
-    const unsigned nopen = fifo ? fwin : n_in, nwarps = T.nwarps();
-    const unsigned per = item_entries(nopen, nwarps);
+    const unsigned nopen = fifo ? fwin : n_in;
+    const unsigned per = item_entries(nopen, T.nwarps());
     const unsigned nchunks = (nopen + per - 1) / per;
     const unsigned nitems = nrank + nt + nchunks;
     const unsigned lane = lane_id();
-    // The warps of the blocks without block merges take their first items by
-    // number (a claim by every warp at once queues on one counter for 2 us);
-    // the rest is claimed.
-    const unsigned wpb = blockDim.x >> 5, own = nhi < nblk ? (nblk - nhi) * wpb : 0u;
-    bool first = T.block() >= nhi;
-    for (;;) {
-      unsigned t = T.wid() - nhi * wpb;
-      if (!first) {
-        if (nitems <= own) break;
-        if (lane == 0) t = own + atomicAdd(&K0.work_next.v, 1u);
+    // While less than half of the blocks have a block merge and two rounds are
+    // enough, the warps of the others take the items by number (claims by every
+    // warp at once queue on one counter: 2 us to start, 2 us to learn that
+    // nothing is left); otherwise all warps claim them one by one.
+    const unsigned wpb = blockDim.x >> 5;
+    const bool bynum = 2u * nhi < nblk && nitems <= 2u * (nblk - nhi) * wpb;
+    const unsigned own = (nblk - nhi) * wpb;  // warps that take items by number
+    unsigned t = T.block() >= nhi ? T.wid() - nhi * wpb : nitems;
+    for (;; t += own) {
+      if (!bynum) {
+        if (lane == 0) t = atomicAdd(&K0.work_next.v, 1u);
         t = __shfl_sync(0xffffffffu, t, 0);
       }
-      first = false;
       if (t >= nitems) break;
       const unsigned long long t0 = globaltimer();
       if (t < nrank) {
@@ -2374,7 +2380,7 @@ __device__ void mq_alloc_region1(const MSlot& sl, QCtl* C) {
 
 __device__ __forceinline__ bool step_empty(const QCtl* C, unsigned i) {
   const CycleCtl& K = C->cyc[i % 3];
-  return ld_volatile(&K.open_count.v) == ld_volatile(&K.head) && ld_volatile(&K.touched_count.v) == 0 &&
+  return ld_volatile(&K.open_count.v) == ld_volatile(&K.head.v) && ld_volatile(&K.touched_count.v) == 0 &&
          ld_volatile(&K.heavy_count.v) == 0;
 }
 
@@ -2390,7 +2396,7 @@ __device__ __forceinline__ unsigned mq_weight(const MSlot& sl, const QCtl* C, un
   }
   if (st >= SL_OUT1) return max(1u, ld_volatile(&C->res_count) + ld_volatile(sl.A.fcount + sl.G.n));
   const CycleCtl& K = C->cyc[C->step % 3];
-  const unsigned w = (ld_volatile(&K.open_count.v) - ld_volatile(&K.head)) + ld_volatile(&K.touched_count.v) +
+  const unsigned w = (ld_volatile(&K.open_count.v) - ld_volatile(&K.head.v)) + ld_volatile(&K.touched_count.v) +
                      8u * ld_volatile(&K.heavy_count.v);
   return w ? w : 1u;  // a running slot always gets a block
 }
