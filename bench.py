@@ -897,7 +897,7 @@ def main():
         "clocks": clk.summary(),
         "open_scanned_per_step": st["open_scanned"] / max(1, st["steps"]),
         "longest_task_us_per_step": {k: v / 1e3 / max(1, st["steps"]) for k, v in
-                                     zip(("block_merge", "warp_merge", "extraction"), st["longest_task_ns"])},
+                                     zip(("merge_part", "merge", "extraction"), st["longest_task_ns"])},
         "window": opt.window,
         "window_choice": "autotuned on the 256x256 ship grid of seed 2 (same recipe, corner query): the fastest "
                          "of 1024 ... 262144" if not args.window else "given",

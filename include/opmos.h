@@ -138,17 +138,17 @@ typedef struct opmos_stats {
   uint64_t open_scanned;   /* OPEN entries read by the extraction scans, summed over steps
                               (an entry read by two passes of one step counts twice) */
   uint64_t open_rewritten; /* OPEN entries copied forward to the next step's OPEN array */
-  uint64_t list_candidates; /* candidates beyond the slots a node has per step (64 in a
+  uint64_t list_candidates; /* candidates beyond the slots a node has per step (56 in a
                                batch, 128 for a single query), merged from the node's lists */
-  uint64_t longest_task_ns[3]; /* summed over steps: the step's longest whole-block merge of a
-                                  node with a large frontier, longest one-warp node merge, and
-                                  longest extraction work item (the step's critical path) */
-  uint64_t heavy_merges;   /* node merges done by one or more whole blocks (a large frontier,
-                              or many candidates in the step) */
+  uint64_t longest_task_ns[3]; /* summed over steps: the step's longest part of a split merge,
+                                  longest merge of a node by one warp, and longest extraction
+                                  work item */
+  uint64_t heavy_merges;   /* node merges split into parts (many candidates, or much to compare
+                              them with) */
   uint64_t heavy_max_candidates; /* summed over steps: the most candidates, and the largest */
-  uint64_t heavy_max_frontier;   /* frontier, of a node merged by whole blocks in the step */
-  uint64_t task_ns[3];     /* summed durations of all block merges (one block each), one-warp
-                              merges and extraction items (one warp each) */
+  uint64_t heavy_max_frontier;   /* frontier, of a node whose merge was split in the step */
+  uint64_t task_ns[3];     /* summed durations of all parts of split merges, merges and extraction
+                              items (one warp each) */
 } opmos_stats;
 
 /* Fill *opt with the defaults (all fields explicit). */

@@ -207,7 +207,7 @@ constexpr uint32_t kWindowCapMin = 16384;  // labels a window may hold at least
 
 // Sizes of one query arena for a given byte budget.
 struct ArenaPlan {
-  uint32_t label_cap, open_cap, win_cap, cand_cap, plog_cap, nslots, lsub, kparts, xcap;
+  uint32_t label_cap, open_cap, win_cap, cand_cap, touch_cap, plog_cap, nslots, lsub, kparts, xcap;
   unsigned long long fpool_words;
   size_t bytes;
   size_t fixed;  // the part that does not grow with the labels
@@ -220,22 +220,21 @@ int plan_arena(const opmos_graph* g, uint32_t D, uint32_t window, size_t budget,
   // depend on thread timing (the front would not), hence the generous cap
   pl->win_cap = std::max<uint32_t>(4 * window, kWindowCapMin);
   pl->cand_cap = pl->win_cap * std::max<uint32_t>(g->maxdeg, 1);
+  pl->touch_cap = (uint32_t)std::min<size_t>(n + 1, pl->cand_cap);
   pl->plog_cap = batch ? (1u << 16) : (1u << 20);
   const size_t ptiles = pl->plog_cap / 32 + 1;
-  // per node: fbase, fcount, fcap, then per candidate set ncand, list heads, heavy flag,
-  // part count, slots; per candidate (two sets): parent, arc, list link, two touched
-  // entries, part count, flag, cost vector; the parts of split merges (two sets)
+  // per node: fbase, fcount, fcap, two champions, then per candidate set ncand, list heads,
+  // split flag, part count, slots; per candidate (two sets): list link, flag, record;
+  // per node a window reaches (two sets): touched entry; the parts of split merges
+  // (two sets)
   pl->lsub = batch ? kLSubBatch : kLSubGrid;
-  pl->nslots = kNodeSlots;
-  pl->kparts = 1;
-  pl->xcap = 0;
-  if (!batch) {
-    pl->nslots = kNodeSlotsGrid;
-    pl->kparts = kPartsMax;
-    pl->xcap = kPartsMax * (uint32_t)std::min<size_t>(n + 1, pl->cand_cap);
-  }
-  size_t fixed = (n + 1) * (8 + 4 + 4 + 2 * (4 + (4u << pl->lsub) + 4 + 4 + 4 * (size_t)pl->nslots)) + 3 * kNB * 4 +
-                 2 * (size_t)pl->cand_cap * (28 + 4 * D) + 2 * (size_t)pl->xcap * 4 + (size_t)pl->plog_cap * 4 * D +
+  pl->nslots = batch ? kNodeSlots : kNodeSlotsGrid;
+  pl->kparts = kPartsMax;
+  // parts of split merges a step may list; when it is full nodes keep the parts they have
+  pl->xcap = (batch ? 1u : 8u) * pl->touch_cap;
+  size_t fixed = (n + 1) * (8 + 4 + 4 + 2 * 4 * (size_t)row_words(D) + 2 * (4 + (4u << pl->lsub) + 4 + 4 + 4 * (size_t)pl->nslots)) + 3 * kNB * 4 +
+                 2 * (size_t)pl->cand_cap * (8 + 4 * (size_t)row_words((int)D + 2)) + 2 * (size_t)pl->touch_cap * 4 +
+                 2 * (size_t)pl->xcap * 8 + (size_t)pl->plog_cap * 4 * D +
                  2 * ((size_t)pl->plog_cap + ptiles) * 4 * D + kPSMax * 4 + 96 * 256;
   pl->fixed = fixed;
   if (budget < fixed + (8u << 20))
@@ -258,21 +257,19 @@ void layout_arena(const opmos_graph* g, uint32_t D, const ArenaPlan& pl, char* b
   A->fbase = carve<uint64_t>(p, n);
   A->fcount = carve<uint32_t>(p, n);
   A->fcap = carve<uint32_t>(p, n);
+  for (int b = 0; b < 2; ++b) A->champ[b] = carve<uint32_t>(p, n * row_words((int)D));
   for (int b = 0; b < 2; ++b) {
     CandSet& cs = A->cs[b];
     cs.ncand = carve<uint32_t>(p, n);
     cs.node_head = carve<int32_t>(p, n << pl.lsub);
     cs.hflag = carve<uint32_t>(p, n);
     cs.hcnt = carve<uint32_t>(p, n);
-    cs.hsplit = carve<uint32_t>(p, pl.cand_cap);
-    cs.xpart = carve<uint32_t>(p, std::max<uint32_t>(pl.xcap, 1));
+    cs.xpart = carve<uint2>(p, pl.xcap);
     cs.cflag = carve<uint32_t>(p, pl.cand_cap);
     cs.cslot = carve<int32_t>(p, n * pl.nslots);
-    cs.cparent = carve<uint32_t>(p, pl.cand_cap);
-    cs.cedge = carve<uint32_t>(p, pl.cand_cap);
     cs.cnext = carve<int32_t>(p, pl.cand_cap);
-    cs.touched = carve<uint32_t>(p, 2 * (size_t)pl.cand_cap);
-    cs.cg = carve<uint32_t>(p, (size_t)pl.cand_cap * D);
+    cs.touched = carve<uint32_t>(p, pl.touch_cap);
+    cs.crow = carve<uint32_t>(p, (size_t)pl.cand_cap * row_words((int)D + 2));
   }
   A->hist = carve<uint32_t>(p, 3 * kNB);
   A->prank = carve<uint32_t>(p, kPSMax);
@@ -295,6 +292,7 @@ void layout_arena(const opmos_graph* g, uint32_t D, const ArenaPlan& pl, char* b
   A->win_cap = pl.win_cap;
   A->cand_cap = pl.cand_cap;
   A->plog_cap = pl.plog_cap;
+  A->touch_cap = pl.touch_cap;
   A->fpool_words = pl.fpool_words;
   A->nslots = pl.nslots;
   A->lsub = pl.lsub;
@@ -526,8 +524,7 @@ int solve_one(const opmos_graph* g, const opmos_heur* heur, uint32_t start, uint
   P.flags = o.flags;
   P.qd = D;
   P.ps_grow = kGridIndexGrow;
-  P.heavy_work = o.window < kSmallWindow ? kHeavyWorkSmallWindow : kHeavyWork;
-  P.part_work = o.window < kSmallWindow ? kPartWork : kPartWorkWide;
+  P.part_work = part_work(D);
   P.time_limit_ns = time_limit_ns();
 
   // large windows take the wide grid (three 256-thread blocks per SM)
@@ -580,7 +577,7 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
   const DevInfo di = device_info();
   cudaStream_t s = (cudaStream_t)o.stream;
   const uint32_t nq = (uint32_t)qlist.size();
-  const int occ = multi_occupancy(D);
+  const int occ = multi_occupancy(D, 0);
   if (occ <= 0) return fail(OPMOS_ERR_CUDA, "multi-query kernel cannot be resident");
   const unsigned blocks = (unsigned)di.sms * (unsigned)std::min(occ, 2);
   ArenaPlan pl;
@@ -600,8 +597,7 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
   P.flags = o.flags;
   P.qd = D;
   P.ps_grow = kMultiIndexGrow;
-  P.heavy_work = kHeavyWork;
-  P.part_work = kPartWork;
+  P.part_work = part_work(D);
   P.time_limit_ns = time_limit_ns();
   std::vector<MSlot> hslots(slots);
   for (unsigned i = 0; i < slots; ++i) {
@@ -705,7 +701,7 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
       cudaMemsetAsync(dres, 0, b_r, s);
       cudaMemcpyAsync(dslots, p_sl, b_sl, cudaMemcpyHostToDevice, s);
       cudaMemcpyAsync(dqs, p_q, b_q, cudaMemcpyHostToDevice, s);
-      const cudaError_t el = launch_multi(D, dslots, ctls, slots, dqs, hctl, dgraphs, dres, nullptr, M, blocks, s);
+      const cudaError_t el = launch_multi(D, dslots, ctls, slots, dqs, hctl, dgraphs, dres, nullptr, M, blocks, 0, s);
       cudaMemcpyAsync(p_r, dres, b_r, cudaMemcpyDeviceToHost, s);
       cudaMemcpyAsync(p_M2, M, sizeof(MCtl), cudaMemcpyDeviceToHost, s);
       e = cudaStreamEndCapture(s, &graph);
@@ -745,7 +741,7 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
-    cudaError_t e = launch_multi(D, dslots, ctls, slots, dqs, hctl, dgraphs, dres, nullptr, M, blocks, s);
+    cudaError_t e = launch_multi(D, dslots, ctls, slots, dqs, hctl, dgraphs, dres, nullptr, M, blocks, 0, s);
     cudaEventRecord(e1, s);
     cudaError_t e2 =
         e == cudaSuccess ? cudaMemcpyAsync(hres.data(), dres, nq * sizeof(QResult), cudaMemcpyDeviceToHost, s) : e;
@@ -1250,8 +1246,7 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       sl.P.flags = o.flags;
       sl.P.qd = sv->dmax;
       sl.P.ps_grow = kMultiIndexGrow;
-      sl.P.heavy_work = kHeavyWork;
-      sl.P.part_work = kPartWork;
+      sl.P.part_work = part_work(sv->dmax);
       sl.P.time_limit_ns = time_limit_ns();
       sl.state = SL_FREE;
     }
@@ -1272,11 +1267,11 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       server_free(sv);
       return cuda_fail(e, "server set-up");
     }
-    const int occ = multi_occupancy(sv->dmax);
+    const int occ = multi_occupancy(sv->dmax, kServeBlockSmem);
     const unsigned full = (unsigned)di.sms * (unsigned)std::min(occ, 2);
     sv->blocks = full > 2 * kServeHeurBlocks ? full - 2 * kServeHeurBlocks : std::max(1u, full / 2);
     e = launch_multi(sv->dmax, dslots, ctls, sv->nslots, (MQuery*)dev_of(sv->hq), (unsigned*)dev_of(sv->hctl), dgraphs,
-                     (QResult*)dev_of(sv->hres), (unsigned*)dev_of(sv->hdone), M, sv->blocks, sv->kstream);
+                     (QResult*)dev_of(sv->hres), (unsigned*)dev_of(sv->hdone), M, sv->blocks, kServeBlockSmem, sv->kstream);
     if (e != cudaSuccess) {
       server_free(sv);
       return cuda_fail(e, "server kernel launch");

@@ -37,25 +37,24 @@ constexpr int kSub = 256;    // F[1] cells per F[0] bucket; a bin is 2^s2 consec
 constexpr unsigned kChunk = 32;       // most OPEN entries per extraction work item
 constexpr unsigned kRankQ = 1024;     // P entries per rank work item of an index rebuild
 constexpr unsigned kPSMax = 32768;    // largest P indexed by the sorted snapshot
-// candidates x frontier entries from which a node's merge takes a whole block:
-// lower for small windows (a step is short, its longest one-warp merge sets
-// its length), higher for large windows and batches (block merges are most
-// of the work)
-constexpr unsigned kHeavyWorkSmallWindow = 512;
-constexpr unsigned kHeavyWork = 2048;
-constexpr unsigned kSmallWindow = 16384;
-constexpr unsigned kHeavyCands = 32;      // ... and so are nodes reached by more candidates in a step
-// A block merge whose candidates x frontier entries exceed the part work is
-// split into parts (up to kPartsMax, each a whole block), each part holding
-// at least kPartCands candidates when the candidates are split; the part
-// work is larger on the wide grid, whose blocks are three to an SM.
-constexpr unsigned kPartWork = 1u << 17;
-constexpr unsigned kPartWorkWide = 1u << 18;
-constexpr unsigned kPartsMax = 16;
-constexpr unsigned kPartCands = 64;
+constexpr unsigned kSmallWindow = 16384;  // larger windows take the wide grid
+// A node's merge is split into parts, one warp each, of about part_work(d)
+// comparisons or fewer, kPartsMax at most: a warp alone issues an instruction
+// every 4-5 cycles, so this many take it about 5 us, a step's other work.
+// Measured (kPartWork = 3,000 / 6,000 / 12,000 / 24,000): 256x256 grid d=3 at
+// W = 262,144 134 / 121 / 110 / 108 ms; 160x160 d=3 31.7 / 32.5 / 32.1 / 32.2;
+// 96x96 d=5 first in first out 7.5 / 7.2 / 7.6 / 8.6; route d=12 8.6 / 8.4 /
+// 8.3 / 8.8; 128 queries d=5 40 / 37 / 36 / 36.
+constexpr unsigned kPartWork = 12288;
+constexpr unsigned kPartsMax = 128;
+constexpr unsigned kPartShares = 8;  // most shares of one group of 32 candidates
+inline unsigned part_work(unsigned d) { return kPartWork / (1u + d / 4u); }
 constexpr unsigned kPartPruned = 1u << 16;  // added to a node's part counter by a part that pruned
-constexpr unsigned kHeavyBusy = 0xFFFFFFFFu;  // hflag while the node is being listed
-constexpr unsigned kNodeSlots = 64;       // candidate slots per node and step in batch mode
+constexpr unsigned kSplitParts = 0xFFFFu;     // hflag: parts the node's merge is split into (0: none)
+constexpr unsigned kSplitDone = 1u << 30;     // ... its last part has finished
+constexpr unsigned kSplitSeen = 1u << 31;     // ... its own item has been skipped
+constexpr unsigned kNoPart = 0xFFFFFFFFu;     // a place of xpart that holds no part
+constexpr unsigned kNodeSlots = 56;       // candidate slots per node and step in batch mode
 constexpr unsigned kNodeSlotsGrid = 128;  // ... for a single query (whole-grid search)
 // Lists per node for the candidates beyond the slots (log2): the lanes of a
 // warp walk them side by side, so gathering k of them costs about
@@ -81,13 +80,13 @@ enum StatIdx {
   S_OSCAN,    // OPEN entries read by the extraction scans
   S_OKEEP,    // OPEN entries copied to the next step's OPEN array
   S_OVF,      // candidates beyond a node's slots (merged through the node's list)
-  S_MAXH,     // sum over steps of the longest heavy (block) merge of the step, ns
-  S_MAXL,     // ... of the longest light (warp) merge
+  S_MAXH,     // sum over steps of the longest part of a split merge of the step, ns
+  S_MAXL,     // ... of the longest merge by one warp
   S_MAXX,     // ... of the longest extraction work item
-  S_NHEAVY,   // heavy merges
-  S_MAXNC,    // sum over steps of the most candidates a block-merged node of the step had
-  S_MAXF,     // ... of the largest frontier a block-merged node of the step had
-  S_SUMH,     // summed durations of block merges (one block each), ns
+  S_NHEAVY,   // merges split into parts
+  S_MAXNC,    // sum over steps of the most candidates a node of a split merge of the step had
+  S_MAXF,     // ... of the largest frontier a node of a split merge of the step had
+  S_SUMH,     // summed durations of merge parts (one warp each), ns
   S_SUML,     // ... of one-warp merges (one warp each)
   S_SUMX,     // ... of extraction work items (one warp each)
   kNStat
@@ -95,13 +94,14 @@ enum StatIdx {
 
 // Two shapes of the single-query grid: one 512-thread block per SM for short
 // steps (windows below kSmallWindow), three 256-thread blocks per SM for large
-// windows, where block merges are most of a step and the merges of three
-// blocks overlap on one SM (registers are capped at 85 a thread then, and
-// some spill; two blocks with 128 registers were 9% slower, four with 64
-// no faster).
+// windows, whose steps have several work items for every warp (registers are
+// capped at 85 a thread then, and some spill).
 constexpr unsigned kGridThreads = 512;
 constexpr unsigned kGridWideThreads = 256;
 constexpr unsigned kGridWideBlocksPerSM = 3;
+
+// Words of a row that holds w words and is read 16 bytes at a time.
+__host__ __device__ constexpr int row_words(int w) { return w <= 2 ? w : (w + 3) / 4 * 4; }
 
 struct GraphDev {
   uint32_t n, m, d, maxdeg;
@@ -130,9 +130,8 @@ struct CycleCtl {
   // a block's first warp reads counter l (kRecWords; see Search::step).
   Hot<unsigned> open_count;         // entries of step i's OPEN array (FIFO: the ring's tail)
   Hot<unsigned> head;               // FIFO: the ring position window i+1 starts at (0 otherwise)
-  Hot<unsigned> touched_count;      // nodes window i's candidates reach with a small frontier (one warp each)
-  Hot<unsigned> heavy_count;        // ... with a large frontier (one block each)
-  Hot<unsigned> part_count;         // parts of split heavy merges listed in xpart
+  Hot<unsigned> touched_count;      // nodes window i's candidates reach
+  Hot<unsigned> part_count;         // places of xpart claimed for parts of split merges
   Hot<unsigned> plen;               // P-log length every reader uses in step i
   Hot<unsigned> lbase;              // labels that existed when step i began
   Hot<unsigned> win_min;            // smallest F[0] among the labels of window i
@@ -144,15 +143,14 @@ struct CycleCtl {
   // counters claimed from
   Hot<unsigned> win_count;          // labels of window i
   Hot<unsigned> cand_count;         // candidates of window i (merged in step i)
-  Hot<unsigned> work_next;          // dynamic claims: index-rank items, light merges, extraction chunks
-  Hot<unsigned> heavy_next;         // dynamic claims of heavy merges (parts first)
-  unsigned tmax[5];                 // longest heavy merge, light merge, extraction item of step i (ns);
-                                    // most candidates and largest frontier of a heavy merge
+  Hot<unsigned> work_next;          // dynamic claims of work items
+  unsigned tmax[5];                 // longest merge part, merge, extraction item of step i (ns);
+                                    // most candidates and largest frontier of a split merge
 };
 // The record's words a step reads: the counters above (the last one in two
 // words), the bins of its histogram and the P index.
 enum RecWord {
-  RW_OPEN, RW_HEAD, RW_TOUCHED, RW_HEAVY, RW_PARTS, RW_PLEN, RW_LBASE, RW_WMIN, RW_WPREV, RW_WMAX, RW_F1LO, RW_F1HI,
+  RW_OPEN, RW_HEAD, RW_TOUCHED, RW_PARTS, RW_PLEN, RW_LBASE, RW_WMIN, RW_WPREV, RW_WMAX, RW_F1LO, RW_F1HI,
   RW_KEYLO, RW_KEYHI, RW_BINS, RW_PIDX = RW_BINS + 5, kRecWords = RW_PIDX + 10
 };
 static_assert(kRecWords <= 32, "one lane a word");
@@ -213,18 +211,14 @@ struct CandSet {
   int32_t* cslot;      // (n+1) * nslots: the first nslots of them
   int32_t* node_head;  // (n+1) << lsub: the rest, in 2^lsub lists per node linked by cnext (the
                        // j-th candidate beyond the slots joins list j mod 2^lsub)
-  uint32_t* hflag;     // n+1: 0, or h + 1 once the node is listed as the h-th heavy node (merged by
-                       // whole blocks), kHeavyBusy while it is being listed
-  uint32_t* hcnt;      // n+1: parts of a split block merge finished so far (low 16 bits), plus
+  uint32_t* hflag;     // n+1: parts the node's merge is split into (kSplitParts), kSplitDone, kSplitSeen
+  uint32_t* hcnt;      // n+1: parts of a split merge finished so far (low 16 bits), plus
                        // kPartPruned for each part that pruned a frontier entry
-  uint32_t* hsplit;    // cand_cap: parts the h-th heavy node's merge is split into (1: not split)
-  uint32_t* xpart;     // parts of split merges, h << 4 | part (kPartsMax per heavy node at most)
+  uint2* xpart;        // xcap: parts of split merges, (node or kNoPart, part)
   uint32_t* cflag;     // cand_cap: candidate dropped by a part of a split merge
-  uint32_t* cparent;
-  uint32_t* cedge;
   int32_t* cnext;
-  uint32_t* cg;        // d * cand_cap
-  uint32_t* touched;   // 2 * cand_cap: every node reached from the front, block-merged ones from the back
+  uint32_t* crow;      // cand_cap records of row_words(d + 2) words: costs, arc, parent label
+  uint32_t* touched;   // touch_cap: every node reached
 };
 
 // Pointers into one query's arena (one slot).
@@ -232,6 +226,7 @@ struct QArena {
   uint64_t* fbase;     // n+1
   uint32_t* fcount;    // n+1
   uint32_t* fcap;      // n+1
+  uint32_t* champ[2];  // (n+1) rows: a label of each node that drops candidates at the expansion
   CandSet cs[2];
   uint32_t* lg;        // d * label_cap
   uint32_t* lnode;
@@ -252,11 +247,11 @@ struct QArena {
   uint32_t win_cap;
   uint32_t cand_cap;
   uint32_t plog_cap;
-  uint32_t pad;
+  uint32_t touch_cap;  // nodes a window can reach: min(n + 1, cand_cap)
   unsigned long long fpool_words;
   uint32_t nslots;     // candidate slots per node and step (the rest go to the node's lists)
   uint32_t lsub;       // log2 of the lists per node
-  uint32_t kparts;     // most parts a block merge is split into (1: never split)
+  uint32_t kparts;     // most parts a merge is split into
   uint32_t xcap;       // entries of each candidate set's xpart
 };
 
@@ -271,8 +266,7 @@ struct QParams {
   uint32_t flags;
   uint32_t qd;            // objectives the query uses (<= the kernel's D; the rest read as 0)
   uint32_t ps_grow;       // the P index is rebuilt once the log outgrows it by 32 + count >> ps_grow
-  uint32_t heavy_work;    // candidates x frontier entries from which a node is merged by a whole block
-  uint32_t part_work;     // ... per part of a split block merge
+  uint32_t part_work;     // candidates x frontier entries of one part of a split merge
   unsigned long long time_limit_ns;
 };
 
@@ -393,7 +387,6 @@ __device__ __forceinline__ unsigned grid_barrier(BarWord* b, unsigned target) {
 
 // Whole cooperative grid on one query.
 struct GridTeam {
-  static constexpr bool kSplitMerges = true;  // block merges may be split into parts
   __device__ __forceinline__ unsigned tid() const { return blockIdx.x * blockDim.x + threadIdx.x; }
   __device__ __forceinline__ unsigned nthreads() const { return gridDim.x * blockDim.x; }
   __device__ __forceinline__ unsigned wid() const { return tid() >> 5; }

@@ -66,9 +66,9 @@ int grid_occupancy(bool wide);
 template <int D>
 cudaError_t launch_multi_d(MSlot* slots, QCtl* ctls, unsigned nslots, const MQuery* queue, unsigned* hctl,
                            const GraphDev* graphs, QResult* results, unsigned* done_flags, MCtl* M, unsigned blocks,
-                           cudaStream_t s);
+                           size_t smem, cudaStream_t s);
 template <int D>
-int multi_occupancy_d();
+int multi_occupancy_d(size_t smem);
 
 // Dispatch on the objective count, 1..OPMOS_MAX_D (search_dispatch.cu).
 cudaError_t launch_search_grid(unsigned d, const GraphDev& G, const QArena& A, QCtl* C, const QParams& P,
@@ -76,8 +76,8 @@ cudaError_t launch_search_grid(unsigned d, const GraphDev& G, const QArena& A, Q
 int search_occupancy(unsigned d, bool wide);
 cudaError_t launch_multi(unsigned d, MSlot* slots, QCtl* ctls, unsigned nslots, const MQuery* queue,
                          unsigned* hctl, const GraphDev* graphs, QResult* results, unsigned* done_flags, MCtl* M,
-                         unsigned blocks, cudaStream_t s);
-int multi_occupancy(unsigned d);
+                         unsigned blocks, size_t smem, cudaStream_t s);
+int multi_occupancy(unsigned d, size_t smem);
 
 // Ideal-point heuristic jobs: h_out[v] = shortest v->goal distance under
 // objective k (Sec. 4), one thread block per job.
@@ -90,9 +90,11 @@ int record_error(int code, const char* msg);
 
 // smem: shared memory a block may take. kHeurSmem by default; kHeurSmemServed
 // beside a resident multi-query kernel, which leaves a block's place (its
-// shared memory, registers and threads) free on the SMs it does not fill.
+// shared memory, registers and threads) free on the SMs it does not fill: the
+// server launches its kernel with kServeBlockSmem a block for that.
 constexpr size_t kHeurSmem = 200u << 10;
-constexpr size_t kHeurSmemServed = 38u << 10;
+constexpr size_t kServeBlockSmem = 72u << 10;
+constexpr size_t kHeurSmemServed = 68u << 10;
 cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                              size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta,
                              unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem = kHeurSmem);

@@ -44,15 +44,15 @@ int search_occupancy(unsigned d, bool wide) {
 
 cudaError_t launch_multi(unsigned d, MSlot* slots, QCtl* ctls, unsigned nslots, const MQuery* queue,
                          unsigned* hctl, const GraphDev* graphs, QResult* results, unsigned* done_flags, MCtl* M,
-                         unsigned blocks, cudaStream_t s) {
-#define CALL(D) launch_multi_d<D>(slots, ctls, nslots, queue, hctl, graphs, results, done_flags, M, blocks, s)
+                         unsigned blocks, size_t smem, cudaStream_t s) {
+#define CALL(D) launch_multi_d<D>(slots, ctls, nslots, queue, hctl, graphs, results, done_flags, M, blocks, smem, s)
   OPMOS_DISPATCH_D(d, CALL)
 #undef CALL
   return cudaErrorInvalidValue;
 }
 
-int multi_occupancy(unsigned d) {
-#define CALL(D) multi_occupancy_d<D>()
+int multi_occupancy(unsigned d, size_t smem) {
+#define CALL(D) multi_occupancy_d<D>(smem)
   OPMOS_DISPATCH_D(d, CALL)
 #undef CALL
   return 0;

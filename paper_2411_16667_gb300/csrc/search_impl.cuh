@@ -8,10 +8,9 @@
 // extracted while the current one is processed):
 //
 //   merge (window i)     the candidates produced by expanding window i are
-//                        merged node by node, one warp per target node (a
-//                        whole block when candidates x frontier entries are
-//                        many, split into parts of one block each when they
-//                        are very many):
+//                        merged node by node, one warp per target node (split
+//                        into parts of one warp each when there is much to
+//                        compare):
 //                        resolved against each other (in-batch dominance and
 //                        duplicates), against the node's frontier alpha(v')
 //                        (Algorithm 1: weakly dominated candidates are dropped,
@@ -29,8 +28,9 @@
 //                        weakly dominates (PruneOPEN of Algorithm 1, applied
 //                        lazily); window labels are expanded at once along
 //                        their out-arcs (g' = g + c(e), dropped when h(v') is
-//                        infinite) into the other candidate set; all other
-//                        entries are carried to OPEN_{i+1}.
+//                        infinite or the node's champion -- one accepted label
+//                        of it -- dominates it) into the other candidate set;
+//                        all other entries are carried to OPEN_{i+1}.
 //
 // Labels created by merge i therefore become extractable from window i+2 on:
 // the same one-step lag as the paper's asynchronous scheme, which leaves the
@@ -58,12 +58,15 @@
 // the goal costs logged since; a rebuild runs over three steps (rank,
 // scatter, tiles) and is then published.
 //
-// A node is only ever merged by one warp (or block) per step, so frontier
-// updates need no locks. All waits are bounded (see GridTeam::sync).
+// A node's frontier is only ever written by one warp per step (the parts of a
+// split merge read it, and the last one to finish writes), so updates need no
+// locks. All waits are bounded (see GridTeam::sync).
 #pragma once
 
 #include "opmos_dev.cuh"
 #include "search.cuh"
+
+#include <algorithm>
 
 namespace opmos {
 namespace detail {
@@ -118,30 +121,26 @@ __device__ inline unsigned block_exclusive_scan(unsigned x, unsigned* s_warp, un
   return r;
 }
 
-constexpr unsigned kHC = 256;  // candidates a block merge holds at once
+// Dynamic shared memory of the search kernels: 32 rows of DP words a warp (see
+// Search::rows).
+__device__ __forceinline__ uint32_t* row_space() {
+  extern __shared__ __align__(16) uint32_t s_rows[];
+  return s_rows;
+}
 
 struct Shared {
   alignas(16) unsigned hist[kNB];  // this block's share of the next OPEN's histogram
   unsigned warp[33];
   unsigned f_min, b1_max, bstar;
   unsigned pmax[3];
-  unsigned claim[2];
   // what this block's extraction items found (next bins), added to the global
   // record once a step
   unsigned long long min_key;
   unsigned win_min, win_max, f1lo, f1hi;
   unsigned rec[32];    // the step's record (RecWord)
   PIdx pd;             // the P index as this step sees it
-  // the candidates of a block-merged node (up to kHC at a time)
-  uint32_t hc[OPMOS_MAX_D][kHC];
-  int hcid[kHC];
-  uint32_t hedge[kHC], hpar[kHC];
-  unsigned halive[kHC / 32], hkill[kHC / 32], hpkill[kHC / 32];
-  int hlist[32];       // cursors of the block-merged node's lists
-  unsigned mq_ncand, mq_next, m_nb, m_ok, m_lb, m_cap, m_plen, m_more;
-  unsigned long long m_fb;
-  unsigned tmax[5];    // this block's longest heavy merge, light merge, extraction item (ns);
-                       // most candidates and largest frontier of its heavy merges
+  unsigned tmax[5];    // this block's longest merge part, merge, extraction item (ns); most
+                       // candidates and largest frontier of its split merges
 };
 
 // Histogram bin of an OPEN key (F0 << 32 | F1): the key's cell is
@@ -181,9 +180,10 @@ __device__ __forceinline__ bool z_less(const uint32_t (&a)[MD], const uint32_t (
 
 template <int D>
 struct Search {
+  static constexpr int DP = row_words(D);      // words of a champion's row
+  static constexpr int CW = row_words(D + 2);  // words of a candidate's record: costs, arc, parent
   // frontier tiles loaded per round of a scan: fewer at high d (registers)
-  static constexpr int kU = D <= 4 ? 4 : (D <= 8 ? 2 : 1);
-  static constexpr int kUH = D <= 8 ? 2 : 1;
+  static constexpr int kU = D <= 4 ? 4 : (D <= 12 ? 2 : 1);
   static constexpr int kPT = D <= 4 ? 4 : (D <= 8 ? 2 : 1);  // P-index tiles loaded per round
 
   const GraphDev& G;
@@ -231,6 +231,8 @@ struct Search {
       A.fbase[v] = 0;
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
+#pragma unroll
+        for (int k = 0; k < DP; ++k) A.champ[b][(size_t)v * DP + k] = kInf;
         for (unsigned j = 0; j < (1u << A.lsub); ++j) A.cs[b].node_head[((size_t)v << A.lsub) + j] = kNil;
         A.cs[b].ncand[v] = 0;
         A.cs[b].hflag[v] = 0;
@@ -249,9 +251,7 @@ struct Search {
     K.win_max.v = 0;
     K.cand_count.v = 0;
     K.touched_count.v = 0;
-    K.heavy_count.v = 0;
     K.work_next.v = 0;
-    K.heavy_next.v = 0;
     K.part_count.v = 0;
     K.f1lo.v = kInf;
     K.f1hi.v = 0;
@@ -435,11 +435,11 @@ struct Search {
     if (alive) pos = atomicAdd(&cs.ncand[v2], 1u);
     c = __shfl_sync(0xffffffffu, c, lead) + __popc(am & lanemask_lt());
     if (alive) {
-      cs.cparent[c] = parent;
-      cs.cedge[c] = e;
-      cs.cflag[c] = 0u;
+      uint32_t rec[CW];
 #pragma unroll
-      for (int k = 0; k < D; ++k) cs.cg[(size_t)k * A.cand_cap + c] = g2[k];
+      for (int k = 0; k < CW; ++k) rec[k] = k < D ? g2[k % D] : k == D ? e : k == D + 1 ? parent : 0u;
+      vec_store(cs.crow + (size_t)c * CW, rec);
+      cs.cflag[c] = 0u;
       if (pos < A.nslots) {
         cs.cslot[(size_t)v2 * A.nslots + pos] = (int)c;
       } else {  // list (pos - nslots) mod 2^lsub of the node, so all its lists grow evenly
@@ -448,12 +448,9 @@ struct Search {
         st[S_OVF]++;
       }
     }
-    // Every node is listed among the light ones (one warp each) on its
-    // first candidate. A node with a large frontier, or reached by many
-    // candidates, is also listed once at the far end of the touched array
-    // (hflag decides; the array holds 2 * cand_cap entries) and merged by
-    // whole blocks; its light item then only clears hflag. Only light items
-    // touch hflag during the merge, so a block merge never races a warp.
+    // Every node is listed once, on its first candidate (one warp merges it). A
+    // node with much to compare has its merge split into hflag[v] parts, listed
+    // apart; its own item is skipped then.
     const unsigned fm = __ballot_sync(0xffffffffu, alive && pos == 0);
     if (fm) {
       const unsigned l0 = __ffs(fm) - 1;
@@ -462,24 +459,20 @@ struct Search {
       t = __shfl_sync(0xffffffffu, t, l0) + __popc(fm & lanemask_lt());
       if (alive && pos == 0) cs.touched[t] = v2;
     }
-    // A node is merged by a whole block once its candidates x frontier
-    // entries reach P.heavy_work (checked at 1, 4, 8 and 16 candidates: the
-    // work of a one-warp merge grows with that product; at the goal node n,
-    // with candidates x P), and always past kHeavyCands candidates (a warp
-    // would take them in two batches).
-    if (alive) {
-      const unsigned nc = pos + 1u;
-      const bool list = pos == kHeavyCands || ((nc == 1u || nc == 4u || nc == 8u || nc == 16u) &&
-                                               (unsigned long long)nc * fc >= P.heavy_work);
-      // at 64, 128, 256, ... candidates the merge may be split further
-      const bool grow = A.kparts > 1u && pos > kHeavyCands && ((pos + 1u) & pos) == 0u;
-      // (the P test of a goal candidate skips most of P through the index tiles)
-      if (list || grow) heavy_list(cs, K1, v2, parts_for(pos + 1u, fc >> (v2 == G.n ? 3 : 0)), list);
+    // A merge is split once its candidates x what each is compared with (and
+    // the 128 or so comparisons' time it costs anyway) exceed P.part_work: looked at as the candidates reach 1, 2, 4, 8, ... A candidate
+    // meets the frontier and, if it survives, P: few entries of P with few
+    // objectives (the index tiles cover three), most of it with many. At the
+    // goal node n there is P alone.
+    if (alive && ((pos + 1u) & pos) == 0u) {
+      const unsigned want = parts_for(pos + 1u, 128u + pos + (v2 == G.n ? psnap >> kPGoal : fc + (psnap >> kPNode)));
+      if (want > 1u) split_merge(cs, K1, v2, want);
     }
   }
 
-  // Parts a block merge of nc candidates against F frontier entries is split
-  // into: a power of two, each part about P.part_work comparisons or fewer.
+  // Parts a merge of nc candidates of F comparisons each is split into: a power
+  // of two, each part about P.part_work comparisons or fewer.
+  static constexpr unsigned kPNode = D <= 4 ? 5 : (D <= 6 ? 3 : (D <= 8 ? 2 : 0)), kPGoal = D <= 4 ? 2 : (D <= 6 ? 1 : 0);
   __device__ unsigned parts_for(unsigned nc, unsigned F) const {
     const unsigned long long w = (unsigned long long)nc * F;
     unsigned k = 1;
@@ -487,44 +480,22 @@ struct Search {
     return k;
   }
 
-  // Lists node v as a heavy node (list), or raises the parts of its merge to
-  // want as its candidates grow. The lister holds hflag at kHeavyBusy until
-  // the node's index h and part count are written, then publishes h + 1; a
-  // raise that finds the node not yet published is dropped (the next one, at
-  // twice the candidates, tries again). Every new part is recorded in xpart;
-  // parts already recorded keep their numbers.
-  __device__ void heavy_list(const CandSet& cs, CycleCtl& K1, uint32_t v, unsigned want, bool list) {
-    unsigned h, r0;
-    if (list) {
-      if (atomicCAS(&cs.hflag[v], 0u, kHeavyBusy) != 0u) return;  // listed already
-      h = atomicAdd(&K1.heavy_count.v, 1u);
-      cs.touched[2u * A.cand_cap - 1u - h] = v;
-      cs.hsplit[h] = want;
-      r0 = 0;
-    } else {
-      const unsigned f = ld_volatile(&cs.hflag[v]);
-      if (f == 0u || f == kHeavyBusy) return;
-      h = f - 1u;
-      unsigned old = ld_volatile(&cs.hsplit[h]);
-      for (;;) {
-        if (want <= old) return;
-        const unsigned seen = atomicCAS(&cs.hsplit[h], old, want);
-        if (seen == old) break;
-        old = seen;
-      }
-      r0 = old > 1u ? old : 0u;  // parts [old, want), or all of them when the merge was not split
-    }
-    if (want > 1u) {
-      const unsigned j = atomicAdd(&K1.part_count.v, want - r0);
-      if (j + (want - r0) > A.xcap)
-        set_error(C, OPMOS_ERR_CAPACITY);
-      else
-        for (unsigned r = r0; r < want; ++r) cs.xpart[j + r - r0] = h << 4 | r;
-    }
-    if (list) {
-      __threadfence();
-      atomicExch(&cs.hflag[v], h + 1u);
-    }
+  // Raises the parts node v's merge is split into to want, and lists the new
+  // ones. Candidates arrive together, so the node's count of parts is raised by
+  // one atomic maximum whose return tells which parts are new (a protocol in
+  // which one candidate listed the node and later ones raised it lost most
+  // raises: nodes of 400 candidates were merged in 2 parts, 190 us). The
+  // places of the list are claimed first: a count never exceeds the parts
+  // listed, and when the list is full the node keeps the parts it has (none:
+  // one warp merges it). Places claimed in vain hold kNoPart.
+  __device__ void split_merge(const CandSet& cs, CycleCtl& K1, uint32_t v, unsigned want) {
+    const unsigned seen = ld_volatile(&cs.hflag[v]);
+    if (want <= seen) return;
+    const unsigned j = atomicAdd(&K1.part_count.v, want - seen), end = j + (want - seen);
+    unsigned old = want;  // nothing new when the list is full
+    if (end <= A.xcap) old = atomicMax(&cs.hflag[v], want);
+    for (unsigned x = j; x < min(end, A.xcap); ++x)
+      cs.xpart[x] = old + (x - j) < want ? make_uint2(v, old + (x - j)) : make_uint2(kNoPart, 0u);
   }
 
   // A window label as its lane holds it.
@@ -563,9 +534,9 @@ struct Search {
 #pragma unroll
       for (int k = 0; k < D; ++k) F[k] = want ? l.g[k] + hk(k, l.v) : 0u;
       if (pd.count && since < pd.mark)
-        p_filter(alive, F, pd.mark, psnap, pd.count, pd.ntiles, pd.cur, pcmp);
+        p_filter(alive, F, pd.mark, psnap, pd.count, 0, pd.ntiles, pd.cur, pcmp);
       else
-        p_filter(alive, F, since, psnap, 0, 0, 0, pcmp);
+        p_filter(alive, F, since, psnap, 0, 0, 0, 0, pcmp);
     }
     return alive;
   }
@@ -611,7 +582,13 @@ struct Search {
             st[S_CAND]++;
           }
           fc = A.fcount[v2];
-          if (!goal) alive = hk(0, v2) != kInf;  // else the goal is unreachable from v2
+          if (!goal) {
+            // dropped when the goal is unreachable from v2, or the best label
+            // v2 had when the step began dominates it
+            uint32_t ch[D];
+            champion(A.champ[cyc & 1u], v2, ch);
+            alive = hk(0, v2) != kInf && !weakly_le<D>(ch, g2);
+          }
         }
         add_candidates(cs, K1, alive, v2, par, e, g2, fc);
       }
@@ -747,142 +724,272 @@ struct Search {
     expand_labels(take, own, cs, K1);
   }
 
-  // F against the P index + the logged goal costs log[t0, t1): clears alive
-  // for candidates a solution weakly dominates (Algorithm 1). Every lane of
-  // the warp calls it; pcmp counts vector comparisons (lane 0's count is the
-  // warp's).
-  __device__ __forceinline__ void p_filter(bool& alive, const uint32_t (&F)[D], unsigned t0, unsigned t1,
-                                           unsigned pcount, unsigned pntiles, unsigned pbuf,
-                                           unsigned long long& pcmp) {
-    p_filter(alive, F, t0, t1, pcount, 0u, pntiles, pntiles, pbuf, pcmp);
+  // ---------------- rows: up to 32 vectors every lane of the warp reads ----------------
+  // A warp keeps the vectors it tests against many others (candidates with
+  // their arcs, or their F) in shared memory, one row of RP words each: a lane
+  // holds one entry of the other side, and the row all lanes read comes in
+  // RP / 4 loads instead of D shuffles.
+  static constexpr int RP = row_words(D + 1);
+  __device__ __forceinline__ uint32_t* rows() const { return row_space() + (threadIdx.x & ~31u) * RP; }
+  __device__ __forceinline__ void put_row(const uint32_t (&x)[D], uint32_t edge = 0) const {
+    uint32_t r[RP];
+#pragma unroll
+    for (int k = 0; k < RP; ++k) r[k] = k < D ? x[k % D] : k == D ? edge : 0u;
+    __syncwarp();  // earlier readers are done
+    vec_store(rows() + lane_id() * RP, r);
+    __syncwarp();
+  }
+  __device__ __forceinline__ void get_row(unsigned j, uint32_t (&x)[D]) const {
+    uint32_t r[RP];
+    vec_load(rows() + j * RP, r);
+#pragma unroll
+    for (int k = 0; k < D; ++k) x[k] = r[k];
+  }
+  __device__ __forceinline__ void get_row(unsigned j, uint32_t (&x)[D], uint32_t& edge) const {
+    uint32_t r[RP];
+    vec_load(rows() + j * RP, r);
+#pragma unroll
+    for (int k = 0; k < D; ++k) x[k] = r[k];
+    edge = r[D];
+  }
+  // Rows of W words, 16 bytes at a time (W = 1 or a multiple of 2).
+  template <int W>
+  __device__ __forceinline__ static void vec_load(const uint32_t* r, uint32_t (&x)[W]) {
+    if constexpr (W % 4 == 0) {
+#pragma unroll
+      for (int q = 0; q < W / 4; ++q) {
+        const uint4 v = reinterpret_cast<const uint4*>(r)[q];
+        x[4 * q] = v.x;
+        x[4 * q + 1] = v.y;
+        x[4 * q + 2] = v.z;
+        x[4 * q + 3] = v.w;
+      }
+    } else if constexpr (W % 2 == 0) {
+#pragma unroll
+      for (int q = 0; q < W / 2; ++q) {
+        const uint2 v = reinterpret_cast<const uint2*>(r)[q];
+        x[2 * q] = v.x;
+        x[2 * q + 1] = v.y;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < W; ++k) x[k] = r[k];
+    }
+  }
+  template <int W>
+  __device__ __forceinline__ static void vec_store(uint32_t* r, const uint32_t (&x)[W]) {
+    if constexpr (W % 4 == 0) {
+#pragma unroll
+      for (int q = 0; q < W / 4; ++q)
+        reinterpret_cast<uint4*>(r)[q] = make_uint4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < W; ++k) r[k] = x[k];
+    }
   }
 
-  // The same over the index tiles [tg_lo, tg_hi) of pntiles only (tg_lo a
-  // multiple of 32): the slice one warp of a block takes.
+  // F against tiles [tlo, thi) of the P index (pcount entries) + the logged goal
+  // costs log[t0, t1): clears alive for candidates a solution weakly dominates
+  // (Algorithm 1). Every lane of the warp calls it (its rows are overwritten);
+  // pcmp counts vector comparisons (lane 0's count is the warp's).
+  //
+  // The chain is what it costs (a handful of candidates, tiles in L2): the log's
+  // tail and the tile minima are loaded together, every candidate's passing
+  // tiles are found first (lane j keeps candidate j's), and then kPT of those
+  // tiles are loaded at a time, whichever candidates they belong to. With many
+  // objectives (kPFlat) nearly every tile passes, and the entries are scanned
+  // outright.
+  static constexpr bool kPFlat = D > 6;
   __device__ void p_filter(bool& alive, const uint32_t (&F)[D], unsigned t0, unsigned t1, unsigned pcount,
-                           unsigned tg_lo, unsigned tg_hi, unsigned pntiles, unsigned pbuf,
-                           unsigned long long& pcmp) {
+                           unsigned tlo, unsigned thi, unsigned pbuf, unsigned long long& pcmp) {
     const unsigned lane = lane_id();
     unsigned long long cnt = 0;
-    constexpr int UT = kU;  // tail tiles loaded per round
-    for (unsigned r0 = t0; r0 < t1; r0 += 32 * UT) {
-      if (!__any_sync(0xffffffffu, alive)) break;
-      uint32_t pt[UT][D];
+    unsigned am = __ballot_sync(0xffffffffu, alive);
+    if (!am || (t0 >= t1 && tlo >= thi)) return;
+    const uint32_t* ps = A.ps[pbuf];
+    const uint32_t* pst = A.pst[pbuf];
+    const size_t tcap = A.plog_cap / 32 + 1;
+    uint32_t tm[D];  // tile minima, one tile a lane
 #pragma unroll
-      for (int u = 0; u < UT; ++u) {
-        const unsigned jj = r0 + u * 32 + lane;
-#pragma unroll
-        for (int k = 0; k < D; ++k) pt[u][k] = jj < t1 ? A.plog[(size_t)k * A.plog_cap + jj] : kInf;
-      }
-#pragma unroll
-      for (int u = 0; u < UT; ++u) {
-        const unsigned j0 = r0 + u * 32;
-        unsigned amask = __ballot_sync(0xffffffffu, alive);
-        if (j0 >= t1 || !amask) break;
-        const bool vp = j0 + lane < t1;
-        cnt += (unsigned long long)__popc(amask) * min(32u, t1 - j0);
-        while (amask) {
-          const unsigned j = __ffs(amask) - 1;
-          amask &= amask - 1;
-          uint32_t Fj[D];
-#pragma unroll
-          for (int k = 0; k < D; ++k) Fj[k] = __shfl_sync(0xffffffffu, F[k], j);
-          const bool wd = vp && weakly_le<D>(pt[u], Fj);
-          if (__ballot_sync(0xffffffffu, wd) && lane == j) alive = false;
-        }
-      }
+    for (int k = 0; k < D; ++k) tm[k] = !kPFlat && tlo + lane < thi ? pst[(size_t)k * tcap + tlo + lane] : kInf;
+    put_row(F);
+    p_scan(am, A.plog, t0, t1, cnt);
+    if (kPFlat) {
+      p_scan(am, ps, tlo * 32, min(thi * 32, pcount), cnt);
+      alive = (am >> lane) & 1u;
+      if (lane == 0) pcmp += cnt;
+      return;
     }
-    if (pcount) {
-      const uint32_t* ps = A.ps[pbuf];
-      const uint32_t* pst = A.pst[pbuf];
-      const size_t tcap = A.plog_cap / 32 + 1;
-      constexpr int U = kU;  // tile-minimum groups loaded per round
-      for (unsigned tg0 = tg_lo; tg0 < tg_hi; tg0 += 32 * U) {
-        if (!__any_sync(0xffffffffu, alive)) break;
-        uint32_t tm[U][D];
+    for (unsigned tg = tlo; tg < thi && am; tg += 32) {
+      if (tg != tlo) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned tl = tg0 + u * 32 + lane;
+        for (int k = 0; k < D; ++k) tm[k] = tg + lane < thi ? pst[(size_t)k * tcap + tg + lane] : kInf;
+      }
+      cnt += (unsigned long long)__popc(am) * min(32u, thi - tg);
+      unsigned pm = 0;  // lane j: the tiles candidate j still has to be tested against
+      for (unsigned todo = am; todo;) {
+        unsigned j[2];
+        next_two(todo, j);
 #pragma unroll
-          for (int k = 0; k < D; ++k) tm[u][k] = tl < tg_hi ? pst[(size_t)k * tcap + tl] : kInf;
+        for (int x = 0; x < 2; ++x) {
+          uint32_t Fj[D];
+          get_row(j[x], Fj);
+          const unsigned m = __ballot_sync(0xffffffffu, tg + lane < thi && weakly_le<D>(tm, Fj));
+          if (lane == j[x]) pm = m;
         }
+      }
+      // (candidate, tile) pairs, one tile of up to kPT candidates a round -- or
+      // several tiles of one candidate when fewer are left
+      for (;;) {
+        unsigned open = __ballot_sync(0xffffffffu, pm != 0u);
+        if (!open) break;
+        unsigned jq[kPT], eq[kPT];
+        unsigned turn = open;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned tg = tg0 + u * 32;
-          unsigned amask = __ballot_sync(0xffffffffu, alive);
-          if (tg >= tg_hi || !amask) break;
-          const bool vt = tg + lane < tg_hi;
-          while (amask) {
-            const unsigned j = __ffs(amask) - 1;
-            amask &= amask - 1;
-            uint32_t Fj[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) Fj[k] = __shfl_sync(0xffffffffu, F[k], j);
-            unsigned pm = __ballot_sync(0xffffffffu, vt && weakly_le<D>(tm[u], Fj));
-            cnt += min(32u, tg_hi - tg);
-            bool dead = false;
-            while (pm && !dead) {
-              // up to kPT passing tiles per round: their loads overlap
-              unsigned tt[kPT];
-#pragma unroll
-              for (int q = 0; q < kPT; ++q) {
-                tt[q] = pm ? __ffs(pm) - 1 : 32u;
-                pm &= pm - 1;
-              }
-              uint32_t p[kPT][D];
-              bool ve[kPT];
-#pragma unroll
-              for (int q = 0; q < kPT; ++q) {
-                const unsigned e = (tg + tt[q]) * 32 + lane;
-                ve[q] = tt[q] < 32u && e < pcount;
-#pragma unroll
-                for (int k = 0; k < D; ++k) p[q][k] = ve[q] ? ps[(size_t)k * A.plog_cap + e] : kInf;
-              }
-#pragma unroll
-              for (int q = 0; q < kPT; ++q) {
-                dead |= __ballot_sync(0xffffffffu, ve[q] && weakly_le<D>(p[q], Fj)) != 0;
-                cnt += tt[q] < 32u ? 32 : 0;
-              }
+        for (int q = 0; q < kPT; ++q) {
+          if (!turn) turn = open;
+          jq[q] = 32u;
+          eq[q] = pcount;
+          if (open) {
+            jq[q] = __ffs(turn) - 1;
+            turn &= turn - 1;
+            const unsigned m = __shfl_sync(0xffffffffu, pm, jq[q]);
+            eq[q] = (tg + __ffs(m) - 1) * 32 + lane;
+            if (lane == jq[q]) pm &= pm - 1;
+            if (!(m & (m - 1))) {  // that was its last tile
+              open &= ~(1u << jq[q]);
+              turn &= ~(1u << jq[q]);
             }
-            if (dead && lane == j) alive = false;
+            cnt += 32;
           }
         }
+        uint32_t p[kPT][D];
+#pragma unroll
+        for (int q = 0; q < kPT; ++q)
+#pragma unroll
+          for (int k = 0; k < D; ++k) p[q][k] = eq[q] < pcount ? ps[(size_t)k * A.plog_cap + eq[q]] : kInf;
+        unsigned gone = 0;
+#pragma unroll
+        for (int q = 0; q < kPT; ++q) {
+          if (jq[q] > 31u) break;
+          uint32_t Fj[D];
+          get_row(jq[q], Fj);
+          if (eq[q] < pcount && weakly_le<D>(p[q], Fj)) gone |= 1u << jq[q];
+        }
+        gone = __reduce_or_sync(0xffffffffu, gone);
+        am &= ~gone;
+        if ((gone >> lane) & 1u) pm = 0;
       }
     }
+    alive = (am >> lane) & 1u;
     if (lane == 0) pcmp += cnt;
   }
 
-  // ---------------- merge of window i's candidates (Algorithm 1: frontier checks, goal branch) ----------------
-  // (a) in-batch: lanes holding candidates; a candidate another one strictly
-  // dominates, or that equals one with a smaller arc id, is dropped.
-  __device__ __forceinline__ bool in_batch_alive(const uint32_t (&c)[D], uint32_t my_edge, bool valid, unsigned nb) {
+  // The rows of am against entries [t0, t1) of a list of goal costs, all of them.
+  __device__ __forceinline__ void p_scan(unsigned& am, const uint32_t* list, unsigned t0, unsigned t1,
+                                         unsigned long long& cnt) const {
     const unsigned lane = lane_id();
-    bool alive = valid;
-    for (unsigned j = 0; j < nb; ++j) {
-      uint32_t cj[D];
+    for (unsigned r0 = t0; r0 < t1 && am; r0 += 32 * kU) {
+      uint32_t pt[kU][D];
 #pragma unroll
-      for (int k = 0; k < D; ++k) cj[k] = __shfl_sync(0xffffffffu, c[k], j);
-      const uint32_t ej = __shfl_sync(0xffffffffu, my_edge, j);
-      if (alive && lane != j &&
-          (dominates<D>(cj, c) || (equal<D>(cj, c) && (ej < my_edge || (ej == my_edge && j < lane)))))
-        alive = false;
-    }
-    return alive;
-  }
-
-  // A frontier entry m created in this step (id >= lbase) that candidate j
-  // equals takes j's parent and arc if j's arc id is smaller, so the path kept
-  // for a cost does not depend on the order in which candidates arrived.
-  __device__ __forceinline__ void adopt_smaller_arc(unsigned eqmask, unsigned j, uint32_t mid, uint32_t my_edge,
-                                                    uint32_t my_par) {
-    const uint32_t ej = __shfl_sync(0xffffffffu, my_edge, j);
-    const uint32_t pj = __shfl_sync(0xffffffffu, my_par, j);
-    if ((eqmask >> lane_id()) & 1u) {
-      if (ej < A.ledge[mid]) {
-        A.ledge[mid] = ej;
-        A.lparent[mid] = pj;
+      for (int u = 0; u < kU; ++u) {
+        const unsigned jj = r0 + u * 32 + lane;
+#pragma unroll
+        for (int k = 0; k < D; ++k) pt[u][k] = jj < t1 ? list[(size_t)k * A.plog_cap + jj] : kInf;
+      }
+      cnt += (unsigned long long)__popc(am) * min(32u * kU, t1 - r0);
+      const int nu = (int)min((unsigned)kU, (t1 - r0 + 31) / 32);
+      for (unsigned todo = am; todo;) {
+        unsigned j[2];
+        next_two(todo, j);
+        uint32_t Fj[2][D];
+        bool wd[2] = {false, false};
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          get_row(j[x], Fj[x]);
+#pragma unroll
+          for (int u = 0; u < kU; ++u) {
+            if (u >= nu) break;
+            wd[x] |= r0 + u * 32 + lane < t1 && weakly_le<D>(pt[u], Fj[x]);
+          }
+        }
+        am &= ~__reduce_or_sync(0xffffffffu, (wd[0] ? 1u << j[0] : 0u) | (wd[1] ? 1u << j[1] : 0u));
       }
     }
+  }
+
+  // The next two set bits of todo, taken out of it (the last one twice).
+  __device__ __forceinline__ static void next_two(unsigned& todo, unsigned (&j)[2]) {
+    j[0] = j[1] = __ffs(todo) - 1;
+    todo &= todo - 1;
+    if (todo) {
+      j[1] = __ffs(todo) - 1;
+      todo &= todo - 1;
+    }
+  }
+
+  // ---------------- merge of window i's candidates (Algorithm 1: frontier checks, goal branch) ----------------
+  // Up to 32 candidates of one node, lane j holding candidate j (and its row).
+  struct Batch {
+    uint32_t c[D];
+    uint32_t edge, par;
+    bool alive;
+  };
+  // kU tiles of 32 frontier entries, lane l holding entry l of each.
+  struct Round {
+    uint32_t m[kU][D];
+    uint32_t mid[kU];
+  };
+  __device__ __forceinline__ Round load_round(unsigned r0, unsigned hi, uint64_t fb, unsigned cap, bool ids) const {
+    Round t;
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const unsigned i = r0 + u * 32 + lane_id();
+      const bool vm = i < hi;
+#pragma unroll
+      for (int k = 0; k < D; ++k) t.m[u][k] = vm ? A.fpool[fb + (size_t)k * cap + i] : kInf;
+      t.mid[u] = ids && vm ? A.fpool[fb + (size_t)D * cap + i] : 0u;
+    }
+    return t;
+  }
+  // The lanes' candidates (kNil: none).
+  __device__ __forceinline__ Batch load_batch(const CandSet& cs, int mine) const {
+    Batch b;
+    b.alive = mine != kNil;
+    uint32_t rec[CW];
+#pragma unroll
+    for (int k = 0; k < CW; ++k) rec[k] = kInf;
+    if (b.alive) vec_load(cs.crow + (size_t)mine * CW, rec);
+#pragma unroll
+    for (int k = 0; k < D; ++k) b.c[k] = rec[k];
+    b.edge = rec[D];
+    b.par = rec[D + 1];
+    return b;
+  }
+  // A batch against itself: a candidate another one strictly dominates, or that
+  // equals one with a smaller arc id, is dropped (a dropped one drops nothing
+  // more: what it dominates is dominated by what dropped it). Leaves the batch
+  // in the rows.
+  __device__ __forceinline__ void resolve_batch(Batch& b) const {
+    const unsigned lane = lane_id();
+    put_row(b.c, b.edge);
+    unsigned am = __ballot_sync(0xffffffffu, b.alive);
+    for (unsigned todo = am; todo;) {
+      unsigned j[2];
+      next_two(todo, j);
+      uint32_t cj[2][D], ej[2];
+      bool dies = false;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        get_row(j[x], cj[x], ej[x]);
+        if (lane != j[x] && weakly_le<D>(cj[x], b.c))
+          dies |= !weakly_le<D>(b.c, cj[x]) || ej[x] < b.edge || (ej[x] == b.edge && j[x] < lane);
+      }
+      const unsigned gone = __ballot_sync(0xffffffffu, dies);
+      am &= ~gone;
+      todo &= ~gone;
+    }
+    b.alive = (am >> lane) & 1u;
   }
 
   // A label created in this step and pruned in it is taken back out of the
@@ -891,910 +998,536 @@ struct Search {
     if (id >= lbase && v != G.n) atomicSub(&S.hist[bin_of(key_of(g, v), bpn)], 1u);
   }
 
-  __device__ void merge_batch(uint32_t v, int mine, unsigned nb, CycleCtl& K1) {
-    const CandSet& cs = A.cs[cyc & 1u];
+  // The batch against frontier entries [lo, hi) at fb, cap: candidates an entry
+  // weakly dominates die, entries a candidate strictly dominates are pruned
+  // (label dead from the next step on). WRITE: the entries that stay are moved together from lo on, and the
+  // end of them is returned; an entry created in this step (id >= lbase) that
+  // a candidate equals takes its parent and arc if its arc id is smaller, so
+  // the path kept for a cost does not depend on the order in which candidates
+  // arrived. Otherwise the entries are only read (several warps share the
+  // frontier), and pruned tells whether one was marked.
+  //
+  // kU tiles of 32 entries are loaded per round (t: the first round, loaded by
+  // the caller beside the candidates) and every live candidate's row is read
+  // once a round: 2 D compares a pair and a vote for two candidates.
+  template <bool WRITE>
+  __device__ unsigned scan_frontier(uint32_t v, Batch& b, unsigned lo, unsigned hi, uint64_t fb, unsigned cap,
+                                    Round& t, bool& pruned_any, unsigned long long& fcmp) {
+    constexpr int U = kU;
     const unsigned lane = lane_id();
-    const bool is_goal = (v == G.n);  // the virtual node standing for P
-    uint32_t c[D];
-    const bool valid = lane < nb;
+    unsigned am = __ballot_sync(0xffffffffu, b.alive), out = lo;
+    const uint32_t(&m)[U][D] = t.m;
+    const uint32_t(&mid)[U] = t.mid;
+    for (unsigned r0 = lo; r0 < hi; r0 += 32 * U) {
+      if (!am && (!WRITE || out == r0)) {  // nothing left to test and nothing moved: the rest stays in place
+        out = hi;
+        break;
+      }
+      if (r0 != lo) t = load_round(r0, hi, fb, cap, WRITE);  // (the caller has loaded the first)
+      const int nu = (int)min((unsigned)U, (hi - r0 + 31) / 32);  // tiles of the round that hold entries
+      bool pr[U];
 #pragma unroll
-    for (int k = 0; k < D; ++k) c[k] = valid ? cs.cg[(size_t)k * A.cand_cap + mine] : 0u;
-    const uint32_t my_edge = valid ? cs.cedge[mine] : kInf;
-    const uint32_t my_par = valid ? cs.cparent[mine] : kInf;
-    bool alive = in_batch_alive(c, my_edge, valid, nb);
-    uint64_t fb = A.fbase[v];
-    unsigned cap = A.fcap[v];
-    const unsigned fc = A.fcount[v];
-    unsigned out = fc;
-    unsigned long long fcmp = 0, pcmp = 0;
-    if (is_goal) {
-      // (b') at the goal alpha(v_g) is P: one weak-dominance test against the
-      // P index and every goal cost logged since it was built (this warp is
-      // the only writer of the log in this step). P members a new solution
-      // dominates are dropped once, at output (Prune(P, l) of Algorithm 1).
-      const unsigned plen = ld_volatile(&C->plog_len.v);
-      const PIdx& pd = S.pd;
-      p_filter(alive, c, pd.count ? pd.mark : 0u, plen, pd.count, pd.ntiles, pd.cur, pcmp);
-    } else {
-      // (b) against the frontier alpha(v), compacting it in place; kU tiles
-      // of 32 entries are loaded per round
-      out = 0;
-      constexpr int U = kU;
-      bool done = false;
-      for (unsigned r0 = 0; r0 < fc && !done; r0 += 32 * U) {
-        uint32_t m[U][D];
-        uint32_t mid[U];
+      for (int u = 0; u < U; ++u) pr[u] = false;
+      fcmp += (unsigned long long)__popc(am) * min(32u * U, hi - r0);
+      // two candidates an iteration (the last one twice when they are odd): a
+      // warp alone waits for its own chain of compares and votes
+      for (unsigned todo = am; todo;) {
+        unsigned j[2];
+        next_two(todo, j);
+        uint32_t cj[2][D];
+        get_row(j[0], cj[0]);
+        get_row(j[1], cj[1]);
+        bool dies[2] = {false, false}, same = false;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          if (u >= nu) break;
+          const bool vm = r0 + u * 32 + lane < hi;
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const bool le_mc = vm && weakly_le<D>(m[u], cj[x]);
+            const bool le_cm = vm && weakly_le<D>(cj[x], m[u]);
+            dies[x] |= le_mc;
+            pr[u] |= le_cm && !le_mc;
+            if (WRITE) same |= le_cm && le_mc && mid[u] >= lbase;
+          }
+        }
+        const unsigned gone = __reduce_or_sync(0xffffffffu, (dies[0] ? 1u << j[0] : 0u) | (dies[1] ? 1u << j[1] : 0u));
+        if (!gone) continue;
+        am &= ~gone;
+        if (WRITE && __any_sync(0xffffffffu, same)) {
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const uint32_t ej = __shfl_sync(0xffffffffu, b.edge, j[x]), pj = __shfl_sync(0xffffffffu, b.par, j[x]);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const bool eq = r0 + u * 32 + lane < hi && mid[u] >= lbase && weakly_le<D>(m[u], cj[x]) &&
+                              weakly_le<D>(cj[x], m[u]);
+              if (eq && ej < A.ledge[mid[u]]) {
+                A.ledge[mid[u]] = ej;
+                A.lparent[mid[u]] = pj;
+              }
+            }
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const unsigned i = r0 + u * 32 + lane;
+        if (pr[u]) {
+          const uint32_t id = WRITE ? mid[u] : A.fpool[fb + (size_t)D * cap + i];
+          A.ldead[id] = cyc;
+          if (WRITE) unhist(m[u], v, id);
+          st[S_PRUNED]++;
+          pruned_any = true;
+        }
+      }
+      if (WRITE) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const unsigned i = r0 + u * 32 + lane;
-          const bool vm = i < fc;
-#pragma unroll
-          for (int k = 0; k < D; ++k) m[u][k] = vm ? A.fpool[fb + (size_t)k * cap + i] : kInf;
-          mid[u] = vm ? A.fpool[fb + (size_t)D * cap + i] : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned i0 = r0 + u * 32;
-          if (i0 >= fc) {
-            done = true;
-            break;
-          }
-          const unsigned i = i0 + lane;
-          const bool vm = i < fc;
-          bool pruned = false;
-          unsigned amask = __ballot_sync(0xffffffffu, alive);
-          if (amask == 0 && out == i0) {
-            // nothing left to test and nothing moved: the rest stays in place
-            out = fc;
-            done = true;
-            break;
-          }
-          fcmp += (unsigned long long)__popc(amask) * min(32u, fc - i0);
-          const bool fresh = vm && mid[u] >= lbase;
-          while (amask) {
-            const unsigned j = __ffs(amask) - 1;
-            amask &= amask - 1;
-            uint32_t cj[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) cj[k] = __shfl_sync(0xffffffffu, c[k], j);
-            const bool le_mc = vm && weakly_le<D>(m[u], cj);
-            const bool le_cm = vm && weakly_le<D>(cj, m[u]);
-            if (__ballot_sync(0xffffffffu, le_mc) && lane == j) alive = false;
-            const unsigned eqm = __ballot_sync(0xffffffffu, fresh && le_mc && le_cm);
-            if (eqm) adopt_smaller_arc(eqm, j, mid[u], my_edge, my_par);
-            pruned |= le_cm && !le_mc;
-          }
-          const bool keep = vm && !pruned;
-          if (vm && pruned) {
-            A.ldead[mid[u]] = cyc;
-            unhist(m[u], v, mid[u]);
-            st[S_PRUNED]++;
-          }
+          const bool keep = i < hi && !pr[u];
           const unsigned km = __ballot_sync(0xffffffffu, keep);
           const unsigned pos = out + __popc(km & lanemask_lt());
-          __syncwarp();
+          // (every lane's entries of the round are in registers: a tile's
+          // places may overwrite entries of its round only)
           if (keep && pos != i) {
 #pragma unroll
             for (int k = 0; k < D; ++k) A.fpool[fb + (size_t)k * cap + pos] = m[u][k];
             A.fpool[fb + (size_t)D * cap + pos] = mid[u];
           }
-          __syncwarp();
           out += __popc(km);
         }
       }
     }
-    merge_finish(v, mine, c, valid, alive, out, fb, cap, K1, fcmp, pcmp);
+    b.alive = (am >> lane) & 1u;
+    __syncwarp();
+    return out;
   }
 
-  // The end of a batch's merge, by one warp, lane j holding candidate j:
-  // (c) F against P (Algorithm 1) at an ordinary node, then (d) survivors
-  // become labels and join alpha(v) and the next OPEN (or the P log at the
-  // goal). A candidate P rejects has still pruned the frontier entries it
-  // dominates (as in Algorithm 1, where Prune precedes the P test). out =
-  // live frontier entries left after (b); fb, cap = the frontier block.
-  __device__ void merge_finish(uint32_t v, int mine, const uint32_t (&c)[D], bool valid, bool alive, unsigned out,
-                               uint64_t fb, unsigned cap, CycleCtl& K1, unsigned long long fcmp,
-                               unsigned long long pcmp, bool p_done = false) {
-    const CandSet& cs = A.cs[cyc & 1u];
-    const unsigned lane = lane_id();
-    const bool is_goal = (v == G.n);
-    if (!is_goal && !p_done && __any_sync(0xffffffffu, alive)) {
-      uint32_t F[D];
+  // F against share x of n of P (Algorithm 1) for the batch: the index's tiles
+  // and the log behind it, up to t1. hv: the node's heuristic, 0 at the goal
+  // node n.
+  __device__ __forceinline__ void batch_ptest(const uint32_t (&hv)[D], Batch& b, unsigned t1, unsigned x, unsigned n,
+                                              unsigned long long& pcmp) {
+    if (!__any_sync(0xffffffffu, b.alive)) return;
+    const PIdx& pd = S.pd;
+    uint32_t F[D];
 #pragma unroll
-      for (int k = 0; k < D; ++k) F[k] = c[k] + (valid ? hk(k, v) : 0u);
-      const PIdx& pd = S.pd;
-      p_filter(alive, F, pd.count ? pd.mark : 0u, psnap, pd.count, pd.ntiles, pd.cur, pcmp);
+    for (int k = 0; k < D; ++k) F[k] = b.alive ? b.c[k] + hv[k] : kInf;
+    const unsigned t0 = pd.count ? pd.mark : 0u, tiles = pd.count ? pd.ntiles : 0u, tail = t1 - min(t0, t1);
+    p_filter(b.alive, F, t0 + (unsigned)((uint64_t)tail * x / n), t0 + (unsigned)((uint64_t)tail * (x + 1) / n), pd.count,
+             (unsigned)((uint64_t)tiles * x / n), (unsigned)((uint64_t)tiles * (x + 1) / n), pd.cur, pcmp);
+  }
+
+  // A node's champion is the accepted label of the smallest cost sum. A candidate
+  // it weakly dominates would be dropped by the merge (a label once accepted is
+  // in the frontier or was pruned by one that dominates whatever it dominates),
+  // so the expansion drops it at once: a third to two thirds of all candidates
+  // (two thirds to three quarters are dominated by some label). The rows are a
+  // pair by step parity: step i reads rows i & 1 and writes the others, so a row
+  // is never read half written; an older champion is as valid as a new one.
+  __device__ __forceinline__ static void champion(const uint32_t* rows, uint32_t v, uint32_t (&x)[D]) {
+    uint32_t r[DP];
+    vec_load(rows + (size_t)v * DP, r);
+#pragma unroll
+    for (int k = 0; k < D; ++k) x[k] = r[k];
+  }
+  __device__ __forceinline__ static uint32_t cost_sum(const uint32_t (&x)[D]) {
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int k = 0; k < D; ++k) sum += x[k];
+    return (uint32_t)min(sum, (unsigned long long)kInf);
+  }
+  __device__ __forceinline__ void update_champion(uint32_t v, const Batch& b) {
+    uint32_t c0[D], c1[D];
+    uint32_t* const next = A.champ[(cyc & 1u) ^ 1u] + (size_t)v * DP;
+    champion(A.champ[cyc & 1u], v, c0);
+    champion(A.champ[(cyc & 1u) ^ 1u], v, c1);
+    const uint32_t mine = b.alive ? cost_sum(b.c) : kInf;
+    const uint32_t best = warp_min(mine);
+    const unsigned who = __ballot_sync(0xffffffffu, b.alive && mine == best);
+    const uint32_t s0 = cost_sum(c0), s1 = cost_sum(c1);
+    __syncwarp();  // the rows are read before one is written
+    if (best < min(s0, s1)) {
+      if (lane_id() == (unsigned)__ffs(who) - 1) {
+#pragma unroll
+        for (int k = 0; k < D; ++k) next[k] = b.c[k];
+      }
+    } else if (s0 < s1 && lane_id() == 0) {
+#pragma unroll
+      for (int k = 0; k < D; ++k) next[k] = c0[k];
     }
-    // (d) survivors become labels, join alpha(v), OPEN (or the P log at the goal)
-    const unsigned smask = __ballot_sync(0xffffffffu, alive);
+  }
+
+  // The batch's survivors become labels and join alpha(v) -- `out` live entries
+  // at fb, cap, moved to a block of twice the size when full -- and the next
+  // OPEN, or at the goal node n the P log. Returns alpha(v)'s new size. The
+  // warp is the only one at the node. A candidate P rejected has still pruned
+  // the frontier entries it dominates (as in Algorithm 1, where Prune precedes
+  // the P test).
+  __device__ unsigned insert_batch(uint32_t v, const uint32_t (&hv)[D], const Batch& b, unsigned out, uint64_t& fb,
+                                   unsigned& cap, CycleCtl& K1) {
+    const unsigned lane = lane_id();
+    const bool is_goal = v == G.n, fifo = (P.flags & OPMOS_FLAG_FIFO) != 0;
+    const unsigned smask = __ballot_sync(0xffffffffu, b.alive);
     const unsigned ns = __popc(smask);
-    if (ns) {
-      unsigned lb = 0;
-      if (lane == 0) lb = atomicAdd(&C->n_labels.v, ns);
-      lb = __shfl_sync(0xffffffffu, lb, 0);
-      const bool over_budget = lb + ns > P.label_budget;
-      if (lb + ns > A.label_cap || over_budget) {
-        if (lane == 0) set_error(C, (lb + ns > A.label_cap) ? OPMOS_ERR_CAPACITY : OPMOS_ERR_BUDGET);
-      } else {
-        if (lane == 0) atomicMax(&K1.lbase.v, lb + ns);
-        const unsigned need = out + ns;
-        if (need > cap) {
-          // grow: new block of twice the size, copy the live entries
-          const unsigned tile = P.tile;
-          unsigned ncap = max(2u * need, tile);
-          ncap = (ncap + tile - 1) / tile * tile;
-          unsigned long long nb0 = 0;
-          if (lane == 0) nb0 = atomicAdd(&C->f_words.v, (unsigned long long)(D + 1) * ncap);
-          nb0 = __shfl_sync(0xffffffffu, nb0, 0);
-          if (nb0 + (unsigned long long)(D + 1) * ncap > A.fpool_words) {
-            if (lane == 0) set_error(C, OPMOS_ERR_CAPACITY);
-            return;
-          }
-          for (unsigned i = lane; i < out; i += 32) {
+    if (!ns) return out;
+    // label ids and places in the next OPEN, claimed side by side
+    unsigned lb = 0, ob = 0, plen = 0;
+    if (lane == 0) {
+      lb = atomicAdd(&C->n_labels.v, ns);
+      if (!is_goal) ob = atomicAdd(fifo ? &C->fifo_tail.v : &K1.open_count.v, ns);
+      if (is_goal) plen = ld_volatile(&C->plog_len.v);  // this warp is the log's only writer
+    }
+    if (!is_goal) update_champion(v, b);
+    lb = __shfl_sync(0xffffffffu, lb, 0);
+    ob = __shfl_sync(0xffffffffu, ob, 0);
+    plen = __shfl_sync(0xffffffffu, plen, 0);
+    if (lb + ns > A.label_cap || lb + ns > P.label_budget) {
+      if (lane == 0) set_error(C, (lb + ns > A.label_cap) ? OPMOS_ERR_CAPACITY : OPMOS_ERR_BUDGET);
+      return out;
+    }
+    if (is_goal ? plen + ns > A.plog_cap : (fifo ? ob - fifo_head : ob) + ns > A.open_cap) {
+      if (lane == 0) set_error(C, OPMOS_ERR_CAPACITY);
+      return out;
+    }
+    if (lane == 0) atomicMax(&K1.lbase.v, lb + ns);
+    const unsigned need = out + ns;
+    if (need > cap) {
+      // grow: new block of twice the size, copy the live entries
+      const unsigned tile = P.tile;
+      unsigned ncap = max(2u * need, tile);
+      ncap = (ncap + tile - 1) / tile * tile;
+      unsigned long long nb0 = 0;
+      if (lane == 0) nb0 = atomicAdd(&C->f_words.v, (unsigned long long)(D + 1) * ncap);
+      nb0 = __shfl_sync(0xffffffffu, nb0, 0);
+      if (nb0 + (unsigned long long)(D + 1) * ncap > A.fpool_words) {
+        if (lane == 0) set_error(C, OPMOS_ERR_CAPACITY);
+        return out;
+      }
+      for (unsigned i = lane; i < out; i += 32) {
 #pragma unroll
-            for (int k = 0; k <= D; ++k) A.fpool[nb0 + (size_t)k * ncap + i] = A.fpool[fb + (size_t)k * cap + i];
-          }
-          fb = nb0;
-          cap = ncap;
-          if (lane == 0) {
-            A.fbase[v] = fb;
-            A.fcap[v] = cap;
-          }
-        }
-        unsigned plen = 0;
-        if (is_goal) {
-          plen = __shfl_sync(0xffffffffu, ld_volatile(&C->plog_len.v), 0);  // read before lane 0 raises it
-          if (plen + ns > A.plog_cap) {
-            if (lane == 0) set_error(C, OPMOS_ERR_CAPACITY);
-            return;
-          }
-        }
-        if (alive) {
-          const unsigned r = __popc(smask & lanemask_lt());
-          const unsigned id = lb + r;
-#pragma unroll
-          for (int k = 0; k < D; ++k) A.lg[(size_t)k * A.label_cap + id] = c[k];
-          A.lnode[id] = is_goal ? P.goal : v;
-          A.lparent[id] = cs.cparent[mine];
-          A.ledge[id] = cs.cedge[mine];
-          A.lpver[id] = psnap;
-          A.ldead[id] = kAlive;
-#pragma unroll
-          for (int k = 0; k < D; ++k) A.fpool[fb + (size_t)k * cap + out + r] = c[k];
-          A.fpool[fb + (size_t)D * cap + out + r] = id;
-          if (is_goal) {
-#pragma unroll
-            for (int k = 0; k < D; ++k) A.plog[(size_t)k * A.plog_cap + plen + r] = c[k];
-          } else {
-            push_open(id, c, v, K1);
-          }
-        }
-        if (is_goal && lane == 0) {
-          __threadfence();
-          *reinterpret_cast<volatile unsigned*>(&C->plog_len.v) = plen + ns;
-          atomicMax(&K1.plen.v, plen + ns);
-        }
-        out += ns;
+        for (int k = 0; k <= D; ++k) A.fpool[nb0 + (size_t)k * ncap + i] = A.fpool[fb + (size_t)k * cap + i];
+      }
+      fb = nb0;
+      cap = ncap;
+      if (lane == 0) {
+        A.fbase[v] = fb;
+        A.fcap[v] = cap;
       }
     }
+    if (b.alive) {
+      const unsigned r = __popc(smask & lanemask_lt());
+      const unsigned id = lb + r;
+#pragma unroll
+      for (int k = 0; k < D; ++k) A.lg[(size_t)k * A.label_cap + id] = b.c[k];
+      A.lnode[id] = is_goal ? P.goal : v;
+      A.lparent[id] = b.par;
+      A.ledge[id] = b.edge;
+      A.lpver[id] = psnap;
+      A.ldead[id] = kAlive;
+#pragma unroll
+      for (int k = 0; k < D; ++k) A.fpool[fb + (size_t)k * cap + out + r] = b.c[k];
+      A.fpool[fb + (size_t)D * cap + out + r] = id;
+      if (is_goal) {
+#pragma unroll
+        for (int k = 0; k < D; ++k) A.plog[(size_t)k * A.plog_cap + plen + r] = b.c[k];
+      } else if (fifo) {
+        // the ring's tail (positions [head, tail) of this step are never written over)
+        A.oid[0][(ob + r) % A.open_cap] = id;
+      } else {
+        // the array of step i+1, counted in its histogram
+        const uint64_t key = ((uint64_t)(b.c[0] + hv[0]) << 32) | (D > 1 ? b.c[1 % D] + hv[1 % D] : 0u);
+        const unsigned nxt = (cyc & 1u) ^ 1u;
+        A.okey[nxt][ob + r] = key;
+        A.oid[nxt][ob + r] = id;
+        atomicAdd(&S.hist[bin_of(key, bpn)], 1u);
+      }
+    }
+    __syncwarp();
     if (lane == 0) {
-      A.fcount[v] = out;
+      if (is_goal) {  // the log entries are written before they are published
+        __threadfence();
+        *reinterpret_cast<volatile unsigned*>(&C->plog_len.v) = plen + ns;
+        atomicMax(&K1.plen.v, plen + ns);
+      } else if (fifo) {
+        atomicMax(&K1.open_count.v, ob + ns);
+      }
       st[S_INSERTED] += ns;
+    }
+    return need;
+  }
+
+  // A node's candidates of one step in groups of up to 32: first the slots, 32
+  // at a time, then 32 / L rounds of its L = 2^lsub lists at a time: lane x
+  // walks list x mod L and holds its candidate of round x / L of the group.
+  struct Groups {
+    uint32_t v;
+    unsigned in_slots, nslot_groups;
+    int lcur;        // the lane's position in its list
+    unsigned lnext;  // the list group lcur stands at
+  };
+  __device__ __forceinline__ unsigned ngroups(unsigned nc) const {
+    const unsigned ns = min(nc, A.nslots);
+    return (ns + 31) / 32 + (nc - ns + 31) / 32;
+  }
+  __device__ __forceinline__ int list_step(const CandSet& cs, int c, unsigned n) const {
+    for (; n && c != kNil; --n) c = cs.cnext[c];
+    return c;
+  }
+  __device__ __forceinline__ Groups open_groups(const CandSet& cs, uint32_t v, unsigned nc) const {
+    Groups q;
+    q.v = v;
+    q.in_slots = min(nc, A.nslots);
+    q.nslot_groups = (q.in_slots + 31) / 32;
+    q.lnext = 0;
+    q.lcur = kNil;
+    if (nc > q.in_slots) {
+      const unsigned list = lane_id() & ((1u << A.lsub) - 1u);
+      q.lcur = list_step(cs, cs.node_head[((size_t)v << A.lsub) + list], lane_id() >> A.lsub);
+    }
+    return q;
+  }
+  // The lane's candidate of group g (kNil: none); g must not decrease.
+  __device__ __forceinline__ int group(const CandSet& cs, Groups& q, unsigned g) const {
+    if (g < q.nslot_groups) {
+      const unsigned s = g * 32 + lane_id();
+      return s < q.in_slots ? cs.cslot[(size_t)q.v * A.nslots + s] : kNil;
+    }
+    q.lcur = list_step(cs, q.lcur, (g - q.nslot_groups - q.lnext) << (5 - A.lsub));
+    q.lnext = g - q.nslot_groups;
+    return q.lcur;
+  }
+  // The node's candidate set is empty again (the set is reused two steps later).
+  __device__ __forceinline__ void clear_groups(const CandSet& cs, uint32_t v, unsigned nc) const {
+    const unsigned lane = lane_id();
+    __syncwarp();  // every lane has read what it needs
+    if (lane == 0) cs.ncand[v] = 0;
+    if (nc > A.nslots && lane < (1u << A.lsub)) cs.node_head[((size_t)v << A.lsub) + lane] = kNil;
+  }
+
+  __device__ __forceinline__ void node_h(uint32_t v, uint32_t (&hv)[D]) const {
+#pragma unroll
+    for (int k = 0; k < D; ++k) hv[k] = v == G.n ? 0u : hk(k, v);
+  }
+
+  // One node's merge by one warp, 32 candidates at a time:
+  // (b) against the frontier alpha(v), compacted in place; at the goal node n
+  // alpha is P: one weak-dominance test against the P index and every goal
+  // cost logged since it was built (P members a new solution dominates are
+  // dropped once, at output: Prune(P, l) of Algorithm 1); (c) F against P;
+  // (d) survivors join alpha(v) and the next OPEN.
+  __device__ void merge_node(uint32_t v, CycleCtl& K1) {
+    const CandSet& cs = A.cs[cyc & 1u];
+    const unsigned lane = lane_id();
+    // the node's words and its first slots, in one round of loads
+    const unsigned nc = cs.ncand[v];
+    uint64_t fb = A.fbase[v];
+    unsigned cap = A.fcap[v], fc = A.fcount[v];
+    const unsigned fc0 = fc;
+    const int slot0 = lane < A.nslots ? cs.cslot[(size_t)v * A.nslots + lane] : kNil;
+    uint32_t hv[D];
+    node_h(v, hv);
+    Groups q = open_groups(cs, v, nc);
+    const unsigned ng = ngroups(nc);
+    unsigned long long fcmp = 0, pcmp = 0;
+    bool pruned = false;
+    for (unsigned g = 0; g < ng; ++g) {
+      const int mine = g ? group(cs, q, g) : (lane < q.in_slots ? slot0 : kNil);
+      Batch b = load_batch(cs, mine);
+      Round t = load_round(0u, v == G.n ? 0u : fc, fb, cap, true);
+      resolve_batch(b);
+      if (v == G.n) {
+        batch_ptest(hv, b, __shfl_sync(0xffffffffu, ld_volatile(&C->plog_len.v), 0), 0u, 1u, pcmp);
+      } else {
+        fc = scan_frontier<true>(v, b, 0u, fc, fb, cap, t, pruned, fcmp);
+        batch_ptest(hv, b, psnap, 0u, 1u, pcmp);
+      }
+      fc = insert_batch(v, hv, b, fc, fb, cap, K1);
+    }
+    clear_groups(cs, v, nc);
+    if (lane == 0) {
+      if (fc != fc0) A.fcount[v] = fc;
       st[S_FCMP] += fcmp;
       st[S_PCMP] += pcmp;
     }
   }
 
-  // A new label joins the next OPEN: the array of step i+1 (counted in its
-  // histogram) or, with OPMOS_FLAG_FIFO, the ring's tail (positions
-  // [head, tail) of this step are never written over).
-  __device__ __forceinline__ void push_open(uint32_t id, const uint32_t (&c)[D], uint32_t v, CycleCtl& K1) {
-    if (P.flags & OPMOS_FLAG_FIFO) {
-      const unsigned o = agg_inc(&C->fifo_tail.v);
-      if (o - fifo_head < A.open_cap) {
-        A.oid[0][o % A.open_cap] = id;
-        atomicMax(&K1.open_count.v, o + 1u);
-      } else {
-        set_error(C, OPMOS_ERR_CAPACITY);
+  // The batch's live candidates (in the rows) against the node's candidates of
+  // groups [glo, ghi): one that another strictly dominates, or that equals one
+  // with a smaller arc id, dies (no two candidates of a node have the same
+  // costs and the same arc). The next group's records are loaded while one is tested.
+  __device__ void test_groups(const CandSet& cs, uint32_t v, unsigned nc, Batch& b, unsigned glo, unsigned ghi) {
+    const unsigned lane = lane_id();
+    unsigned am = __ballot_sync(0xffffffffu, b.alive);
+    Groups q = open_groups(cs, v, nc);
+    int o = glo < ghi ? group(cs, q, glo) : kNil;
+    Batch t = load_batch(cs, o);
+    for (unsigned g = glo; g < ghi && am; ++g) {
+      const int o2 = g + 1 < ghi ? group(cs, q, g + 1) : kNil;
+      const Batch t2 = load_batch(cs, o2);
+      for (unsigned todo = am; todo;) {
+        unsigned j[2];
+        next_two(todo, j);
+        unsigned gone = 0;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          uint32_t cj[D], ej;
+          get_row(j[x], cj, ej);
+          if (t.alive && weakly_le<D>(t.c, cj)) {
+            // (one that equals it in cost and arc is the candidate itself)
+            if (!weakly_le<D>(cj, t.c) || t.edge < ej) gone |= 1u << j[x];
+          }
+        }
+        am &= ~__reduce_or_sync(0xffffffffu, gone);
       }
-      return;
+      t = t2;
     }
-    const uint64_t key = key_of(c, v);
-    const unsigned o = agg_inc(&K1.open_count.v);
-    if (o < A.open_cap) {
-      const unsigned nxt = (cyc & 1u) ^ 1u;
-      A.okey[nxt][o] = key;
-      A.oid[nxt][o] = id;
-      atomicAdd(&S.hist[bin_of(key, bpn)], 1u);
-    } else {
-      set_error(C, OPMOS_ERR_CAPACITY);
-    }
+    b.alive = (am >> lane) & 1u;
   }
 
-  // A warp's cursor over node v's candidates of one step: the slots 32 at a
-  // time, then the node's 2^lsub lists, lane j walking list j. Opening it
-  // reads and clears the node's count and list heads (the set is reused two
-  // steps later).
-  struct Cursor {
-    unsigned ncand;  // candidates of the node this step
-    unsigned next;   // next slot index to read
-    int lcur;        // lane j < 2^lsub: its position in list j (kNil at the end)
-  };
-  __device__ __forceinline__ Cursor open_cursor(const CandSet& cs, uint32_t v) {
+  // Part r of a merge split into k parts (a power of two; decided while the
+  // node's candidates arrived), one warp. What can drop a candidate -- the
+  // node's other candidates, the frontier, P -- is only read, so the parts are
+  // independent: ka shares of the candidates (groups a, a + ka, ... of 32, or
+  // 16, 8 or 4 lanes of one group while there are more parts than groups)
+  // times kb ranges of all three. Shares of the candidates come first, as a
+  // candidate's early exit stays within one part then. Frontier entries a
+  // candidate strictly dominates are marked pruned (ldead = cyc); candidates
+  // that die get cflag set. Dominance is transitive and the frontier is an
+  // antichain, so it does not matter that a part does not see the deaths of the
+  // others. The last part to finish (a counter per node; nobody waits) compacts
+  // the frontier if a part pruned, and inserts what no part dropped.
+  //
+  // One warp a part, not a block: a block merge of the same work was 40 us of
+  // block barriers and round trips between them for 3 us of comparisons, while
+  // warps wait for nobody and many share an SM.
+  __device__ void merge_part(uint32_t v, unsigned r, unsigned k, CycleCtl& K1) {
+    const CandSet& cs = A.cs[cyc & 1u];
     const unsigned lane = lane_id();
-    Cursor q;
-    q.ncand = cs.ncand[v];
-    q.next = 0;
-    // lists holding something: min(candidates beyond the slots, 2^lsub)
-    const unsigned nl = q.ncand > A.nslots ? min(q.ncand - A.nslots, 1u << A.lsub) : 0u;
-    int32_t* heads = cs.node_head + ((size_t)v << A.lsub);
-    q.lcur = lane < nl ? heads[lane] : kNil;
+    const bool goal = v == G.n;
+    const unsigned nc = cs.ncand[v], F = A.fcount[v];
+    uint64_t fb = A.fbase[v];
+    unsigned cap = A.fcap[v];
+    uint32_t hv[D];
+    node_h(v, hv);
+    const unsigned plen = goal ? __shfl_sync(0xffffffffu, ld_volatile(&C->plog_len.v), 0) : psnap;
+    const unsigned ng = ngroups(nc);
+    unsigned ka = k, sub = 1;  // sub: shares of a group of 32
+    while (ka > 1u && ka / 2 >= ng) {
+      ka >>= 1;
+      if (sub < kPartShares) sub <<= 1;
+    }
+    const unsigned ks = ka * sub, kb = k / ks;
+    const unsigned a = (r % ks) / sub, bb = r / ks;
+    const unsigned width = 32u / sub, l0 = (r % ks) % sub * width;  // this part's lanes of a group
+    const unsigned lo = (unsigned)((uint64_t)F * bb / kb), hi = goal ? 0u : (unsigned)((uint64_t)F * (bb + 1) / kb);
+    unsigned long long fcmp = 0, pcmp = 0;
+    bool pruned = false;
+    {
+      Groups q = open_groups(cs, v, nc);
+      // (parts beyond the shares times the ranges have nothing to do)
+      for (unsigned g = r < ks * kb ? a : ng; g < ng; g += ka) {
+        const int mine = group(cs, q, g);
+        Batch b = load_batch(cs, mine);
+        Round t = load_round(lo, hi, fb, cap, false);
+        const bool own = lane - l0 < width;
+        b.alive = b.alive && own;
+        put_row(b.c, b.edge);
+        if (!goal) scan_frontier<false>(v, b, lo, hi, fb, cap, t, pruned, fcmp);
+        test_groups(cs, v, nc, b, ng * bb / kb, ng * (bb + 1) / kb);
+        batch_ptest(hv, b, plen, bb, kb, pcmp);
+        if (own && mine != kNil && !b.alive) cs.cflag[mine] = 1u;
+      }
+    }
+    // the part counter's low 16 bits count finished parts; kPartPruned is
+    // added by a part that pruned a frontier entry
+    const unsigned pr = __any_sync(0xffffffffu, pruned) ? kPartPruned : 0u;
+    __threadfence();
     __syncwarp();
-    if (lane == 0) cs.ncand[v] = 0;
-    if (lane < nl) heads[lane] = kNil;
-    return q;
-  }
-  __device__ __forceinline__ bool cursor_more(const Cursor& q) const {
-    return q.next < min(q.ncand, A.nslots) || __any_sync(0xffffffffu, q.lcur != kNil);
-  }
-  // Next batch (up to 32): the lane's candidate (kNil if none) and the batch
-  // size in *nb; the batch's candidates sit in lanes 0 .. *nb - 1.
-  __device__ __forceinline__ int next_batch(const CandSet& cs, uint32_t v, Cursor& q, unsigned* nb) {
-    const unsigned lane = lane_id();
-    int mine = kNil;
-    const unsigned in_slots = min(q.ncand, A.nslots);
-    if (q.next < in_slots) {
-      const unsigned n = min(32u, in_slots - q.next);
-      if (lane < n) mine = cs.cslot[(size_t)v * A.nslots + q.next + lane];
-      q.next += n;
-      *nb = n;
-    } else {
-      // rounds over the lists side by side: the lanes still inside a list
-      // hand their candidates to lanes n, n+1, ... and step on
-      unsigned n = 0;
-      for (;;) {
-        const unsigned bal = __ballot_sync(0xffffffffu, q.lcur != kNil);
-        if (bal == 0u || n >= 32u) break;
-        const unsigned cnt = __popc(bal);
-        const unsigned t = lane - n;  // this lane receives the t-th candidate of the round
-        const bool recv = lane >= n && t < cnt;
-        const int got = __shfl_sync(0xffffffffu, q.lcur, recv ? nth_bit(bal, t) : 0u);
-        if (recv) mine = got;
-        if (q.lcur != kNil && n + __popc(bal & lanemask_lt()) < 32u) q.lcur = cs.cnext[q.lcur];
-        n = min(32u, n + cnt);
-      }
-      *nb = n;
-    }
-    return mine;
-  }
-
-  // One node's merge by one warp.
-  __device__ void merge_node(uint32_t v, CycleCtl& K1) {
-    const CandSet& cs = A.cs[cyc & 1u];
-    Cursor q = open_cursor(cs, v);
-    do {
-      unsigned nb = 0;
-      const int mine = next_batch(cs, v, q, &nb);
-      merge_batch(v, mine, nb, K1);
-    } while (cursor_more(q));
-  }
-
-  // Merge of a node with a large frontier, or many candidates, by the whole
-  // block (every thread calls it). Up to kHC candidates at a time sit in
-  // shared memory (the node's slots, then its list):
-  //  (a) every thread resolves one candidate against all the others (strict
-  //      dominance; of equal ones the smallest arc id stays);
-  //  (b) all warps scan the frontier in rounds of nwarps * 32 * kUH entries,
-  //      each warp kUH tiles of 32 against every live candidate, and compact
-  //      it in place: a round's reads all precede the first barrier, its
-  //      writes land below the round's start, so they never overwrite an
-  //      entry another warp still has to read. Candidates killed by one warp
-  //      are dropped by the others from the next round on; a candidate that a
-  //      frontier entry weakly dominates never dominates another entry (the
-  //      frontier is an antichain), so the entries each candidate prunes do
-  //      not depend on when its death is seen;
-  //  (c) F against P, 32 candidates per warp, the P log tail and the index
-  //      tiles split between the warps that hold the same candidates;
-  //  (d) survivors become labels, join alpha(v) and the next OPEN.
-  __device__ void merge_heavy(uint32_t v, CycleCtl& K1) {
-    open_block_cursor(A.cs[cyc & 1u], v, false);
-    __syncthreads();
-    heavy_groups(v, K1, false);
-  }
-
-  // Warp 0 opens node v's cursor for a block merge in shared memory:
-  // S.mq_ncand candidates, slots from S.mq_next (past the slots if
-  // slots_done), list positions in S.hlist. A block barrier must follow.
-  __device__ void open_block_cursor(const CandSet& cs, uint32_t v, bool slots_done) {
-    if (threadIdx.x < 32) {
-      const Cursor q = open_cursor(cs, v);
-      S.hlist[threadIdx.x] = q.lcur;
-      if (threadIdx.x == 0) {
-        S.mq_ncand = q.ncand;
-        S.mq_next = slots_done ? min(q.ncand, A.nslots) : 0u;
-      }
-    }
-  }
-
-  // The next group (up to kHC, one per thread) of a block merge's candidates, into S.hcid;
-  // returns its size (every thread), 0 once none is left. First the slot
-  // rows S.mq_next, S.mq_next + 1, ... below nrows, row j being slot
-  // first + j * stride, then the lists whose cursors sit in S.hlist, walked
-  // side by side by warp 0. With filtered, candidates a part of a split merge
-  // dropped are skipped (and the group still fills while any are left).
-  __device__ unsigned gather_group(const CandSet& cs, uint32_t v, unsigned nrows, unsigned first, unsigned stride,
-                                   bool filtered) {
-    const unsigned tid = threadIdx.x;
-    const unsigned hcap = min(kHC, blockDim.x);  // one candidate per thread
-    unsigned s0 = S.mq_next, n0 = 0;
-    if (!filtered) {  // every slot below the count holds a candidate
-      n0 = s0 < nrows ? min(hcap, nrows - s0) : 0u;
-      if (tid < n0) S.hcid[tid] = cs.cslot[(size_t)v * A.nslots + first + (s0 + tid) * stride];
-      s0 += n0;
-    }
-    while (s0 < nrows && n0 < hcap) {  // (uniform: s0 and n0 are the same in every thread)
-      const unsigned take = min(hcap - n0, nrows - s0);
-      int c = kNil;
-      if (tid < take) c = cs.cslot[(size_t)v * A.nslots + first + (s0 + tid) * stride];
-      const bool keep = c != kNil && __ldcg(cs.cflag + c) == 0u;
-      unsigned cnt;
-      const unsigned pos = block_exclusive_scan(keep ? 1u : 0u, S.warp, cnt);  // (every thread has read mq_next)
-      if (keep) S.hcid[n0 + pos] = c;
-      n0 += cnt;
-      s0 += take;
-    }
-    __syncthreads();
-    if (tid < 32) {
-      int cur = S.hlist[tid];
-      unsigned n = n0;
-      for (;;) {
-        const bool live = cur != kNil;
-        if (!__any_sync(0xffffffffu, live) || n >= hcap) break;
-        const bool kp = live && (!filtered || __ldcg(cs.cflag + cur) == 0u);
-        const unsigned bal = __ballot_sync(0xffffffffu, kp);
-        const unsigned rk = __popc(bal & lanemask_lt());
-        const bool put = kp && n + rk < hcap;
-        if (put) S.hcid[n + rk] = cur;
-        if (put || (live && !kp)) cur = cs.cnext[cur];
-        n = min(hcap, n + __popc(bal));
-      }
-      S.hlist[tid] = cur;
-      const bool more = s0 < nrows || __any_sync(0xffffffffu, cur != kNil);
-      if (tid == 0) {
-        S.mq_next = s0;
-        S.m_nb = n;
-        S.m_more = more;
-      }
-    }
-    __syncthreads();
-    return S.m_nb;
-  }
-
-  // A gathered group's costs, arcs and parents into shared memory; the
-  // group's kill words cleared. A block barrier must follow.
-  __device__ void load_group(const CandSet& cs, unsigned nb) {
-    const unsigned tid = threadIdx.x;
-    if (tid < nb) {
-      const int c = S.hcid[tid];
+    unsigned done = 0;
+    if (lane == 0) done = atomicAdd(&cs.hcnt[v], 1u + pr) + 1u + pr;
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if ((done & (kPartPruned - 1u)) == k) {
+      __threadfence();
+      unsigned out = F;
+      if (done >= kPartPruned) out = compact_pruned(fb, cap, F);
+      Groups q = open_groups(cs, v, nc);
+      int pend = kNil;  // lanes 0 .. np-1: survivors to insert
+      unsigned np = 0;
+      for (unsigned g0 = 0; g0 < ng; g0 += 4) {  // four groups' flags side by side
+        int mine[4];
+        uint32_t gone[4];
 #pragma unroll
-      for (int k = 0; k < D; ++k) S.hc[k][tid] = cs.cg[(size_t)k * A.cand_cap + c];
-      S.hedge[tid] = cs.cedge[c];
-      S.hpar[tid] = cs.cparent[c];
-    }
-    if (tid < kHC / 32) {
-      S.halive[tid] = 0;
-      S.hkill[tid] = 0;
-      S.hpkill[tid] = 0;
-    }
-  }
-
-  // In-set resolution of a group (Sec. 5's Dup&Dom): candidate tid dies when
-  // another strictly dominates it or equals it with a smaller (arc, index);
-  // the survivors' words go to S.halive. A block barrier must follow.
-  __device__ void group_inset(unsigned nb) {
-    const unsigned tid = threadIdx.x, lane = lane_id(), w = tid >> 5;
-    bool alive = tid < nb;
-    if (alive) {
-      uint32_t ct[D];
+        for (int x = 0; x < 4; ++x) mine[x] = g0 + x < ng ? group(cs, q, g0 + x) : kNil;
 #pragma unroll
-      for (int k = 0; k < D; ++k) ct[k] = S.hc[k][tid];
-      const uint32_t et = S.hedge[tid];
-      for (unsigned j = 0; j < nb && alive; ++j) {
-        if (j == tid) continue;
-        uint32_t cj[D];
+        for (int x = 0; x < 4; ++x) gone[x] = mine[x] != kNil ? __ldcg(cs.cflag + mine[x]) : 1u;
 #pragma unroll
-        for (int k = 0; k < D; ++k) cj[k] = S.hc[k][j];
-        const uint32_t ej = S.hedge[j];
-        if (dominates<D>(cj, ct) || (equal<D>(cj, ct) && (ej < et || (ej == et && j < tid)))) alive = false;
-      }
-    }
-    const unsigned am = __ballot_sync(0xffffffffu, alive);
-    if (lane == 0 && w < kHC / 32) S.halive[w] = am;
-  }
-
-  // F against P for the live candidates of group word q, this warp taking
-  // slice sl of nsl of the P log entries [t0, t1) and of the first nt index
-  // tiles; the ones P dominates are flagged in S.hpkill. At the goal node n,
-  // F = g (h(n) = 0).
-  __device__ void group_ptest(uint32_t v, unsigned q, unsigned nsl, unsigned sl, unsigned t0, unsigned t1,
-                              unsigned nt) {
-    const unsigned lane = lane_id();
-    const unsigned word = S.halive[q] & ~S.hkill[q];
-    if (!word || sl >= nsl) return;
-    const PIdx& pd = S.pd;
-    const unsigned jj = q * 32 + lane;
-    uint32_t F[D];
-#pragma unroll
-    for (int k = 0; k < D; ++k) F[k] = S.hc[k][jj] + (v == G.n ? 0u : hk(k, v));
-    bool alive = (word >> lane) & 1u;
-    const unsigned tper = ((t1 - min(t0, t1) + nsl - 1) / nsl + 31) / 32 * 32;
-    const unsigned lo = min(t1, t0 + sl * tper), hi = min(t1, lo + tper);
-    const unsigned gper = ((nt + nsl - 1) / nsl + 31) / 32 * 32;
-    const unsigned glo = min(nt, sl * gper), ghi = min(nt, glo + gper);
-    unsigned long long pcmp = 0;
-    p_filter(alive, F, lo, hi, pd.count, glo, ghi, nt, pd.cur, pcmp);
-    st[S_PCMP] += pcmp;
-    const unsigned pk = __ballot_sync(0xffffffffu, !alive) & word;
-    if (lane == 0 && pk) atomicOr(&S.hpkill[q], pk);
-  }
-
-  // The group loop of a block merge, from the cursor in shared memory
-  // (S.mq_ncand candidates, slots from S.mq_next, then the lists at
-  // S.hlist). filtered: the survivors of a split merge's parts (the ones
-  // without cflag), already checked against the frontier's first `old`
-  // entries, so only the entries the loop itself inserts are scanned. At the
-  // goal node n there is no frontier scan: alpha(n) is P, and candidates meet
-  // P through the P index and log, up to the entries this merge appended
-  // (from entry pfrom on only, when filtered: the parts tested the rest).
-  __device__ void heavy_groups(uint32_t v, CycleCtl& K1, bool filtered, unsigned old = 0, unsigned pfrom = 0) {
-    const bool goal = v == G.n;
-    constexpr int U = kUH;
-    constexpr unsigned NW = kHC / 32;  // candidate words
-    const CandSet& cs = A.cs[cyc & 1u];
-    const unsigned tid = threadIdx.x, lane = lane_id(), w = tid >> 5, nw = blockDim.x >> 5;
-    const unsigned in_slots = min(S.mq_ncand, A.nslots);
-    for (;;) {
-      const unsigned nb = gather_group(cs, v, in_slots, 0u, 1u, filtered);
-      if (nb == 0) break;
-      const unsigned nwords = (nb + 31) / 32;
-      load_group(cs, nb);
-      __syncthreads();
-      // (a) in-set resolution
-      group_inset(nb);
-      __syncthreads();
-      // (b) the frontier
-      const uint64_t fb = A.fbase[v];
-      const unsigned cap = A.fcap[v];
-      const unsigned fc = A.fcount[v];
-      unsigned out = goal ? fc : old;
-      unsigned long long fcmp = 0;
-      const unsigned R = nw * 32u * U;
-      for (unsigned r0 = out; r0 < fc; r0 += R) {
-        const unsigned base = r0 + w * 32u * U;
-        uint32_t m[U][D];
-        uint32_t mid[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned i = base + u * 32 + lane;
-          const bool vm = i < fc;
-#pragma unroll
-          for (int k = 0; k < D; ++k) m[u][k] = vm ? A.fpool[fb + (size_t)k * cap + i] : kInf;
-          mid[u] = vm ? A.fpool[fb + (size_t)D * cap + i] : 0u;
-        }
-        unsigned kill[NW], km[U], wtot = 0;
-#pragma unroll
-        for (unsigned q = 0; q < NW; ++q) kill[q] = 0;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned i0 = base + u * 32;
-          const unsigned i = i0 + lane;
-          const bool vm = i < fc;
-          const bool fresh = vm && mid[u] >= lbase;
-          bool pruned = false;
-          if (i0 < fc) {
-#pragma unroll
-            for (unsigned q = 0; q < NW; ++q) {
-              if (q >= nwords) break;
-              // one lane's view of the kills other warps add meanwhile
-              unsigned am = __shfl_sync(0xffffffffu, S.halive[q] & ~S.hkill[q] & ~kill[q], 0);
-              fcmp += (unsigned long long)__popc(am) * min(32u, fc - i0);
-              while (am) {
-                const unsigned j = __ffs(am) - 1;
-                am &= am - 1;
-                const unsigned jj = q * 32 + j;
-                uint32_t cj[D];
-#pragma unroll
-                for (int k = 0; k < D; ++k) cj[k] = S.hc[k][jj];
-                const bool le_mc = vm && weakly_le<D>(m[u], cj);
-                const bool le_cm = vm && weakly_le<D>(cj, m[u]);
-                if (__ballot_sync(0xffffffffu, le_mc)) kill[q] |= 1u << j;
-                if (fresh && le_mc && le_cm && S.hedge[jj] < A.ledge[mid[u]]) {
-                  A.ledge[mid[u]] = S.hedge[jj];
-                  A.lparent[mid[u]] = S.hpar[jj];
-                }
-                pruned |= le_cm && !le_mc;
-              }
-            }
+        for (int x = 0; x < 4; ++x) {
+          const unsigned bal = __ballot_sync(0xffffffffu, gone[x] == 0u), cnt = __popc(bal);
+          if (np + cnt > 32u) {
+            out = insert_batch(v, hv, load_batch(cs, pend), out, fb, cap, K1);
+            pend = kNil;
+            np = 0;
           }
-          if (vm && pruned) {
-            A.ldead[mid[u]] = cyc;
-            unhist(m[u], v, mid[u]);
-            st[S_PRUNED]++;
-          }
-          km[u] = __ballot_sync(0xffffffffu, vm && !pruned);
-          wtot += __popc(km[u]);
-        }
-        if (lane == 0) {
-          S.warp[w] = wtot;
-#pragma unroll
-          for (unsigned q = 0; q < NW; ++q)
-            if (kill[q]) atomicOr(&S.hkill[q], kill[q]);
-        }
-        __syncthreads();  // (1) all reads of this round are done
-        const unsigned x = lane < nw ? S.warp[lane] : 0u;
-        unsigned incl = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= (unsigned)o) incl += y;
-        }
-        const unsigned wpre = __shfl_sync(0xffffffffu, incl - x, w);
-        const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-        unsigned pos = out + wpre;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned i = base + u * 32 + lane;
-          const bool keep = (km[u] >> lane) & 1u;
-          const unsigned p = pos + __popc(km[u] & lanemask_lt());
-          if (keep && p != i) {
-#pragma unroll
-            for (int k = 0; k < D; ++k) A.fpool[fb + (size_t)k * cap + p] = m[u][k];
-            A.fpool[fb + (size_t)D * cap + p] = mid[u];
-          }
-          pos += __popc(km[u]);
-        }
-        bool any = false;
-#pragma unroll
-        for (unsigned q = 0; q < NW; ++q) any |= (S.halive[q] & ~S.hkill[q]) != 0;
-        __syncthreads();  // (2) S.warp and S.hkill read by every warp
-        const unsigned seen = min(r0 + R, fc);
-        out += total;
-        if (!any && out == seen) {
-          // no candidate left to test and nothing moved: the rest stays in place
-          out = fc;
-          break;
+          const unsigned t = lane - np;  // this lane receives the t-th survivor of the group
+          const bool recv = lane >= np && t < cnt;
+          const int got = __shfl_sync(0xffffffffu, mine[x], recv ? nth_bit(bal, t) : 0u);
+          if (recv) pend = got;
+          np += cnt;
         }
       }
-      if (lane == 0) st[S_FCMP] += fcmp;
-      // (c) F against P: warp w takes candidate word w % nwords and one of the
-      // nw / nwords slices of the P log tail and of the index tiles
-      {
-        const unsigned pl = goal ? ld_volatile(&C->plog_len.v) : psnap;
-        if (goal && filtered)
-          group_ptest(v, w % nwords, nw / nwords, w / nwords, pfrom, pl, 0u);
-        else
-          group_ptest(v, w % nwords, nw / nwords, w / nwords, S.pd.count ? S.pd.mark : 0u, pl,
-                      S.pd.count ? S.pd.ntiles : 0u);
+      if (np) out = insert_batch(v, hv, load_batch(cs, pend), out, fb, cap, K1);
+      clear_groups(cs, v, nc);
+      if (lane == 0) {
+        cs.hcnt[v] = 0;
+        if (out != F) A.fcount[v] = out;
+        if (atomicOr(&cs.hflag[v], kSplitDone) & kSplitSeen) cs.hflag[v] = 0;
       }
-      __syncthreads();
-      // (d) survivors become labels, join alpha(v) and the next OPEN
-      const bool surv = tid < nb && (((S.halive[w % NW] & ~S.hkill[w % NW] & ~S.hpkill[w % NW]) >> lane) & 1u);
-      heavy_insert(v, K1, surv, out, fb, cap);
-      const bool more = S.m_more;
-      __syncthreads();  // the next group reuses the shared candidate arrays
-      if (!more) break;
+    }
+    if (lane == 0) {
+      st[S_FCMP] += fcmp;
+      st[S_PCMP] += pcmp;
     }
   }
 
-  // Survivors of a block merge (thread tid holds candidate tid in shared
-  // memory; surv tells whether it survived) become labels, join alpha(v) --
-  // out live entries at fb, cap, grown when full -- and the next OPEN, or at
-  // the goal node n the P log. Returns alpha(v)'s new size (the block must
-  // pass a barrier before the shared candidate arrays are reused).
-  __device__ unsigned heavy_insert(uint32_t v, CycleCtl& K1, bool surv, unsigned out, uint64_t fb, unsigned cap) {
-    const unsigned tid = threadIdx.x, lane = lane_id(), w = tid >> 5, nw = blockDim.x >> 5;
-    const bool goal = v == G.n;
-    const unsigned smask = __ballot_sync(0xffffffffu, surv);
-    if (lane == 0) S.warp[w] = __popc(smask);
-    __syncthreads();
-    unsigned pre = 0, ntot = 0;
-    for (unsigned q = 0; q < nw; ++q) {
-      const unsigned c = S.warp[q];
-      pre += q < w ? c : 0u;
-      ntot += c;
-    }
-    const unsigned rank = pre + __popc(smask & lanemask_lt());
-    if (tid == 0) {
-      S.m_ok = 0;
-      S.m_fb = fb;
-      S.m_cap = cap;
-      if (ntot) {
-        const unsigned lb = atomicAdd(&C->n_labels.v, ntot);
-        S.m_lb = lb;
-        if (lb + ntot > A.label_cap || lb + ntot > P.label_budget) {
-          set_error(C, (lb + ntot > A.label_cap) ? OPMOS_ERR_CAPACITY : OPMOS_ERR_BUDGET);
-        } else if (goal && ld_volatile(&C->plog_len.v) + ntot > A.plog_cap) {
-          set_error(C, OPMOS_ERR_CAPACITY);
-        } else {
-          atomicMax(&K1.lbase.v, lb + ntot);
-          S.m_ok = 1;
-          S.m_plen = goal ? ld_volatile(&C->plog_len.v) : 0u;  // this block is the log's only writer
-          if (out + ntot > cap) {  // grow: a new block of twice the size
-            const unsigned tile = P.tile;
-            unsigned ncap = max(2u * (out + ntot), tile);
-            ncap = (ncap + tile - 1) / tile * tile;
-            const unsigned long long nb0 = atomicAdd(&C->f_words.v, (unsigned long long)(D + 1) * ncap);
-            if (nb0 + (unsigned long long)(D + 1) * ncap > A.fpool_words) {
-              set_error(C, OPMOS_ERR_CAPACITY);
-              S.m_ok = 0;
-            } else {
-              S.m_fb = nb0;
-              S.m_cap = ncap;
-            }
-          }
-        }
-      }
-    }
-    __syncthreads();
-    const unsigned ok = S.m_ok;
-    if (ok) {
-      const uint64_t nfb = S.m_fb;
-      const unsigned ncap = S.m_cap;
-      if (nfb != fb) {
-        for (unsigned x = tid; x < out; x += blockDim.x)
-#pragma unroll
-          for (int k = 0; k <= D; ++k) A.fpool[nfb + (size_t)k * ncap + x] = A.fpool[fb + (size_t)k * cap + x];
-      }
-      if (surv) {
-        const unsigned id = S.m_lb + rank;
-        uint32_t c[D];
-#pragma unroll
-        for (int k = 0; k < D; ++k) c[k] = S.hc[k][tid];
-#pragma unroll
-        for (int k = 0; k < D; ++k) A.lg[(size_t)k * A.label_cap + id] = c[k];
-        A.lnode[id] = goal ? P.goal : v;
-        A.lparent[id] = S.hpar[tid];
-        A.ledge[id] = S.hedge[tid];
-        A.lpver[id] = psnap;
-        A.ldead[id] = kAlive;
-#pragma unroll
-        for (int k = 0; k < D; ++k) A.fpool[nfb + (size_t)k * ncap + out + rank] = c[k];
-        A.fpool[nfb + (size_t)D * ncap + out + rank] = id;
-        if (goal) {
-#pragma unroll
-          for (int k = 0; k < D; ++k) A.plog[(size_t)k * A.plog_cap + S.m_plen + rank] = c[k];
-        } else {
-          push_open(id, c, v, K1);
-        }
-      }
-      if (goal) {
-        __syncthreads();  // the log entries are written before they are published
-        if (tid == 0) {
-          __threadfence();
-          *reinterpret_cast<volatile unsigned*>(&C->plog_len.v) = S.m_plen + ntot;
-          atomicMax(&K1.plen.v, S.m_plen + ntot);
-        }
-      }
-      if (tid == 0) {
-        A.fbase[v] = nfb;
-        A.fcap[v] = ncap;
-        A.fcount[v] = out + ntot;
-        st[S_INSERTED] += ntot;
-      }
-    } else if (tid == 0) {
-      A.fcount[v] = out;
-    }
-    return ok ? out + ntot : out;
-  }
-
-  // Compaction of a frontier after a split merge: the entries whose label
-  // was pruned in this step (ldead == cyc, written by other blocks: read past
-  // L1) are removed; returns the live count. Rounds as in heavy_groups (b).
+  // Compaction of a frontier after a split merge, by one warp: the entries
+  // whose label was pruned in this step (ldead == cyc, written by other warps:
+  // read past L1) are removed; returns the live count.
   __device__ unsigned compact_pruned(uint64_t fb, unsigned cap, unsigned F) {
-    constexpr int U = kUH;
-    const unsigned lane = lane_id(), w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const unsigned R = nw * 32u * U;
+    constexpr int U = kU;
+    const unsigned lane = lane_id();
     unsigned out = 0;
-    for (unsigned r0 = 0; r0 < F; r0 += R) {
-      const unsigned base = r0 + w * 32u * U;
+    for (unsigned r0 = 0; r0 < F; r0 += 32 * U) {
       uint32_t m[U][D];
       uint32_t mid[U];
-      unsigned km[U], wtot = 0;
+      bool keep[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const unsigned i = base + u * 32 + lane;
+        const unsigned i = r0 + u * 32 + lane;
         const bool vm = i < F;
 #pragma unroll
         for (int k = 0; k < D; ++k) m[u][k] = vm ? A.fpool[fb + (size_t)k * cap + i] : 0u;
         mid[u] = vm ? A.fpool[fb + (size_t)D * cap + i] : 0u;
-        km[u] = __ballot_sync(0xffffffffu, vm && __ldcg(A.ldead + mid[u]) != cyc);
-        wtot += __popc(km[u]);
+        keep[u] = vm;
       }
-      if (lane == 0) S.warp[w] = wtot;
-      __syncthreads();  // (1) all reads of this round are done
-      const unsigned x = lane < nw ? S.warp[lane] : 0u;
-      unsigned incl = x;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= (unsigned)o) incl += y;
-      }
-      const unsigned wpre = __shfl_sync(0xffffffffu, incl - x, w);
-      const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
-      unsigned pos = out + wpre;
+      for (int u = 0; u < U; ++u) keep[u] = keep[u] && __ldcg(A.ldead + mid[u]) != cyc;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const unsigned i = base + u * 32 + lane;
-        const bool keep = (km[u] >> lane) & 1u;
-        const unsigned p = pos + __popc(km[u] & lanemask_lt());
-        if (keep && p != i) {
+        const unsigned i = r0 + u * 32 + lane;
+        const unsigned km = __ballot_sync(0xffffffffu, keep[u]);
+        const unsigned pos = out + __popc(km & lanemask_lt());
+        if (keep[u] && pos != i) {
 #pragma unroll
-          for (int k = 0; k < D; ++k) A.fpool[fb + (size_t)k * cap + p] = m[u][k];
-          A.fpool[fb + (size_t)D * cap + p] = mid[u];
+          for (int k = 0; k < D; ++k) A.fpool[fb + (size_t)k * cap + pos] = m[u][k];
+          A.fpool[fb + (size_t)D * cap + pos] = mid[u];
         }
-        pos += __popc(km[u]);
+        out += __popc(km);
       }
-      __syncthreads();  // (2) S.warp read by every warp
-      out += total;
     }
+    __syncwarp();
     return out;
-  }
-
-  // Shape of a merge split into k parts: ka shares of the candidates (ka
-  // divides k, each share kPartCands candidates or more) times kb = k / ka
-  // ranges of the frontier. Splitting the candidates keeps each candidate's
-  // early exit in one scan, so it is preferred.
-  __device__ static void part_shape(unsigned k, unsigned nc, unsigned& ka, unsigned& kb) {
-    const unsigned amax = max(1u, nc / kPartCands);
-    ka = 1;
-    for (unsigned x = 2; x <= k; ++x)
-      if (k % x == 0 && x <= amax) ka = x;
-    kb = k / ka;
-  }
-
-  // Part r of a block merge split into k parts (k >= 2; decided while the
-  // node's candidates arrived). With the shape (ka, kb), part r = b * ka + a
-  // takes share a of the candidates -- slots a, a + ka, ... and lists a,
-  // a + ka, ... -- kHC at a time, and frontier entries [b F / kb,
-  // (b+1) F / kb), read only:
-  //  (a) in-set resolution within each group;
-  //  (b) frontier entries a candidate strictly dominates are marked pruned
-  //      (ldead = cyc); candidates an entry weakly dominates die;
-  // and the candidates that died get cflag set. Each dies only when a
-  // candidate of its group or a frontier entry dominates it, and every entry
-  // some candidate strictly dominates is marked (dominance is transitive and
-  // the frontier is an antichain). The last part to finish (a counter per
-  // node; nobody waits) compacts the frontier if a part pruned, then merges
-  // the surviving candidates as one block merge does -- against each other,
-  // the entries it inserts and P -- so P tests only the survivors. At the goal
-  // node n, whose alpha is P, the parts split the candidates only and test
-  // them against P; the last part tests the survivors against the log
-  // entries it appends itself.
-  __device__ void merge_part(uint32_t v, unsigned r, unsigned k, CycleCtl& K1) {
-    constexpr int U = kUH;
-    constexpr unsigned NW = kHC / 32;
-    const CandSet& cs = A.cs[cyc & 1u];
-    const unsigned tid = threadIdx.x, lane = lane_id(), w = tid >> 5, nw = blockDim.x >> 5;
-    const unsigned F = A.fcount[v];
-    const unsigned nc = cs.ncand[v];
-    const uint64_t fb = A.fbase[v];
-    const unsigned cap = A.fcap[v];
-    const bool goal = v == G.n;  // no frontier ranges: the parts test their shares against P
-    unsigned ka = k, kb = 1;
-    if (!goal) part_shape(k, nc, ka, kb);
-    const unsigned a = r % ka, b = r / ka;
-    const unsigned lo = (unsigned)((uint64_t)F * b / kb), hi = goal ? 0u : (unsigned)((uint64_t)F * (b + 1) / kb);
-    const unsigned ns = min(nc, A.nslots), nl = nc - ns;
-    if (tid < 32) {  // this share's lists (the node's heads stay until the last part resets them)
-      const unsigned j = a + tid * ka;
-      S.hlist[tid] = (j < (1u << A.lsub) && j < nl) ? cs.node_head[((size_t)v << A.lsub) + j] : kNil;
-      if (tid == 0) S.mq_next = 0;
-    }
-    __syncthreads();
-    const unsigned nrows = ns > a ? (ns - a + ka - 1) / ka : 0u;
-    unsigned long long fcmp = 0;
-    bool any_pruned = false;
-    for (;;) {
-      const unsigned nb = gather_group(cs, v, nrows, a, ka, false);
-      if (nb == 0) break;
-      const unsigned nwords = (nb + 31) / 32;
-      load_group(cs, nb);
-      __syncthreads();
-      group_inset(nb);
-      __syncthreads();
-      // (b) the frontier range, read only, until no candidate of the group lives
-      for (unsigned r0 = lo + w * 32u * U; r0 < hi; r0 += nw * 32u * U) {
-        bool any = false;
-#pragma unroll
-        for (unsigned q = 0; q < NW; ++q) any |= q < nwords && (S.halive[q] & ~S.hkill[q]) != 0u;
-        if (!__any_sync(0xffffffffu, any)) break;
-        uint32_t m[U][D];
-        uint32_t mid[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned i = r0 + u * 32 + lane;
-          const bool vm = i < hi;
-#pragma unroll
-          for (int kk = 0; kk < D; ++kk) m[u][kk] = vm ? A.fpool[fb + (size_t)kk * cap + i] : kInf;
-          mid[u] = vm ? A.fpool[fb + (size_t)D * cap + i] : 0u;
-        }
-        unsigned kill[NW];
-#pragma unroll
-        for (unsigned q = 0; q < NW; ++q) kill[q] = 0;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const unsigned i0 = r0 + u * 32;
-          const bool vm = i0 + lane < hi;
-          bool pruned = false;
-          if (i0 < hi) {
-#pragma unroll
-            for (unsigned q = 0; q < NW; ++q) {
-              if (q >= nwords) break;
-              // one lane's view of the kills other warps add meanwhile
-              unsigned am = __shfl_sync(0xffffffffu, S.halive[q] & ~S.hkill[q] & ~kill[q], 0);
-              fcmp += (unsigned long long)__popc(am) * min(32u, hi - i0);
-              while (am) {
-                const unsigned j = __ffs(am) - 1;
-                am &= am - 1;
-                uint32_t cj[D];
-#pragma unroll
-                for (int kk = 0; kk < D; ++kk) cj[kk] = S.hc[kk][q * 32 + j];
-                const bool le_mc = vm && weakly_le<D>(m[u], cj);
-                const bool le_cm = vm && weakly_le<D>(cj, m[u]);
-                if (__ballot_sync(0xffffffffu, le_mc)) kill[q] |= 1u << j;
-                pruned |= le_cm && !le_mc;
-              }
-            }
-          }
-          if (vm && pruned) {
-            A.ldead[mid[u]] = cyc;
-            st[S_PRUNED]++;
-            any_pruned = true;
-          }
-        }
-        if (lane == 0) {
-#pragma unroll
-          for (unsigned q = 0; q < NW; ++q)
-            if (kill[q]) atomicOr(&S.hkill[q], kill[q]);
-        }
-      }
-      __syncthreads();
-      if (goal) {  // P as the parts see it: no part appends to the log
-        group_ptest(v, w % nwords, nw / nwords, w / nwords, S.pd.count ? S.pd.mark : 0u,
-                    ld_volatile(&C->plog_len.v), S.pd.count ? S.pd.ntiles : 0u);
-        __syncthreads();
-      }
-      if (tid < nb) {
-        const unsigned q = tid >> 5, bit = 1u << (tid & 31);
-        if (((S.hkill[q] | S.hpkill[q]) & bit) || !(S.halive[q] & bit)) cs.cflag[S.hcid[tid]] = 1u;
-      }
-      const bool more = S.m_more;
-      __syncthreads();  // the next group reuses the shared arrays
-      if (!more) break;
-    }
-    if (lane == 0) st[S_FCMP] += fcmp;
-    // the part counter's low 16 bits count finished parts; kPartPruned is
-    // added by a part that pruned a frontier entry
-    const unsigned pr = __syncthreads_or(any_pruned) ? kPartPruned : 0u;
-    __threadfence();
-    if (tid == 0) {
-      const unsigned c = atomicAdd(&cs.hcnt[v], 1u + pr) + 1u + pr;
-      S.m_ok = (c & (kPartPruned - 1u)) == k ? (c >= kPartPruned ? 2u : 1u) : 0u;
-    }
-    __syncthreads();
-    const unsigned ok = S.m_ok;
-    if (!ok) return;
-    // the last part of the node: the survivors of every share
-    __threadfence();
-    open_block_cursor(cs, v, false);
-    if (tid == 0) cs.hcnt[v] = 0;
-    unsigned out = F;
-    if (ok == 2u) {  // some part pruned an entry: compact
-      out = compact_pruned(fb, cap, F);
-      if (tid == 0) A.fcount[v] = out;
-    }
-    __syncthreads();
-    heavy_groups(v, K1, true, out, ld_volatile(&C->plog_len.v));
   }
 
   // ---------------- P index rebuild (three steps, then published) ----------------
@@ -1906,31 +1639,6 @@ struct Search {
     if (threadIdx.x == 0) C->pidx[(i + 1) & 1u] = nd;
   }
 
-  // Block-merge item t of a step: a part of a split merge (t < np), or a
-  // heavy node's whole merge, skipped when it is split.
-  __device__ void heavy_item(unsigned t, unsigned np, unsigned cur, CycleCtl& K1, bool split) {
-    const unsigned x = t < np ? A.cs[cur].xpart[t] : (t - np) << 4;
-    const unsigned h = x >> 4, r = x & 15u;
-    const unsigned k = A.cs[cur].hsplit[h];
-    const uint32_t v = A.cs[cur].touched[2u * A.cand_cap - 1u - h];
-    if (t >= np && k > 1u) return;
-    if (threadIdx.x == 0 && r == 0) {  // read before the merge clears them
-      S.tmax[3] = max(S.tmax[3], A.cs[cur].ncand[v]);
-      S.tmax[4] = max(S.tmax[4], A.fcount[v]);
-    }
-    const unsigned long long t0 = globaltimer();
-    if (split && k > 1u)
-      merge_part(v, r, k, K1);
-    else
-      merge_heavy(v, K1);
-    if (threadIdx.x == 0) {
-      const unsigned long long dt = globaltimer() - t0;
-      S.tmax[0] = max(S.tmax[0], (unsigned)min(dt, 0xFFFFFFFFull));
-      st[S_NHEAVY] += r == 0;
-      st[S_SUMH] += dt;
-    }
-  }
-
   // ---------------- one step ----------------
   // Returns false (on every block alike) when the search is over: OPEN_i
   // holds no entry and window i produced no candidate.
@@ -1966,11 +1674,11 @@ struct Search {
     __syncthreads();
     const unsigned* rec = S.rec;
     const unsigned head = rec[RW_HEAD], tail = rec[RW_OPEN];
-    const unsigned nt = rec[RW_TOUCHED], nh = rec[RW_HEAVY], np = rec[RW_PARTS];
+    const unsigned nt = rec[RW_TOUCHED], np = min(rec[RW_PARTS], A.xcap);
     const Measured ms{(unsigned long long)rec[RW_KEYHI] << 32 | rec[RW_KEYLO], rec[RW_F1LO], rec[RW_F1HI],
                       rec[RW_WMIN], rec[RW_WPREV], rec[RW_WMAX]};
     const unsigned n_in = min(tail - head, A.open_cap);  // FIFO: ring tail - head
-    if (n_in == 0 && nt == 0 && nh == 0) return false;
+    if (n_in == 0 && nt == 0) return false;
     cyc = i;
     fifo_head = head;
     const unsigned fwin = min(n_in, P.window);  // FIFO: ring positions window i+1 takes
@@ -2008,51 +1716,47 @@ struct Search {
       st[S_TSEL] += t - *tlap;
       *tlap = t;
     }
-    // block merges first (the longest single tasks): the parts of split
-    // merges (recorded in xpart while the candidates arrived), then one item
-    // per heavy node, skipped when the node's merge is split
-    // The first one of each block is its own number, later ones are claimed.
-    const unsigned nhi = np + nh, nblk = T.nblocks();
-    for (unsigned t = T.block(), turn = 0; t < nhi; turn ^= 1u) {
-      const unsigned mine = t;
-      heavy_item(mine, np, cur, K1, Team::kSplitMerges);
-      if (nhi <= nblk) break;
-      if (threadIdx.x == 0) S.claim[turn] = nblk + atomicAdd(&K0.heavy_next.v, 1u);
-      __syncthreads();
-      t = S.claim[turn];
-    }
-    // warp items: index-rank items, light merges, extraction chunks
+    // work items, one warp each: parts of split merges (the longest), index-rank
+    // items, merges, extraction chunks
     const PIdx& pd = S.pd;
     const unsigned nrank = (D >= 2 && pd.state == 1) ? ((pd.k + 31) / 32) * ((pd.k + kRankQ - 1) / kRankQ) : 0u;
-    const unsigned nopen = fifo ? fwin : n_in;
-    const unsigned per = item_entries(nopen, T.nwarps());
+    const unsigned nopen = fifo ? fwin : n_in, nwarps = T.nwarps();
+    const unsigned per = item_entries(nopen, nwarps);
     const unsigned nchunks = (nopen + per - 1) / per;
-    const unsigned nitems = nrank + nt + nchunks;
+    const unsigned nitems = np + nrank + nt + nchunks;
     const unsigned lane = lane_id();
-    // While less than half of the blocks have a block merge and two rounds are
-    // enough, the warps of the others take the items by number (claims by every
-    // warp at once queue on one counter: 2 us to start, 2 us to learn that
-    // nothing is left); otherwise all warps claim them one by one.
-    const unsigned wpb = blockDim.x >> 5;
-    const bool bynum = 2u * nhi < nblk && nitems <= 2u * (nblk - nhi) * wpb;
-    const unsigned own = (nblk - nhi) * wpb;  // warps that take items by number
-    unsigned t = T.block() >= nhi ? T.wid() - nhi * wpb : nitems;
-    for (;; t += own) {
-      if (!bynum) {
-        if (lane == 0) t = atomicAdd(&K0.work_next.v, 1u);
-        t = __shfl_sync(0xffffffffu, t, 0);
-      }
-      if (t >= nitems) break;
+    // The first item of a warp goes by its number, neighbouring items to
+    // different blocks; the rest is claimed (claims by every warp at once queue
+    // on one counter: 2 us).
+    for (unsigned t = (threadIdx.x >> 5) * T.nblocks() + T.block(); t < nitems;) {
       const unsigned long long t0 = globaltimer();
-      if (t < nrank) {
-        rank_item(t);
-      } else if (t < nrank + nt) {
-        const uint32_t v = A.cs[cur].touched[t - nrank];
+      if (t < np) {
+        const uint2 x = A.cs[cur].xpart[t];
+        const uint32_t v = x.x;
+        if (v != kNoPart) {
+          const unsigned r = x.y, k = A.cs[cur].hflag[v] & kSplitParts;
+          if (lane == 0 && r == 0) {  // read before the merge clears them
+            atomicMax(&S.tmax[3], A.cs[cur].ncand[v]);
+            atomicMax(&S.tmax[4], A.fcount[v]);
+            st[S_NHEAVY]++;
+          }
+          __syncwarp();
+          merge_part(v, r, k, K1);
+          if (lane == 0) {
+            const unsigned long long dt = globaltimer() - t0;
+            atomicMax(&S.tmax[0], (unsigned)min(dt, 0xFFFFFFFFull));
+            st[S_SUMH] += dt;
+          }
+        }
+      } else if (t < np + nrank) {
+        rank_item(t - np);
+      } else if (t < np + nrank + nt) {
+        const uint32_t v = A.cs[cur].touched[t - np - nrank];
         uint32_t* hf = A.cs[cur].hflag + v;
-        const uint32_t listed = *hf;
-        __syncwarp();  // every lane has read it before lane 0 clears it
-        if (listed) {
-          if (lane == 0) *hf = 0;  // merged by a block this step
+        const uint32_t split = *hf;
+        __syncwarp();  // every lane has read it before lane 0 changes it
+        if (split) {  // merged in parts this step; this item or the last part clears the word
+          if (lane == 0 && (atomicOr(hf, kSplitSeen) & kSplitDone)) *hf = 0;
         } else {
           merge_node(v, K1);
         }
@@ -2062,7 +1766,7 @@ struct Search {
           st[S_SUML] += dt;
         }
       } else {
-        const unsigned c = t - nrank - nt;
+        const unsigned c = t - np - nrank - nt;
         if (fifo)
           extract_fifo(head + c * per, head + min(fwin, (c + 1) * per), K1);
         else
@@ -2073,6 +1777,9 @@ struct Search {
           st[S_SUMX] += dt;
         }
       }
+      if (nitems <= nwarps) break;
+      if (lane == 0) t = nwarps + atomicAdd(&K0.work_next.v, 1u);
+      t = __shfl_sync(0xffffffffu, t, 0);
     }
     index_strided_work(T);
     __syncthreads();
@@ -2323,7 +2030,6 @@ __global__ void __launch_bounds__(NT, NB) search_grid_kernel(GraphDev G, QArena 
 // work, at least one block), so large and small queries advance side by side.
 // ---------------------------------------------------------------------------
 struct SubTeam {
-  static constexpr bool kSplitMerges = false;  // a query's arena has kparts = 1
   unsigned j, nb;
   __device__ __forceinline__ unsigned tid() const { return j * blockDim.x + threadIdx.x; }
   __device__ __forceinline__ unsigned nthreads() const { return nb * blockDim.x; }
@@ -2380,8 +2086,7 @@ __device__ void mq_alloc_region1(const MSlot& sl, QCtl* C) {
 
 __device__ __forceinline__ bool step_empty(const QCtl* C, unsigned i) {
   const CycleCtl& K = C->cyc[i % 3];
-  return ld_volatile(&K.open_count.v) == ld_volatile(&K.head.v) && ld_volatile(&K.touched_count.v) == 0 &&
-         ld_volatile(&K.heavy_count.v) == 0;
+  return ld_volatile(&K.open_count.v) == ld_volatile(&K.head.v) && ld_volatile(&K.touched_count.v) == 0;
 }
 
 // Work units of a slot that enters the iteration in state st (0: none). INIT
@@ -2397,7 +2102,7 @@ __device__ __forceinline__ unsigned mq_weight(const MSlot& sl, const QCtl* C, un
   if (st >= SL_OUT1) return max(1u, ld_volatile(&C->res_count) + ld_volatile(sl.A.fcount + sl.G.n));
   const CycleCtl& K = C->cyc[C->step % 3];
   const unsigned w = (ld_volatile(&K.open_count.v) - ld_volatile(&K.head.v)) + ld_volatile(&K.touched_count.v) +
-                     8u * ld_volatile(&K.heavy_count.v);
+                     ld_volatile(&K.part_count.v);
   return w ? w : 1u;  // a running slot always gets a block
 }
 
@@ -2598,43 +2303,52 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
 // ---------------------------------------------------------------------------
 // host launchers, explicitly instantiated per objective count
 // ---------------------------------------------------------------------------
+// Dynamic shared memory of a block of nt threads (the warps' rows), with the
+// kernel allowed that much.
+template <int D>
+size_t row_bytes(const void* kernel, unsigned nt, size_t at_least = 0) {
+  const size_t bytes = std::max(at_least, (size_t)nt * detail::Search<D>::RP * 4);
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  return bytes;
+}
+
 template <int D>
 cudaError_t launch_grid(const GraphDev& G, const QArena& A, QCtl* C, const QParams& P, const OutPool& O,
                         QResult* R, bool wide, unsigned blocks, cudaStream_t s) {
   void* args[] = {(void*)&G, (void*)&A, (void*)&C, (void*)&P, (void*)&O, (void*)&R};
-  if (wide)
-    return cudaLaunchCooperativeKernel(
-        (void*)detail::search_grid_kernel<D, kGridWideThreads, kGridWideBlocksPerSM>, dim3(blocks),
-        dim3(kGridWideThreads), args, 0, s);
-  return cudaLaunchCooperativeKernel((void*)detail::search_grid_kernel<D, kGridThreads, 1>, dim3(blocks),
-                                     dim3(kGridThreads), args, 0, s);
+  const void* kernel = wide ? (const void*)detail::search_grid_kernel<D, kGridWideThreads, kGridWideBlocksPerSM>
+                            : (const void*)detail::search_grid_kernel<D, kGridThreads, 1>;
+  const unsigned nt = wide ? kGridWideThreads : kGridThreads;
+  return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(nt), args, row_bytes<D>(kernel, nt), s);
 }
 
 template <int D>
 int grid_occupancy(bool wide) {
+  const void* kernel = wide ? (const void*)detail::search_grid_kernel<D, kGridWideThreads, kGridWideBlocksPerSM>
+                            : (const void*)detail::search_grid_kernel<D, kGridThreads, 1>;
+  const unsigned nt = wide ? kGridWideThreads : kGridThreads;
   int nb = 0;
-  if (wide)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &nb, detail::search_grid_kernel<D, kGridWideThreads, kGridWideBlocksPerSM>, kGridWideThreads, 0);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, detail::search_grid_kernel<D, kGridThreads, 1>,
-                                                  kGridThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, (int)nt, row_bytes<D>(kernel, nt));
   return nb;
 }
 
 template <int D>
 cudaError_t launch_multi_d(MSlot* slots, QCtl* ctls, unsigned nslots, const MQuery* queue, unsigned* hctl,
                            const GraphDev* graphs, QResult* results, unsigned* done_flags, MCtl* M, unsigned blocks,
-                           cudaStream_t s) {
+                           size_t smem, cudaStream_t s) {
   void* args[] = {(void*)&slots, (void*)&ctls, (void*)&nslots, (void*)&queue, (void*)&hctl,
                   (void*)&graphs, (void*)&results, (void*)&done_flags, (void*)&M};
-  return cudaLaunchCooperativeKernel((void*)detail::multi_kernel<D>, dim3(blocks), dim3(kMultiThreads), args, 0, s);
+  const void* kernel = (const void*)detail::multi_kernel<D>;
+  return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kMultiThreads), args,
+                                     row_bytes<D>(kernel, kMultiThreads, smem), s);
 }
 
 template <int D>
-int multi_occupancy_d() {
+int multi_occupancy_d(size_t smem) {
+  const void* kernel = (const void*)detail::multi_kernel<D>;
   int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, detail::multi_kernel<D>, kMultiThreads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, (int)kMultiThreads,
+                                                row_bytes<D>(kernel, kMultiThreads, smem));
   return nb;
 }
 

@@ -14,8 +14,8 @@ namespace opmos {
                                       QResult*, bool, unsigned, cudaStream_t);                                   \
   template int grid_occupancy<D>(bool);                                                                         \
   template cudaError_t launch_multi_d<D>(MSlot*, QCtl*, unsigned, const MQuery*, unsigned*, const GraphDev*,     \
-                                         QResult*, unsigned*, MCtl*, unsigned, cudaStream_t);                   \
-  template int multi_occupancy_d<D>();
+                                         QResult*, unsigned*, MCtl*, unsigned, size_t, cudaStream_t);           \
+  template int multi_occupancy_d<D>(size_t);
 
 #define OPMOS_IN_GROUP(D) (OPMOS_D_FIRST <= (D) && (D) <= OPMOS_D_LAST)
 #if OPMOS_IN_GROUP(1)

@@ -39,9 +39,9 @@ T* take(char*& p, size_t count) {
   return reinterpret_cast<T*>(a);
 }
 
-// One node (node 0) merged as in step 0: one warp or the whole block.
+// One node (node 0) merged as in step 0 by one warp: whole, or part by part.
 template <int D>
-__global__ void __launch_bounds__(kGridThreads, 1) merge_hook_kernel(GraphDev G, QArena A, QCtl* C, QParams P,
+__global__ void __launch_bounds__(32, 1) merge_hook_kernel(GraphDev G, QArena A, QCtl* C, QParams P,
                                                                      OutPool O, unsigned lbase, unsigned block) {
   __shared__ Shared S;
   Search<D> X(G, A, C, P, O, S);
@@ -54,14 +54,9 @@ __global__ void __launch_bounds__(kGridThreads, 1) merge_hook_kernel(GraphDev G,
     for (int i = 0; i < kNB; ++i) S.hist[i] = 0;
   }
   __syncthreads();
-  if (block >= 2) {  // a merge split into `block` parts, one after the other (the last one finishes)
-    for (unsigned r = 0; r < block; ++r) {
-      X.merge_part(0u, r, block, C->cyc[1]);
-      __syncthreads();
-    }
-  } else if (block) {
-    X.merge_heavy(0u, C->cyc[1]);
-  } else if (threadIdx.x < 32) {
+  if (block) {  // a merge split into `block` parts, one after the other (the last one finishes)
+    for (unsigned r = 0; r < block; ++r) X.merge_part(0u, r, block, C->cyc[1]);
+  } else {
     X.merge_node(0u, C->cyc[1]);
   }
 }
@@ -74,9 +69,9 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   const uint32_t label_cap = nfront + ncand + 64, cand_cap = ncand + 64, open_cap = ncand + 64;
   const uint32_t fcap0 = (nfront + 31) / 32 * 32 + 32;
   const size_t fpool_words = (size_t)(D + 1) * (fcap0 + 4 * (nfront + ncand) + 256);
-  size_t bytes = 64 * 256 + sizeof(QCtl) + (size_t)D * 4 * (n + 1) + 8 * 4 * (n + 1) +
+  size_t bytes = 80 * 256 + sizeof(QCtl) + (size_t)D * 4 * (n + 1) + 8 * 4 * (n + 1) +
                  2 * (4 * (n + 1) * (3 + slots + (1u << lsub))) +
-                 2 * (size_t)cand_cap * (32 + 4 * D) + 2 * 4 * (n + 1) + (size_t)label_cap * (4 * D + 20) + fpool_words * 4 +
+                 2 * (size_t)cand_cap * (40 + 4 * D) + 2 * 4 * (n + 1) + (size_t)label_cap * (4 * D + 20) + fpool_words * 4 +
                  2 * (size_t)open_cap * 12 + 3 * kNB * 4 + kPSMax * 4 + 64 * 4 * D * 6;
   DevBuf mem;
   cudaError_t e = cudaMalloc(&mem.p, bytes);
@@ -89,20 +84,18 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   A.fbase = take<uint64_t>(p, n + 1);
   A.fcount = take<uint32_t>(p, n + 1);
   A.fcap = take<uint32_t>(p, n + 1);
+  for (int b = 0; b < 2; ++b) A.champ[b] = take<uint32_t>(p, (n + 1) * row_words(D));
   for (int b = 0; b < 2; ++b) {
     CandSet& cs = A.cs[b];
     cs.ncand = take<uint32_t>(p, n + 1);
     cs.node_head = take<int32_t>(p, (size_t)(n + 1) << lsub);
     cs.hflag = take<uint32_t>(p, n + 1);
     cs.hcnt = take<uint32_t>(p, n + 1);
-    cs.hsplit = take<uint32_t>(p, cand_cap);
     cs.cflag = take<uint32_t>(p, cand_cap);
     cs.cslot = take<int32_t>(p, (size_t)(n + 1) * slots);
-    cs.cparent = take<uint32_t>(p, cand_cap);
-    cs.cedge = take<uint32_t>(p, cand_cap);
     cs.cnext = take<int32_t>(p, cand_cap);
     cs.touched = take<uint32_t>(p, 2 * (size_t)cand_cap);
-    cs.cg = take<uint32_t>(p, (size_t)cand_cap * D);
+    cs.crow = take<uint32_t>(p, (size_t)cand_cap * row_words(D + 2));
   }
   A.lg = take<uint32_t>(p, (size_t)label_cap * D);
   A.lnode = take<uint32_t>(p, label_cap);
@@ -124,6 +117,7 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   A.open_cap = open_cap;
   A.win_cap = cand_cap;
   A.cand_cap = cand_cap;
+  A.touch_cap = cand_cap;
   A.plog_cap = 64;
   A.fpool_words = fpool_words;
   A.nslots = slots;
@@ -141,13 +135,14 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
     }
     fimg[(size_t)D * fcap0 + i] = i;
   }
-  std::vector<uint32_t> cpar(cand_cap, 0), cedge(cand_cap, 0), cg((size_t)cand_cap * D, 0);
+  const uint32_t cw = row_words(D + 2);
+  std::vector<uint32_t> crow((size_t)cand_cap * cw, 0);
   std::vector<int32_t> cnext(cand_cap, kNil), cslot((size_t)(n + 1) * slots, kNil),
       head((size_t)(n + 1) << lsub, kNil);
   for (uint32_t j = 0; j < ncand; ++j) {
-    cpar[j] = j;
-    cedge[j] = arc[j];
-    for (int k = 0; k < D; ++k) cg[(size_t)k * cand_cap + j] = cand[(size_t)j * D + k];
+    for (int k = 0; k < D; ++k) crow[(size_t)j * cw + k] = cand[(size_t)j * D + k];
+    crow[(size_t)j * cw + D] = arc[j];
+    crow[(size_t)j * cw + D + 1] = j;
     if (j < slots) {
       cslot[j] = (int32_t)j;
     } else {  // list (j - slots) mod 2^lsub, newest first, as the expansion's exchanges leave it
@@ -185,10 +180,8 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   up(cs.ncand, ncand_v, 8);
   up(cs.node_head, head.data(), head.size() * 4);
   up(cs.cslot, cslot.data(), cslot.size() * 4);
-  up(cs.cparent, cpar.data(), cpar.size() * 4);
-  up(cs.cedge, cedge.data(), cedge.size() * 4);
   up(cs.cnext, cnext.data(), cnext.size() * 4);
-  up(cs.cg, cg.data(), cg.size() * 4);
+  up(cs.crow, crow.data(), crow.size() * 4);
   std::vector<int32_t> nil1((size_t)(n + 1) << lsub, kNil);
   up(A.cs[1].node_head, nil1.data(), nil1.size() * 4);
   if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook upload: %s", cudaGetErrorString(e));
@@ -205,10 +198,9 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   P.label_budget = label_cap;
   P.qd = D;
   P.ps_grow = 6;
-  P.heavy_work = kHeavyWork;
-  P.part_work = kPartWork;
+  P.part_work = part_work(D);
   OutPool O{nullptr, 0, nullptr};
-  merge_hook_kernel<D><<<1, kGridThreads>>>(G, A, C, P, O, nfront, block);
+  merge_hook_kernel<D><<<1, 32, 32 * Search<D>::RP * 4>>>(G, A, C, P, O, nfront, block);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook kernel: %s", cudaGetErrorString(e));
@@ -270,7 +262,7 @@ int opmos_test_merge(uint32_t d, uint32_t nfront, const uint32_t* front, uint32_
     if (!out_cost || !out_origin || !out_count || (nfront && !front) || (ncand && (!cand || !cand_arc)))
       return hook_fail(OPMOS_ERR_INVALID_ARG, "NULL argument");
     if (slots == 0 || slots > 4096) return hook_fail(OPMOS_ERR_INVALID_ARG, "slots must be in [1, 4096]");
-    if (block > kPartsMax) return hook_fail(OPMOS_ERR_INVALID_ARG, "block must be 0..%u", kPartsMax);
+    if (block > 16u) return hook_fail(OPMOS_ERR_INVALID_ARG, "block must be 0..16");
     if (nfront > (1u << 20) || ncand > (1u << 20)) return hook_fail(OPMOS_ERR_INVALID_ARG, "inputs too large");
     unsigned lsub = 0;
     while ((1u << lsub) < lists && lsub < 5) ++lsub;
@@ -309,8 +301,8 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
       return hook_fail(OPMOS_ERR_INVALID_ARG, "bad window, bins or size");
     constexpr int D = 2;
     const uint32_t cap = n + 64;
-    size_t bytes = 64 * 256 + sizeof(QCtl) + 4 * 2 * 3 + 4 * 3 * 16 + 2 * (size_t)cap * 12 + (size_t)cap * (4 * D + 20) +
-                   3 * kNB * 4 + 2 * ((size_t)cap * (32 + 4 * D) + 4 * 3 * 44) + 64 * 4 * D * 6 + kPSMax * 4;
+    size_t bytes = 80 * 256 + sizeof(QCtl) + 4 * 2 * 3 + 4 * 3 * 16 + 2 * (size_t)cap * 12 + (size_t)cap * (4 * D + 20) +
+                   3 * kNB * 4 + 2 * ((size_t)cap * (40 + 4 * D) + 4 * 3 * 44) + 64 * 4 * D * 6 + kPSMax * 4;
     DevBuf mem;
     cudaError_t e = cudaMalloc(&mem.p, bytes);
     if (e != cudaSuccess) return hook_fail(OPMOS_ERR_OUT_OF_MEMORY, "test hook: %s", cudaGetErrorString(e));
@@ -324,20 +316,18 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
     A.fbase = take<uint64_t>(p, 3);
     A.fcount = take<uint32_t>(p, 3);
     A.fcap = take<uint32_t>(p, 3);
+    for (int b = 0; b < 2; ++b) A.champ[b] = take<uint32_t>(p, 3 * row_words(D));
     for (int b = 0; b < 2; ++b) {
       CandSet& cs = A.cs[b];
       cs.ncand = take<uint32_t>(p, 3);
       cs.node_head = take<int32_t>(p, 3);
       cs.hflag = take<uint32_t>(p, 3);
       cs.hcnt = take<uint32_t>(p, 3);
-      cs.hsplit = take<uint32_t>(p, cap);
       cs.cflag = take<uint32_t>(p, cap);
       cs.cslot = take<int32_t>(p, 3 * 32);
-      cs.cparent = take<uint32_t>(p, cap);
-      cs.cedge = take<uint32_t>(p, cap);
       cs.cnext = take<int32_t>(p, cap);
       cs.touched = take<uint32_t>(p, 2 * (size_t)cap);
-      cs.cg = take<uint32_t>(p, (size_t)cap * D);
+      cs.crow = take<uint32_t>(p, (size_t)cap * row_words(D + 2));
     }
     A.lg = take<uint32_t>(p, (size_t)cap * D);
     A.lnode = take<uint32_t>(p, cap);
@@ -359,6 +349,7 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
     A.open_cap = cap;
     A.win_cap = cap;  // no cap on the window here: the bins alone decide
     A.cand_cap = cap;
+    A.touch_cap = cap;
     A.plog_cap = 64;
     A.fpool_words = 64;
     A.nslots = 32;
@@ -406,12 +397,11 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
     P.label_budget = cap;
     P.qd = D;
     P.ps_grow = 6;
-    P.heavy_work = kHeavyWork;
-    P.part_work = kPartWork;
+    P.part_work = part_work(D);
     const BinParams bp{bins[0], bins[1], bins[2], bins[3], bins[4]};
     OutPool O{nullptr, 0, nullptr};
     window_hist_kernel<<<64, 256>>>(A, n, bp, A.hist + 1 * kNB);
-    window_hook_kernel<<<1, kGridThreads>>>(G, A, C, P, O, n, bp, d_bstar);
+    window_hook_kernel<<<1, kGridThreads, kGridThreads * Search<2>::RP * 4>>>(G, A, C, P, O, n, bp, d_bstar);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook kernel: %s", cudaGetErrorString(e));
