@@ -81,17 +81,6 @@ __device__ __forceinline__ unsigned long long warp_min64(unsigned long long x) {
   return (unsigned long long)hi << 32 | lo;
 }
 
-__device__ __forceinline__ void flush_stats(QCtl* C, unsigned long long (&st)[kNStat]) {
-#pragma unroll
-  for (int i = 0; i < kNStat; ++i) {
-    unsigned long long v = st[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane_id() == 0 && v) atomicAdd(&C->stats[i], v);
-    st[i] = 0;
-  }
-}
-
 // Block-wide exclusive scan of one value per thread; returns the block total.
 __device__ inline unsigned block_exclusive_scan(unsigned x, unsigned* s_warp, unsigned& total) {
   const unsigned lane = lane_id(), w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -139,9 +128,22 @@ struct Shared {
   unsigned win_min, win_max, f1lo, f1hi;
   unsigned rec[32];    // the step's record (RecWord)
   PIdx pd;             // the P index as this step sees it
+  unsigned cnt[kNStat];  // this block's counters since the last flush (see flush_counts)
   unsigned tmax[5];    // this block's longest merge part, merge, extraction item (ns); most
                        // candidates and largest frontier of its split merges
 };
+
+// Adds the block's counters to the query's. Every thread calls it, between
+// block barriers that separate it from the counting. (Counters in shared memory
+// are added to by one lane a work item; 26 of 64 bits in every thread took 52
+// registers.) With `full` set only the ones near their 32 bits are added.
+__device__ __forceinline__ void flush_counts(QCtl* C, Shared& S, unsigned full = 1u) {
+  const unsigned i = threadIdx.x - 64u;
+  if (i < (unsigned)kNStat && S.cnt[i] >= full) {
+    atomicAdd(&C->stats[i], (unsigned long long)S.cnt[i]);
+    S.cnt[i] = 0;
+  }
+}
 
 // Histogram bin of an OPEN key (F0 << 32 | F1): the key's cell is
 // q * kSub + x, q = (F0 - b0) / delta its F[0] bucket and x = (F1 - b1) >> s1
@@ -192,7 +194,6 @@ struct Search {
   const QParams& P;
   const OutPool& O;
   Shared& S;
-  unsigned long long st[kNStat];
   // fixed for one step
   unsigned cyc = 0;    // step number i
   unsigned psnap = 0;  // P-log prefix every F-against-P test of step i uses
@@ -202,9 +203,12 @@ struct Search {
 
   __device__ Search(const GraphDev& g, const QArena& a, QCtl* c, const QParams& p, const OutPool& o,
                     Shared& s)
-      : G(g), A(a), C(c), P(p), O(o), S(s) {
-#pragma unroll
-    for (int i = 0; i < kNStat; ++i) st[i] = 0;
+      : G(g), A(a), C(c), P(p), O(o), S(s) {}
+
+  __device__ __forceinline__ void count(int what, unsigned n) const { atomicAdd(&S.cnt[what], n); }
+  // One lane counts for the warp.
+  __device__ __forceinline__ void count_lane0(int what, unsigned n) const {
+    if (lane_id() == 0 && n) atomicAdd(&S.cnt[what], n);
   }
 
   // h_k(v) and c_k(e); objectives the query does not use read as 0, which
@@ -317,7 +321,7 @@ struct Search {
     C->fifo_tail.v = K.open_count.v;
     C->plog_len.v = (s == t) ? 1u : 0u;
     K.plen.v = C->plog_len.v;
-    st[S_INSERTED] += 1;
+    count(S_INSERTED, 1u);
   }
 
   // ---------------- window selection (Algorithm 2: NUM_POP lowest labels) ----------------
@@ -445,7 +449,7 @@ struct Search {
       } else {  // list (pos - nslots) mod 2^lsub of the node, so all its lists grow evenly
         const unsigned j = (pos - A.nslots) & ((1u << A.lsub) - 1u);
         cs.cnext[c] = atomicExch(&cs.node_head[((size_t)v2 << A.lsub) + j], (int)c);
-        st[S_OVF]++;
+        count(S_OVF, 1u);
       }
     }
     // Every node is listed once, on its first candidate (one warp merges it). A
@@ -525,7 +529,7 @@ struct Search {
   }
   // Lazy PruneOPEN: F against the goal costs logged since the label's last
   // check (through the P index when that check predates it).
-  __device__ __forceinline__ bool still_open(bool want, const Label& l, unsigned long long& pcmp) {
+  __device__ __forceinline__ bool still_open(bool want, const Label& l, unsigned& pcmp) {
     const unsigned since = warp_min(want ? l.since : kInf);
     bool alive = want;
     if (since < psnap) {
@@ -553,6 +557,7 @@ struct Search {
     unsigned L = P.lanes;
     while (L < 32u && __popc(hits) * L <= 16u) L <<= 1;
     const unsigned lane = lane_id(), groups = 32u / L, grp = lane / L, gl = lane % L;
+    unsigned arcs = 0;
     while (hits) {
       const unsigned src = nth_bit(hits, grp);
       const bool has = src < 32u;
@@ -567,6 +572,7 @@ struct Search {
       const unsigned rounds = warp_max(deg);
       for (unsigned r = 0; r < rounds; r += L) {
         bool alive = gl + r < deg;
+        arcs += __popc(__ballot_sync(0xffffffffu, alive && !goal));
         uint32_t v2 = G.n, par = lid, e = e0 + gl + r, g2[D];
 #pragma unroll
         for (int k = 0; k < D; ++k) g2[k] = g[k];
@@ -579,7 +585,6 @@ struct Search {
             v2 = __ldg(G.col + e);
 #pragma unroll
             for (int k = 0; k < D; ++k) g2[k] += ck(k, e);
-            st[S_CAND]++;
           }
           fc = A.fcount[v2];
           if (!goal) {
@@ -594,6 +599,7 @@ struct Search {
       }
       for (unsigned r = 0; r < groups && hits; ++r) hits &= hits - 1;
     }
+    count_lane0(S_CAND, arcs);
   }
 
   // ---------------- extraction of window i+1 from OPEN_i ----------------
@@ -634,21 +640,19 @@ struct Search {
       id = A.oid[cur][i];
       dead = A.ldead[id];
       want = bin_of(key, bp) <= S.bstar;
-      st[S_OSCAN]++;
     }
     const Label own = load_label(want, id);
-    if (valid) {
-      if (dead < cyc) {
-        st[S_DEAD]++;
-        want = false;
-      } else {
-        keep = !want;
-      }
-    }
-    unsigned long long pcmp = 0;
+    const bool gone = valid && dead < cyc;
+    if (gone)
+      want = false;
+    else
+      keep = valid && !want;
+    unsigned pcmp = 0;
     bool take = still_open(want, own, pcmp);
-    st[S_PCMP] += pcmp;
-    if (want && !take) st[S_GOALPRUNED]++;
+    count_lane0(S_PCMP, pcmp);
+    count_lane0(S_OSCAN, __popc(__ballot_sync(0xffffffffu, valid)));
+    count_lane0(S_DEAD, __popc(__ballot_sync(0xffffffffu, gone)));
+    count_lane0(S_GOALPRUNED, __popc(__ballot_sync(0xffffffffu, want && !take)));
     if (n_in > A.win_cap && take) {  // else the window cannot be full
       if (agg_inc(&K1.win_count.v) >= A.win_cap) {
         take = false;
@@ -662,7 +666,7 @@ struct Search {
     if (km && lane == 0) ob = atomicAdd(&K1.open_count.v, __popc(km));
     const unsigned tm = __ballot_sync(0xffffffffu, take);
     if (tm) {
-      if (take) st[S_EXTRACTED]++;
+      count_lane0(S_EXTRACTED, __popc(tm));
       const unsigned wmin = warp_min(take ? (unsigned)(key >> 32) : kInf);
       const unsigned wmax = warp_max(take ? (unsigned)(key >> 32) : 0u);
       if (lane == 0) {
@@ -678,7 +682,6 @@ struct Search {
         if (o < A.open_cap) {
           A.okey[nxt][o] = key;
           A.oid[nxt][o] = id;
-          st[S_OKEEP]++;
           const unsigned b = bin_of(key, bpn);
           atomicAdd(&S.hist[b], 1u);
           inbins = b < (unsigned)kNB - 1;
@@ -686,6 +689,7 @@ struct Search {
           set_error(C, OPMOS_ERR_CAPACITY);
         }
       }
+      count_lane0(S_OKEEP, __popc(km));
       const unsigned long long kmin = warp_min64(keep ? key : ~0ull);
       const unsigned f1lo = warp_min(inbins ? (uint32_t)key : kInf), f1hi = warp_max(inbins ? (uint32_t)key : 0u);
       if (lane == 0) {
@@ -711,16 +715,16 @@ struct Search {
     if (valid) {
       id = A.oid[0][pos % A.open_cap];
       dead = A.ldead[id];
-      st[S_OSCAN]++;
     }
     const Label own = load_label(valid, id);
     const bool want = valid && dead >= cyc;
-    if (valid && !want) st[S_DEAD]++;
-    unsigned long long pcmp = 0;
+    unsigned pcmp = 0;
     const bool take = still_open(want, own, pcmp);
-    st[S_PCMP] += pcmp;
-    if (want && !take) st[S_GOALPRUNED]++;
-    if (take) st[S_EXTRACTED]++;
+    count_lane0(S_PCMP, pcmp);
+    count_lane0(S_OSCAN, __popc(__ballot_sync(0xffffffffu, valid)));
+    count_lane0(S_DEAD, __popc(__ballot_sync(0xffffffffu, valid && !want)));
+    count_lane0(S_GOALPRUNED, __popc(__ballot_sync(0xffffffffu, want && !take)));
+    count_lane0(S_EXTRACTED, __popc(__ballot_sync(0xffffffffu, take)));
     expand_labels(take, own, cs, K1);
   }
 
@@ -801,9 +805,9 @@ struct Search {
   // outright.
   static constexpr bool kPFlat = D > 6;
   __device__ void p_filter(bool& alive, const uint32_t (&F)[D], unsigned t0, unsigned t1, unsigned pcount,
-                           unsigned tlo, unsigned thi, unsigned pbuf, unsigned long long& pcmp) {
+                           unsigned tlo, unsigned thi, unsigned pbuf, unsigned& pcmp) {
     const unsigned lane = lane_id();
-    unsigned long long cnt = 0;
+    unsigned cnt = 0;
     unsigned am = __ballot_sync(0xffffffffu, alive);
     if (!am || (t0 >= t1 && tlo >= thi)) return;
     const uint32_t* ps = A.ps[pbuf];
@@ -825,7 +829,7 @@ struct Search {
 #pragma unroll
         for (int k = 0; k < D; ++k) tm[k] = tg + lane < thi ? pst[(size_t)k * tcap + tg + lane] : kInf;
       }
-      cnt += (unsigned long long)__popc(am) * min(32u, thi - tg);
+      cnt += __popc(am) * min(32u, thi - tg);
       unsigned pm = 0;  // lane j: the tiles candidate j still has to be tested against
       for (unsigned todo = am; todo;) {
         unsigned j[2];
@@ -887,7 +891,7 @@ struct Search {
 
   // The rows of am against entries [t0, t1) of a list of goal costs, all of them.
   __device__ __forceinline__ void p_scan(unsigned& am, const uint32_t* list, unsigned t0, unsigned t1,
-                                         unsigned long long& cnt) const {
+                                         unsigned& cnt) const {
     const unsigned lane = lane_id();
     for (unsigned r0 = t0; r0 < t1 && am; r0 += 32 * kU) {
       uint32_t pt[kU][D];
@@ -897,7 +901,7 @@ struct Search {
 #pragma unroll
         for (int k = 0; k < D; ++k) pt[u][k] = jj < t1 ? list[(size_t)k * A.plog_cap + jj] : kInf;
       }
-      cnt += (unsigned long long)__popc(am) * min(32u * kU, t1 - r0);
+      cnt += __popc(am) * min(32u * kU, t1 - r0);
       const int nu = (int)min((unsigned)kU, (t1 - r0 + 31) / 32);
       for (unsigned todo = am; todo;) {
         unsigned j[2];
@@ -1012,7 +1016,7 @@ struct Search {
   // once a round: 2 D compares a pair and a vote for two candidates.
   template <bool WRITE>
   __device__ unsigned scan_frontier(uint32_t v, Batch& b, unsigned lo, unsigned hi, uint64_t fb, unsigned cap,
-                                    Round& t, bool& pruned_any, unsigned long long& fcmp) {
+                                    Round& t, bool& pruned_any, unsigned& fcmp) {
     constexpr int U = kU;
     const unsigned lane = lane_id();
     unsigned am = __ballot_sync(0xffffffffu, b.alive), out = lo;
@@ -1028,7 +1032,7 @@ struct Search {
       bool pr[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) pr[u] = false;
-      fcmp += (unsigned long long)__popc(am) * min(32u * U, hi - r0);
+      fcmp += __popc(am) * min(32u * U, hi - r0);
       // two candidates an iteration (the last one twice when they are odd): a
       // warp alone waits for its own chain of compares and votes
       for (unsigned todo = am; todo;) {
@@ -1077,7 +1081,7 @@ struct Search {
           const uint32_t id = WRITE ? mid[u] : A.fpool[fb + (size_t)D * cap + i];
           A.ldead[id] = cyc;
           if (WRITE) unhist(m[u], v, id);
-          st[S_PRUNED]++;
+          count(S_PRUNED, 1u);
           pruned_any = true;
         }
       }
@@ -1108,7 +1112,7 @@ struct Search {
   // and the log behind it, up to t1. hv: the node's heuristic, 0 at the goal
   // node n.
   __device__ __forceinline__ void batch_ptest(const uint32_t (&hv)[D], Batch& b, unsigned t1, unsigned x, unsigned n,
-                                              unsigned long long& pcmp) {
+                                              unsigned& pcmp) {
     if (!__any_sync(0xffffffffu, b.alive)) return;
     const PIdx& pd = S.pd;
     uint32_t F[D];
@@ -1253,7 +1257,7 @@ struct Search {
       } else if (fifo) {
         atomicMax(&K1.open_count.v, ob + ns);
       }
-      st[S_INSERTED] += ns;
+      count(S_INSERTED, ns);
     }
     return need;
   }
@@ -1330,7 +1334,7 @@ struct Search {
     node_h(v, hv);
     Groups q = open_groups(cs, v, nc);
     const unsigned ng = ngroups(nc);
-    unsigned long long fcmp = 0, pcmp = 0;
+    unsigned fcmp = 0, pcmp = 0;
     bool pruned = false;
     for (unsigned g = 0; g < ng; ++g) {
       const int mine = g ? group(cs, q, g) : (lane < q.in_slots ? slot0 : kNil);
@@ -1348,8 +1352,8 @@ struct Search {
     clear_groups(cs, v, nc);
     if (lane == 0) {
       if (fc != fc0) A.fcount[v] = fc;
-      st[S_FCMP] += fcmp;
-      st[S_PCMP] += pcmp;
+      count(S_FCMP, fcmp);
+      count(S_PCMP, pcmp);
     }
   }
 
@@ -1422,7 +1426,7 @@ struct Search {
     const unsigned a = (r % ks) / sub, bb = r / ks;
     const unsigned width = 32u / sub, l0 = (r % ks) % sub * width;  // this part's lanes of a group
     const unsigned lo = (unsigned)((uint64_t)F * bb / kb), hi = goal ? 0u : (unsigned)((uint64_t)F * (bb + 1) / kb);
-    unsigned long long fcmp = 0, pcmp = 0;
+    unsigned fcmp = 0, pcmp = 0;
     bool pruned = false;
     {
       Groups q = open_groups(cs, v, nc);
@@ -1485,10 +1489,8 @@ struct Search {
         if (atomicOr(&cs.hflag[v], kSplitDone) & kSplitSeen) cs.hflag[v] = 0;
       }
     }
-    if (lane == 0) {
-      st[S_FCMP] += fcmp;
-      st[S_PCMP] += pcmp;
-    }
+    count_lane0(S_FCMP, fcmp);
+    count_lane0(S_PCMP, pcmp);
   }
 
   // Compaction of a frontier after a split merge, by one warp: the entries
@@ -1692,11 +1694,11 @@ struct Search {
     if (T.leader_block()) {
       if (threadIdx.x == 64) {
         // the longest tasks of step i-1 (its slot is K2)
-        st[S_MAXH] += K2.tmax[0];
-        st[S_MAXL] += K2.tmax[1];
-        st[S_MAXX] += K2.tmax[2];
-        st[S_MAXNC] += K2.tmax[3];
-        st[S_MAXF] += K2.tmax[4];
+        count(S_MAXH, K2.tmax[0]);
+        count(S_MAXL, K2.tmax[1]);
+        count(S_MAXX, K2.tmax[2]);
+        count(S_MAXNC, K2.tmax[3]);
+        count(S_MAXF, K2.tmax[4]);
         clear_cycle(K2);
         // values step i+1 starts from; the writers of this step raise them
         atomicMax(&K1.plen.v, psnap);
@@ -1713,7 +1715,7 @@ struct Search {
     __syncthreads();
     if (T.leader() && tlap) {
       const unsigned long long t = globaltimer();
-      st[S_TSEL] += t - *tlap;
+      count(S_TSEL, (unsigned)(t - *tlap));
       *tlap = t;
     }
     // work items, one warp each: parts of split merges (the longest), index-rank
@@ -1738,14 +1740,14 @@ struct Search {
           if (lane == 0 && r == 0) {  // read before the merge clears them
             atomicMax(&S.tmax[3], A.cs[cur].ncand[v]);
             atomicMax(&S.tmax[4], A.fcount[v]);
-            st[S_NHEAVY]++;
+            count(S_NHEAVY, 1u);
           }
           __syncwarp();
           merge_part(v, r, k, K1);
           if (lane == 0) {
             const unsigned long long dt = globaltimer() - t0;
             atomicMax(&S.tmax[0], (unsigned)min(dt, 0xFFFFFFFFull));
-            st[S_SUMH] += dt;
+            count(S_SUMH, (unsigned)dt);
           }
         }
       } else if (t < np + nrank) {
@@ -1763,7 +1765,7 @@ struct Search {
         if (lane == 0) {
           const unsigned long long dt = globaltimer() - t0;
           atomicMax(&S.tmax[1], (unsigned)min(dt, 0xFFFFFFFFull));
-          st[S_SUML] += dt;
+          count(S_SUML, (unsigned)dt);
         }
       } else {
         const unsigned c = t - np - nrank - nt;
@@ -1774,7 +1776,7 @@ struct Search {
         if (lane == 0) {
           const unsigned long long dt = globaltimer() - t0;
           atomicMax(&S.tmax[2], (unsigned)min(dt, 0xFFFFFFFFull));
-          st[S_SUMX] += dt;
+          count(S_SUMX, (unsigned)dt);
         }
       }
       if (nitems <= nwarps) break;
@@ -1784,6 +1786,7 @@ struct Search {
     index_strided_work(T);
     __syncthreads();
     if (threadIdx.x < 5 && S.tmax[threadIdx.x]) atomicMax(&K0.tmax[threadIdx.x], S.tmax[threadIdx.x]);
+    flush_counts(C, S, 1u << 30);
     if (threadIdx.x == 32) {
       if (S.min_key != ~0ull) atomicMin(&K1.min_key.v, S.min_key);
       if (S.win_min != kInf) {
@@ -1799,7 +1802,7 @@ struct Search {
       if (S.hist[x]) atomicAdd(&A.hist[r1 * kNB + x], S.hist[x]);
     if (T.leader() && tlap) {
       const unsigned long long t = globaltimer();
-      st[S_TWORK] += t - *tlap;
+      count(S_TWORK, (unsigned)(t - *tlap));
       *tlap = t;
     }
     return true;
@@ -1833,7 +1836,7 @@ struct Search {
       }
       if (dom) {
         A.ldead[A.fpool[fb + (size_t)D * cap + i]] = 0;
-        st[S_PRUNED]++;
+        count(S_PRUNED, 1u);
       } else {
         ++kept;
       }
@@ -1971,6 +1974,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
   __shared__ Shared S;
   const GridTeam T;
   Search<D> X(G, A, C, P, O, S);
+  if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
   X.init_zero(T);
   bool ok = T.sync(C);
   X.init_seed(T, false);
@@ -1983,7 +1987,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
     ok = T.sync(C);
     if (T.leader()) {
       const unsigned long long t = globaltimer();
-      X.st[S_TSYNC] += t - tph;
+      X.count(S_TSYNC, (unsigned)(t - tph));
       tph = t;
     }
     ++step;
@@ -1991,11 +1995,14 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
   if (ok) {
     if (T.leader()) C->res_count = 0;
     ok = T.sync(C) && X.output(T);
-    if (T.leader()) X.st[S_TOUT] += globaltimer() - tph;
+    if (T.leader()) X.count(S_TOUT, (unsigned)(globaltimer() - tph));
   }
-  X.st[S_STEPS] = T.leader() ? step : 0;
-  X.st[S_GOALINS] = T.leader() ? ld_volatile(&C->plog_len.v) : 0;
-  flush_stats(C, X.st);
+  if (T.leader()) {
+    X.count(S_STEPS, step);
+    X.count(S_GOALINS, ld_volatile(&C->plog_len.v));
+  }
+  __syncthreads();
+  flush_counts(C, S);
   T.sync(C);
   if (T.leader()) {
     __threadfence();
@@ -2066,7 +2073,11 @@ __device__ inline void mq_write_result(const MSlot& sl, unsigned slot, QCtl* C, 
   R->f_words = C->f_words.v;
   C->stats[S_STEPS] = C->step;
   C->stats[S_GOALINS] = C->plog_len.v;
-  for (int i = 0; i < kNStat; ++i) R->stats[i] = C->stats[i];
+  unsigned long long st[kNStat];
+#pragma unroll
+  for (int i = 0; i < kNStat; ++i) st[i] = __ldcg(&C->stats[i]);
+#pragma unroll
+  for (int i = 0; i < kNStat; ++i) R->stats[i] = st[i];
   if (done_flags) {
     __threadfence_system();  // the record is visible before its completion flag
     *reinterpret_cast<volatile unsigned*>(&done_flags[ri]) = 1u;
@@ -2084,59 +2095,42 @@ __device__ void mq_alloc_region1(const MSlot& sl, QCtl* C) {
   C->res_off = off;
 }
 
-__device__ __forceinline__ bool step_empty(const QCtl* C, unsigned i) {
-  const CycleCtl& K = C->cyc[i % 3];
-  return ld_volatile(&K.open_count.v) == ld_volatile(&K.head.v) && ld_volatile(&K.touched_count.v) == 0;
-}
-
-// Work units of a slot that enters the iteration in state st (0: none). INIT
-// and the scan part of the output get one block; the other output parts a
-// share like search steps.
-__device__ __forceinline__ unsigned mq_weight(const MSlot& sl, const QCtl* C, unsigned st, bool& single) {
-  single = false;
-  if (st == SL_FREE || st == SL_HELD) return 0;
-  if (st == SL_INIT || st == SL_OUT3) {
-    single = true;
-    return 1u;
-  }
-  if (st >= SL_OUT1) return max(1u, ld_volatile(&C->res_count) + ld_volatile(sl.A.fcount + sl.G.n));
-  const CycleCtl& K = C->cyc[C->step % 3];
-  const unsigned w = (ld_volatile(&K.open_count.v) - ld_volatile(&K.head.v)) + ld_volatile(&K.touched_count.v) +
-                     ld_volatile(&K.part_count.v);
-  return w ? w : 1u;  // a running slot always gets a block
-}
-
-// Virtual blocks of the iteration (block 0, once every slot's state is set):
-// a slot gets a share of the grid in proportion to its work, at least one
-// block; M->pref holds the prefix sums. One block computes them for all: a
-// block that read the weights for itself could see counters the iteration's
-// work already moves, and take another slot's work.
-__device__ inline void mq_assign(const MSlot* slots, const QCtl* ctls, unsigned nslots, MCtl* M) {
+// Virtual blocks of the iteration, from every slot's weight (block 0; w[x]: the
+// work units of slot threadIdx.x + x * blockDim.x, 0 for none, kOneBlock for
+// work of one block). Every slot with work gets one block, and the blocks left
+// are shared out in proportion to the work: no more virtual blocks than blocks,
+// as long as there are blocks for all, since one that takes two makes the
+// iteration twice as long for everyone. M->pref holds the prefix sums. One block
+// computes them for all: a block that read the weights for itself could see
+// counters the iteration's work already moves, and take another slot's work.
+constexpr unsigned kOneBlock = 0xFFFFFFFFu;
+constexpr unsigned kSlotsPerThread = (kMaxSlots + kMultiThreads - 1) / kMultiThreads;
+__device__ inline void mq_assign(const unsigned (&w)[kSlotsPerThread], unsigned nslots, MCtl* M) {
   __shared__ unsigned long long s_wtot;
-  __shared__ unsigned s_scan[33];
-  if (threadIdx.x == 0) s_wtot = 0;
+  __shared__ unsigned s_active, s_scan[33];
+  if (threadIdx.x == 0) {
+    s_wtot = 0;
+    s_active = 0;
+  }
   __syncthreads();
   unsigned long long wloc = 0;
-  for (unsigned q = threadIdx.x; q < nslots; q += blockDim.x) {
-    bool single;
-    const unsigned w = mq_weight(slots[q], &ctls[q], slots[q].state, single);
-    if (!single) wloc += w;
+  unsigned active = 0;
+#pragma unroll
+  for (unsigned x = 0; x < kSlotsPerThread; ++x) {
+    active += w[x] != 0u;
+    if (w[x] != kOneBlock) wloc += w[x];
   }
   if (wloc) atomicAdd(&s_wtot, wloc);
+  if (active) atomicAdd(&s_active, active);
   __syncthreads();
-  const unsigned long long wtot = s_wtot > 0 ? s_wtot : 1, B = gridDim.x;
+  const unsigned long long wtot = s_wtot > 0 ? s_wtot : 1;
+  const unsigned long long spare = gridDim.x > s_active ? gridDim.x - s_active : 0u;
   unsigned carry = 0;
-  for (unsigned c0 = 0; c0 < nslots; c0 += blockDim.x) {
-    const unsigned q = c0 + threadIdx.x;
-    unsigned nbq = 0;
-    if (q < nslots) {
-      bool single;
-      const unsigned w = mq_weight(slots[q], &ctls[q], slots[q].state, single);
-      if (single)
-        nbq = 1;
-      else if (w)
-        nbq = (unsigned)min(B, max(1ull, (w * B + wtot - 1) / wtot));
-    }
+#pragma unroll
+  for (unsigned x = 0; x < kSlotsPerThread; ++x) {
+    const unsigned q = threadIdx.x + x * blockDim.x;
+    if (x * blockDim.x >= nslots) break;
+    const unsigned nbq = w[x] == 0u ? 0u : w[x] == kOneBlock ? 1u : 1u + (unsigned)(w[x] * spare / wtot);
     unsigned total;
     const unsigned ex = block_exclusive_scan(nbq, s_scan, total);
     if (q < nslots) M->pref[q] = carry + ex;
@@ -2155,22 +2149,32 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
   const unsigned q_count = ld_volatile(&hctl[HC_TAIL]);
   const unsigned qcap = M->qcap;
   const unsigned after_out = M->hold ? SL_HELD : SL_FREE;
-  for (unsigned q = threadIdx.x; q < nslots; q += blockDim.x) {
+  unsigned w[kSlotsPerThread];  // work units of this thread's slots in the iteration
+#pragma unroll
+  for (unsigned x = 0; x < kSlotsPerThread; ++x) {
+    w[x] = 0;
+    const unsigned q = threadIdx.x + x * blockDim.x;
+    if (q >= nslots) continue;
     MSlot& sl = slots[q];
     QCtl* C = &ctls[q];
     unsigned st = sl.state;
-    if (st == SL_RUN) {
-      const unsigned step = C->step + 1;
+    if (st == SL_RUN || st == SL_INIT) {
+      // the step that comes next, from one round of loads
+      const unsigned step = st == SL_RUN ? __ldcg(&C->step) + 1u : 0u;
+      const CycleCtl& K = C->cyc[step % 3];
+      const unsigned err = ld_volatile(&C->error), open = __ldcg(&K.open_count.v) - __ldcg(&K.head.v),
+                     touched = __ldcg(&K.touched_count.v), parts = __ldcg(&K.part_count.v);
+      const bool late = st == SL_RUN && globaltimer() - C->t_start > sl.P.time_limit_ns;
       C->step = step;
-      if (ld_volatile(&C->error) || step_empty(C, step))
+      if (err || (open == 0 && touched == 0)) {
         st = SL_OUT1;
-      else if (globaltimer() - C->t_start > sl.P.time_limit_ns) {
+      } else if (late) {
         atomicCAS(&C->error, 0u, (unsigned)OPMOS_ERR_TIMEOUT);
         st = SL_OUT1;
+      } else {
+        st = SL_RUN;
+        w[x] = max(1u, open / 4u + touched + parts);
       }
-      if (st == SL_OUT1) C->res_count = 0;
-    } else if (st == SL_INIT) {
-      st = (ld_volatile(&C->error) || step_empty(C, 0)) ? SL_OUT1 : SL_RUN;
       if (st == SL_OUT1) C->res_count = 0;
     } else if (st == SL_OUT1 || st == SL_OUT2 || st == SL_OUT3 || st == SL_OUT4) {
       // one output part per iteration; an error ends the output early
@@ -2221,10 +2225,14 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
       }
     }
     sl.state = st;
+    if (st == SL_INIT || st == SL_OUT3)
+      w[x] = kOneBlock;
+    else if (st == SL_OUT1 || st == SL_OUT2 || st == SL_OUT4)
+      w[x] = max(1u, __ldcg(sl.A.fcount + sl.G.n) / 4u);
     if (st != SL_FREE) atomicAdd(&s_busy, 1u);
   }
   __syncthreads();
-  mq_assign(slots, ctls, nslots, M);
+  mq_assign(w, nslots, M);
   if (threadIdx.x == 0) {
     M->iter++;
     const unsigned closing = ld_volatile(&hctl[HC_CLOSING]);
@@ -2234,14 +2242,16 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
 }
 
 template <int D>
-__device__ void mq_work(MSlot* slots, QCtl* ctls, unsigned q, unsigned j, unsigned nb, Shared& S) {
-  const QArena A = slots[q].A;
-  const QParams P = slots[q].P;
-  const GraphDev G = slots[q].G;
-  const OutPool O = slots[q].O;
-  const unsigned st = slots[q].state;
+__device__ void mq_work(MSlot* slots, QCtl* ctls, unsigned q, unsigned j, unsigned nb, Shared& S, MSlot& s_slot) {
+  // the slot's record in shared memory (a copy in every thread's local memory
+  // was 500 bytes a thread an iteration)
+  static_assert(sizeof(MSlot) % 4 == 0, "MSlot");
+  for (unsigned x = threadIdx.x; x < sizeof(MSlot) / 4; x += blockDim.x)
+    reinterpret_cast<unsigned*>(&s_slot)[x] = __ldcg(reinterpret_cast<const unsigned*>(&slots[q]) + x);
+  __syncthreads();
+  const unsigned st = s_slot.state;
   QCtl* C = &ctls[q];
-  Search<D> X(G, A, C, P, O, S);
+  Search<D> X(s_slot.G, s_slot.A, C, s_slot.P, s_slot.O, S);
   if (st == SL_INIT) {
     const BlockTeam T;
     X.init_zero(T);
@@ -2260,11 +2270,13 @@ __device__ void mq_work(MSlot* slots, QCtl* ctls, unsigned q, unsigned j, unsign
   } else if (st == SL_RUN) {
     X.step(SubTeam{j, nb}, C->step, nullptr);
   }
-  flush_stats(C, X.st);
+  __syncthreads();
+  flush_counts(C, S);
 }
 
 template <int D>
-__device__ void mq_phase(MSlot* slots, QCtl* ctls, unsigned nslots, MCtl* M, Shared& S, unsigned* s_pref) {
+__device__ void mq_phase(MSlot* slots, QCtl* ctls, unsigned nslots, MCtl* M, Shared& S, MSlot& s_slot,
+                         unsigned* s_pref) {
   for (unsigned q = threadIdx.x; q <= nslots; q += blockDim.x) s_pref[q] = ld_volatile(&M->pref[q]);
   __syncthreads();
   const unsigned B = gridDim.x;
@@ -2277,7 +2289,7 @@ __device__ void mq_phase(MSlot* slots, QCtl* ctls, unsigned nslots, MCtl* M, Sha
     }
     const unsigned q = lo;
     const unsigned j = v - s_pref[q], nb = s_pref[q + 1] - s_pref[q];
-    mq_work<D>(slots, ctls, q, j, nb, S);
+    mq_work<D>(slots, ctls, q, j, nb, S, s_slot);
     __syncthreads();
   }
 }
@@ -2287,13 +2299,15 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
     multi_kernel(MSlot* slots, QCtl* ctls, unsigned nslots, const MQuery* queue, unsigned* hctl,
                  const GraphDev* graphs, QResult* results, unsigned* done_flags, MCtl* M) {
   __shared__ Shared S;
+  __shared__ MSlot s_slot;
   __shared__ unsigned s_pref[kMaxSlots + 1];
+  if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
   unsigned target = 0;
   for (;;) {
     if (blockIdx.x == 0) mq_schedule<D>(slots, ctls, nslots, queue, hctl, graphs, M, results, done_flags);
     if (!mq_barrier(M, target)) return;
     if (ld_volatile(&M->done)) return;
-    mq_phase<D>(slots, ctls, nslots, M, S, s_pref);
+    mq_phase<D>(slots, ctls, nslots, M, S, s_slot, s_pref);
     if (!mq_barrier(M, target)) return;
   }
 }
