@@ -92,13 +92,14 @@ enum StatIdx {
   kNStat
 };
 
-// Two shapes of the single-query grid: one 512-thread block per SM for short
-// steps (windows below kSmallWindow), three 256-thread blocks per SM for large
-// windows, whose steps have several work items for every warp (registers are
-// capped at 85 a thread then, and some spill).
-constexpr unsigned kGridThreads = 512;
+// Two shapes of the single-query grid: one 384-thread block per SM for short
+// steps (windows below kSmallWindow; 512 threads were 1-4% slower, 256 as fast),
+// two 256-thread blocks per SM for large windows, whose steps have several work
+// items for every warp (256x256 grid, W = 262,144: 97 ms; three blocks, whose
+// 80 registers a thread spill, 102 ms, four 103 ms).
+constexpr unsigned kGridThreads = 384;
 constexpr unsigned kGridWideThreads = 256;
-constexpr unsigned kGridWideBlocksPerSM = 3;
+constexpr unsigned kGridWideBlocksPerSM = 2;
 
 // Words of a row that holds w words and is read 16 bytes at a time.
 __host__ __device__ constexpr int row_words(int w) { return w <= 2 ? w : (w + 3) / 4 * 4; }
