@@ -120,7 +120,7 @@ __device__ __forceinline__ uint32_t* row_space() {
 struct Shared {
   alignas(16) unsigned hist[kNB];  // this block's share of the next OPEN's histogram
   unsigned warp[33];
-  unsigned f_min, b1_max, bstar;
+  unsigned f_min, b1_max;  // see select_window
   unsigned pmax[3];
   // what this block's extraction items found (next bins), added to the global
   // record once a step
@@ -325,64 +325,75 @@ struct Search {
   }
 
   // ---------------- window selection (Algorithm 2: NUM_POP lowest labels) ----------------
-  // Bins [0, b*] where b* is the largest bin whose cumulative count is <= W,
-  // but at least the first non-empty bin (the overflow bin is never taken).
-  // Every block computes the same b* into S.bstar. all: OPEN holds at most W
-  // entries, so every bin but the last has a cumulative count within W and
-  // b* is kNB - 2 without reading the histogram.
-  __device__ void select_window(const unsigned* gh, bool all = false) {
-    constexpr unsigned kPer = kNB / 256;  // bins per thread: blocks have 256 threads or more
-    static_assert(kGridThreads >= 256 && kGridWideThreads >= 256 && kMultiThreads >= 256, "kPer");
-    if (all) {
-      if (threadIdx.x == 0) S.bstar = kNB - 2;
-      for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
-      __syncthreads();
-      return;
-    }
-    const unsigned per = (kNB + blockDim.x - 1) / blockDim.x;
-    // the histogram (other SMs added to it: read past L1) staged in shared
-    // memory with 16-byte loads, then each thread takes `per` consecutive bins
-    {
-      const uint4* g4 = reinterpret_cast<const uint4*>(gh);
-      uint4* s4 = reinterpret_cast<uint4*>(S.hist);
-      for (unsigned x = threadIdx.x; x < kNB / 4; x += blockDim.x) s4[x] = __ldcg(g4 + x);
-    }
+  // OPEN's histogram in registers: the block's first 8 warps take 512 bins each,
+  // lane l the bins 4 (32 j + l) .. + 3 of them in q[j] (16-byte loads, whole
+  // lines). Other SMs added to it: read past L1. A step issues the loads before
+  // it waits for its record, which says whether they are needed.
+  struct Bins {
+    uint4 q[4];
+  };
+  static_assert(kNB == 8 * 512 && kGridThreads >= 256 && kGridWideThreads >= 256 && kMultiThreads >= 256, "Bins");
+  __device__ __forceinline__ static Bins load_bins(const unsigned* gh) {
+    Bins h;
+    const uint4* g4 = reinterpret_cast<const uint4*>(gh) + (threadIdx.x >> 5) * 128 + lane_id();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h.q[j] = threadIdx.x < 256u ? __ldcg(g4 + 32 * j) : make_uint4(0u, 0u, 0u, 0u);
+    return h;
+  }
+  // The window is the bins [0, b*], b* the largest bin whose cumulative count is
+  // <= W, but at least the first non-empty bin (the overflow bin is never
+  // taken). all: OPEN holds at most W entries, so every bin but the last has a
+  // cumulative count within W. Every block finds the same b*; bstar() gives it
+  // after the next block barrier. One thread holds the bin where the count
+  // passes W and one the first entry, so they write without atomics. (Loading
+  // the bins after the record, staging them in shared memory, a block scan and
+  // atomics by every thread made a step of the 160x160 ship grid 13.5 us
+  // instead of 12.5, one of the 32x32 grid 11.5 instead of 10.9.)
+  __device__ void select_window(const Bins& h, bool all) {
     if (threadIdx.x == 0) {
+      S.b1_max = all ? kNB - 2 : 0;
       S.f_min = kNB;
-      S.b1_max = 0;
     }
-    __syncthreads();
-    const unsigned b0 = threadIdx.x * per;
-    unsigned loc[kPer];
-    unsigned sum = 0;
+    if (all) return;
+    const unsigned w = threadIdx.x >> 5, lane = lane_id();
+    unsigned sum[4], incl[4];
 #pragma unroll
-    for (unsigned j = 0; j < kPer; ++j) {
-      loc[j] = (j < per && b0 + j < (unsigned)kNB) ? S.hist[b0 + j] : 0u;
-      sum += loc[j];
-    }
-    unsigned total;
-    unsigned run = block_exclusive_scan(sum, S.warp, total);
-    unsigned fmin = kNB, b1 = 0;
-    bool any_b1 = false;
+    for (int j = 0; j < 4; ++j) sum[j] = incl[j] = h.q[j].x + h.q[j].y + h.q[j].z + h.q[j].w;
 #pragma unroll
-    for (unsigned j = 0; j < kPer; ++j) {
-      const unsigned b = b0 + j;
-      run += loc[j];
-      if (j < per && b < (unsigned)kNB - 1) {
-        if (loc[j] && b < fmin) fmin = b;
-        if (run <= P.window) {
-          b1 = b;
-          any_b1 = true;
-        }
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl[j], o);
+        if (lane >= (unsigned)o) incl[j] += y;
       }
+    unsigned tot[4], all4 = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      tot[j] = __shfl_sync(0xffffffffu, incl[j], 31);
+      all4 += tot[j];
     }
-    if (fmin < kNB) atomicMin(&S.f_min, fmin);
-    if (any_b1) atomicMax(&S.b1_max, b1);
+    if (lane == 0 && w < 8) S.warp[w] = all4;
     __syncthreads();
-    if (threadIdx.x == 0) S.bstar = max(S.b1_max, S.f_min == (unsigned)kNB ? 0u : S.f_min);
-    // S.hist starts the next OPEN's histogram empty
-    for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
-    __syncthreads();
+    if (w >= 8) return;
+    unsigned before = 0;
+#pragma unroll
+    for (unsigned x = 0; x < 8; ++x) before += x < w ? S.warp[x] : 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      unsigned run = before + incl[j] - sum[j];  // the count before the lane's four bins
+      const unsigned c[4] = {h.q[j].x, h.q[j].y, h.q[j].z, h.q[j].w};
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const unsigned bin = w * 512 + j * 128 + lane * 4 + x;
+        if (run == 0 && c[x] && bin < kNB - 1) S.f_min = bin;
+        if (run <= P.window && (run + c[x] > P.window || bin == kNB - 1)) S.b1_max = bin ? bin - 1 : 0u;
+        run += c[x];
+      }
+      before += tot[j];
+    }
+  }
+  __device__ __forceinline__ unsigned bstar() const {
+    return max(S.b1_max, S.f_min == (unsigned)kNB ? 0u : S.f_min);
   }
 
   // Bins of the histogram of OPEN_{i+1}, from what step i-1 measured (the
@@ -639,7 +650,7 @@ struct Search {
       key = A.okey[cur][i];
       id = A.oid[cur][i];
       dead = A.ldead[id];
-      want = bin_of(key, bp) <= S.bstar;
+      want = bin_of(key, bp) <= bstar();
     }
     const Label own = load_label(want, id);
     const bool gone = valid && dead < cyc;
@@ -1330,8 +1341,14 @@ struct Search {
     unsigned cap = A.fcap[v], fc = A.fcount[v];
     const unsigned fc0 = fc;
     const int slot0 = lane < A.nslots ? cs.cslot[(size_t)v * A.nslots + lane] : kNil;
+    const uint32_t split = cs.hflag[v];
     uint32_t hv[D];
     node_h(v, hv);
+    __syncwarp();  // every lane has read the word before lane 0 changes it
+    if (split) {   // merged in parts this step; this item or the last part clears the word
+      if (lane == 0 && (atomicOr(&cs.hflag[v], kSplitSeen) & kSplitDone)) cs.hflag[v] = 0;
+      return;
+    }
     Groups q = open_groups(cs, v, nc);
     const unsigned ng = ngroups(nc);
     unsigned fcmp = 0, pcmp = 0;
@@ -1652,6 +1669,7 @@ struct Search {
     CycleCtl& K1 = C->cyc[r1];
     CycleCtl& K2 = C->cyc[r2];
     const bool fifo = (P.flags & OPMOS_FLAG_FIFO) != 0;
+    const Bins bins = load_bins(A.hist + r0 * kNB);
     // Everything the step reads of its record, by one warp a block in one round
     // of loads, a lane a word (every warp reading every word was 36,000 loads
     // of 15 lines a step: 2.7 us).
@@ -1689,7 +1707,7 @@ struct Search {
     // bins OPEN_i's histogram was built on
     const BinParams bp{rec[RW_BINS], rec[RW_BINS + 1], rec[RW_BINS + 2], rec[RW_BINS + 3], rec[RW_BINS + 4]};
     bpn = next_bins(ms);
-    select_window(A.hist + r0 * kNB, n_in <= P.window);
+    select_window(bins, fifo || n_in <= P.window);
     for (unsigned x = T.tid(); x < kNB; x += T.nthreads()) A.hist[r2 * kNB + x] = 0;
     if (T.leader_block()) {
       if (threadIdx.x == 64) {
@@ -1754,14 +1772,7 @@ struct Search {
         rank_item(t - np);
       } else if (t < np + nrank + nt) {
         const uint32_t v = A.cs[cur].touched[t - np - nrank];
-        uint32_t* hf = A.cs[cur].hflag + v;
-        const uint32_t split = *hf;
-        __syncwarp();  // every lane has read it before lane 0 changes it
-        if (split) {  // merged in parts this step; this item or the last part clears the word
-          if (lane == 0 && (atomicOr(hf, kSplitSeen) & kSplitDone)) *hf = 0;
-        } else {
-          merge_node(v, K1);
-        }
+        merge_node(v, K1);
         if (lane == 0) {
           const unsigned long long dt = globaltimer() - t0;
           atomicMax(&S.tmax[1], (unsigned)min(dt, 0xFFFFFFFFull));
@@ -1798,8 +1809,18 @@ struct Search {
         atomicMax(&K1.f1hi.v, S.f1hi);
       }
     }
-    for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x)
-      if (S.hist[x]) atomicAdd(&A.hist[r1 * kNB + x], S.hist[x]);
+    // (a thread empties what it adds: S.hist is zero again for the next step)
+    for (unsigned x = threadIdx.x; x < kNB / 4; x += blockDim.x) {
+      uint4& q = reinterpret_cast<uint4*>(S.hist)[x];
+      const uint4 h = q;
+      if (!(h.x | h.y | h.z | h.w)) continue;
+      q = make_uint4(0u, 0u, 0u, 0u);
+      unsigned* to = A.hist + r1 * kNB + 4 * x;
+      if (h.x) atomicAdd(to, h.x);
+      if (h.y) atomicAdd(to + 1, h.y);
+      if (h.z) atomicAdd(to + 2, h.z);
+      if (h.w) atomicAdd(to + 3, h.w);
+    }
     if (T.leader() && tlap) {
       const unsigned long long t = globaltimer();
       count(S_TWORK, (unsigned)(t - *tlap));
@@ -1975,6 +1996,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
   const GridTeam T;
   Search<D> X(G, A, C, P, O, S);
   if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
+  for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
   X.init_zero(T);
   bool ok = T.sync(C);
   X.init_seed(T, false);
@@ -2302,6 +2324,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
   __shared__ MSlot s_slot;
   __shared__ unsigned s_pref[kMaxSlots + 1];
   if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
+  for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
   unsigned target = 0;
   for (;;) {
     if (blockIdx.x == 0) mq_schedule<D>(slots, ctls, nslots, queue, hctl, graphs, M, results, done_flags);

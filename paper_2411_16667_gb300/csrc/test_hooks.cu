@@ -244,9 +244,11 @@ __global__ void __launch_bounds__(kGridThreads, 1) window_hook_kernel(GraphDev G
   X.lbase = n;
   X.bpn = bp;
   if (threadIdx.x == 0) S.pd = PIdx{};
+  for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
   __syncthreads();
-  X.select_window(A.hist + 1 * kNB);  // leaves S.hist empty for the extraction
-  if (threadIdx.x == 0) *bstar = S.bstar;
+  X.select_window(X.load_bins(A.hist + 1 * kNB), false);
+  __syncthreads();
+  if (threadIdx.x == 0) *bstar = X.bstar();
   const unsigned nchunks = (n + kChunk - 1) / kChunk;
   for (unsigned c = threadIdx.x >> 5; c < nchunks; c += blockDim.x >> 5) X.extract_chunk(c, n, kChunk, bp, C->cyc[2]);
 }
