@@ -1337,6 +1337,17 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       server_free(sv);
       return cuda_fail(e, "server set-up");
     }
+    // Load the heuristic kernels of every graph now, by launches without jobs: a
+    // kernel is loaded at its first launch, which may wait until the device is
+    // idle, and the resident kernel never ends while submit waits.
+    for (uint32_t i = 0; i < ngraphs && e == cudaSuccess; ++i)
+      e = launch_heuristic(graphs[i]->dev, sv->djobs, 0, sv->hscratch, 5 * (size_t)sv->shape.n + 64, 1, graphs[i]->delta,
+                           sv->hkctr, sv->hkctr + 1, sv->hstream, kHeurSmemServed);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(sv->hstream);
+    if (e != cudaSuccess) {
+      server_free(sv);
+      return cuda_fail(e, "server heuristic kernels");
+    }
     const int occ = multi_occupancy(sv->dmax, kServeBlockSmem);
     const unsigned full = (unsigned)di.sms * (unsigned)std::min(occ, 2);
     sv->blocks = full > 2 * kServeHeurBlocks ? full - 2 * kServeHeurBlocks : std::max(1u, full / 2);
