@@ -334,8 +334,8 @@ int compute_heuristic(const opmos_graph* g, uint32_t D, const uint32_t* goals, u
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   cudaEventRecord(e0, s);
-  cudaError_t e = launch_heuristic(g->dev, djobs, njobs, (uint32_t*)scratch, spb, blocks, g->delta, ctr,
-                                   ctr + 1, s);
+  cudaError_t e = launch_heuristic(g->dev, djobs, njobs, (uint32_t*)scratch, spb, blocks, g->delta, ctr, ctr + 1, s,
+                                   kHeurSmem, (unsigned)di.sms);
   cudaEventRecord(e1, s);
   if (e != cudaSuccess) {
     cudaEventDestroy(e0);
@@ -1196,6 +1196,7 @@ void server_free(opmos_server* sv) {
     *reinterpret_cast<volatile unsigned*>(&sv->hctl[HC_CLOSING]) = 2;  // stop now
     for (unsigned i = 0; i < sv->nslots; ++i) *reinterpret_cast<volatile unsigned*>(&sv->hctl[HC_RELEASE + i]) = 1;
     cudaStreamSynchronize(sv->kstream);
+    --resident_servers;
   }
   if (sv->dmem) cudaFree(sv->dmem);
   if (sv->hmem) cudaFreeHost(sv->hmem);
@@ -1362,6 +1363,7 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       return cuda_fail(e, "server kernel launch");
     }
     sv->running = true;
+    ++resident_servers;
     *out = sv;
     return OPMOS_OK;
   });

@@ -22,11 +22,14 @@
 //                  kFlagsNodes nodes
 //   kFlagsGlobal   list heads only: larger graphs
 // Measured, one thread per node and all lists in global memory -> here: 97x89
-// ship grid, d = 3 (distances shared) 1.37 -> 0.28 ms; 160x160 2.7 -> 0.52;
-// 256x256, d = 5 (flags shared) 4.4 -> 1.5; road-like graph of 199,809 nodes,
-// d = 4 (flags shared) 16 -> 4.8 ms: 1,400 rounds of 3.4 us.
+// ship grid, d = 3 (distances shared) 1.37 -> 0.26 ms; 160x160 2.7 -> 0.49;
+// 256x256, d = 5 (flags shared) 4.4 -> 1.44; road-like graph of 199,809 nodes,
+// d = 4 (flags shared) 16 -> 4.6 ms: 1,400 rounds of 3.3 us. Larger graphs with
+// SMs to spare go to a cluster of blocks below.
 //
 // Scratch per block: near, next, far, far2 (n each) and flags (n).
+#include <algorithm>
+
 #include "opmos_dev.cuh"
 #include "search.cuh"
 
@@ -192,11 +195,233 @@ __global__ void __launch_bounds__(kHeurThreads, 2)
   }
 }
 
+// ---------------------------------------------------------------------------
+// One (goal, k) pair by a cluster of kHeurCluster blocks: for graphs whose
+// distances do not fit one SM's shared memory, while there are SMs to spare
+// (a query's own d pairs; a batch has a pair for every SM). The same search, the
+// nodes dealt out to the blocks (node v is number v / kHeurCluster of block
+// v % kHeurCluster, so neighbours of a grid go to different blocks), each
+// block with its nodes' distances, flags and the heads of their lists in its
+// shared memory.
+//
+// A step: every block relaxes the next nodes of its near list, one arc a lane,
+// and writes the (node, distance) each arc gives into the inbox of the node's
+// block; one cluster barrier; every block takes the minima of its inbox and
+// lists what improved. Only stores and that barrier cross SMs. (Improving the
+// distances by atomics on the other blocks' shared memory was a chain of three
+// returning atomics a round: 1.35 ms instead of 1.12 on the 256x256 grid below.) Inboxes are two by step parity, with a row for
+// every sender, so a slot is a count in the sender's own memory.
+//
+// A single block's round was a chain of ~7,000 cycles, 5,000 of them scattered
+// returning atomics at the L2 for ~130 nodes; a step is 3,600 (1,700 until the
+// last arc is sent, 1,400 for the barrier and the slowest block, 300 for the
+// inbox). Measured, one block -> cluster: 256x256 ship grid, d = 5: 1.44 -> 1.12
+// ms; road-like graph of 199,809 nodes, d = 4: 4.6 -> 2.8 ms, d = 2: 4.1 -> 2.5
+// ms. 256 threads a block were 15-25% slower, 1,024 up to 15%.
+// ---------------------------------------------------------------------------
+constexpr unsigned kHeurCluster = 8;
+constexpr unsigned kClusterThreads = 512;  // also the messages of one block to another in a step
+constexpr unsigned kClusterNear = 1024;    // entries of each near list kept in shared memory
+constexpr unsigned kInboxWords = 2 * kHeurCluster * kClusterThreads * 2;
+
+constexpr size_t cluster_nodes(size_t n) { return (n + kHeurCluster - 1) / kHeurCluster; }
+constexpr size_t cluster_words(size_t n) {
+  return kInboxWords + 2 * kClusterNear + cluster_nodes(n) + 2 * ((cluster_nodes(n) + 31) / 32);
+}
+
+// The address of this block's shared p in block `rank` of the cluster, and
+// stores there.
+__device__ __forceinline__ unsigned peer(const void* p, unsigned rank) {
+  unsigned a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ void peer_store(unsigned a, unsigned x, unsigned y) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kClusterThreads, 1) __cluster_dims__(kHeurCluster, 1, 1)
+    heuristic_cluster_kernel(GraphDev G, const HJob* jobs, uint32_t* scratch, const uint32_t* delta, unsigned* err,
+                             unsigned lpn) {
+  extern __shared__ __align__(8) uint32_t dyn[];
+  __shared__ unsigned s_n[2], s_far_n, s_far2_n, s_fmin;  // entries of the near lists and the far list; smallest far distance
+  __shared__ unsigned s_sent[kHeurCluster], s_near, s_low;  // a step's messages: number to each block, any for a near list, smallest far one
+  __shared__ uint2 s_info[2][kHeurCluster];  // by step parity, from every block: messages | more << 31, smallest far distance
+  const unsigned n = G.n, tid = threadIdx.x, lane = tid & 31u;
+  const unsigned rank = blockIdx.x % kHeurCluster, job = blockIdx.x / kHeurCluster;
+  const unsigned npc = (n + kHeurCluster - 1) / kHeurCluster, words = (npc + 31) / 32;
+  uint2* const inbox = reinterpret_cast<uint2*>(dyn);  // [parity][sender][slot]
+  uint32_t* const heads = dyn + kInboxWords;           // of the near lists
+  uint32_t* const dist = heads + 2 * kClusterNear;
+  uint32_t* const nbit = dist + npc;
+  uint32_t* const fbit = nbit + words;
+  // the ends of the near lists and the far list twice, npc entries each
+  uint32_t* const base = scratch + (size_t)blockIdx.x * 4 * npc;
+  auto append = [&](unsigned l, uint32_t lv) {
+    const unsigned at = atomicAdd(&s_n[l], 1u);
+    if (at < kClusterNear)
+      heads[l * kClusterNear + at] = lv;
+    else
+      base[(size_t)l * npc + at] = lv;
+  };
+  auto mark = [&](uint32_t* bits, uint32_t lv) -> bool {
+    const uint32_t b = 1u << (lv & 31);
+    return !(atomicOr(bits + (lv >> 5), b) & b);
+  };
+  auto unmark = [&](uint32_t* bits, uint32_t lv) { atomicAnd(bits + (lv >> 5), ~(1u << (lv & 31))); };
+  const unsigned grp = tid / lpn, gl = tid % lpn, ngrp = kClusterThreads / lpn;
+  const unsigned k = jobs[job].k, goal = jobs[job].goal;
+  uint32_t* const out = jobs[job].h_out;
+  const uint32_t* rc = G.rcost + (size_t)k * G.m;
+  const unsigned long long dk = delta[k] ? delta[k] : 1u;
+  for (unsigned v = tid; v < npc; v += kClusterThreads) dist[v] = kInf;
+  for (unsigned x = tid; x < 2 * words; x += kClusterThreads) nbit[x] = 0;
+  if (tid < kHeurCluster) s_sent[tid] = 0;
+  if (tid == 0) {
+    s_n[0] = s_n[1] = s_far_n = s_near = 0;
+    s_fmin = s_low = kInf;
+  }
+  __syncthreads();
+  if (tid == 0 && goal % kHeurCluster == rank) {
+    dist[goal / kHeurCluster] = 0;
+    mark(nbit, goal / kHeurCluster);
+    append(1u, goal / kHeurCluster);
+  }
+  cluster_sync();  // nobody writes into a block before its start
+  // the near list being relaxed, the next entry of it and its end (the other
+  // list is being filled); arcs of the lanes' nodes are left
+  unsigned cur = 0, pos = 0, nn = 0, ip = 0, fsel = 0;
+  int left = 0;
+  uint32_t jb = 0, je = 0, du = 0;  // the group's node: next arcs, their end, its distance
+  unsigned long long thr = dk;      // the near lists hold distances < thr
+  unsigned long long steps = 0;
+  const unsigned long long max_steps = 128ull * n + 4096;
+  // every block takes every branch of this loop's end alike: they depend on what
+  // all have exchanged
+  for (;;) {
+    if (++steps > max_steps) {
+      if (tid == 0) atomicCAS(err, 0u, (unsigned)OPMOS_ERR_TIMEOUT);
+      return;
+    }
+    if (!left) {
+      if (pos >= nn) {  // this list is done
+        cur ^= 1u;
+        pos = 0;
+        nn = s_n[cur];
+        if (tid == 0) s_n[cur ^ 1u] = 0;
+      }
+      jb = je = 0;
+      if (pos + grp < nn) {
+        const unsigned i = pos + grp;
+        const uint32_t lu = i < kClusterNear ? heads[cur * kClusterNear + i] : base[(size_t)cur * npc + i];
+        const uint32_t u = lu * kHeurCluster + rank;
+        jb = __ldg(G.rrowptr + u);
+        je = __ldg(G.rrowptr + u + 1);
+        du = dist[lu];
+        if (gl == 0) unmark(nbit, lu);  // an improvement from here on lists it again
+      }
+      pos += ngrp;
+    }
+    if (jb + gl < je) {
+      const uint32_t w = __ldg(G.rsrc + jb + gl);
+      const uint32_t nd = du + __ldg(rc + jb + gl);
+      const unsigned o = w % kHeurCluster;
+      const unsigned slot = atomicAdd(&s_sent[o], 1u);
+      peer_store(peer(inbox + (ip * kHeurCluster + rank) * kClusterThreads + slot, o), w / kHeurCluster, nd);
+      if (nd < thr)
+        s_near = 1;
+      else
+        atomicMin(&s_low, nd);
+    }
+    jb += lpn;
+    left = __syncthreads_or(jb < je);
+    if (tid < kHeurCluster) {
+      const bool more = left || pos < nn || s_n[cur ^ 1u] || s_near;
+      peer_store(peer(&s_info[ip][rank], tid), s_sent[tid] | (more ? 0x80000000u : 0u), min(s_fmin, s_low));
+    }
+    cluster_sync();
+    unsigned more = 0, fmin = kInf;
+#pragma unroll
+    for (unsigned r = 0; r < kHeurCluster; ++r) {
+      more |= s_info[ip][r].x;
+      fmin = min(fmin, s_info[ip][r].y);
+    }
+    if (tid < kHeurCluster) s_sent[tid] = 0;
+    if (tid == 0) {
+      s_near = 0;
+      s_low = kInf;
+    }
+    // the inbox, two warps a sender
+    {
+      constexpr unsigned kWarps = kClusterThreads / 32;
+      const unsigned from = (tid >> 5) % kHeurCluster;
+      const unsigned c = s_info[ip][from].x & 0x7FFFFFFFu;
+      const uint2* in = inbox + (ip * kHeurCluster + from) * kClusterThreads;
+      for (unsigned i = (tid >> 5) / kHeurCluster * 32 + lane; i < c; i += kWarps / kHeurCluster * 32) {
+        const uint2 m = in[i];
+        if (m.y < atomicMin(dist + m.x, m.y)) {
+          if (m.y < thr) {
+            if (mark(nbit, m.x)) append(cur ^ 1u, m.x);
+          } else {
+            atomicMin(&s_fmin, m.y);
+            if (mark(fbit, m.x)) base[(size_t)(2 + fsel) * npc + atomicAdd(&s_far_n, 1u)] = m.x;
+          }
+        }
+      }
+    }
+    ip ^= 1u;
+    __syncthreads();
+    if (more & 0x80000000u) continue;
+    if (fmin == kInf) break;  // no block has a pending distance
+    // pending distances below the old threshold are final; fmin is at most the
+    // smallest of the others. Each block sorts its own far list.
+    const unsigned long long settled = thr;
+    thr = max((unsigned long long)fmin, settled) + dk;
+    const unsigned fn = s_far_n;
+    const uint32_t* const far = base + (size_t)(2 + fsel) * npc;
+    fsel ^= 1u;
+    uint32_t* const far2 = base + (size_t)(2 + fsel) * npc;
+    __syncthreads();
+    if (tid == 0) {
+      s_far2_n = 0;
+      s_fmin = kInf;
+    }
+    __syncthreads();
+    for (unsigned i = tid; i < fn; i += kClusterThreads) {
+      const uint32_t lw = far[i], dw = dist[lw];
+      if (dw < thr) {
+        unmark(fbit, lw);
+        if (dw >= settled && mark(nbit, lw)) append(cur ^ 1u, lw);
+      } else {
+        atomicMin(&s_fmin, dw);
+        far2[atomicAdd(&s_far2_n, 1u)] = lw;
+      }
+    }
+    __syncthreads();
+    if (tid == 0) s_far_n = s_far2_n;
+    __syncthreads();
+  }
+  for (unsigned lv = tid; lv < npc; lv += kClusterThreads) {
+    const unsigned v = lv * kHeurCluster + rank;
+    if (v < n) out[v] = dist[lv];
+  }
+}
+
 // The mode of a graph of n nodes: everything in shared memory while it fits.
 HeurMode heuristic_mode(size_t n, size_t smem) {
   if (heur_words(kDistShared, n) * 4 <= smem) return kDistShared;
   if (heur_words(kFlagsShared, n) * 4 <= smem) return kFlagsShared;
   return kFlagsGlobal;
+}
+
+// Lanes a node: as many as its arcs on average, so one round takes most nodes.
+unsigned lanes_per_node(const GraphDev& G) {
+  unsigned lpn = 4;
+  while (lpn < 32 && (unsigned long long)lpn * G.n < G.m) lpn <<= 1;
+  return lpn;
 }
 
 template <HeurMode MODE>
@@ -207,19 +432,34 @@ cudaError_t launch_mode(const GraphDev& G, const HJob* jobs, unsigned njobs, uin
   const cudaError_t e = cudaFuncSetAttribute((const void*)heuristic_kernel<MODE>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  // lanes a node: as many as its arcs on average, so one round takes most nodes
-  unsigned lpn = 4;
-  while (lpn < 32 && (unsigned long long)lpn * G.n < G.m) lpn <<= 1;
   heuristic_kernel<MODE><<<blocks, kHeurThreads, smem, s>>>(G, jobs, njobs, scratch, scratch_words_per_block, delta,
-                                                            next_job, err, lpn);
+                                                            next_job, err, lanes_per_node(G));
   return cudaGetLastError();
 }
 
 }  // namespace
 
+std::atomic<int> resident_servers{0};
+
 cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                              size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta,
-                             unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem) {
+                             unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem, unsigned sms) {
+  if (resident_servers.load() != 0) {
+    smem = std::min(smem, kHeurSmemServed);
+    sms = 0;
+  }
+  // a cluster a pair where the distances do not fit one block but fit eight,
+  // while every cluster has its SMs at once
+  if (njobs && heuristic_mode(G.n, smem) != kDistShared && njobs * kHeurCluster <= sms &&
+      cluster_words(G.n) * 4 <= smem) {
+    const size_t bytes = cluster_words(G.n) * 4;
+    const cudaError_t e = cudaFuncSetAttribute((const void*)heuristic_cluster_kernel,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    heuristic_cluster_kernel<<<njobs * kHeurCluster, kClusterThreads, bytes, s>>>(G, jobs, scratch, delta, err,
+                                                                                 lanes_per_node(G));
+    return cudaGetLastError();
+  }
   switch (heuristic_mode(G.n, smem)) {
     case kDistShared:
       return launch_mode<kDistShared>(G, jobs, njobs, scratch, scratch_words_per_block, blocks, delta, next_job, err, s);

@@ -1,5 +1,6 @@
 // Host-visible declarations shared by the search kernels and the C ABI layer.
 #pragma once
+#include <atomic>
 
 #include "opmos_dev.cuh"
 
@@ -95,8 +96,13 @@ int record_error(int code, const char* msg);
 constexpr size_t kHeurSmem = 200u << 10;
 constexpr size_t kServeBlockSmem = 72u << 10;
 constexpr size_t kHeurSmemServed = 68u << 10;
+// Resident server kernels of this process. While there is one, the heuristic
+// takes blocks that fit beside it: a cluster, or a block with most of an SM's
+// shared memory, would wait for the server's end.
+extern std::atomic<int> resident_servers;
 cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                              size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta,
-                             unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem = kHeurSmem);
+                             unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem = kHeurSmem,
+                             unsigned sms = 0);
 
 }  // namespace opmos
