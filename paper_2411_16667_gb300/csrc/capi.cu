@@ -217,7 +217,7 @@ constexpr uint32_t kWindowCapMin = 16384;  // labels a window may hold at least
 
 // Sizes of one query arena for a given byte budget.
 struct ArenaPlan {
-  uint32_t label_cap, open_cap, win_cap, cand_cap, touch_cap, plog_cap, nslots, lsub, kparts, xcap;
+  uint32_t label_cap, open_cap, win_cap, cand_cap, touch_cap, plog_cap, nslots, lsub, kparts, xcap, nchamps;
   unsigned long long fpool_words;
   size_t bytes;
   size_t fixed;  // the part that does not grow with the labels
@@ -233,16 +233,18 @@ int plan_arena(const opmos_graph* g, uint32_t D, uint32_t window, size_t budget,
   pl->touch_cap = (uint32_t)std::min<size_t>(n + 1, pl->cand_cap);
   pl->plog_cap = batch ? (1u << 16) : (1u << 20);
   const size_t ptiles = pl->plog_cap / 32 + 1;
-  // per node: fbase, fcount, fcap, two champions, then per candidate set ncand, list heads,
+  // per node: fbase, fcount, fcap, champions (two sets), then per candidate set ncand, list heads,
   // split flag, part count, slots; per candidate (two sets): list link, flag, record;
   // per node a window reaches (two sets): touched entry; the parts of split merges
   // (two sets)
   pl->lsub = batch ? kLSubBatch : kLSubGrid;
-  pl->nslots = batch ? kNodeSlots : kNodeSlotsGrid;
+  pl->nslots = batch ? kNodeSlots - row_words((int)D) : kNodeSlotsGrid;
   pl->kparts = kPartsMax;
   // parts of split merges a step may list; when it is full nodes keep the parts they have
   pl->xcap = (batch ? 1u : 8u) * pl->touch_cap;
-  size_t fixed = (n + 1) * (8 + 4 + 4 + 2 * 4 * (size_t)row_words(D) + 2 * (4 + (4u << pl->lsub) + 4 + 4 + 4 * (size_t)pl->nslots)) + 3 * kNB * 4 +
+  const uint32_t nchamps = pl->nchamps = !batch && window >= kLargeWindow ? kChamps : 1u;
+  size_t fixed = (n + 1) * (8 + 4 + 4 + 2 * 4 * nchamps * (size_t)row_words(D) +
+                           2 * (4 + (4u << pl->lsub) + 4 + 4 + 4 * (size_t)pl->nslots)) + 3 * kNB * 4 +
                  2 * (size_t)pl->cand_cap * (8 + 4 * (size_t)row_words((int)D + 2)) + 2 * (size_t)pl->touch_cap * 4 +
                  2 * (size_t)pl->xcap * 8 + (size_t)pl->plog_cap * 4 * D +
                  2 * ((size_t)pl->plog_cap + ptiles) * 4 * D + kPSMax * 4 + 96 * 256;
@@ -267,7 +269,7 @@ void layout_arena(const opmos_graph* g, uint32_t D, const ArenaPlan& pl, char* b
   A->fbase = carve<uint64_t>(p, n);
   A->fcount = carve<uint32_t>(p, n);
   A->fcap = carve<uint32_t>(p, n);
-  for (int b = 0; b < 2; ++b) A->champ[b] = carve<uint32_t>(p, n * row_words((int)D));
+  for (int b = 0; b < 2; ++b) A->champ[b] = carve<uint32_t>(p, n * pl.nchamps * row_words((int)D));
   for (int b = 0; b < 2; ++b) {
     CandSet& cs = A->cs[b];
     cs.ncand = carve<uint32_t>(p, n);
@@ -304,6 +306,7 @@ void layout_arena(const opmos_graph* g, uint32_t D, const ArenaPlan& pl, char* b
   A->plog_cap = pl.plog_cap;
   A->touch_cap = pl.touch_cap;
   A->fpool_words = pl.fpool_words;
+  A->nchamps = pl.nchamps;
   A->nslots = pl.nslots;
   A->lsub = pl.lsub;
   A->kparts = pl.kparts;
@@ -575,7 +578,7 @@ int solve_one(const opmos_graph* g, const opmos_heur* heur, uint32_t start, uint
   P.flags = o.flags;
   P.qd = D;
   P.ps_grow = kGridIndexGrow;
-  P.part_work = part_work(D);
+  P.part_work = part_work(D, o.window);
   P.time_limit_ns = time_limit_ns();
 
   // large windows take the wide grid (two 256-thread blocks per SM)
@@ -648,7 +651,7 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
   P.flags = o.flags;
   P.qd = D;
   P.ps_grow = kMultiIndexGrow;
-  P.part_work = part_work(D);
+  P.part_work = part_work(D, 0);
   P.time_limit_ns = time_limit_ns();
   std::vector<MSlot> hslots(slots);
   for (unsigned i = 0; i < slots; ++i) {
@@ -1321,7 +1324,7 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       sl.P.flags = o.flags;
       sl.P.qd = sv->dmax;
       sl.P.ps_grow = kMultiIndexGrow;
-      sl.P.part_work = part_work(sv->dmax);
+      sl.P.part_work = part_work(sv->dmax, 0);
       sl.P.time_limit_ns = time_limit_ns();
       sl.state = SL_FREE;
     }

@@ -41,20 +41,35 @@ constexpr unsigned kSmallWindow = 16384;  // larger windows take the wide grid
 // A node's merge is split into parts, one warp each, of about part_work(d)
 // comparisons or fewer, kPartsMax at most: a warp alone issues an instruction
 // every 4-5 cycles, so this many take it about 5 us, a step's other work.
-// Measured (kPartWork = 3,000 / 6,000 / 12,000 / 24,000): 256x256 grid d=3 at
-// W = 262,144 134 / 121 / 110 / 108 ms; 160x160 d=3 31.7 / 32.5 / 32.1 / 32.2;
-// 96x96 d=5 first in first out 7.5 / 7.2 / 7.6 / 8.6; route d=12 8.6 / 8.4 /
-// 8.3 / 8.8; 128 queries d=5 40 / 37 / 36 / 36.
+// Measured (kPartWork = 4,096 / 8,192 / 12,288 / 24,576): 160x160 d=3 27.1 / 27.7
+// / 27.2 / 27.2 ms; 96x96 d=5 first in first out 7.2 / 7.3 / 7.5 / 8.5; route
+// d=12 7.6 / 7.5 / 7.6 / 8.1; 128 queries d=5 26.0 / 24.4 / 24.6 / 24.5; 128x128
+// d=3 at W = 65,536 - / 7.0 (6,144) / 7.3 / 7.5. From kLargeWindow on every warp
+// has several parts a step anyway and what a part costs by itself counts: twice
+// the work, 256x256 grid d=3 at W = 262,144 89 -> 87 ms (344 -> 312 ms on a
+// second seed); four times, 93 (303).
 constexpr unsigned kPartWork = 12288;
+constexpr unsigned kLargeWindow = 131072;
 constexpr unsigned kPartsMax = 128;
 constexpr unsigned kPartShares = 8;  // most shares of one group of 32 candidates
-inline unsigned part_work(unsigned d) { return kPartWork / (1u + d / 4u); }
+inline unsigned part_work(unsigned d, unsigned window) {
+  return (window >= kLargeWindow ? 2 : 1) * kPartWork / (1u + d / 4u);
+}
+// Champions a node has (see Search::champion): a single query with a large
+// window takes several, as merges are most of its steps and its nodes have
+// hundreds of candidates; elsewhere more than one costs the expansion what it
+// saves the merges (1 / 2 / 4 / 7 champions: 256x256 d=3 at W = 262,144 99 / 100 /
+// 89 / 92 ms, on a second seed 372 / 365 / 344 / 341; 128x128 d=3 at W = 65,536
+// 7.0 / 7.1 / 7.3 / 7.8; 97x89 d=3 4.46 / 4.50 / 4.60 / -).
+constexpr unsigned kChamps = 4;
 constexpr unsigned kPartPruned = 1u << 16;  // added to a node's part counter by a part that pruned
 constexpr unsigned kSplitParts = 0xFFFFu;     // hflag: parts the node's merge is split into (0: none)
 constexpr unsigned kSplitDone = 1u << 30;     // ... its last part has finished
 constexpr unsigned kSplitSeen = 1u << 31;     // ... its own item has been skipped
 constexpr unsigned kNoPart = 0xFFFFFFFFu;     // a place of xpart that holds no part
-constexpr unsigned kNodeSlots = 56;       // candidate slots per node and step in batch mode
+// candidate slots per node and step in batch mode, less the words of a
+// champion's row (their memory was the slots')
+constexpr unsigned kNodeSlots = 61;
 constexpr unsigned kNodeSlotsGrid = 128;  // ... for a single query (whole-grid search)
 // Lists per node for the candidates beyond the slots (log2): the lanes of a
 // warp walk them side by side, so gathering k of them costs about
@@ -227,7 +242,8 @@ struct QArena {
   uint64_t* fbase;     // n+1
   uint32_t* fcount;    // n+1
   uint32_t* fcap;      // n+1
-  uint32_t* champ[2];  // (n+1) rows: a label of each node that drops candidates at the expansion
+  uint32_t* champ[2];  // (n+1) x nchamps rows: labels of each node that drop candidates at the expansion
+  uint32_t nchamps;
   CandSet cs[2];
   uint32_t* lg;        // d * label_cap
   uint32_t* lnode;

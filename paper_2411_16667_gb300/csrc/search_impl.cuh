@@ -28,8 +28,8 @@
 //                        weakly dominates (PruneOPEN of Algorithm 1, applied
 //                        lazily); window labels are expanded at once along
 //                        their out-arcs (g' = g + c(e), dropped when h(v') is
-//                        infinite or the node's champion -- one accepted label
-//                        of it -- dominates it) into the other candidate set;
+//                        infinite or a champion of the node -- one of its best
+//                        accepted labels -- dominates it) into the other candidate set;
 //                        all other entries are carried to OPEN_{i+1}.
 //
 // Labels created by merge i therefore become extractable from window i+2 on:
@@ -180,7 +180,9 @@ __device__ __forceinline__ bool z_less(const uint32_t (&a)[MD], const uint32_t (
   return a[dim] < b[dim];
 }
 
-template <int D>
+// kMany: nodes may have several champions (A.nchamps); a test for it at run time
+// made short steps 1% slower.
+template <int D, bool kMany = false>
 struct Search {
   static constexpr int DP = row_words(D);      // words of a champion's row
   static constexpr int CW = row_words(D + 2);  // words of a candidate's record: costs, arc, parent
@@ -242,7 +244,7 @@ struct Search {
     fill(T, A.fbase, 2 * n, 0u);
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
-      fill(T, A.champ[b], n * DP, kInf);
+      fill(T, A.champ[b], n * A.nchamps * DP, kInf);
       fill(T, A.cs[b].node_head, n << A.lsub, (uint32_t)kNil);
       fill(T, A.cs[b].ncand, n, 0u);
       fill(T, A.cs[b].hflag, n, 0u);
@@ -610,11 +612,18 @@ struct Search {
           }
           fc = A.fcount[v2];
           if (!goal) {
-            // dropped when the goal is unreachable from v2, or the best label
-            // v2 had when the step began dominates it
+            // dropped when the goal is unreachable from v2, or a champion v2 had
+            // when the step began dominates it
             uint32_t ch[D];
             champion(A.champ[cyc & 1u], v2, ch);
             alive = hk(0, v2) != kInf && !weakly_le<D>(ch, g2);
+            if (kMany && A.nchamps > 1u && alive) {
+#pragma unroll
+              for (unsigned q = 1; q < kChamps; ++q) {
+                champion(A.champ[cyc & 1u], plane(q) + v2, ch);
+                alive = alive && !weakly_le<D>(ch, g2);
+              }
+            }
           }
         }
         add_candidates(cs, K1, alive, v2, par, e, g2, fc);
@@ -1145,34 +1154,45 @@ struct Search {
              (unsigned)((uint64_t)tiles * x / n), (unsigned)((uint64_t)tiles * (x + 1) / n), pd.cur, pcmp);
   }
 
-  // A node's champion is the accepted label of the smallest cost sum. A candidate
-  // it weakly dominates would be dropped by the merge (a label once accepted is
-  // in the frontier or was pruned by one that dominates whatever it dominates),
-  // so the expansion drops it at once: a third to two thirds of all candidates
+  // A node's champion is the accepted label of the smallest cost sum; further ones
+  // (A.nchamps) are those of sums in which one objective weighs four times the
+  // others, then a quarter. A candidate one of them weakly dominates would be
+  // dropped by the merge (a label once accepted is in the frontier or was pruned by
+  // one that dominates whatever it dominates), so the expansion drops it at once: a third to two thirds of all candidates
   // (two thirds to three quarters are dominated by some label). The rows are a
   // pair by step parity: step i reads rows i & 1 and writes the others, so a row
   // is never read half written; an older champion is as valid as a new one.
-  __device__ __forceinline__ static void champion(const uint32_t* rows, uint32_t v, uint32_t (&x)[D]) {
+  __device__ __forceinline__ static void champion(const uint32_t* rows, size_t v, uint32_t (&x)[D]) {
     uint32_t r[DP];
-    vec_load(rows + (size_t)v * DP, r);
+    vec_load(rows + v * DP, r);
 #pragma unroll
     for (int k = 0; k < D; ++k) x[k] = r[k];
   }
+  // Champion q of node v is row plane(q) + v.
+  __device__ __forceinline__ size_t plane(unsigned q) const { return (size_t)q * (G.n + 1ull); }
+  // The cost sum champion Q is the smallest of.
+  template <unsigned Q>
   __device__ __forceinline__ static uint32_t cost_sum(const uint32_t (&x)[D]) {
     unsigned long long sum = 0;
 #pragma unroll
     for (int k = 0; k < D; ++k) sum += x[k];
+    if constexpr (Q > 0) {
+      constexpr unsigned k = (Q - 1) % D;
+      sum = Q <= (unsigned)D ? sum + 3ull * x[k] : 4ull * sum - 3ull * x[k];
+    }
     return (uint32_t)min(sum, (unsigned long long)kInf);
   }
+  template <unsigned Q>
   __device__ __forceinline__ void update_champion(uint32_t v, const Batch& b) {
     uint32_t c0[D], c1[D];
-    uint32_t* const next = A.champ[(cyc & 1u) ^ 1u] + (size_t)v * DP;
-    champion(A.champ[cyc & 1u], v, c0);
-    champion(A.champ[(cyc & 1u) ^ 1u], v, c1);
-    const uint32_t mine = b.alive ? cost_sum(b.c) : kInf;
+    const size_t row = plane(Q) + v;
+    uint32_t* const next = A.champ[(cyc & 1u) ^ 1u] + row * DP;
+    champion(A.champ[cyc & 1u], row, c0);
+    champion(A.champ[(cyc & 1u) ^ 1u], row, c1);
+    const uint32_t mine = b.alive ? cost_sum<Q>(b.c) : kInf;
     const uint32_t best = warp_min(mine);
     const unsigned who = __ballot_sync(0xffffffffu, b.alive && mine == best);
-    const uint32_t s0 = cost_sum(c0), s1 = cost_sum(c1);
+    const uint32_t s0 = cost_sum<Q>(c0), s1 = cost_sum<Q>(c1);
     __syncwarp();  // the rows are read before one is written
     if (best < min(s0, s1)) {
       if (lane_id() == (unsigned)__ffs(who) - 1) {
@@ -1205,7 +1225,15 @@ struct Search {
       if (!is_goal) ob = atomicAdd(fifo ? &C->fifo_tail.v : &K1.open_count.v, ns);
       if (is_goal) plen = ld_volatile(&C->plog_len.v);  // this warp is the log's only writer
     }
-    if (!is_goal) update_champion(v, b);
+    if (!is_goal) {
+      update_champion<0>(v, b);
+      if (kMany && A.nchamps > 1u) {
+        static_assert(kChamps == 4, "one call each");
+        update_champion<1>(v, b);
+        update_champion<2>(v, b);
+        update_champion<3>(v, b);
+      }
+    }
     lb = __shfl_sync(0xffffffffu, lb, 0);
     ob = __shfl_sync(0xffffffffu, ob, 0);
     plen = __shfl_sync(0xffffffffu, plen, 0);
@@ -2000,12 +2028,12 @@ struct Search {
 // ---------------------------------------------------------------------------
 // Single query on the whole cooperative grid
 // ---------------------------------------------------------------------------
-template <int D>
+template <int D, bool kMany>
 __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QParams& P, const OutPool& O,
                          QResult* R) {
   __shared__ Shared S;
   const GridTeam T;
-  Search<D> X(G, A, C, P, O, S);
+  Search<D, kMany> X(G, A, C, P, O, S);
   if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
   for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
   X.init_zero(T);
@@ -2053,7 +2081,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
 template <int D, unsigned NT, unsigned NB>
 __global__ void __launch_bounds__(NT, NB) search_grid_kernel(GraphDev G, QArena A, QCtl* C, QParams P, OutPool O,
                                                              QResult* R) {
-  run_grid<D>(G, A, C, P, O, R);
+  run_grid<D, (NB > 1)>(G, A, C, P, O, R);
 }
 
 // ---------------------------------------------------------------------------

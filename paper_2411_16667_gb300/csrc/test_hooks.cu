@@ -122,6 +122,7 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   A.fpool_words = fpool_words;
   A.nslots = slots;
   A.lsub = lsub;
+  A.nchamps = 1;
   if ((size_t)(p - base) > bytes) return hook_fail(OPMOS_ERR_CAPACITY, "test hook: layout exceeds its buffer");
   e = cudaMemset(mem.p, 0, bytes);
   // host images of what a step finds: frontier of node 0 (labels 0..nfront-1)
@@ -198,7 +199,7 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   P.label_budget = label_cap;
   P.qd = D;
   P.ps_grow = 6;
-  P.part_work = part_work(D);
+  P.part_work = part_work(D, 0);
   OutPool O{nullptr, 0, nullptr};
   merge_hook_kernel<D><<<1, 32, 32 * Search<D>::RP * 4>>>(G, A, C, P, O, nfront, block);
   e = cudaGetLastError();
@@ -399,7 +400,7 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
     P.label_budget = cap;
     P.qd = D;
     P.ps_grow = 6;
-    P.part_work = part_work(D);
+    P.part_work = part_work(D, 0);
     const BinParams bp{bins[0], bins[1], bins[2], bins[3], bins[4]};
     OutPool O{nullptr, 0, nullptr};
     window_hist_kernel<<<64, 256>>>(A, n, bp, A.hist + 1 * kNB);
