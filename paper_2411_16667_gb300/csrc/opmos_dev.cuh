@@ -186,22 +186,21 @@ struct PIdx {
   unsigned shift[3];                  // per-objective shifts balancing the Z-order
 };
 
-// A grid barrier's arrival count and the error word beside it, read together
-// with one 64-bit load.
-struct alignas(8) BarWord {
-  unsigned count;
+// A grid barrier. state holds the arrivals in its upper half and, in bit 0,
+// whether an error is set; every access to it is of 64 bits, as accesses of
+// different sizes to one place are not ordered with each other. error is the
+// first error's code, written before the bit is set (set_error).
+struct alignas(16) Barrier {
+  unsigned long long state;
   unsigned error;
+  unsigned pad;
 };
+constexpr unsigned long long kBarArrival = 1ull << 32;
+constexpr unsigned long long kBarError = 1ull;
 
 // Per-query control block (global memory).
 struct QCtl {
-  union {
-    BarWord bar;       // single query: the grid barrier
-    struct {
-      unsigned bar_arrivals;
-      unsigned error;  // bar.error
-    };
-  };
+  Barrier bar;         // single query: the grid barrier; bar.error: the query's error, 0 for none
   unsigned done;
   unsigned step;
   unsigned res_count;
@@ -324,7 +323,12 @@ __device__ __forceinline__ unsigned agg_inc(unsigned* ctr) {
   return base + __popc(mask & lanemask_lt());
 }
 
-__device__ __forceinline__ void set_error(QCtl* C, unsigned code) { atomicCAS(&C->error, 0u, code); }
+__device__ __forceinline__ void set_error(Barrier* b, unsigned code) {
+  atomicCAS(&b->error, 0u, code);
+  __threadfence();  // the code before the bit that announces it
+  atomicOr(&b->state, kBarError);
+}
+__device__ __forceinline__ void set_error(QCtl* C, unsigned code) { set_error(&C->bar, code); }
 
 // ---------------------------------------------------------------------------
 // Dominance on d-vectors (Sec. 3): a dominates b iff a <= b componentwise and
@@ -369,33 +373,34 @@ constexpr unsigned long long kBarrierTimeoutNs = 20ull * 1000 * 1000 * 1000;  //
 
 // One block's wait at a grid-wide barrier (one thread calls it, between block
 // barriers): it announces its block and waits until `target` blocks have
-// arrived since the launch; returns the error word. The count only grows, so
-// the last arrival itself releases the others, and the error word is read
-// with it: no reset, no second counter, one fence on each side. Measured
-// with 152 blocks: 1.2 us, against 2.2 us for a counter that the last block
-// resets before it raises a generation. The wait is bounded (gives up with
-// OPMOS_ERR_TIMEOUT, never hangs) and ends early once an error is set.
-__device__ __forceinline__ unsigned grid_barrier(BarWord* b, unsigned target) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
+// arrived since the launch; returns whether no error is set. The count only
+// grows (modulo 2^32: a carry leaves the word), so the last arrival itself
+// releases the others, and the error bit is read with it: no reset, no second
+// counter, one fence on each side. Measured with 152 blocks: 1.2 us, against
+// 2.2 us for a counter that the last block resets before it raises a
+// generation. The wait is bounded (gives up with OPMOS_ERR_TIMEOUT, never
+// hangs) and ends early once an error is set.
+__device__ __forceinline__ bool grid_barrier(Barrier* b, unsigned target) {
+  asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(&b->state), "l"(kBarArrival) : "memory");
   unsigned long long t0 = 0;
   for (unsigned spins = 0;; ++spins) {
     unsigned long long w;
     // relaxed polls and one fence at the end: an acquire per poll would drop
     // the SM's L1 under the blocks still at work on it
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(b) : "memory");
-    const unsigned err = (unsigned)(w >> 32);
-    if ((int)((unsigned)w - target) >= 0) {
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(&b->state) : "memory");
+    const bool err = (w & kBarError) != 0;
+    if ((int)((unsigned)(w >> 32) - target) >= 0) {
       __threadfence();
-      return err;
+      return !err;
     }
     if (spins < 64u) continue;
-    if (err) return err;
+    if (err) return false;
     if ((spins & 255u) == 0u) {
       const unsigned long long t = globaltimer();
       if (t0 == 0) t0 = t;
       if (t - t0 > kBarrierTimeoutNs) {
-        atomicCAS(&b->error, 0u, (unsigned)OPMOS_ERR_TIMEOUT);
-        return OPMOS_ERR_TIMEOUT;
+        set_error(b, (unsigned)OPMOS_ERR_TIMEOUT);
+        return false;
       }
     }
     if (spins > 1024u) __nanosleep(32);
@@ -419,7 +424,7 @@ struct GridTeam {
     __syncthreads();
     if (threadIdx.x == 0) {
       target += gridDim.x;
-      s_ok = grid_barrier(&C->bar, target) == 0u;
+      s_ok = grid_barrier(&C->bar, target);
     }
     __syncthreads();
     return s_ok != 0;
@@ -438,7 +443,7 @@ struct BlockTeam {
   __device__ __forceinline__ bool sync(QCtl* C) const {
     __shared__ unsigned s_ok;
     __syncthreads();
-    if (threadIdx.x == 0) s_ok = ld_volatile(&C->error) == 0;
+    if (threadIdx.x == 0) s_ok = ld_volatile(&C->bar.error) == 0;
     __syncthreads();
     return s_ok != 0;
   }

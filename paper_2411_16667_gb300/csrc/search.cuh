@@ -28,7 +28,7 @@ struct MQuery {    // a queued query
 };
 
 struct MCtl {      // grid-wide control of the multi-query kernel
-  BarWord bar;  // the grid barrier
+  Barrier bar;  // the grid barrier
   unsigned done, pad;
   unsigned q_next, iter, qcap, hold;  // hold: keep slots until the host releases them
   unsigned pref[kMaxSlots + 1];       // virtual blocks of the iteration: prefix sums over the slots

@@ -283,7 +283,7 @@ struct Search {
   __device__ void init_seed(const Team& T, bool reset_ctl) {
     if (!T.leader()) return;
     if (reset_ctl) {
-      C->error = 0;
+      C->bar.error = 0;
       C->done = 0;
       C->res_count = C->res_status = 0;
       C->res_off = C->res_path = C->res_total = 0;
@@ -2067,7 +2067,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
   T.sync(C);
   if (T.leader()) {
     __threadfence();
-    R->status = *reinterpret_cast<volatile unsigned*>(&C->error);
+    R->status = *reinterpret_cast<volatile unsigned*>(&C->bar.error);
     R->count = C->res_count;
     R->off = C->res_off;
     R->path = C->res_path;
@@ -2114,7 +2114,7 @@ __device__ inline bool mq_barrier(MCtl* M, unsigned& target) {
   __syncthreads();
   if (threadIdx.x == 0) {
     target += gridDim.x;
-    s_ok = grid_barrier(&M->bar, target) == 0u;
+    s_ok = grid_barrier(&M->bar, target);
   }
   __syncthreads();
   return s_ok != 0;
@@ -2124,7 +2124,7 @@ __device__ inline void mq_write_result(const MSlot& sl, unsigned slot, QCtl* C, 
                                        unsigned* done_flags, unsigned qcap) {
   const unsigned ri = sl.qidx % qcap;
   QResult* R = &results[ri];
-  R->status = ld_volatile(&C->error);
+  R->status = ld_volatile(&C->bar.error);
   R->slot = slot;
   R->count = C->res_count;
   R->off = C->res_off;
@@ -2152,7 +2152,7 @@ __device__ void mq_alloc_region1(const MSlot& sl, QCtl* C) {
   const unsigned kk_live = ld_volatile(&C->res_count);
   const unsigned long long words = (unsigned long long)kk_live * D + kk_live + 1;
   const unsigned long long off = atomicAdd(O.used, words);
-  if (off + words > O.cap) atomicCAS(&C->error, 0u, (unsigned)OPMOS_ERR_CAPACITY);
+  if (off + words > O.cap) set_error(C, OPMOS_ERR_CAPACITY);
   C->res_off = off;
 }
 
@@ -2223,14 +2223,14 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
       // the step that comes next, from one round of loads
       const unsigned step = st == SL_RUN ? __ldcg(&C->step) + 1u : 0u;
       const CycleCtl& K = C->cyc[step % 3];
-      const unsigned err = ld_volatile(&C->error), open = __ldcg(&K.open_count.v) - __ldcg(&K.head.v),
+      const unsigned err = ld_volatile(&C->bar.error), open = __ldcg(&K.open_count.v) - __ldcg(&K.head.v),
                      touched = __ldcg(&K.touched_count.v), parts = __ldcg(&K.part_count.v);
       const bool late = st == SL_RUN && globaltimer() - C->t_start > sl.P.time_limit_ns;
       C->step = step;
       if (err || (open == 0 && touched == 0)) {
         st = SL_OUT1;
       } else if (late) {
-        atomicCAS(&C->error, 0u, (unsigned)OPMOS_ERR_TIMEOUT);
+        set_error(C, OPMOS_ERR_TIMEOUT);
         st = SL_OUT1;
       } else {
         st = SL_RUN;
@@ -2239,12 +2239,12 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
       if (st == SL_OUT1) C->res_count = 0;
     } else if (st == SL_OUT1 || st == SL_OUT2 || st == SL_OUT3 || st == SL_OUT4) {
       // one output part per iteration; an error ends the output early
-      if (ld_volatile(&C->error) || st == SL_OUT4) {
+      if (ld_volatile(&C->bar.error) || st == SL_OUT4) {
         mq_write_result(sl, q, C, results, done_flags, qcap);
         st = after_out;
       } else if (st == SL_OUT1) {
         mq_alloc_region1<D>(sl, C);
-        if (ld_volatile(&C->error)) {  // no room for the result: report, never write
+        if (ld_volatile(&C->bar.error)) {  // no room for the result: report, never write
           mq_write_result(sl, q, C, results, done_flags, qcap);
           st = after_out;
         } else {
@@ -2316,7 +2316,7 @@ __device__ void mq_work(MSlot* slots, QCtl* ctls, unsigned q, unsigned j, unsign
   if (st == SL_INIT) {
     const BlockTeam T;
     X.init_zero(T);
-    if (threadIdx.x == 0) C->error = 0;
+    if (threadIdx.x == 0) C->bar.error = 0;
     __syncthreads();
     X.init_seed(T, true);
     __syncthreads();

@@ -208,7 +208,7 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   unsigned err = 0;
   uint64_t fb = 0;
   uint32_t fc = 0, cap = 0;
-  e = cudaMemcpy(&err, &C->error, 4, cudaMemcpyDeviceToHost);
+  e = cudaMemcpy(&err, &C->bar.error, 4, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemcpy(&fb, A.fbase, 8, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemcpy(&fc, A.fcount, 4, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess) e = cudaMemcpy(&cap, A.fcap, 4, cudaMemcpyDeviceToHost);
@@ -410,7 +410,7 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
     if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook kernel: %s", cudaGetErrorString(e));
     unsigned kept = 0, err = 0;
     e = cudaMemcpy(&kept, &C->cyc[2].open_count.v, 4, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess) e = cudaMemcpy(&err, &C->error, 4, cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(&err, &C->bar.error, 4, cudaMemcpyDeviceToHost);
     if (e == cudaSuccess) e = cudaMemcpy(bstar, d_bstar, 4, cudaMemcpyDeviceToHost);
     std::vector<uint32_t> kid(kept);
     if (e == cudaSuccess && kept) e = cudaMemcpy(kid.data(), A.oid[0], kept * 4, cudaMemcpyDeviceToHost);
