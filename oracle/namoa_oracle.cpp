@@ -49,6 +49,7 @@ constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kMaxD = 16;
 
 enum { ORC_OK = 0, ORC_INVALID = 1, ORC_OVERFLOW = 2, ORC_BUDGET = 3, ORC_NOMEM = 4 };
+constexpr int kTooWide = -1;  // a cost that does not fit a byte (see Bytes)
 
 struct GraphView {
   uint32_t n;
@@ -165,6 +166,93 @@ inline bool equal(const uint64_t* a, const uint64_t* b, int d) {
   return true;
 }
 
+// Many objectives with small costs: the dominance tests of a search whose
+// front holds 100,000 vectors of 16 objectives take an hour on labels read one
+// after the other. When every cost met fits a byte, each set keeps its vectors
+// by columns as well, and a test takes 16 labels at a time (half a minute).
+// Algorithm, order and counters are the same.
+constexpr int kBytesMinD = 9;
+struct Bytes {
+  uint8_t x[kMaxD];
+};
+// v as bytes; false when an entry does not fit.
+inline bool to_bytes(const uint64_t* v, int d, Bytes* out) {
+  for (int i = 0; i < d; ++i) {
+    if (v[i] > 255) return false;
+    out->x[i] = (uint8_t)v[i];
+  }
+  return true;
+}
+
+// Labels, and their vectors as columns of bytes where the search keeps those.
+struct Set {
+  int d = 0;
+  std::vector<uint32_t> id;
+  std::vector<uint8_t> col[kMaxD];
+  size_t size() const { return id.size(); }
+  void push_back(uint32_t i) { id.push_back(i); }
+  void push_back(uint32_t i, const Bytes& b) {
+    id.push_back(i);
+    for (int k = 0; k < d; ++k) col[k].push_back(b.x[k]);
+  }
+  void erase(size_t i) {
+    id.erase(id.begin() + i);
+    for (int k = 0; k < d; ++k) col[k].erase(col[k].begin() + i);
+  }
+  void erase_id(uint32_t x) {
+    auto it = std::find(id.begin(), id.end(), x);
+    if (it != id.end()) erase(it - id.begin());
+  }
+  // The last label takes the place of label i.
+  void swap_out(size_t i) {
+    id[i] = id.back();
+    id.pop_back();
+    for (int k = 0; k < d; ++k) {
+      col[k][i] = col[k].back();
+      col[k].pop_back();
+    }
+  }
+  // The first label from place `from` on that weakly dominates b (ABOVE: that b
+  // weakly dominates); size() if there is none.
+  template <bool ABOVE>
+  size_t next(const Bytes& b, size_t from) const {
+    typedef uint8_t V __attribute__((vector_size(16)));
+    const size_t n = size();
+    size_t i = from;
+    V bound[kMaxD];
+    if (i + 16 <= n)
+      for (int k = 0; k < d; ++k) bound[k] = V{} + b.x[k];
+    for (; i + 16 <= n; i += 16) {
+      uint64_t m[2] = {~0ull, ~0ull};
+      for (int k = 0; k < d && (m[0] | m[1]); k += 4) {  // a byte stays 0xff while its label qualifies
+        V all = ~V{};
+        for (int j = k; j < d && j < k + 4; ++j) {
+          V c;
+          std::memcpy(&c, &col[j][i], 16);
+          all &= (V)(ABOVE ? c >= bound[j] : c <= bound[j]);
+        }
+        uint64_t a[2];
+        std::memcpy(a, &all, 16);
+        m[0] &= a[0];
+        m[1] &= a[1];
+      }
+      if (m[0] | m[1]) break;  // one of these 16
+    }
+    for (; i < n; ++i) {
+      bool q = true;
+      for (int k = 0; k < d && q; ++k) q = ABOVE ? col[k][i] >= b.x[k] : col[k][i] <= b.x[k];
+      if (q) return i;
+    }
+    return n;
+  }
+  bool equals(size_t i, const Bytes& b) const {
+    for (int k = 0; k < d; ++k)
+      if (col[k][i] != b.x[k]) return false;
+    return true;
+  }
+};
+
+template <bool BYTES>
 struct Namoa {
   const GraphView& G;
   const uint32_t* h;
@@ -185,32 +273,75 @@ struct Namoa {
     }
   };
   std::set<uint32_t, Lex> open;
-  std::vector<std::vector<uint32_t>> gop, gcl;
+  std::vector<Set> gop, gcl;
   std::vector<uint8_t> visited;
-  std::vector<uint32_t> P;
+  Set P;
   Counters cnt;
+  // BYTES: OPEN's F side by side (in no order), every label's place there, and
+  // its g
+  Set open_rows;
+  std::vector<uint32_t> open_at;
+  std::vector<Bytes> gb;
 
   Namoa(const GraphView& g, const uint32_t* hh, uint32_t s, uint32_t t, uint64_t b)
       : G(g), h(hh), start(s), goal(t), d((int)g.d), budget(b), open(Lex{&pool, (int)g.d}),
         gop(g.n), gcl(g.n), visited(g.n, 0) {
     pool.d = d;
+    if (BYTES) {
+      for (auto* sets : {&gop, &gcl})
+        for (Set& s : *sets) s.d = d;
+      P.d = open_rows.d = d;
+    }
   }
 
   uint32_t hv(uint32_t k, uint32_t v) const { return h[(uint64_t)k * G.n + v]; }
   bool h_inf(uint32_t v) const { return hv(0, v) == kInf32; }
 
-  static void erase_id(std::vector<uint32_t>& s, uint32_t id) {
-    auto it = std::find(s.begin(), s.end(), id);
-    if (it != s.end()) s.erase(it);
+  void add(Set& s, uint32_t id) {
+    if (BYTES)
+      s.push_back(id, gb[id]);
+    else
+      s.push_back(id);
+  }
+  // BYTES: label id leaves the rows of OPEN.
+  void open_rows_erase(uint32_t id) {
+    const uint32_t at = open_at[id];
+    open_at[open_rows.id.back()] = at;
+    open_rows.swap_out(at);
   }
 
   // NotDominated(x, P) in the weak reading: no p in P with g(p) <= x.
-  bool not_dominated_by_P(const uint64_t* x) {
-    for (uint32_t p : P) {
-      cnt.comparisons++;
-      if (weakly(pool.g(p), x, d)) return false;
+  bool not_dominated_by_P(const uint64_t* x, const Bytes& x8) {
+    size_t i = 0;
+    if (BYTES)
+      i = P.next<false>(x8, 0);
+    else
+      while (i < P.size() && !weakly(pool.g(P.id[i]), x, d)) ++i;
+    cnt.comparisons += std::min(i + 1, P.size());
+    return i == P.size();
+  }
+  // Removes from s what the vector g strictly dominates (from_open: also from
+  // OPEN); returns how many.
+  size_t prune(Set& s, const uint64_t* g, const Bytes& g8, bool from_open) {
+    const size_t before = s.size();
+    cnt.comparisons += before;
+    for (size_t i = 0;;) {
+      if (BYTES) {
+        i = s.next<true>(g8, i);
+        if (i < s.size() && s.equals(i, g8)) {
+          ++i;
+          continue;
+        }
+      } else {
+        while (i < s.size() && !dominates(g, pool.g(s.id[i]), d)) ++i;
+      }
+      if (i == s.size()) return before - s.size();
+      if (from_open) {
+        open.erase(s.id[i]);
+        if (BYTES) open_rows_erase(s.id[i]);
+      }
+      s.erase(i);
     }
-    return true;
   }
 
   std::chrono::steady_clock::time_point t0;
@@ -228,12 +359,22 @@ struct Namoa {
     pool.gv.insert(pool.gv.end(), g, g + d);
     pool.Fv.insert(pool.Fv.end(), F, F + d);
     *id = (uint32_t)(pool.size() - 1);
+    if (BYTES) {
+      Bytes b;
+      if (!to_bytes(g, d, &b)) return kTooWide;
+      gb.push_back(b);
+    }
     return ORC_OK;
   }
 
-  void open_insert(uint32_t id) {
+  void open_insert(uint32_t id, const Bytes& F8) {
     open.insert(id);
-    gop[pool.node[id]].push_back(id);
+    if (BYTES) {
+      open_at.resize(id + 1);
+      open_at[id] = (uint32_t)open_rows.size();
+      open_rows.push_back(id, F8);
+    }
+    add(gop[pool.node[id]], id);
     visited[pool.node[id]] = 1;
     cnt.inserted++;
     if (open.size() > cnt.max_open) cnt.max_open = open.size();
@@ -245,43 +386,49 @@ struct Namoa {
     uint64_t zero[kMaxD] = {0}, Fs[kMaxD];
     for (int i = 0; i < d; ++i) Fs[i] = h_inf(start) ? kInf64 : hv(i, start);
     uint32_t ls;
+    Bytes g8{}, F8{};
+    if (BYTES && !to_bytes(Fs, d, &F8)) return kTooWide;
     if (int rc = new_label(start, kNone, ~0ull, zero, Fs, &ls)) return rc;
-    open_insert(ls);
+    open_insert(ls, F8);
     // main loop: while OPEN is not empty
     while (!open.empty()) {
       // l <- OPEN.popmin()
       uint32_t l = *open.begin();
       open.erase(open.begin());
+      if (BYTES) open_rows_erase(l);
       cnt.extracted++;
       const uint32_t v = pool.node[l];
       // move l from G_OP(v) to G_CL(v)
-      erase_id(gop[v], l);
-      gcl[v].push_back(l);
+      gop[v].erase_id(l);
+      add(gcl[v], l);
       if (v == goal) {
         cnt.goal_extracted++;
         // goal branch: PruneOPEN(l) over the whole OPEN
-        for (auto it = open.begin(); it != open.end();) {
-          cnt.comparisons++;
-          if (weakly(pool.g(l), pool.F(*it), d)) {
-            erase_id(gop[pool.node[*it]], *it);
-            it = open.erase(it);
+        cnt.comparisons += open.size();
+        if (BYTES) {
+          for (size_t i = 0; (i = open_rows.next<true>(gb[l], i)) < open_rows.size();) {
+            const uint32_t x = open_rows.id[i];
+            gop[pool.node[x]].erase_id(x);
+            open.erase(x);
+            open_rows_erase(x);  // the last one takes its place
             cnt.pruned_open_goal++;
-          } else {
-            ++it;
+          }
+        } else {
+          for (auto it = open.begin(); it != open.end();) {
+            if (weakly(pool.g(l), pool.F(*it), d)) {
+              gop[pool.node[*it]].erase_id(*it);
+              it = open.erase(it);
+              cnt.pruned_open_goal++;
+            } else {
+              ++it;
+            }
           }
         }
         // Prune(P, l)
-        for (size_t i = 0; i < P.size();) {
-          cnt.comparisons++;
-          if (dominates(pool.g(l), pool.g(P[i]), d)) {
-            P.erase(P.begin() + i);
-            cnt.pruned_p++;
-          } else {
-            ++i;
-          }
-        }
+        if (BYTES) g8 = gb[l];
+        cnt.pruned_p += prune(P, pool.g(l), g8, false);
         // insert l into P unless a member weakly dominates it
-        if (not_dominated_by_P(pool.g(l))) P.push_back(l);
+        if (not_dominated_by_P(pool.g(l), g8)) add(P, l);
         continue;
       }
       // expansion of l along the out-arcs of v
@@ -296,63 +443,56 @@ struct Namoa {
           g2[i] = pool.g(l)[i] + G.c(i, e);
           F2[i] = g2[i] + hv(i, vp);
         }
+        if (BYTES && !(to_bytes(g2, d, &g8) && to_bytes(F2, d, &F8))) return kTooWide;
         if (!visited[vp]) {
           // v' never visited: insert l' unless P dominates F(l')
-          if (not_dominated_by_P(F2)) {
+          if (not_dominated_by_P(F2, F8)) {
             uint32_t id;
             if (int rc = new_label(vp, l, e, g2, F2, &id)) return rc;
-            open_insert(id);
+            open_insert(id, F8);
           }
           continue;
         }
-        // Duplicate(l')
-        bool dup = false;
-        for (const auto* S : {&gop[vp], &gcl[vp]})
-          for (uint32_t x : *S) {
-            cnt.comparisons++;
-            if (equal(pool.g(x), g2, d)) dup = true;
+        // Duplicate(l'), then NotDominated(l', G_OP(v')) and NotDominated(l', G_CL(v')):
+        // each compares l' with every label of v'
+        const uint64_t labels = gop[vp].size() + gcl[vp].size();
+        bool dup = false, dominated = false;
+        if (BYTES) {
+          // no label of v' dominates another, so one that equals l' and one
+          // that dominates it are not both there: the first that weakly
+          // dominates it tells which
+          for (const auto* S : {&gop[vp], &gcl[vp]}) {
+            const size_t i = S->template next<false>(g8, 0);
+            if (i == S->size()) continue;
+            (S->equals(i, g8) ? dup : dominated) = true;
+            break;
           }
-        if (dup) continue;
-        // NotDominated(l', G_OP(v')) and NotDominated(l', G_CL(v'))
-        bool dominated = false;
-        for (const auto* S : {&gop[vp], &gcl[vp]})
-          for (uint32_t x : *S) {
-            cnt.comparisons++;
-            if (dominates(pool.g(x), g2, d)) dominated = true;
-          }
-        if (dominated) continue;
+        } else {
+          for (const auto* S : {&gop[vp], &gcl[vp]})
+            for (uint32_t x : S->id)
+              if (equal(pool.g(x), g2, d)) dup = true;
+          if (!dup)
+            for (const auto* S : {&gop[vp], &gcl[vp]})
+              for (uint32_t x : S->id)
+                if (dominates(pool.g(x), g2, d)) dominated = true;
+        }
+        cnt.comparisons += dup ? labels : 2 * labels;
+        if (dup || dominated) continue;
         // Prune(G_CL(v'), l')
-        for (size_t i = 0; i < gcl[vp].size();) {
-          cnt.comparisons++;
-          if (dominates(g2, pool.g(gcl[vp][i]), d)) {
-            gcl[vp].erase(gcl[vp].begin() + i);
-            cnt.pruned_closed++;
-          } else {
-            ++i;
-          }
-        }
+        cnt.pruned_closed += prune(gcl[vp], g2, g8, false);
         // Prune(G_OP(v'), l') and remove the pruned labels from OPEN
-        for (size_t i = 0; i < gop[vp].size();) {
-          cnt.comparisons++;
-          if (dominates(g2, pool.g(gop[vp][i]), d)) {
-            open.erase(gop[vp][i]);
-            gop[vp].erase(gop[vp].begin() + i);
-            cnt.pruned_open++;
-          } else {
-            ++i;
-          }
-        }
+        cnt.pruned_open += prune(gop[vp], g2, g8, true);
         // insert l' unless P dominates F(l')
-        if (not_dominated_by_P(F2)) {
+        if (not_dominated_by_P(F2, F8)) {
           uint32_t id;
           if (int rc = new_label(vp, l, e, g2, F2, &id)) return rc;
-          open_insert(id);
+          open_insert(id, F8);
         }
       }
     }
     cnt.ns = (uint64_t)std::chrono::duration_cast<std::chrono::nanoseconds>(
                  std::chrono::steady_clock::now() - t0).count();
-    for (uint32_t p : P)
+    for (uint32_t p : P.id)
       for (int i = 0; i < d; ++i)
         if (pool.g(p)[i] >= kInf32) return ORC_OVERFLOW;
     return ORC_OK;
@@ -371,6 +511,49 @@ struct oracle_result {
   Counters cnt;
   uint64_t labels = 0;
 };
+
+namespace {
+
+template <bool BYTES>
+int solve(const GraphView& G, const uint32_t* h, uint32_t start, uint32_t goal, uint64_t budget, oracle_result** out) {
+  const uint32_t d = G.d;
+  Namoa<BYTES> S(G, h, start, goal, budget);
+  const int rc = S.run();
+  if (rc && rc != ORC_BUDGET) return rc;
+  auto* r = new oracle_result;
+  r->d = d;
+  r->cnt = S.cnt;
+  r->labels = S.pool.size();
+  if (rc == ORC_BUDGET) {
+    // stopped by the budget: counters only (the front is not final)
+    r->partial = 1;
+    *out = r;
+    return ORC_BUDGET;
+  }
+  std::vector<uint32_t> P = S.P.id;
+  std::sort(P.begin(), P.end(), [&](uint32_t a, uint32_t b) {
+    for (uint32_t i = 0; i < d; ++i)
+      if (S.pool.g(a)[i] != S.pool.g(b)[i]) return S.pool.g(a)[i] < S.pool.g(b)[i];
+    return a < b;
+  });
+  for (uint32_t p : P) {
+    for (uint32_t i = 0; i < d; ++i) r->costs.push_back((uint32_t)S.pool.g(p)[i]);
+    std::vector<uint32_t> nodes;
+    std::vector<uint64_t> edges;
+    for (uint32_t x = p; x != kNone; x = S.pool.parent[x]) {
+      nodes.push_back(S.pool.node[x]);
+      if (S.pool.parent[x] != kNone) edges.push_back(S.pool.edge[x]);
+    }
+    std::reverse(nodes.begin(), nodes.end());
+    std::reverse(edges.begin(), edges.end());
+    r->nodes.push_back(std::move(nodes));
+    r->edges.push_back(std::move(edges));
+  }
+  *out = r;
+  return ORC_OK;
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -401,40 +584,12 @@ int oracle_solve(uint32_t n, uint64_t m, uint32_t d, const uint64_t* rowptr, con
       if (int rc = reverse_dijkstra(G, goal, hbuf.data())) return rc;
       h = hbuf.data();
     }
-    Namoa S(G, h, start, goal, label_budget ? label_budget : ~0ull);
-    const int rc = S.run();
-    if (rc && rc != ORC_BUDGET) return rc;
-    auto* r = new oracle_result;
-    r->d = d;
-    r->cnt = S.cnt;
-    r->labels = S.pool.size();
-    if (rc == ORC_BUDGET) {
-      // stopped by the budget: counters only (the front is not final)
-      r->partial = 1;
-      *out = r;
-      return ORC_BUDGET;
+    const uint64_t budget = label_budget ? label_budget : ~0ull;
+    if (d >= (uint32_t)kBytesMinD) {
+      const int rc = solve<true>(G, h, start, goal, budget, out);
+      if (rc != kTooWide) return rc;
     }
-    std::vector<uint32_t> P = S.P;
-    std::sort(P.begin(), P.end(), [&](uint32_t a, uint32_t b) {
-      for (uint32_t i = 0; i < d; ++i)
-        if (S.pool.g(a)[i] != S.pool.g(b)[i]) return S.pool.g(a)[i] < S.pool.g(b)[i];
-      return a < b;
-    });
-    for (uint32_t p : P) {
-      for (uint32_t i = 0; i < d; ++i) r->costs.push_back((uint32_t)S.pool.g(p)[i]);
-      std::vector<uint32_t> nodes;
-      std::vector<uint64_t> edges;
-      for (uint32_t x = p; x != kNone; x = S.pool.parent[x]) {
-        nodes.push_back(S.pool.node[x]);
-        if (S.pool.parent[x] != kNone) edges.push_back(S.pool.edge[x]);
-      }
-      std::reverse(nodes.begin(), nodes.end());
-      std::reverse(edges.begin(), edges.end());
-      r->nodes.push_back(std::move(nodes));
-      r->edges.push_back(std::move(edges));
-    }
-    *out = r;
-    return ORC_OK;
+    return solve<false>(G, h, start, goal, budget, out);
   } catch (const std::bad_alloc&) {
     return ORC_NOMEM;
   }
