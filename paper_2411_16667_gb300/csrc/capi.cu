@@ -240,8 +240,10 @@ int plan_arena(const opmos_graph* g, uint32_t D, uint32_t window, size_t budget,
   pl->lsub = batch ? kLSubBatch : kLSubGrid;
   pl->nslots = batch ? kNodeSlots - row_words((int)D) : kNodeSlotsGrid;
   pl->kparts = kPartsMax;
-  // parts of split merges a step may list; when it is full nodes keep the parts they have
-  pl->xcap = (batch ? 1u : 8u) * pl->touch_cap;
+  // parts of split merges a step may list: some a node, and enough for every
+  // warp to have several on graphs of few nodes (see Search::next_scale)
+  const uint32_t xnodes = (batch ? 1u : 8u) * pl->touch_cap;
+  pl->xcap = std::max(xnodes, batch ? kPartPlacesBatch : kPartPlacesGrid);
   const uint32_t nchamps = pl->nchamps = !batch && window >= kLargeWindow ? kChamps : 1u;
   size_t fixed = (n + 1) * (8 + 4 + 4 + 2 * 4 * nchamps * (size_t)row_words(D) +
                            2 * (4 + (4u << pl->lsub) + 4 + 4 + 4 * (size_t)pl->nslots)) + 3 * kNB * 4 +
@@ -249,7 +251,8 @@ int plan_arena(const opmos_graph* g, uint32_t D, uint32_t window, size_t budget,
                  2 * (size_t)pl->xcap * 8 + (size_t)pl->plog_cap * 4 * D +
                  2 * ((size_t)pl->plog_cap + ptiles) * 4 * D + kPSMax * 4 + 96 * 256;
   pl->fixed = fixed;
-  if (budget < fixed + (8u << 20))
+  // (what the least places add to small graphs comes out of the 8 MiB)
+  if (budget + 2 * (size_t)(pl->xcap - xnodes) * 8 < fixed + (8u << 20))
     return fail(OPMOS_ERR_CAPACITY, "arena budget %zu too small (fixed part %zu)", budget, fixed);
   const size_t rem = budget - fixed;
   const size_t per_label = 4 * D + 20;  // cost vector, node, parent, arc, P-log mark, death step

@@ -51,6 +51,10 @@ constexpr unsigned kSmallWindow = 16384;  // larger windows take the wide grid
 constexpr unsigned kPartWork = 12288;
 constexpr unsigned kLargeWindow = 131072;
 constexpr unsigned kPartsMax = 128;
+// Least places of the list of a step's parts: eight warps' worth a warp of the
+// grid for a single query, a block's worth of a batch's two an SM in a batch.
+constexpr unsigned kPartPlacesGrid = 16384;
+constexpr unsigned kPartPlacesBatch = 2048;
 constexpr unsigned kPartShares = 8;  // most shares of one group of 32 candidates
 inline unsigned part_work(unsigned d, unsigned window) {
   return (window >= kLargeWindow ? 2 : 1) * kPartWork / (1u + d / 4u);
@@ -147,7 +151,8 @@ struct CycleCtl {
   Hot<unsigned> open_count;         // entries of step i's OPEN array (FIFO: the ring's tail)
   Hot<unsigned> head;               // FIFO: the ring position window i+1 starts at (0 otherwise)
   Hot<unsigned> touched_count;      // nodes window i's candidates reach
-  Hot<unsigned> part_count;         // places of xpart claimed for parts of split merges
+  Hot<unsigned> part_count;         // places of xpart asked for, for parts of split merges
+  Hot<unsigned> part_scale;         // the parts were of part_work << part_scale comparisons
   Hot<unsigned> plen;               // P-log length every reader uses in step i
   Hot<unsigned> lbase;              // labels that existed when step i began
   Hot<unsigned> win_min;            // smallest F[0] among the labels of window i
@@ -166,7 +171,7 @@ struct CycleCtl {
 // The record's words a step reads: the counters above (the last one in two
 // words), the bins of its histogram and the P index.
 enum RecWord {
-  RW_OPEN, RW_HEAD, RW_TOUCHED, RW_PARTS, RW_PLEN, RW_LBASE, RW_WMIN, RW_WPREV, RW_WMAX, RW_F1LO, RW_F1HI,
+  RW_OPEN, RW_HEAD, RW_TOUCHED, RW_PARTS, RW_SCALE, RW_PLEN, RW_LBASE, RW_WMIN, RW_WPREV, RW_WMAX, RW_F1LO, RW_F1HI,
   RW_KEYLO, RW_KEYHI, RW_BINS, RW_PIDX = RW_BINS + 5, kRecWords = RW_PIDX + 10
 };
 static_assert(kRecWords <= 32, "one lane a word");
