@@ -2241,7 +2241,8 @@ __device__ void mq_schedule(MSlot* slots, QCtl* ctls, unsigned nslots, const MQu
       const unsigned step = st == SL_RUN ? __ldcg(&C->step) + 1u : 0u;
       const CycleCtl& K = C->cyc[step % 3];
       const unsigned err = ld_volatile(&C->bar.error), open = __ldcg(&K.open_count.v) - __ldcg(&K.head.v),
-                     touched = __ldcg(&K.touched_count.v), parts = __ldcg(&K.part_count.v);
+                     touched = __ldcg(&K.touched_count.v);
+      const unsigned parts = min(__ldcg(&K.part_count.v), sl.A.xcap);  // (asked for; the list holds so many)
       const bool late = st == SL_RUN && globaltimer() - C->t_start > sl.P.time_limit_ns;
       C->step = step;
       if (err || (open == 0 && touched == 0)) {
