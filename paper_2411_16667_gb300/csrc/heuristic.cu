@@ -424,13 +424,20 @@ unsigned lanes_per_node(const GraphDev& G) {
   return lpn;
 }
 
+// Allows a kernel as much dynamic shared memory as any launch of it may take.
+// The bound belongs to the kernel, not to the launch, and other threads launch
+// it for other graphs (opmos_heuristic_noalloc holds no lock): one that fitted
+// this launch could be lowered by another thread just before it.
+cudaError_t allow_smem(const void* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHeurSmem);
+}
+
 template <HeurMode MODE>
 cudaError_t launch_mode(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                         size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta, unsigned* next_job,
                         unsigned* err, cudaStream_t s) {
   const size_t smem = heur_words(MODE, G.n) * 4;
-  const cudaError_t e = cudaFuncSetAttribute((const void*)heuristic_kernel<MODE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem((const void*)heuristic_kernel<MODE>);
   if (e != cudaSuccess) return e;
   heuristic_kernel<MODE><<<blocks, kHeurThreads, smem, s>>>(G, jobs, njobs, scratch, scratch_words_per_block, delta,
                                                             next_job, err, lanes_per_node(G));
@@ -453,8 +460,7 @@ cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs
   if (njobs && heuristic_mode(G.n, smem) != kDistShared && njobs * kHeurCluster <= sms &&
       cluster_words(G.n) * 4 <= smem) {
     const size_t bytes = cluster_words(G.n) * 4;
-    const cudaError_t e = cudaFuncSetAttribute((const void*)heuristic_cluster_kernel,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    const cudaError_t e = allow_smem((const void*)heuristic_cluster_kernel);
     if (e != cudaSuccess) return e;
     heuristic_cluster_kernel<<<njobs * kHeurCluster, kClusterThreads, bytes, s>>>(G, jobs, scratch, delta, err,
                                                                                  lanes_per_node(G));

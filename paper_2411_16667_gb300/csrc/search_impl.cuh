@@ -2392,13 +2392,14 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
 // ---------------------------------------------------------------------------
 // host launchers, explicitly instantiated per objective count
 // ---------------------------------------------------------------------------
-// Dynamic shared memory of a block of nt threads (the warps' rows), with the
-// kernel allowed that much.
+// Dynamic shared memory of a block of nt threads: the warps' rows, or at_least
+// when that is more. The kernel is allowed the most that any launch of it takes
+// (a server's block), as batches and servers launch it from several threads.
 template <int D>
 size_t row_bytes(const void* kernel, unsigned nt, size_t at_least = 0) {
-  const size_t bytes = std::max(at_least, (size_t)nt * detail::Search<D>::RP * 4);
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  return bytes;
+  const size_t rows = (size_t)nt * detail::Search<D>::RP * 4;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(rows, kServeBlockSmem));
+  return std::max(rows, at_least);
 }
 
 template <int D>
