@@ -1202,7 +1202,8 @@ void server_free(opmos_server* sv) {
     *reinterpret_cast<volatile unsigned*>(&sv->hctl[HC_CLOSING]) = 2;  // stop now
     for (unsigned i = 0; i < sv->nslots; ++i) *reinterpret_cast<volatile unsigned*>(&sv->hctl[HC_RELEASE + i]) = 1;
     cudaStreamSynchronize(sv->kstream);
-    --resident_servers;
+    std::lock_guard<std::mutex> lk(residents.mu);
+    --residents.servers;
   }
   if (sv->dmem) cudaFree(sv->dmem);
   if (sv->hmem) cudaFreeHost(sv->hmem);
@@ -1348,12 +1349,12 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       server_free(sv);
       return cuda_fail(e, "server set-up");
     }
-    // Load the heuristic kernels of every graph now, by launches without jobs: a
-    // kernel is loaded at its first launch, which may wait until the device is
-    // idle, and the resident kernel never ends while submit waits.
-    for (uint32_t i = 0; i < ngraphs && e == cudaSuccess; ++i)
-      e = launch_heuristic(graphs[i]->dev, sv->djobs, 0, sv->hscratch, 5 * (size_t)sv->shape.n + 64, 1, graphs[i]->delta,
-                           sv->hkctr, sv->hkctr + 1, sv->hstream, kHeurSmemServed);
+    // Load the heuristic's kernels now, whatever sizes the graphs have: a kernel is
+    // loaded at its first launch, which may wait until the device is idle, and the
+    // resident kernel never ends while submit, or a heuristic of another graph,
+    // waits.
+    e = cudaMemsetAsync(sv->hkctr, 0, 2 * sizeof(unsigned), sv->hstream);
+    if (e == cudaSuccess) e = load_heuristic(sv->hkctr, sv->hstream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(sv->hstream);
     if (e != cudaSuccess) {
       server_free(sv);
@@ -1362,14 +1363,17 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
     const int occ = multi_occupancy(sv->dmax, kServeBlockSmem);
     const unsigned full = (unsigned)di.sms * (unsigned)std::min(occ, 2);
     sv->blocks = full > 2 * kServeHeurBlocks ? full - 2 * kServeHeurBlocks : std::max(1u, full / 2);
-    e = launch_multi(sv->dmax, dslots, ctls, sv->nslots, (MQuery*)dev_of(sv->hq), (unsigned*)dev_of(sv->hctl), dgraphs,
-                     (QResult*)dev_of(sv->hres), (unsigned*)dev_of(sv->hdone), M, sv->blocks, kServeBlockSmem, sv->kstream);
+    {
+      std::lock_guard<std::mutex> lk(residents.mu);
+      e = launch_multi(sv->dmax, dslots, ctls, sv->nslots, (MQuery*)dev_of(sv->hq), (unsigned*)dev_of(sv->hctl), dgraphs,
+                       (QResult*)dev_of(sv->hres), (unsigned*)dev_of(sv->hdone), M, sv->blocks, kServeBlockSmem, sv->kstream);
+      if (e == cudaSuccess) ++residents.servers;
+    }
     if (e != cudaSuccess) {
       server_free(sv);
       return cuda_fail(e, "server kernel launch");
     }
     sv->running = true;
-    ++resident_servers;
     *out = sv;
     return OPMOS_OK;
   });

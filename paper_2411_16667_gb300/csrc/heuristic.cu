@@ -446,18 +446,28 @@ cudaError_t launch_mode(const GraphDev& G, const HJob* jobs, unsigned njobs, uin
 
 }  // namespace
 
-std::atomic<int> resident_servers{0};
+Residents residents;
+
+cudaError_t load_heuristic(unsigned* ctr, cudaStream_t s) {
+  GraphDev G{};
+  G.n = 1;
+  cudaError_t e = launch_mode<kDistShared>(G, nullptr, 0, nullptr, 0, 1, nullptr, ctr, ctr + 1, s);
+  if (e == cudaSuccess) e = launch_mode<kFlagsShared>(G, nullptr, 0, nullptr, 0, 1, nullptr, ctr, ctr + 1, s);
+  if (e == cudaSuccess) e = launch_mode<kFlagsGlobal>(G, nullptr, 0, nullptr, 0, 1, nullptr, ctr, ctr + 1, s);
+  return e;
+}
 
 cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                              size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta,
                              unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem, unsigned sms) {
-  if (resident_servers.load() != 0) {
+  std::lock_guard<std::mutex> lk(residents.mu);
+  if (residents.servers != 0) {
     smem = std::min(smem, kHeurSmemServed);
     sms = 0;
   }
   // a cluster a pair where the distances do not fit one block but fit eight,
   // while every cluster has its SMs at once
-  if (njobs && heuristic_mode(G.n, smem) != kDistShared && njobs * kHeurCluster <= sms &&
+  if (heuristic_mode(G.n, smem) != kDistShared && njobs * kHeurCluster <= sms &&
       cluster_words(G.n) * 4 <= smem) {
     const size_t bytes = cluster_words(G.n) * 4;
     const cudaError_t e = allow_smem((const void*)heuristic_cluster_kernel);

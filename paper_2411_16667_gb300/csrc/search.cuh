@@ -1,6 +1,6 @@
 // Host-visible declarations shared by the search kernels and the C ABI layer.
 #pragma once
-#include <atomic>
+#include <mutex>
 
 #include "opmos_dev.cuh"
 
@@ -98,8 +98,17 @@ constexpr size_t kServeBlockSmem = 72u << 10;
 constexpr size_t kHeurSmemServed = 68u << 10;
 // Resident server kernels of this process. While there is one, the heuristic
 // takes blocks that fit beside it: a cluster, or a block with most of an SM's
-// shared memory, would wait for the server's end.
-extern std::atomic<int> resident_servers;
+// shared memory, would wait for the server's end. A heuristic looks and launches
+// under mu, and a server's kernel is launched and counted under it, so that none
+// starts in between.
+struct Residents {
+  std::mutex mu;
+  int servers = 0;
+};
+extern Residents residents;
+// Loads the heuristic's kernels that run beside a server, by launches without
+// jobs (ctr: two zero words of device memory).
+cudaError_t load_heuristic(unsigned* ctr, cudaStream_t s);
 cudaError_t launch_heuristic(const GraphDev& G, const HJob* jobs, unsigned njobs, uint32_t* scratch,
                              size_t scratch_words_per_block, unsigned blocks, const uint32_t* delta,
                              unsigned* next_job, unsigned* err, cudaStream_t s, size_t smem = kHeurSmem,
