@@ -60,6 +60,11 @@ OPMOS_API int opmos_test_merge(uint32_t d, uint32_t nfront, const uint32_t* fron
 OPMOS_API int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const uint8_t* dead,
                                 uint32_t window, const uint32_t* bins, uint8_t* taken, uint32_t* bstar);
 
+/* A block's counters (opmos_stats): each of the n values is added to one counter
+ * by a warp, `steps` times over with a step's end after each; *sum is what the
+ * query's counter holds afterwards. */
+OPMOS_API int opmos_test_count(uint32_t n, const uint64_t* add, uint32_t steps, uint64_t* sum);
+
 #ifdef __cplusplus
 }
 #endif

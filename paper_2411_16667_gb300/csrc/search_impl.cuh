@@ -128,7 +128,8 @@ struct Shared {
   unsigned win_min, win_max, f1lo, f1hi;
   unsigned rec[32];    // the step's record (RecWord)
   PIdx pd;             // the P index as this step sees it
-  unsigned cnt[kNStat];  // this block's counters since the last flush (see flush_counts)
+  // this block's counters since the last flush, cnt + (high << 16) each (see flush_counts)
+  unsigned cnt[kNStat], high[kNStat];
   unsigned tmax[5];    // this block's longest merge part, merge, extraction item (ns); most
                        // candidates and largest frontier of its split merges
 };
@@ -136,13 +137,19 @@ struct Shared {
 // Adds the block's counters to the query's. Every thread calls it, between
 // block barriers that separate it from the counting. (Counters in shared memory
 // are added to by one lane a work item; 26 of 64 bits in every thread took 52
-// registers.) With `full` set only the ones near their 32 bits are added.
+// registers.) With `full` set only the ones that large are added. A step adds
+// less than 2^31 labels or candidates to a block's counters; of what may be more,
+// times and comparisons, see Search::count_big.
+constexpr unsigned kFlushAt = 1u << 30;  // at a step's end
 __device__ __forceinline__ void flush_counts(QCtl* C, Shared& S, unsigned full = 1u) {
   const unsigned i = threadIdx.x - 64u;
-  if (i < (unsigned)kNStat && S.cnt[i] >= full) {
-    atomicAdd(&C->stats[i], (unsigned long long)S.cnt[i]);
-    S.cnt[i] = 0;
+  if (i < (unsigned)kNStat && (S.cnt[i] | S.high[i]) >= full) {
+    atomicAdd(&C->stats[i], S.cnt[i] + ((unsigned long long)S.high[i] << 16));
+    S.cnt[i] = S.high[i] = 0;
   }
+}
+__device__ __forceinline__ void clear_counts(Shared& S) {
+  if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = S.high[threadIdx.x] = 0;
 }
 
 // Histogram bin of an OPEN key (F0 << 32 | F1): the key's cell is
@@ -210,6 +217,25 @@ struct Search {
       : G(g), A(a), C(c), P(p), O(o), S(s) {}
 
   __device__ __forceinline__ void count(int what, unsigned n) const { atomicAdd(&S.cnt[what], n); }
+  // A counter that a step may carry past 32 bits (times, comparisons), at most
+  // once a work item: 16 bits go to one word, the others to a second, which a
+  // step of less than the barrier's time limit cannot fill; empty_counts comes
+  // before the first is full. (Looking whether an addition wrapped made steps 2%
+  // longer, adding large values to the query's counter instead 1%.)
+  __device__ __forceinline__ void count_big(int what, unsigned long long n) const {
+    atomicAdd(&S.cnt[what], (unsigned)n & 0xFFFFu);
+    atomicAdd(&S.high[what], (unsigned)(n >> 16));
+  }
+  static constexpr unsigned kFlushItems = 1024;
+  static_assert((unsigned long long)(kGridThreads / 32) * kFlushItems * 0xFFFFu + kFlushAt < 1ull << 32 &&
+                    kGridWideThreads <= kGridThreads && kMultiThreads <= kGridThreads, "a step's counts");
+  // By one warp beside others that count, every kFlushItems of its work items.
+  __device__ void empty_counts() const {
+    const unsigned i = lane_id();
+    if (i >= (unsigned)kNStat) return;
+    const unsigned long long n = atomicExch(&S.cnt[i], 0u) + ((unsigned long long)atomicExch(&S.high[i], 0u) << 16);
+    if (n) atomicAdd(&C->stats[i], n);
+  }
   // One lane counts for the warp.
   __device__ __forceinline__ void count_lane0(int what, unsigned n) const {
     if (lane_id() == 0 && n) atomicAdd(&S.cnt[what], n);
@@ -568,7 +594,7 @@ struct Search {
   }
   // Lazy PruneOPEN: F against the goal costs logged since the label's last
   // check (through the P index when that check predates it).
-  __device__ __forceinline__ bool still_open(bool want, const Label& l, unsigned& pcmp) {
+  __device__ __forceinline__ bool still_open(bool want, const Label& l, unsigned long long& pcmp) {
     const unsigned since = warp_min(want ? l.since : kInf);
     bool alive = want;
     if (since < psnap) {
@@ -693,9 +719,9 @@ struct Search {
       want = false;
     else
       keep = valid && !want;
-    unsigned pcmp = 0;
+    unsigned long long pcmp = 0;
     bool take = still_open(want, own, pcmp);
-    count_lane0(S_PCMP, pcmp);
+    if (lane_id() == 0 && pcmp) count_big(S_PCMP, pcmp);
     count_lane0(S_OSCAN, __popc(__ballot_sync(0xffffffffu, valid)));
     count_lane0(S_DEAD, __popc(__ballot_sync(0xffffffffu, gone)));
     count_lane0(S_GOALPRUNED, __popc(__ballot_sync(0xffffffffu, want && !take)));
@@ -764,9 +790,9 @@ struct Search {
     }
     const Label own = load_label(valid, id);
     const bool want = valid && dead >= cyc;
-    unsigned pcmp = 0;
+    unsigned long long pcmp = 0;
     const bool take = still_open(want, own, pcmp);
-    count_lane0(S_PCMP, pcmp);
+    if (lane_id() == 0 && pcmp) count_big(S_PCMP, pcmp);
     count_lane0(S_OSCAN, __popc(__ballot_sync(0xffffffffu, valid)));
     count_lane0(S_DEAD, __popc(__ballot_sync(0xffffffffu, valid && !want)));
     count_lane0(S_GOALPRUNED, __popc(__ballot_sync(0xffffffffu, want && !take)));
@@ -852,7 +878,7 @@ struct Search {
   // d = 16, 17,539 solutions 101 ms instead of 80; 6x8x24 route, d = 12, 16,268
   // solutions 65 instead of 52, 1,381 solutions 3.7 instead of 3.6.)
   __device__ void p_filter(bool& alive, const uint32_t (&F)[D], unsigned t0, unsigned t1, unsigned pcount,
-                           unsigned tlo, unsigned thi, unsigned pbuf, unsigned& pcmp) {
+                           unsigned tlo, unsigned thi, unsigned pbuf, unsigned long long& pcmp) {
     const unsigned lane = lane_id();
     unsigned cnt = 0;
     unsigned am = __ballot_sync(0xffffffffu, alive);
@@ -1057,7 +1083,7 @@ struct Search {
   // once a round: 2 D compares a pair and a vote for two candidates.
   template <bool WRITE>
   __device__ unsigned scan_frontier(uint32_t v, Batch& b, unsigned lo, unsigned hi, uint64_t fb, unsigned cap,
-                                    Round& t, bool& pruned_any, unsigned& fcmp) {
+                                    Round& t, bool& pruned_any, unsigned long long& fcmp) {
     constexpr int U = kU;
     const unsigned lane = lane_id();
     unsigned am = __ballot_sync(0xffffffffu, b.alive), out = lo;
@@ -1153,7 +1179,7 @@ struct Search {
   // and the log behind it, up to t1. hv: the node's heuristic, 0 at the goal
   // node n.
   __device__ __forceinline__ void batch_ptest(const uint32_t (&hv)[D], Batch& b, unsigned t1, unsigned x, unsigned n,
-                                              unsigned& pcmp) {
+                                              unsigned long long& pcmp) {
     if (!__any_sync(0xffffffffu, b.alive)) return;
     const PIdx& pd = S.pd;
     uint32_t F[D];
@@ -1400,7 +1426,7 @@ struct Search {
     }
     Groups q = open_groups(cs, v, nc);
     const unsigned ng = ngroups(nc);
-    unsigned fcmp = 0, pcmp = 0;
+    unsigned long long fcmp = 0, pcmp = 0;
     bool pruned = false;
     for (unsigned g = 0; g < ng; ++g) {
       const int mine = g ? group(cs, q, g) : (lane < q.in_slots ? slot0 : kNil);
@@ -1418,8 +1444,8 @@ struct Search {
     clear_groups(cs, v, nc);
     if (lane == 0) {
       if (fc != fc0) A.fcount[v] = fc;
-      count(S_FCMP, fcmp);
-      count(S_PCMP, pcmp);
+      count_big(S_FCMP, fcmp);
+      count_big(S_PCMP, pcmp);
     }
   }
 
@@ -1492,7 +1518,7 @@ struct Search {
     const unsigned a = (r % ks) / sub, bb = r / ks;
     const unsigned width = 32u / sub, l0 = (r % ks) % sub * width;  // this part's lanes of a group
     const unsigned lo = (unsigned)((uint64_t)F * bb / kb), hi = goal ? 0u : (unsigned)((uint64_t)F * (bb + 1) / kb);
-    unsigned fcmp = 0, pcmp = 0;
+    unsigned long long fcmp = 0, pcmp = 0;
     bool pruned = false;
     {
       Groups q = open_groups(cs, v, nc);
@@ -1555,8 +1581,10 @@ struct Search {
         if (atomicOr(&cs.hflag[v], kSplitDone) & kSplitSeen) cs.hflag[v] = 0;
       }
     }
-    count_lane0(S_FCMP, fcmp);
-    count_lane0(S_PCMP, pcmp);
+    if (lane == 0) {
+      count_big(S_FCMP, fcmp);
+      count_big(S_PCMP, pcmp);
+    }
   }
 
   // Compaction of a frontier after a split merge, by one warp: the entries
@@ -1762,11 +1790,11 @@ struct Search {
     if (T.leader_block()) {
       if (threadIdx.x == 64) {
         // the longest tasks of step i-1 (its slot is K2)
-        count(S_MAXH, K2.tmax[0]);
-        count(S_MAXL, K2.tmax[1]);
-        count(S_MAXX, K2.tmax[2]);
-        count(S_MAXNC, K2.tmax[3]);
-        count(S_MAXF, K2.tmax[4]);
+        count_big(S_MAXH, K2.tmax[0]);
+        count_big(S_MAXL, K2.tmax[1]);
+        count_big(S_MAXX, K2.tmax[2]);
+        count_big(S_MAXNC, K2.tmax[3]);
+        count_big(S_MAXF, K2.tmax[4]);
         clear_cycle(K2);
         // values step i+1 starts from; the writers of this step raise them
         atomicMax(&K1.plen.v, psnap);
@@ -1784,7 +1812,7 @@ struct Search {
     __syncthreads();
     if (T.leader() && tlap) {
       const unsigned long long t = globaltimer();
-      count(S_TSEL, (unsigned)(t - *tlap));
+      count_big(S_TSEL, t - *tlap);
       *tlap = t;
     }
     // work items, one warp each: parts of split merges (the longest), index-rank
@@ -1796,6 +1824,7 @@ struct Search {
     const unsigned nchunks = (nopen + per - 1) / per;
     const unsigned nitems = np + nrank + nt + nchunks;
     const unsigned lane = lane_id();
+    unsigned done = 0;  // items of this warp
     // The first item of a warp goes by its number, neighbouring items to
     // different blocks; the rest is claimed (claims by every warp at once queue
     // on one counter: 2 us).
@@ -1816,7 +1845,7 @@ struct Search {
           if (lane == 0) {
             const unsigned long long dt = globaltimer() - t0;
             atomicMax(&S.tmax[0], (unsigned)min(dt, 0xFFFFFFFFull));
-            count(S_SUMH, (unsigned)dt);
+            count_big(S_SUMH, dt);
           }
         }
       } else if (t < np + nrank) {
@@ -1827,7 +1856,7 @@ struct Search {
         if (lane == 0) {
           const unsigned long long dt = globaltimer() - t0;
           atomicMax(&S.tmax[1], (unsigned)min(dt, 0xFFFFFFFFull));
-          count(S_SUML, (unsigned)dt);
+          count_big(S_SUML, dt);
         }
       } else {
         const unsigned c = t - np - nrank - nt;
@@ -1838,17 +1867,18 @@ struct Search {
         if (lane == 0) {
           const unsigned long long dt = globaltimer() - t0;
           atomicMax(&S.tmax[2], (unsigned)min(dt, 0xFFFFFFFFull));
-          count(S_SUMX, (unsigned)dt);
+          count_big(S_SUMX, dt);
         }
       }
       if (nitems <= nwarps) break;
+      if (++done % kFlushItems == 0) empty_counts();
       if (lane == 0) t = nwarps + atomicAdd(&K0.work_next.v, 1u);
       t = __shfl_sync(0xffffffffu, t, 0);
     }
     index_strided_work(T);
     __syncthreads();
     if (threadIdx.x < 5 && S.tmax[threadIdx.x]) atomicMax(&K0.tmax[threadIdx.x], S.tmax[threadIdx.x]);
-    flush_counts(C, S, 1u << 30);
+    flush_counts(C, S, kFlushAt);
     if (threadIdx.x == 32) {
       if (S.min_key != ~0ull) atomicMin(&K1.min_key.v, S.min_key);
       if (S.win_min != kInf) {
@@ -1874,7 +1904,7 @@ struct Search {
     }
     if (T.leader() && tlap) {
       const unsigned long long t = globaltimer();
-      count(S_TWORK, (unsigned)(t - *tlap));
+      count_big(S_TWORK, t - *tlap);
       *tlap = t;
     }
     return true;
@@ -2046,7 +2076,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
   __shared__ Shared S;
   const GridTeam T;
   Search<D, kMany> X(G, A, C, P, O, S);
-  if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
+  clear_counts(S);
   for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
   X.init_zero(T);
   bool ok = T.sync(C);
@@ -2060,7 +2090,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
     ok = T.sync(C);
     if (T.leader()) {
       const unsigned long long t = globaltimer();
-      X.count(S_TSYNC, (unsigned)(t - tph));
+      X.count_big(S_TSYNC, t - tph);
       tph = t;
     }
     ++step;
@@ -2068,7 +2098,7 @@ __device__ void run_grid(const GraphDev& G, const QArena& A, QCtl* C, const QPar
   if (ok) {
     if (T.leader()) C->res_count = 0;
     ok = T.sync(C) && X.output(T);
-    if (T.leader()) X.count(S_TOUT, (unsigned)(globaltimer() - tph));
+    if (T.leader()) X.count_big(S_TOUT, globaltimer() - tph);
   }
   if (T.leader()) {
     X.count(S_STEPS, step);
@@ -2375,7 +2405,7 @@ __global__ void __launch_bounds__(kMultiThreads, 2)
   __shared__ Shared S;
   __shared__ MSlot s_slot;
   __shared__ unsigned s_pref[kMaxSlots + 1];
-  if (threadIdx.x < kNStat) S.cnt[threadIdx.x] = 0;
+  clear_counts(S);
   for (unsigned x = threadIdx.x; x < kNB; x += blockDim.x) S.hist[x] = 0;
   unsigned target = 0;
   for (;;) {

@@ -254,9 +254,49 @@ __global__ void __launch_bounds__(kGridThreads, 1) window_hook_kernel(GraphDev G
   for (unsigned c = threadIdx.x >> 5; c < nchunks; c += blockDim.x >> 5) X.extract_chunk(c, n, kChunk, bp, C->cyc[2]);
 }
 
+// A block counts as in a step: each value by one lane of a warp, warp after warp,
+// `steps` times over, with a step's end after each.
+__global__ void __launch_bounds__(kMultiThreads, 1) count_hook_kernel(GraphDev G, QArena A, QCtl* C, QParams P,
+                                                                      OutPool O, const unsigned long long* add,
+                                                                      unsigned n, unsigned steps) {
+  __shared__ Shared S;
+  clear_counts(S);
+  __syncthreads();
+  Search<2> X(G, A, C, P, O, S);
+  for (unsigned s = 0; s < steps; ++s) {
+    unsigned done = 0;
+    for (unsigned i = threadIdx.x >> 5; i < n; i += blockDim.x >> 5) {
+      if (lane_id() == 0) X.count_big(S_FCMP, add[i]);
+      __syncwarp();
+      if (++done % X.kFlushItems == 0) X.empty_counts();
+    }
+    __syncthreads();
+    flush_counts(C, S, kFlushAt);
+    __syncthreads();
+  }
+  flush_counts(C, S);
+}
+
 }  // namespace
 
 extern "C" {
+
+int opmos_test_count(uint32_t n, const uint64_t* add, uint32_t steps, uint64_t* sum) {
+  if (!add || !sum || n == 0) return hook_fail(OPMOS_ERR_INVALID_ARG, "NULL argument or nothing to add");
+  DevBuf ctl, vals;
+  cudaError_t e = cudaMalloc(&ctl.p, sizeof(QCtl));
+  if (e == cudaSuccess) e = cudaMalloc(&vals.p, n * sizeof(uint64_t));
+  if (e == cudaSuccess) e = cudaMemset(ctl.p, 0, sizeof(QCtl));
+  if (e == cudaSuccess) e = cudaMemcpy(vals.p, add, n * sizeof(uint64_t), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook: %s", cudaGetErrorString(e));
+  QCtl* C = static_cast<QCtl*>(ctl.p);
+  count_hook_kernel<<<1, kMultiThreads>>>(GraphDev{}, QArena{}, C, QParams{}, OutPool{},
+                                          static_cast<const unsigned long long*>(vals.p), n, steps);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpy(sum, &C->stats[S_FCMP], sizeof(uint64_t), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook kernel: %s", cudaGetErrorString(e));
+  return OPMOS_OK;
+}
 
 int opmos_test_merge(uint32_t d, uint32_t nfront, const uint32_t* front, uint32_t ncand, const uint32_t* cand,
                      const uint32_t* cand_arc, uint32_t block, uint32_t slots, uint32_t lists,

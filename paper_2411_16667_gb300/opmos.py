@@ -22,7 +22,7 @@ FLAG_GRAPH = 2
 FLAG_FIFO = 4
 MAX_D = 16
 
-TEST_EXPORTS = ("opmos_test_merge", "opmos_test_window")  # include/opmos_test.h
+TEST_EXPORTS = ("opmos_test_merge", "opmos_test_window", "opmos_test_count")  # include/opmos_test.h
 EXPORTS = ("opmos_default_options", "opmos_device_count", "opmos_graph_create", "opmos_graph_destroy",
            "opmos_heuristic", "opmos_heuristic_copy", "opmos_heuristic_destroy", "opmos_solve",
            "opmos_solve_batch", "opmos_result_count", "opmos_result_d", "opmos_result_costs",
@@ -104,6 +104,7 @@ def lib(path: str | None = None):
         L.opmos_heuristic_noalloc.argtypes = [vp, u32, u32, vp, vp]
         L.opmos_test_merge.argtypes = [u32, u32, vp, u32, vp, vp, u32, u32, u32, vp, vp, ctypes.POINTER(u32)]
         L.opmos_test_window.argtypes = [u32, vp, vp, vp, u32, vp, vp, ctypes.POINTER(u32)]
+        L.opmos_test_count.argtypes = [u32, vp, u32, ctypes.POINTER(ctypes.c_uint64)]
         _lib = L
     return _lib
 
@@ -359,3 +360,12 @@ def opmos_test_window(f0, f1, dead, window: int, bins):
     _check(lib().opmos_test_window(n, _ptr(f0), _ptr(f1), _ptr(dead), window, _ptr(bins), _ptr(taken),
                                    ctypes.byref(bstar)), "opmos_test_window")
     return taken[:n].astype(bool), int(bstar.value)
+
+
+def opmos_test_count(add, steps: int) -> int:
+    """What a query's counter holds after a block has added the values ``steps``
+    times over."""
+    add = np.ascontiguousarray(add, np.uint64)
+    out = ctypes.c_uint64()
+    _check(lib().opmos_test_count(len(add), _ptr(add), steps, ctypes.byref(out)), "opmos_test_count")
+    return int(out.value)
