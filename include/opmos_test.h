@@ -24,10 +24,9 @@ extern "C" {
  * dropped, frontier labels a candidate strictly dominates are pruned -- and
  * the in-batch resolution of Sec. 5's Dup&Dom), exactly as a search step runs
  * it on the device: one warp (block = 0), or a merge split into `block` =
- * 1..16 parts of one warp (shares of the candidates times ranges of what they
- * are compared with; run one after the other, the last one finishes the
- * node), with candidates taken from the node's slots and then its overflow
- * lists. The frontier must be mutually
+ * 1..128 parts of one warp (shares of the candidates times ranges of what they
+ * are compared with; side by side, the last one to end finishes the node), with
+ * candidates taken from the node's slots and then its overflow lists. The frontier must be mutually
  * non-dominated and cost-unique, as in a search. No solution set is
  * involved.
  *   d: 1, 2, 3, 4, 5, 8, 12 or 16 (other values: OPMOS_ERR_INVALID_ARG).

@@ -39,26 +39,27 @@ T* take(char*& p, size_t count) {
   return reinterpret_cast<T*>(a);
 }
 
-// One node (node 0) merged as in step 0 by one warp: whole, or part by part.
+// One node (node 0) merged as in step 0: by one warp, or its parts by a warp each,
+// side by side.
+constexpr unsigned kHookThreads = 256;
 template <int D>
-__global__ void __launch_bounds__(32, 1) merge_hook_kernel(GraphDev G, QArena A, QCtl* C, QParams P,
-                                                                     OutPool O, unsigned lbase, unsigned block) {
+__global__ void __launch_bounds__(kHookThreads, 1) merge_hook_kernel(GraphDev G, QArena A, QCtl* C, QParams P,
+                                                                     OutPool O, unsigned lbase, unsigned parts) {
   __shared__ Shared S;
   Search<D> X(G, A, C, P, O, S);
   X.cyc = 0;
   X.psnap = 0;
   X.lbase = lbase;
-  X.bpn = BinParams{0u, 0u, 0u, 1u, 0u};
-  if (threadIdx.x == 0) {
-    S.pd = PIdx{};
-    for (int i = 0; i < kNB; ++i) S.hist[i] = 0;
-  }
+  X.bpn = BinParams{0, 0, 0, 1, 0};
+  if (threadIdx.x == 0) S.pd = PIdx{};
+  for (unsigned i = threadIdx.x; i < kNB; i += blockDim.x) S.hist[i] = 0;
+  clear_counts(S);
   __syncthreads();
-  if (block) {  // a merge split into `block` parts, one after the other (the last one finishes)
-    for (unsigned r = 0; r < block; ++r) X.merge_part(0u, r, block, C->cyc[1]);
-  } else {
+  const unsigned w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w < parts)
+    X.merge_part(0u, w, parts, C->cyc[1]);
+  else if (w == 0)
     X.merge_node(0u, C->cyc[1]);
-  }
 }
 
 template <int D>
@@ -201,7 +202,8 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   P.ps_grow = 6;
   P.part_work = part_work(D, 0);
   OutPool O{nullptr, 0, nullptr};
-  merge_hook_kernel<D><<<1, 32, 32 * Search<D>::RP * 4>>>(G, A, C, P, O, nfront, block);
+  const unsigned blocks = std::max(1u, (block * 32u + kHookThreads - 1) / kHookThreads);
+  merge_hook_kernel<D><<<blocks, kHookThreads, kHookThreads * Search<D>::RP * 4>>>(G, A, C, P, O, nfront, block);
   e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return hook_fail(OPMOS_ERR_CUDA, "test hook kernel: %s", cudaGetErrorString(e));
@@ -305,7 +307,7 @@ int opmos_test_merge(uint32_t d, uint32_t nfront, const uint32_t* front, uint32_
     if (!out_cost || !out_origin || !out_count || (nfront && !front) || (ncand && (!cand || !cand_arc)))
       return hook_fail(OPMOS_ERR_INVALID_ARG, "NULL argument");
     if (slots == 0 || slots > 4096) return hook_fail(OPMOS_ERR_INVALID_ARG, "slots must be in [1, 4096]");
-    if (block > 16u) return hook_fail(OPMOS_ERR_INVALID_ARG, "block must be 0..16");
+    if (block > kPartsMax) return hook_fail(OPMOS_ERR_INVALID_ARG, "block must be 0..%u", kPartsMax);
     if (nfront > (1u << 20) || ncand > (1u << 20)) return hook_fail(OPMOS_ERR_INVALID_ARG, "inputs too large");
     unsigned lsub = 0;
     while ((1u << lsub) < lists && lsub < 5) ++lsub;

@@ -330,9 +330,8 @@ class opmos_server:
 def opmos_test_merge(front, cand, cand_arc, block, slots: int = 32, lists: int = 1):
     """Device merge of one node (frontier rows ``front``, candidate rows
     ``cand`` with arc ids ``cand_arc``; the first ``slots`` in the node's
-    slots, the rest in ``lists`` overflow lists) by one warp (block 0), one
-    block (1) or a block merge split into ``block`` = 2..16 parts;
-    returns (costs, origins) of the frontier after the merge (origin <
+    slots, the rest in ``lists`` overflow lists) by one warp (block 0) or in
+    ``block`` = 1..128 parts of a warp each; returns (costs, origins) of the frontier after the merge (origin <
     len(front): that entry; else len(front) + candidate index)."""
     front = np.ascontiguousarray(front, np.uint32)
     cand = np.ascontiguousarray(cand, np.uint32)
