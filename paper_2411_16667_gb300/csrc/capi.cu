@@ -581,7 +581,7 @@ int solve_one(const opmos_graph* g, const opmos_heur* heur, uint32_t start, uint
   P.flags = o.flags;
   P.qd = D;
   P.ps_grow = kGridIndexGrow;
-  P.part_work = part_work(D, o.window);
+  P.part_work = part_work(D);
   P.time_limit_ns = time_limit_ns();
 
   // large windows take the wide grid (two 256-thread blocks per SM)
@@ -589,6 +589,7 @@ int solve_one(const opmos_graph* g, const opmos_heur* heur, uint32_t start, uint
   int occ = search_occupancy(D, wide);
   if (occ <= 0) return fail(OPMOS_ERR_CUDA, "search kernel cannot be resident");
   const unsigned blocks = (unsigned)di.sms * (unsigned)std::min(occ, wide ? (int)kGridWideBlocksPerSM : 1);
+  P.parts_most = parts_most(A.xcap, blocks * (wide ? kGridWideThreads : kGridThreads) / 32);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -654,7 +655,8 @@ int run_multi(const opmos_graph* g, uint32_t D, const opmos_options& o, const st
   P.flags = o.flags;
   P.qd = D;
   P.ps_grow = kMultiIndexGrow;
-  P.part_work = part_work(D, 0);
+  P.part_work = part_work(D);
+  P.parts_most = parts_most(pl.xcap, blocks * kMultiThreads / 32);
   P.time_limit_ns = time_limit_ns();
   std::vector<MSlot> hslots(slots);
   for (unsigned i = 0; i < slots; ++i) {
@@ -1309,6 +1311,9 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
     sv->hkctr = carve<unsigned>(dp, 16);
     sv->hscratch = carve<uint32_t>(dp, kServeHeurBlocks * spb);
     sv->hring = carve<uint32_t>(dp, sv->qcap * hstride);
+    const int occ = multi_occupancy(sv->dmax, kServeBlockSmem);
+    const unsigned full = (unsigned)di.sms * (unsigned)std::min(occ, 2);
+    sv->blocks = full > 2 * kServeHeurBlocks ? full - 2 * kServeHeurBlocks : std::max(1u, full / 2);
     std::vector<MSlot> hslots(sv->nslots);
     for (unsigned i = 0; i < sv->nslots; ++i) {
       char* base = carve<char>(dp, per_slot);
@@ -1328,7 +1333,8 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       sl.P.flags = o.flags;
       sl.P.qd = sv->dmax;
       sl.P.ps_grow = kMultiIndexGrow;
-      sl.P.part_work = part_work(sv->dmax, 0);
+      sl.P.part_work = part_work(sv->dmax);
+      sl.P.parts_most = parts_most(pl.xcap, sv->blocks * kMultiThreads / 32);
       sl.P.time_limit_ns = time_limit_ns();
       sl.state = SL_FREE;
     }
@@ -1360,9 +1366,6 @@ int opmos_server_create(const opmos_graph* const* graphs, uint32_t ngraphs, cons
       server_free(sv);
       return cuda_fail(e, "server heuristic kernels");
     }
-    const int occ = multi_occupancy(sv->dmax, kServeBlockSmem);
-    const unsigned full = (unsigned)di.sms * (unsigned)std::min(occ, 2);
-    sv->blocks = full > 2 * kServeHeurBlocks ? full - 2 * kServeHeurBlocks : std::max(1u, full / 2);
     {
       std::lock_guard<std::mutex> lk(residents.mu);
       e = launch_multi(sv->dmax, dslots, ctls, sv->nslots, (MQuery*)dev_of(sv->hq), (unsigned*)dev_of(sv->hctl), dgraphs,

@@ -40,25 +40,31 @@ constexpr unsigned kPSMax = 32768;    // largest P indexed by the sorted snapsho
 constexpr unsigned kSmallWindow = 16384;  // larger windows take the wide grid
 // A node's merge is split into parts, one warp each, of about part_work(d)
 // comparisons or fewer, kPartsMax at most: a warp alone issues an instruction
-// every 4-5 cycles, so this many take it about 5 us, a step's other work.
+// every 4-5 cycles, so this many take it 5 to 10 us, about a short step's other
+// work. (The longest part of a step takes longer where a node needs more than
+// kPartsMax, and the last part of a node also inserts what survives: 40-90 us a
+// step on the 256x256 grid, W = 262,144.)
 // Measured (kPartWork = 4,096 / 8,192 / 12,288 / 24,576): 160x160 d=3 27.1 / 27.7
 // / 27.2 / 27.2 ms; 96x96 d=5 first in first out 7.2 / 7.3 / 7.5 / 8.5; route
 // d=12 7.6 / 7.5 / 7.6 / 8.1; 128 queries d=5 26.0 / 24.4 / 24.6 / 24.5; 128x128
-// d=3 at W = 65,536 - / 7.0 (6,144) / 7.3 / 7.5. From kLargeWindow on every warp
-// has several parts a step anyway and what a part costs by itself counts: twice
-// the work, 256x256 grid d=3 at W = 262,144 89 -> 87 ms (344 -> 312 ms on a
-// second seed); four times, 93 (303).
+// d=3 at W = 65,536 - / 7.0 (6,144) / 7.3 / 7.5.
+// Once every warp of the grid has kPartsPerWarp parts a step, what a part costs by
+// itself counts, and parts grow (see Search::next_scale).
 constexpr unsigned kPartWork = 12288;
 constexpr unsigned kLargeWindow = 131072;
 constexpr unsigned kPartsMax = 128;
+constexpr unsigned kPartsPerWarp = 4;
 // Least places of the list of a step's parts: eight warps' worth a warp of the
 // grid for a single query, a block's worth of a batch's two an SM in a batch.
 constexpr unsigned kPartPlacesGrid = 16384;
 constexpr unsigned kPartPlacesBatch = 2048;
-constexpr unsigned kPartShares = 8;  // most shares of one group of 32 candidates
-inline unsigned part_work(unsigned d, unsigned window) {
-  return (window >= kLargeWindow ? 2 : 1) * kPartWork / (1u + d / 4u);
+// Parts a step should list at most, with a list of xcap places on a grid of so many
+// warps.
+inline unsigned parts_most(unsigned xcap, unsigned warps) {
+  return xcap / 2 < kPartsPerWarp * warps ? xcap / 2 : kPartsPerWarp * warps;
 }
+constexpr unsigned kPartShares = 8;  // most shares of one group of 32 candidates
+inline unsigned part_work(unsigned d) { return kPartWork / (1u + d / 4u); }
 // Champions a node has (see Search::champion): a single query with a large
 // window takes several, as merges are most of its steps and its nodes have
 // hundreds of candidates; elsewhere more than one costs the expansion what it
@@ -288,6 +294,7 @@ struct QParams {
   uint32_t qd;            // objectives the query uses (<= the kernel's D; the rest read as 0)
   uint32_t ps_grow;       // the P index is rebuilt once the log outgrows it by 32 + count >> ps_grow
   uint32_t part_work;     // candidates x frontier entries of one part of a split merge
+  uint32_t parts_most;    // parts a step should list at most (see Search::next_scale)
   unsigned long long time_limit_ns;
 };
 

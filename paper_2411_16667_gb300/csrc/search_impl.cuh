@@ -538,14 +538,21 @@ struct Search {
   }
   // The scale of the parts listed in this step, from the places asked for in the
   // last one (asked) at scale s: doubled until half the list would have held
-  // them, halved when a sixteenth would. The list is filled first come first
-  // served, and a merge that finds it full is left to one warp: with many
-  // objectives and a large front every node asks for all its parts (d = 12
-  // route of 1,153 nodes, 16,268 solutions, W = 4,096: 100,000 places of 9,232 a
-  // step, one-warp merges of 3.7 ms each step, 310 ms instead of 46).
+  // them and the grid's warps had had kPartsPerWarp each, halved when an eighth
+  // of that would do.
+  // The list is filled first come first served, and a merge that finds it full is
+  // left to one warp: with many objectives and a large front every node asks for
+  // all its parts (d = 12 route of 1,153 nodes, 16,268 solutions, W = 4,096:
+  // 100,000 places of 9,232 a step, one-warp merges of 3.7 ms each step, 310 ms
+  // instead of 46).
+  // And once the warps have their parts, what a part costs by itself counts:
+  // 256x256 grid d=3 at W = 131,072 133 -> 129 ms, second seed 228 -> 208. (Parts of
+  // twice the work for every window from 131,072 on, whatever there was to do, made
+  // that 134 and 212 ms, and steps of fewer parts longer: 96x96 d=5 10.0 ms instead
+  // of 8.6, 128x128 d=3 11.0 instead of 9.8.)
   __device__ __forceinline__ unsigned next_scale(unsigned asked, unsigned s) const {
-    if (asked < A.xcap / 16) return s ? s - 1u : 0u;
-    for (; asked > A.xcap / 2 && s < kMaxScale; asked >>= 1) ++s;
+    if (asked < P.parts_most / 8) return s ? s - 1u : 0u;
+    for (; asked > P.parts_most && s < kMaxScale; asked >>= 1) ++s;
     return s;
   }
 

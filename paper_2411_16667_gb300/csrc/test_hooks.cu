@@ -200,7 +200,8 @@ int merge_hook(uint32_t nfront, const uint32_t* front, uint32_t ncand, const uin
   P.label_budget = label_cap;
   P.qd = D;
   P.ps_grow = 6;
-  P.part_work = part_work(D, 0);
+  P.part_work = part_work(D);
+  P.parts_most = kPartPlacesGrid;
   OutPool O{nullptr, 0, nullptr};
   const unsigned blocks = std::max(1u, (block * 32u + kHookThreads - 1) / kHookThreads);
   merge_hook_kernel<D><<<blocks, kHookThreads, kHookThreads * Search<D>::RP * 4>>>(G, A, C, P, O, nfront, block);
@@ -442,7 +443,8 @@ int opmos_test_window(uint32_t n, const uint32_t* f0, const uint32_t* f1, const 
     P.label_budget = cap;
     P.qd = D;
     P.ps_grow = 6;
-    P.part_work = part_work(D, 0);
+    P.part_work = part_work(D);
+    P.parts_most = kPartPlacesGrid;
     const BinParams bp{bins[0], bins[1], bins[2], bins[3], bins[4]};
     OutPool O{nullptr, 0, nullptr};
     window_hist_kernel<<<64, 256>>>(A, n, bp, A.hist + 1 * kNB);
