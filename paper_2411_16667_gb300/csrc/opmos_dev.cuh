@@ -51,11 +51,10 @@ constexpr unsigned kSmallWindow = 16384;  // larger windows take the wide grid
 // Once every warp of the grid has kPartsPerWarp parts a step, what a part costs by
 // itself counts, and parts grow (see Search::next_scale).
 constexpr unsigned kPartWork = 12288;
-constexpr unsigned kLargeWindow = 131072;
 constexpr unsigned kPartsMax = 128;
 constexpr unsigned kPartsPerWarp = 4;
-// Least places of the list of a step's parts: eight warps' worth a warp of the
-// grid for a single query, a block's worth of a batch's two an SM in a batch.
+// Least places of the list of a step's parts: nine for every warp of the grid for a
+// single query, about one in a batch.
 constexpr unsigned kPartPlacesGrid = 16384;
 constexpr unsigned kPartPlacesBatch = 2048;
 // Parts a step should list at most, with a list of xcap places on a grid of so many
@@ -66,12 +65,17 @@ inline unsigned parts_most(unsigned xcap, unsigned warps) {
 constexpr unsigned kPartShares = 8;  // most shares of one group of 32 candidates
 inline unsigned part_work(unsigned d) { return kPartWork / (1u + d / 4u); }
 // Champions a node has (see Search::champion): a single query with a large
-// window takes several, as merges are most of its steps and its nodes have
-// hundreds of candidates; elsewhere more than one costs the expansion what it
-// saves the merges (1 / 2 / 4 / 7 champions: 256x256 d=3 at W = 262,144 99 / 100 /
-// 89 / 92 ms, on a second seed 372 / 365 / 344 / 341; 128x128 d=3 at W = 65,536
-// 7.0 / 7.1 / 7.3 / 7.8; 97x89 d=3 4.46 / 4.50 / 4.60 / -).
+// window has room for several. They pay where nodes have hundreds of candidates a
+// step, and there the further ones are kept up to date: by merges of kChampCands
+// candidates or more. (1 champion / 4 at every merge / 4 at such merges, W =
+// 131,072: 256x256 d=3 139 / 129 / 129 ms, second seed 226 / 208 / 207, 200x200 60
+// / 53.5 / 53.4; 128x128 d=3 6.2 / 6.4 / 6.2, 64x64 d=3 2.05 / 2.23 / 2.13, 97x97
+// d=1 1.52 / 1.64 / 1.52; from 16 or 64 candidates on within 1% of from 32. Before
+// large merges were split as they are now: 128x128 d=3 at W = 65,536, 1 / 2 / 4 / 7
+// champions 7.0 / 7.1 / 7.3 / 7.8 ms; 97x89 d=3 4.46 / 4.50 / 4.60 / -.)
+constexpr unsigned kLargeWindow = 131072;
 constexpr unsigned kChamps = 4;
+constexpr unsigned kChampCands = 32;
 constexpr unsigned kPartPruned = 1u << 16;  // added to a node's part counter by a part that pruned
 constexpr unsigned kSplitParts = 0xFFFFu;     // hflag: parts the node's merge is split into (0: none)
 constexpr unsigned kSplitDone = 1u << 30;     // ... its last part has finished

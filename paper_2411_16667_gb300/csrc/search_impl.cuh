@@ -1255,7 +1255,7 @@ struct Search {
   // the frontier entries it dominates (as in Algorithm 1, where Prune precedes
   // the P test).
   __device__ unsigned insert_batch(uint32_t v, const uint32_t (&hv)[D], const Batch& b, unsigned out, uint64_t& fb,
-                                   unsigned& cap, CycleCtl& K1) {
+                                   unsigned& cap, CycleCtl& K1, unsigned nc) {
     const unsigned lane = lane_id();
     const bool is_goal = v == G.n, fifo = (P.flags & OPMOS_FLAG_FIFO) != 0;
     const unsigned smask = __ballot_sync(0xffffffffu, b.alive);
@@ -1270,7 +1270,7 @@ struct Search {
     }
     if (!is_goal) {
       update_champion<0>(v, b);
-      if (kMany && A.nchamps > 1u) {
+      if (kMany && A.nchamps > 1u && nc >= kChampCands) {
         static_assert(kChamps == 4, "one call each");
         update_champion<1>(v, b);
         update_champion<2>(v, b);
@@ -1446,7 +1446,7 @@ struct Search {
         fc = scan_frontier<true>(v, b, 0u, fc, fb, cap, t, pruned, fcmp);
         batch_ptest(hv, b, psnap, 0u, 1u, pcmp);
       }
-      fc = insert_batch(v, hv, b, fc, fb, cap, K1);
+      fc = insert_batch(v, hv, b, fc, fb, cap, K1, nc);
     }
     clear_groups(cs, v, nc);
     if (lane == 0) {
@@ -1569,7 +1569,7 @@ struct Search {
         for (int x = 0; x < 4; ++x) {
           const unsigned bal = __ballot_sync(0xffffffffu, gone[x] == 0u), cnt = __popc(bal);
           if (np + cnt > 32u) {
-            out = insert_batch(v, hv, load_batch(cs, pend), out, fb, cap, K1);
+            out = insert_batch(v, hv, load_batch(cs, pend), out, fb, cap, K1, nc);
             pend = kNil;
             np = 0;
           }
@@ -1580,7 +1580,7 @@ struct Search {
           np += cnt;
         }
       }
-      if (np) out = insert_batch(v, hv, load_batch(cs, pend), out, fb, cap, K1);
+      if (np) out = insert_batch(v, hv, load_batch(cs, pend), out, fb, cap, K1, nc);
       clear_groups(cs, v, nc);
       if (lane == 0) {
         cs.hcnt[v] = 0;
