@@ -138,8 +138,9 @@ typedef struct opmos_stats {
   uint64_t open_scanned;   /* OPEN entries read by the extraction scans, summed over steps
                               (an entry read by two passes of one step counts twice) */
   uint64_t open_rewritten; /* OPEN entries copied forward to the next step's OPEN array */
-  uint64_t list_candidates; /* candidates beyond the slots a node has per step (56 in a
-                               batch, 128 for a single query), merged from the node's lists */
+  uint64_t list_candidates; /* candidates beyond the slots a node has per step (128 for a
+                               single query, 45 to 60 in a batch, fewer with more objectives),
+                               merged from the node's lists */
   uint64_t longest_task_ns[3]; /* summed over steps: the step's longest part of a split merge,
                                   longest merge of a node by one warp, and longest extraction
                                   work item */
@@ -193,9 +194,11 @@ OPMOS_API void opmos_heuristic_destroy(opmos_heur* h);
  *     reads the kernel's status word back) and returns when the result is
  *     complete.
  *   Speed: the fixed array holds the worklists of 2 thread blocks, so the
- *     d_used single-objective searches run at most 2 at a time (opmos_heuristic
- *     runs all of them at once); for d_used > 2 the call takes up to
- *     ceil(d_used / 2) times as long. Errors: INVALID_ARG, CAPACITY, TIMEOUT, CUDA. */
+ *     d_used single-objective searches run at most 2 at a time, one block each
+ *     (opmos_heuristic runs all of them at once, with a cluster of 8 blocks each
+ *     on graphs of more than 44,332 nodes): the call takes up to
+ *     ceil(d_used / 2) times as long, and 1.3 to 1.6 times that on such graphs.
+ *     Errors: INVALID_ARG, CAPACITY, TIMEOUT, CUDA. */
 OPMOS_API int opmos_heuristic_noalloc(const opmos_graph* g, uint32_t goal, uint32_t d_used,
                                       uint32_t* h_out_device, void* stream);
 

@@ -252,13 +252,12 @@ struct Search {
   __device__ __forceinline__ uint64_t key_of(const uint32_t (&g)[D], uint32_t v) const {
     return ((uint64_t)(g[0] + hk(0, v)) << 32) | (D > 1 ? g[1 % D] + hk(1 % D, v) : 0u);
   }
-  __device__ __forceinline__ bool dead_now(uint32_t id) const { return A.ldead[id] < cyc; }
 
   // ---------------- initialisation (Algorithm 1) ----------------
   // Empty frontiers, candidate sets and histograms (the empty sets Algorithm
   // 1 starts from). The team must pass a barrier before init_seed.
-  // Whole arrays in turn, 16 bytes a thread: a batch starts a query on one or
-  // two blocks, and every other query of the iteration waits for them. (A thread
+  // Whole arrays in turn, 16 bytes a thread: a batch starts a query on one block,
+  // and every other query of the iteration waits for it. (A thread
   // that set its node's words in every array wrote 32 sectors an instruction;
   // 400 queries on 128x128 nodes took 41.3 ms instead of 35.0.) Stores that are
   // the first to leave the L2, for most nodes are not reached soon: with plain
