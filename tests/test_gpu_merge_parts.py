@@ -30,7 +30,9 @@ def op():
 @pytest.mark.parametrize("parts", [1, 2, 4, 8, 16, 32, 64, 128])
 @pytest.mark.parametrize("d,nf,nc,slots,lists", [
     (3, 0, 20, 32, 32), (2, 5, 32, 32, 1), (3, 300, 7, 128, 32), (5, 4000, 30, 128, 8), (4, 200, 33, 32, 32),
-    (8, 90, 64, 128, 32), (3, 3000, 1000, 128, 32), (12, 60, 500, 64, 8), (16, 700, 100, 45, 8), (1, 1, 40, 60, 8)])
+    (8, 90, 64, 128, 32), (3, 3000, 1000, 128, 32), (12, 60, 500, 64, 8), (16, 700, 100, 45, 8), (1, 1, 40, 60, 8),
+    # removed entries: frontiers of one round of the compaction, one more, many; one candidate alone
+    (3, 256, 40, 128, 32), (3, 257, 40, 128, 32), (4, 255, 9, 128, 32), (3, 3000, 1, 128, 32), (5, 2500, 3, 60, 8)])
 def test_any_number_of_parts(op, parts, d, nf, nc, slots, lists):
     rng = np.random.default_rng(parts + 1000 * nf + nc + d)
     hi = 40 if nf < 400 else 400
