@@ -521,16 +521,26 @@ struct Search {
     // objectives (the index tiles cover three), most of it with many. At the
     // goal node n there is P alone.
     if (alive && ((pos + 1u) & pos) == 0u) {
-      const unsigned want = parts_for(pos + 1u, 128u + pos + (v2 == G.n ? psnap >> kPGoal : fc + (psnap >> kPNode)));
+      const unsigned want = parts_for(pos + 1u, 128u + pos + (v2 == G.n ? psnap >> kPGoal : fc + (psnap >> kPNode)),
+                                      v2 == G.n ? 0u : fc);
       if (want > 1u) split_merge(cs, K1, v2, want);
     }
   }
 
   // Parts a merge of nc candidates of F comparisons each is split into: a power
-  // of two, each part about P.part_work << pscale comparisons or fewer.
+  // of two, each part about P.part_work << pscale comparisons or fewer. scan: the
+  // frontier entries the candidates meet. However few they are, one warp takes a
+  // round of loads for 32 kU entries, 0.5 us, so an entry beyond the first four
+  // rounds counts as kScanCands comparisons by itself. (One candidate against 4,000
+  // entries took 20 us, and every step of the 256x256 grid, d = 3, had one: W =
+  // 1,024 1,111 ms instead of 1,299, W = 256 3,410 instead of 3,980. Counted from
+  // the first entry on, graphs of small frontiers split merges for nothing: 110x110,
+  // d = 5, W = 256 51.5 ms instead of 46.9.)
+  static constexpr unsigned kScanCands = 7, kScanFree = 128 * kU;
   static constexpr unsigned kPNode = D <= 4 ? 5 : (D <= 6 ? 3 : (D <= 8 ? 2 : 0)), kPGoal = D <= 4 ? 2 : (D <= 6 ? 1 : 0);
-  __device__ unsigned parts_for(unsigned nc, unsigned F) const {
-    const unsigned long long w = (unsigned long long)nc * F;
+  __device__ unsigned parts_for(unsigned nc, unsigned F, unsigned scan) const {
+    unsigned long long w = (unsigned long long)nc * F;
+    if (scan > kScanFree) w += kScanCands * (scan - kScanFree);
     unsigned k = 1;
     while (k < A.kparts && w > ((unsigned long long)P.part_work << pscale) * k) k <<= 1;
     return k;
@@ -1494,7 +1504,8 @@ struct Search {
   // independent: ka shares of the candidates (groups a, a + ka, ... of 32, or
   // 16, 8 or 4 lanes of one group while there are more parts than groups)
   // times kb ranges of all three. Shares of the candidates come first, as a
-  // candidate's early exit stays within one part then. Frontier entries a
+  // candidate's early exit stays within one part then, while they hold about
+  // kShareCands candidates. Frontier entries a
   // candidate strictly dominates are marked pruned (ldead = cyc); candidates
   // that die get cflag set. Dominance is transitive and the frontier is an
   // antichain, so it does not matter that a part does not see the deaths of the
@@ -1504,6 +1515,7 @@ struct Search {
   // One warp a part, not a block: a block merge of the same work was 40 us of
   // block barriers and round trips between them for 3 us of comparisons, while
   // warps wait for nobody and many share an SM.
+  static constexpr unsigned kShareCands = 4;
   __device__ void merge_part(uint32_t v, unsigned r, unsigned k, CycleCtl& K1) {
     const CandSet& cs = A.cs[cyc & 1u];
     const unsigned lane = lane_id();
@@ -1518,7 +1530,7 @@ struct Search {
     unsigned ka = k, sub = 1;  // sub: shares of a group of 32
     while (ka > 1u && ka / 2 >= ng) {
       ka >>= 1;
-      if (sub < kPartShares) sub <<= 1;
+      if (sub < kPartShares && sub * kShareCands < nc) sub <<= 1;
     }
     const unsigned ks = ka * sub, kb = k / ks;
     const unsigned a = (r % ks) / sub, bb = r / ks;
