@@ -71,8 +71,8 @@ CPU_SAMPLE_LABELS = 1_500_000
 # among them) they were taken with: a launch whose digest has no entry (the
 # sources changed, or another window was chosen) reports null.
 TRAFFIC = {
-    "7368f652d975998e": 6032931840 + 4144625152,  # W = 262144
-    "903b9a5f7ee557e5": 2759832064 + 2360845056,  # W = 65536
+    "edf1f5962d020bf8": 3300093440 + 2056360960,  # W = 262144
+    "78269fa65b4900c0": 1128617216 + 1117462784,  # W = 65536
 }
 
 
