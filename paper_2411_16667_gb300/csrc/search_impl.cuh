@@ -1449,6 +1449,12 @@ struct Search {
       Batch b = load_batch(cs, mine);
       Round t = load_round(0u, v == G.n ? 0u : fc, fb, cap, true);
       resolve_batch(b);
+      // Where parts have grown, merges of several groups are left to one warp, and a
+      // label that a later group's candidate prunes again has cost its place in the
+      // arena: the later groups are looked at first (256x256 grid, d = 3, W = 262,144,
+      // 58.2 -> 56.5 M labels, same time). For single queries with large windows only,
+      // whose arenas fill; elsewhere it made searches 1% longer.
+      if (kMany && pscale && ng <= 16u && g + 1u < ng) test_groups(cs, v, nc, b, g + 1u, ng);
       if (v == G.n) {
         batch_ptest(hv, b, __shfl_sync(0xffffffffu, ld_volatile(&C->plog_len.v), 0), 0u, 1u, pcmp);
       } else {
