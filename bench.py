@@ -71,8 +71,8 @@ CPU_SAMPLE_LABELS = 1_500_000
 # among them) they were taken with: a launch whose digest has no entry (the
 # sources changed, or another window was chosen) reports null.
 TRAFFIC = {
-    "edf1f5962d020bf8": 3300093440 + 2056360960,  # W = 262144
-    "78269fa65b4900c0": 1128617216 + 1117462784,  # W = 65536
+    "f87b21b896569de9": 3271756800 + 2037555968,  # W = 262144
+    "77e352a3fd7c992b": 1119077376 + 1114801664,  # W = 65536
 }
 
 
